@@ -10,25 +10,25 @@
 #include <string.h>
 
 #include <algorithm>
-#include <map>
 
 #include "kvp_internal.h"
 
 namespace {
 
 constexpr uint64_t kAlign = 1024;
+constexpr uint64_t kPlanAlign = 64;    // arrays of a plan blob
 inline uint64_t round_up(uint64_t x, uint64_t a) { return (x + a - 1) / a * a; }
 
 struct ws_layout {
-    uint64_t status, inv_freq, slots, slot_stride, slot_plan, slot_sched, slot_k, slot_v, partial_o, partial_ml, q_scratch, total;
+    uint64_t status, half_turns, slots, slot_stride, slot_plan, slot_sched, slot_k, slot_v, partial_o, partial_ml, q_scratch, total;
     uint64_t rows_bytes;
 };
 
 constexpr int kMaxCtas = 256;          // upper bound on persistent CTAs (one per SM)
 
-// Work list of the two-stream attention kernel: [cta_begin: kMaxCtas + 1 ints][works][merge items].
+// Work list of the two-stream attention kernel: [cta_begin][works][merge items], packed.
 struct sched_layout {
-    uint64_t works, merges, total;
+    uint64_t total;
     int32_t max_works, max_merges;
 };
 
@@ -40,9 +40,8 @@ sched_layout schedule_layout(const kvp_config *c)
     const int64_t units = (int64_t)c->max_batch * c->n_kv_heads * tiles_q;
     s.max_works = (int32_t)std::min<int64_t>(units + kMaxCtas, 1 << 24);
     s.max_merges = 2 * kMaxCtas + 8 + (int32_t)std::min<int64_t>(units, KVP_MAX_SPLIT_UNITS);   // every unit has one with KVP_PARTIAL
-    s.works = round_up(4 * (kMaxCtas + 1), 256);
-    s.merges = round_up(s.works + sizeof(kvp_work) * (uint64_t)s.max_works, 256);
-    s.total = round_up(s.merges + sizeof(kvp_merge_item) * (uint64_t)s.max_merges, 256);
+    s.total = round_up(4 * (kMaxCtas + 1) + sizeof(kvp_work) * (uint64_t)s.max_works +
+                           sizeof(kvp_merge_item) * (uint64_t)s.max_merges + 2 * kPlanAlign, 256);
     return s;
 }
 
@@ -73,14 +72,26 @@ kvp_plan_layout plan_layout(const kvp_config *c)
     p.max_tiles = (int32_t)((c->max_batch * ((int64_t)c->max_prefix_tokens / KVP_TILE_KEYS + 2) + c->max_slots +
                              c->max_ws_rows / KVP_TILE_KEYS + 8) * lists);
     p.max_chunks = c->max_ws_rows / KVP_CHUNK_ROWS + p.max_segs + 8;
+    p.upload = sizeof(kvp_item) * (uint64_t)p.max_items + sizeof(kvp_tile) * (uint64_t)p.max_tiles +
+               sizeof(kvp_chunk) * (uint64_t)p.max_chunks + sizeof(kvp_seg) * (uint64_t)p.max_segs + 4ull * p.max_rope +
+               4ull * c->max_compressed * c->n_layers * c->n_kv_heads + 6 * kPlanAlign;
+    p.total = round_up(p.upload, 256) + sizeof(float2) * (uint64_t)p.max_rope * (c->head_dim / 2);
+    return p;
+}
+
+// The arrays of one assembly packed back to back, so that an upload moves what is used and not the capacities.
+kvp_plan_offsets plan_offsets(const kvp_assembly_host &as, size_t n_kept, int planes)
+{
+    kvp_plan_offsets p;
     uint64_t o = 0;
-    p.items = o;  o = round_up(o + sizeof(kvp_item) * p.max_items, 256);
-    p.tiles = o;  o = round_up(o + sizeof(kvp_tile) * (uint64_t)p.max_tiles, 256);
-    p.chunks = o; o = round_up(o + sizeof(kvp_chunk) * p.max_chunks, 256);
-    p.segs = o;   o = round_up(o + sizeof(kvp_seg) * p.max_segs, 256);
-    p.rope = o;   o = round_up(o + sizeof(float2) * (uint64_t)p.max_rope * (c->head_dim / 2), 256);
-    p.kept = o;   o = round_up(o + 4ull * c->max_compressed * c->n_layers * c->n_kv_heads, 256);
-    p.total = o;
+    p.items = o;  o = round_up(o + sizeof(kvp_item) * as.items.size(), kPlanAlign);
+    p.tiles = o;  o = round_up(o + sizeof(kvp_tile) * as.tiles.size(), kPlanAlign);
+    p.chunks = o; o = round_up(o + sizeof(kvp_chunk) * as.chunks.size(), kPlanAlign);
+    p.segs = o;   o = round_up(o + sizeof(kvp_seg) * as.segs.size(), kPlanAlign);
+    p.kept = o;   o = round_up(o + 4 * n_kept * planes, kPlanAlign);
+    p.delta = o;  o += 4 * as.delta.size();
+    p.upload = o;
+    p.rope = round_up(o, 256);
     return p;
 }
 
@@ -91,7 +102,7 @@ ws_layout workspace_layout(const kvp_config *c)
     const kvp_plan_layout p = plan_layout(c);
     uint64_t o = 0;
     w.status = o;   o += 256;
-    w.inv_freq = o; o = round_up(o + 8 * 64, kAlign);
+    w.half_turns = o; o = round_up(o + 8 * 64, kAlign);
     w.rows_bytes = round_up((uint64_t)c->n_layers * c->n_kv_heads * c->max_ws_rows * c->head_dim * e, kAlign);
     w.slot_plan = 0;
     w.slot_sched = round_up(p.total, kAlign);
@@ -180,12 +191,14 @@ kvp_plan_dev plan_dev(const kvp_ctx *ctx, int slot)
 {
     char *base = ctx->slot_plan_dev[slot];
     kvp_plan_dev p;
-    p.items = reinterpret_cast<const kvp_item *>(base + ctx->pl.items);
-    p.tiles = reinterpret_cast<const kvp_tile *>(base + ctx->pl.tiles);
-    p.chunks = reinterpret_cast<const kvp_chunk *>(base + ctx->pl.chunks);
-    p.segs = reinterpret_cast<const kvp_seg *>(base + ctx->pl.segs);
-    p.rope = reinterpret_cast<const float2 *>(base + ctx->pl.rope);
-    p.kept = reinterpret_cast<const int32_t *>(base + ctx->pl.kept);
+    const kvp_plan_offsets &off = ctx->slots[slot].off;
+    p.items = reinterpret_cast<const kvp_item *>(base + off.items);
+    p.tiles = reinterpret_cast<const kvp_tile *>(base + off.tiles);
+    p.chunks = reinterpret_cast<const kvp_chunk *>(base + off.chunks);
+    p.segs = reinterpret_cast<const kvp_seg *>(base + off.segs);
+    p.rope = reinterpret_cast<const float2 *>(base + off.rope);
+    p.delta = reinterpret_cast<const int32_t *>(base + off.delta);
+    p.kept = reinterpret_cast<const int32_t *>(base + off.kept);
     p.item_stride = ctx->slots[slot].item_stride;
     p.n_planes = ctx->shape.n_layers * ctx->shape.n_kv_heads;
     return p;
@@ -208,24 +221,19 @@ int find_slot(kvp_ctx *ctx, int32_t assembly_id)
 // fewer tiles.  Counted in single-stream tiles.
 constexpr int kPieceCost = 4;
 
-struct schedule_t {
-    std::vector<int32_t> cta_begin;
-    std::vector<kvp_work> works;
-    std::vector<kvp_merge_item> merges;
-    int32_t n_ctas = 0, n_slots = 0, max_pieces = 1;
-};
-
 // q_lens: nullptr, or one query length per request (<= q_len, the stride of the padded tensors); a request's
 // work records and merge items then carry its own length.
 // opts: KVP_PARTIAL - every unit writes partial slots and gets merge items (even with one piece or none);
 // KVP_SKIP_QUERY_BLOCK - a unit's range starts behind the causal tiles of the query's own keys.
 int32_t plan_schedule(kvp_ctx *ctx, const kvp_assembly_host &as, int layer, int q_len, int q_pos0, const int32_t *q_lens,
-                      uint32_t opts, schedule_t &out)
+                      uint32_t opts, kvp_schedule &out)
 {
     const kvp_shape &sh = ctx->shape;
     const bool force_partial = (opts & KVP_PARTIAL) != 0, skip_tail = (opts & KVP_SKIP_QUERY_BLOCK) != 0;
-    struct unit_t { int32_t b, hk, row_base, mode, n_all, first_piece, n_pieces, q_len, t_first, tile_begin, tail_row0, n_tail; };
-    std::vector<unit_t> units;
+    typedef kvp_schedule::unit unit_t;
+    typedef kvp_schedule::cut cut_t;
+    std::vector<unit_t> &units = out.units;
+    units.clear();
     const int max_rows = sh.group * q_len;
     int64_t total = 0;
     // Row blocks outermost: the units of one (request, kv head) - which stream the same K/V - then lie a
@@ -249,7 +257,8 @@ int32_t plan_schedule(kvp_ctx *ctx, const kvp_assembly_host &as, int layer, int 
                 u.n_tail = n_tail;
                 u.tile_begin = item.tile_begin;
                 u.tail_row0 = item.tail_row0;
-                u.first_piece = u.n_pieces = 0;
+                u.n_pieces = 0;
+                u.slot = -1;
                 units.push_back(u);
                 total += (int64_t)(u.n_all - u.t_first) * (u.mode ? 1 : 2) + kPieceCost;
             }
@@ -263,11 +272,13 @@ int32_t plan_schedule(kvp_ctx *ctx, const kvp_assembly_host &as, int layer, int 
     // not less than a minimum that keeps tiny launches on few CTAs); every piece pays kPieceCost on top of its
     // tiles, a piece is at least two tiles long (or the whole unit), and without splitting a unit goes to the CTA
     // that holds its larger part.  The last CTA of the run takes all that is left, so g CTAs always suffice.
-    struct cut_t { int32_t u, t; };
-    std::vector<cut_t> cuts;
+    std::vector<cut_t> &cuts = out.cuts;
+    cuts.clear();
     const int64_t min_budget = 8 + kPieceCost;
     auto fill = [&](size_t u_begin, size_t u_end, int g, std::vector<cut_t> *rec) -> int {
-        std::vector<int64_t> after(u_end - u_begin + 1, 0);           // weight of the units behind unit u
+        std::vector<int64_t> &after = out.after;                      // weight of the units behind unit u
+        after.resize(u_end - u_begin + 1);
+        after[u_end - u_begin] = 0;
         for (size_t u = u_end; u > u_begin; --u) {
             const unit_t &x = units[u - 1];
             const int64_t wgt = x.n_all == x.t_first ? 0 : (int64_t)(x.n_all - x.t_first) * (x.mode ? 1 : 2) + kPieceCost;
@@ -367,7 +378,8 @@ int32_t plan_schedule(kvp_ctx *ctx, const kvp_assembly_host &as, int layer, int 
     }
     if (aligned) {
         const int rm = n_rb - 1;                                  // the row block with the most causal tiles
-        std::vector<cut_t> model;
+        std::vector<cut_t> &model = out.model;
+        model.clear();
         fill(rb_begin[rm], rb_begin[rm + 1], G / n_rb, &model);
         for (int r = 0; r < n_rb; ++r) {
             const size_t before = cuts.size();
@@ -392,76 +404,64 @@ int32_t plan_schedule(kvp_ctx *ctx, const kvp_assembly_host &as, int layer, int 
     }
     cuts.push_back({(int32_t)units.size(), 0});
 
+    // emission order: the j-th CTAs of all row blocks next to each other
+    std::vector<int32_t> &order = out.order;
+    order.clear();
+    const int n_cuts = (int)cuts.size() - 1;
+    if (per_block) {
+        int most = 0;
+        for (int r = 0; r < n_rb; ++r) most = std::max(most, rb_used[r]);
+        for (int j = 0; j < most; ++j)
+            for (int r = 0, off = 0; r < n_rb; off += rb_used[r], ++r)
+                if (j < rb_used[r]) order.push_back(off + j);
+    } else {
+        for (int c = 0; c < n_cuts; ++c) order.push_back(c);
+    }
     std::vector<kvp_work> &works = out.works;
     std::vector<int32_t> &cta_begin = out.cta_begin;
-    struct cta_rec { std::vector<kvp_work> ws; std::vector<int32_t> unit; };
-    std::vector<cta_rec> recs;
-    for (size_t c = 0; c + 1 < cuts.size(); ++c) {
-        const cut_t a = cuts[c], z = cuts[c + 1];
-        cta_rec rec;
+    works.clear();
+    cta_begin.clear();
+    out.work_unit.clear();
+    for (int32_t idx : order) {
+        const cut_t a = cuts[idx], z = cuts[idx + 1];
+        const size_t first = works.size();
         for (int32_t u = a.u; u <= z.u && u < (int32_t)units.size(); ++u) {
-            const int32_t lo = (u == a.u) ? a.t : units[u].t_first;
-            const int32_t hi = (u == z.u) ? z.t : units[u].n_all;
+            unit_t &x = units[u];
+            const int32_t lo = (u == a.u) ? a.t : x.t_first;
+            const int32_t hi = (u == z.u) ? z.t : x.n_all;
             if (hi <= lo) continue;
-            kvp_work w;
-            w.b = units[u].b; w.hk = units[u].hk; w.row_base = units[u].row_base;
-            w.mode = units[u].mode | (units[u].q_len << 8);       // a request's own query length rides in the upper bits
-            w.tile_lo = lo; w.n_tiles = hi - lo; w.slot0 = w.slot1 = -1;
-            w.tile_begin = units[u].tile_begin; w.tail_row0 = units[u].tail_row0; w.pad[0] = w.pad[1] = 0;
-            rec.ws.push_back(w);
-            rec.unit.push_back(u);
+            // (a request's own query length rides in the upper bits of the mode)
+            works.push_back({x.b, x.hk, x.row_base, x.mode | (x.q_len << 8), lo, hi - lo, -1, -1, x.tile_begin, x.tail_row0, {0, 0}});
+            out.work_unit.push_back(u);
+            ++x.n_pieces;
         }
-        recs.push_back(rec);
+        if (works.size() > first) cta_begin.push_back((int32_t)first);
     }
-    // emission order: the j-th CTAs of all row blocks next to each other
-    std::vector<int> order;
-    if (per_block) {
-        std::vector<int> off(n_rb + 1, 0);
-        for (int r = 0; r < n_rb; ++r) off[r + 1] = off[r] + rb_used[r];
-        for (int j = 0; (int)order.size() < off[n_rb]; ++j)
-            for (int r = 0; r < n_rb; ++r)
-                if (j < rb_used[r]) order.push_back(off[r] + j);
-    } else {
-        for (size_t c = 0; c < recs.size(); ++c) order.push_back((int)c);
-    }
-    std::vector<std::vector<int32_t>> unit_pieces(units.size());
-    for (int idx : order) {
-        const cta_rec &rec = recs[idx];
-        if (rec.ws.empty()) continue;
-        cta_begin.push_back((int32_t)works.size());
-        for (size_t i = 0; i < rec.ws.size(); ++i) {
-            unit_pieces[rec.unit[i]].push_back((int32_t)works.size());
-            works.push_back(rec.ws[i]);
-        }
-    }
-    for (size_t u = 0; u < units.size(); ++u) units[u].n_pieces = (int32_t)unit_pieces[u].size();
     const int n_ctas = (int)cta_begin.size();
     cta_begin.push_back((int32_t)works.size());
 
     std::vector<kvp_merge_item> &merges = out.merges;
+    merges.clear();
     int32_t n_slots = 0, max_pieces = 1;
-    for (size_t ui = 0; ui < units.size(); ++ui) {
-        const unit_t &u = units[ui];
+    for (unit_t &u : units) {
         if (u.n_pieces <= 1 && !force_partial) continue;
         max_pieces = std::max(max_pieces, u.n_pieces);
-        const int32_t base = n_slots;
-        for (int i = 0; i < u.n_pieces; ++i) {
-            kvp_work &w = works[unit_pieces[ui][i]];
-            w.slot0 = base + i;
-            if (u.mode == 0) w.slot1 = base + u.n_pieces + i;
-        }
-        kvp_merge_item m;
-        memset(&m, 0, sizeof m);
-        m.b = u.b; m.hk = u.hk; m.row_base = u.row_base; m.slot0 = base; m.n_slots = u.n_pieces;
-        m.pad[0] = u.q_len;
+        u.slot = n_slots;
+        kvp_merge_item m = {u.b, u.hk, u.row_base, u.slot, u.n_pieces, {u.q_len, 0, 0}};
         merges.push_back(m);
         n_slots += u.n_pieces;
         if (u.mode == 0) {
             m.row_base = u.row_base + KVP_TILE_ROWS;
-            m.slot0 = base + u.n_pieces;
+            m.slot0 = n_slots;
             merges.push_back(m);
             n_slots += u.n_pieces;
         }
+    }
+    for (size_t i = 0; i < works.size(); ++i) {                    // the pieces of a unit take its slots in emission order
+        unit_t &u = units[out.work_unit[i]];
+        if (u.slot < 0) continue;
+        works[i].slot0 = u.slot++;
+        if (u.mode == 0) works[i].slot1 = works[i].slot0 + u.n_pieces;
     }
     if (n_ctas > kMaxCtas || (int)works.size() > ctx->sched_max_works || (int)merges.size() > ctx->sched_max_merges ||
         n_slots > KVP_MAX_SPLIT_UNITS)
@@ -477,38 +477,47 @@ int32_t plan_schedule(kvp_ctx *ctx, const kvp_assembly_host &as, int layer, int 
 int32_t build_schedule(kvp_ctx *ctx, kvp_assembly_host &as, int slot, int layer, int q_len, int q_pos0, const int32_t *q_lens,
                        uint32_t opts, cudaStream_t st)
 {
-    schedule_t sc;
+    kvp_schedule &sc = ctx->plan;
     const int32_t rc = plan_schedule(ctx, as, layer, q_len, q_pos0, q_lens, opts, sc);
     if (rc != KVP_OK) return rc;
-    const std::vector<int32_t> &cta_begin = sc.cta_begin;
-    const std::vector<kvp_work> &works = sc.works;
-    const std::vector<kvp_merge_item> &merges = sc.merges;
-    const int n_ctas = sc.n_ctas;
-    const int32_t max_pieces = sc.max_pieces;
-    KVP_CUDA(ctx, cudaEventSynchronize(ctx->sched_event[slot]));          // staging buffer free again?
-    char *h = ctx->slot_sched_host[slot];
-    memcpy(h, cta_begin.data(), 4 * cta_begin.size());
-    memcpy(h + ctx->sched_off_works, works.data(), sizeof(kvp_work) * works.size());
-    memcpy(h + ctx->sched_off_merges, merges.data(), sizeof(kvp_merge_item) * merges.size());
+    const uint32_t off_works = (uint32_t)round_up(4 * sc.cta_begin.size(), kPlanAlign);
+    const uint32_t off_merges = (uint32_t)round_up(off_works + sizeof(kvp_work) * sc.works.size(), kPlanAlign);
+    const size_t used = off_merges + sizeof(kvp_merge_item) * sc.merges.size();
+    const int ring = ctx->sched_next;
+    ctx->sched_next = (ring + 1) % KVP_SCHED_RING;
+    KVP_CUDA(ctx, cudaEventSynchronize(ctx->sched_event[ring]));          // staging buffer free again?
+    char *h = ctx->sched_ring[ring];
+    memcpy(h, sc.cta_begin.data(), 4 * sc.cta_begin.size());
+    memcpy(h + off_works, sc.works.data(), sizeof(kvp_work) * sc.works.size());
+    memcpy(h + off_merges, sc.merges.data(), sizeof(kvp_merge_item) * sc.merges.size());
     const int li = as.item_stride ? layer : 0;                   // which of the assembly's work lists
-    char *d = ctx->slot_sched_dev[slot] + ctx->sched_bytes * li;
-    KVP_CUDA(ctx, cudaMemcpyAsync(d, h, 4 * cta_begin.size(), cudaMemcpyHostToDevice, st));
-    KVP_CUDA(ctx, cudaMemcpyAsync(d + ctx->sched_off_works, h + ctx->sched_off_works, sizeof(kvp_work) * works.size(),
-                                  cudaMemcpyHostToDevice, st));
-    if (!merges.empty())
-        KVP_CUDA(ctx, cudaMemcpyAsync(d + ctx->sched_off_merges, h + ctx->sched_off_merges,
-                                      sizeof(kvp_merge_item) * merges.size(), cudaMemcpyHostToDevice, st));
-    KVP_CUDA(ctx, cudaEventRecord(ctx->sched_event[slot], st));
+    KVP_CUDA(ctx, cudaMemcpyAsync(ctx->slot_sched_dev[slot] + ctx->sched_bytes * li, h, used, cudaMemcpyHostToDevice, st));
+    KVP_CUDA(ctx, cudaEventRecord(ctx->sched_event[ring], st));
     kvp_assembly_host::sched_state &ss = as.sched[li];
     ss.q_len = q_len;
     ss.q_lens.assign(q_lens ? q_lens : nullptr, q_lens ? q_lens + as.batch : nullptr);
     ss.q_pos0 = q_pos0;
     ss.opts = opts;
-    ss.ctas = n_ctas;
-    ss.works = (int32_t)works.size();
-    ss.merges = (int32_t)merges.size();
-    ss.slots = max_pieces;
+    ss.ctas = sc.n_ctas;
+    ss.works = (int32_t)sc.works.size();
+    ss.merges = (int32_t)sc.merges.size();
+    ss.slots = sc.max_pieces;
+    ss.off_works = off_works;
+    ss.off_merges = off_merges;
     return KVP_OK;
+}
+
+// Whether the work list built for q_len tokens behind `from` appended rows also serves `to`: the list holds causal
+// tile counts, not positions, so it stays the same until a unit's last token enters another 128-key tile (a decode
+// step changes it once in 128 steps).
+bool same_causal_tiles(const kvp_shape &sh, int q_len, int from, int to)
+{
+    const int n_rows = sh.group * q_len;
+    for (int row_base = 0; row_base < n_rows; row_base += 2 * KVP_TILE_ROWS) {
+        const int last = std::min(n_rows - 1, row_base + 2 * KVP_TILE_ROWS - 1) / sh.group;
+        if ((from + last) / KVP_TILE_KEYS != (to + last) / KVP_TILE_KEYS) return false;
+    }
+    return true;
 }
 
 thread_local std::string g_create_error;
@@ -561,8 +570,6 @@ int32_t kvp_create(const kvp_config *cfg, kvp_ctx **out)
     ctx->pl = plan_layout(cfg);
     {
         const sched_layout sl = schedule_layout(cfg);
-        ctx->sched_off_works = sl.works;
-        ctx->sched_off_merges = sl.merges;
         ctx->sched_bytes = sl.total;
         ctx->sched_max_works = sl.max_works;
         ctx->sched_max_merges = sl.max_merges;
@@ -606,28 +613,32 @@ int32_t kvp_create(const kvp_config *cfg, kvp_ctx **out)
     ctx->partial_ml = (float2 *)(ws + w.partial_ml);
     ctx->q_scratch = ws + w.q_scratch;
 
+    // angles are formed on the device as (position offset) x (theta_i / pi), in half turns: sincospi reduces exactly
+    std::vector<double> half_turns;
+    for (double f : ctx->inv_freq) half_turns.push_back((double)((long double)f / acosl(-1.0L)));
+    ctx->half_turns = reinterpret_cast<const double *>(ws + w.half_turns);
     if (cudaMemset(cfg->pool, 0, 2 * plane_bytes) != cudaSuccess ||
         cudaMemset(cfg->workspace, 0, w.total) != cudaSuccess ||
-        cudaMemcpy(ws + w.inv_freq, ctx->inv_freq.data(), 8 * ctx->inv_freq.size(), cudaMemcpyHostToDevice) !=
-            cudaSuccess ||
+        cudaMemcpy(ws + w.half_turns, half_turns.data(), 8 * half_turns.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaDeviceSynchronize() != cudaSuccess)
         return bail(KVP_ERR_CUDA, "clearing pool/workspace failed");
 
+    // one pinned block for all staging buffers: a cudaHostAlloc takes a millisecond or two
+    const uint64_t plan_stage = round_up(ctx->pl.upload, 256);
+    if (cudaHostAlloc((void **)&ctx->staging, plan_stage * cfg->max_assemblies + ctx->sched_bytes * KVP_SCHED_RING,
+                      cudaHostAllocDefault) != cudaSuccess)
+        return bail(KVP_ERR_CUDA, "pinned staging allocation failed");
     for (int a = 0; a < cfg->max_assemblies; ++a) {
-        char *h = nullptr;
         cudaEvent_t ev;
-        if (cudaHostAlloc((void **)&h, ctx->pl.total, cudaHostAllocDefault) != cudaSuccess ||
-            cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess)
-            return bail(KVP_ERR_CUDA, "pinned staging allocation failed");
-        ctx->slot_plan_host.push_back(h);
+        if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess)
+            return bail(KVP_ERR_CUDA, "staging event creation failed");
+        ctx->slot_plan_host.push_back(ctx->staging + plan_stage * a);
         ctx->slot_event.push_back(ev);
-        char *hs = nullptr;
-        cudaEvent_t evs;
-        if (cudaHostAlloc((void **)&hs, ctx->sched_bytes, cudaHostAllocDefault) != cudaSuccess ||
-            cudaEventCreateWithFlags(&evs, cudaEventDisableTiming) != cudaSuccess)
-            return bail(KVP_ERR_CUDA, "pinned staging allocation failed");
-        ctx->slot_sched_host.push_back(hs);
-        ctx->sched_event.push_back(evs);
+    }
+    for (int r = 0; r < KVP_SCHED_RING; ++r) {
+        ctx->sched_ring[r] = ctx->staging + plan_stage * cfg->max_assemblies + ctx->sched_bytes * r;
+        if (cudaEventCreateWithFlags(&ctx->sched_event[r], cudaEventDisableTiming) != cudaSuccess)
+            return bail(KVP_ERR_CUDA, "staging event creation failed");
     }
 
     if (cudaStreamCreateWithFlags(&ctx->load_stream, cudaStreamNonBlocking) != cudaSuccess ||
@@ -668,10 +679,9 @@ int32_t kvp_destroy(kvp_ctx *ctx)
     if (!ctx->host_only) {
         cudaSetDevice(ctx->cfg.device);
         cudaDeviceSynchronize();
-        for (char *h : ctx->slot_plan_host) cudaFreeHost(h);
+        if (ctx->staging) cudaFreeHost(ctx->staging);
         for (cudaEvent_t e : ctx->slot_event) cudaEventDestroy(e);
-        for (char *h : ctx->slot_sched_host) cudaFreeHost(h);
-        for (cudaEvent_t e : ctx->sched_event) cudaEventDestroy(e);
+        for (cudaEvent_t e : ctx->sched_event) if (e) cudaEventDestroy(e);
         for (auto &w : ctx->tev) for (auto &v : w) for (cudaEvent_t e : v) cudaEventDestroy(e);
         for (cudaEvent_t e : ctx->load_done) cudaEventDestroy(e);
         if (ctx->load_fence) cudaEventDestroy(ctx->load_fence);
@@ -849,9 +859,17 @@ static int32_t assemble_impl(kvp_ctx *ctx, int32_t batch, const int32_t *slot_of
             return fail(ctx, KVP_ERR_NOT_FOUND, "assemble: unknown adapter id %d", adapter_ids[s]);
     }
     const bool rebase = flags & KVP_REBASE, mat = flags & KVP_MATERIALIZE;
-    const int half = cfg.head_dim / 2;
 
-    kvp_assembly_host as;
+    kvp_assembly_host &as = ctx->build;      // built here, swapped into its slot at the end
+    as.items.clear();
+    as.segs.clear();
+    as.tiles.clear();
+    as.chunks.clear();
+    as.delta.assign(1, 0);
+    as.appended.clear();
+    as.sched.clear();
+    as.ragged = false;
+    as.last_q_len = 0;
     as.flags = flags;
     as.batch = batch;
     as.shard = pos_base != nullptr;
@@ -869,22 +887,33 @@ static int32_t assemble_impl(kvp_ctx *ctx, int32_t batch, const int32_t *slot_of
     }
     as.waits_loads = host_origin && !ctx->host_only && (ctx->loads_recorded || !to_load.empty());
     const bool waits_loads = as.waits_loads;
-    std::map<int32_t, int32_t> rope_of;        // delta -> rope-table index (0 = identity)
-    std::vector<int32_t> rope_delta(1, 0);
-    rope_of[0] = 0;
-    std::vector<kvp_chunk> chunks;
+    // delta -> rope-table index (0 = identity): open addressing over a power of two, entries are indices + 1
+    size_t hash_size = 64;
+    while (hash_size < 8 * (size_t)n_slots) hash_size *= 2;
+    ctx->rope_hash.assign(hash_size, 0);
+    auto rope_of = [&](int32_t delta) -> int32_t {
+        if (delta == 0) return 0;
+        for (size_t i = (uint32_t)delta * 2654435769u >> 7;; ++i) {
+            int32_t &e = ctx->rope_hash[i & (hash_size - 1)];
+            if (e == 0) {
+                as.delta.push_back(delta);
+                e = (int32_t)as.delta.size();
+            }
+            if (as.delta[e - 1] == delta) return e - 1;
+        }
+    };
+    if (cfg.max_compressed > 0) ctx->kept_row_of.assign(ctx->packets.size(), -1);
     int64_t ws_cursor = 0;
 
     auto add_chunks = [&](int32_t src, int32_t dst, int32_t n, int32_t rope) {
         for (int32_t o = 0; o < n; o += KVP_CHUNK_ROWS)
-            chunks.push_back({src + o, dst + o, std::min<int32_t>(KVP_CHUNK_ROWS, n - o), rope});
+            as.chunks.push_back({src + o, dst + o, std::min<int32_t>(KVP_CHUNK_ROWS, n - o), rope});
     };
     auto add_tiles = [&](int16_t src, int32_t row0, int32_t n, int32_t rope) {
         for (int32_t o = 0; o < n; o += KVP_TILE_KEYS)
             as.tiles.push_back({row0 + o, (int16_t)std::min<int32_t>(KVP_TILE_KEYS, n - o), src, rope, 0});
     };
-    std::map<int32_t, int32_t> kept_row_of;    // compressed packet id -> row of the kept table
-    std::vector<int32_t> kept_packets;
+    std::vector<int32_t> kept_packets;         // compressed packets in use: row r of the kept table is packet kept_packets[r]
     struct item_build { kvp_item it; int32_t stage0, staged; };
     std::vector<item_build> builds;
 
@@ -909,22 +938,17 @@ static int32_t assemble_impl(kvp_ctx *ctx, int32_t batch, const int32_t *slot_of
                 e.len = sg->n;
                 e.dst_pos0 = (int32_t)t;
                 e.delta = rebase ? (int32_t)(t + (pos_base ? pos_base[b] : 0) - sg->pos0) : 0;
-                auto f = rope_of.find(e.delta);
-                if (f == rope_of.end()) {
-                    f = rope_of.emplace(e.delta, (int32_t)rope_delta.size()).first;
-                    rope_delta.push_back(e.delta);
-                }
-                e.rope = f->second;
+                e.rope = rope_of(e.delta);
                 e.pad[0] = -1;                   // workspace row of a staged copy, if any
                 e.pad[1] = k;                    // 0 header, 1 document, 2 trailer
                 e.pad[2] = -1;                   // row of the kept table (compressed document)
                 if (k == 1 && !sg->kept.empty()) {
-                    auto kr = kept_row_of.find(packet_ids[s]);
-                    if (kr == kept_row_of.end()) {
-                        kr = kept_row_of.emplace(packet_ids[s], (int32_t)kept_packets.size()).first;
+                    int32_t &row = ctx->kept_row_of[packet_ids[s]];
+                    if (row < 0) {
+                        row = (int32_t)kept_packets.size();
                         kept_packets.push_back(packet_ids[s]);
                     }
-                    e.pad[2] = kr->second;
+                    e.pad[2] = row;
                 }
                 if (!mat && k != 1) staged += sg->n;
                 as.segs.push_back(e);
@@ -992,12 +1016,12 @@ static int32_t assemble_impl(kvp_ctx *ctx, int32_t batch, const int32_t *slot_of
             }
             as.items.push_back(it);
         }
-    if ((int)as.tiles.size() > ctx->pl.max_tiles || (int)chunks.size() > ctx->pl.max_chunks ||
+    if ((int)as.tiles.size() > ctx->pl.max_tiles || (int)as.chunks.size() > ctx->pl.max_chunks ||
         (int)as.items.size() > ctx->pl.max_items ||
-        (int)rope_delta.size() > ctx->pl.max_rope || (int)as.segs.size() > ctx->pl.max_segs)
+        (int)as.delta.size() > ctx->pl.max_rope || (int)as.segs.size() > ctx->pl.max_segs)
         return fail(ctx, KVP_ERR_CAPACITY, "assemble: plan tables overflow");
-    as.n_chunks = (int32_t)chunks.size();
-    as.n_rope = (int32_t)rope_delta.size();
+    const int planes = cfg.n_layers * cfg.n_kv_heads;
+    as.off = plan_offsets(as, kept_packets.size(), planes);
 
     const int32_t id = ctx->next_assembly++;
     const int slot = id % cfg.max_assemblies;
@@ -1007,30 +1031,18 @@ static int32_t assemble_impl(kvp_ctx *ctx, int32_t batch, const int32_t *slot_of
         KVP_CUDA(ctx, cudaSetDevice(cfg.device));
         KVP_CUDA(ctx, cudaEventSynchronize(ctx->slot_event[slot]));      // staging buffer free again?
         char *h = ctx->slot_plan_host[slot];
-        memcpy(h + ctx->pl.items, as.items.data(), sizeof(kvp_item) * as.items.size());
-        memcpy(h + ctx->pl.tiles, as.tiles.data(), sizeof(kvp_tile) * as.tiles.size());
-        memcpy(h + ctx->pl.chunks, chunks.data(), sizeof(kvp_chunk) * chunks.size());
-        memcpy(h + ctx->pl.segs, as.segs.data(), sizeof(kvp_seg) * as.segs.size());
-        float2 *rt = reinterpret_cast<float2 *>(h + ctx->pl.rope);
-        for (size_t r = 0; r < rope_delta.size(); ++r)
-            for (int i = 0; i < half; ++i) {
-                const double a = (double)rope_delta[r] * ctx->inv_freq[i];      // angle in double: Delta reaches 1e5
-                rt[r * half + i] = make_float2((float)cos(a), (float)sin(a));
-            }
-        const uint64_t used = ctx->pl.rope + sizeof(float2) * rope_delta.size() * half;
-        KVP_CUDA(ctx, cudaMemcpyAsync(ctx->slot_plan_dev[slot], h, used, cudaMemcpyHostToDevice, st));
-        if (!kept_packets.empty()) {
-            const size_t planes = (size_t)cfg.n_layers * cfg.n_kv_heads;
-            int32_t *kt = reinterpret_cast<int32_t *>(h + ctx->pl.kept);
-            for (size_t r = 0; r < kept_packets.size(); ++r)
-                memcpy(kt + r * planes, ctx->packets[kept_packets[r]].kept.data(), 4 * planes);
-            KVP_CUDA(ctx, cudaMemcpyAsync(ctx->slot_plan_dev[slot] + ctx->pl.kept, kt, 4 * planes * kept_packets.size(),
-                                          cudaMemcpyHostToDevice, st));
-        }
+        memcpy(h + as.off.items, as.items.data(), sizeof(kvp_item) * as.items.size());
+        memcpy(h + as.off.tiles, as.tiles.data(), sizeof(kvp_tile) * as.tiles.size());
+        memcpy(h + as.off.chunks, as.chunks.data(), sizeof(kvp_chunk) * as.chunks.size());
+        memcpy(h + as.off.segs, as.segs.data(), sizeof(kvp_seg) * as.segs.size());
+        memcpy(h + as.off.delta, as.delta.data(), 4 * as.delta.size());
+        for (size_t r = 0; r < kept_packets.size(); ++r)
+            memcpy(h + as.off.kept + 4 * r * planes, ctx->packets[kept_packets[r]].kept.data(), 4 * (size_t)planes);
+        KVP_CUDA(ctx, cudaMemcpyAsync(ctx->slot_plan_dev[slot], h, as.off.upload, cudaMemcpyHostToDevice, st));
         KVP_CUDA(ctx, cudaEventRecord(ctx->slot_event[slot], st));
     }
-    const int32_t n_chunks = as.n_chunks;
-    ctx->slots[slot] = std::move(as);
+    const int32_t n_chunks = (int32_t)as.chunks.size(), n_rope = (int32_t)as.delta.size();
+    std::swap(ctx->slots[slot], ctx->build);
     *assembly_id = id;
     if (ctx->host_only) {
         for (int32_t id : to_load) ctx->packet_src[id].resident = true;
@@ -1043,8 +1055,8 @@ static int32_t assemble_impl(kvp_ctx *ctx, int32_t batch, const int32_t *slot_of
         if (mat && waits_loads)                                   // the gather reads every layer of the documents
             KVP_CUDA(ctx, cudaStreamWaitEvent(st, ctx->load_done[ctx->shape.n_layers - 1], 0));
         KVP_CUDA(ctx, time_edge(ctx, 1, 0, st));
-        KVP_CUDA(ctx, kvp_launch_gather(ctx->shape, plan_dev(ctx, slot), n_chunks, ctx->pool_k, ctx->pool_v,
-                                        ctx->slot_k[slot], ctx->slot_v[slot], st));
+        KVP_CUDA(ctx, kvp_launch_gather(ctx->shape, plan_dev(ctx, slot), n_chunks, n_rope, ctx->half_turns, ctx->pool_k,
+                                        ctx->pool_v, ctx->slot_k[slot], ctx->slot_v[slot], st));
         KVP_CUDA(ctx, time_edge(ctx, 1, 1, st));
     }
     return KVP_OK;
@@ -1152,7 +1164,6 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
     if (rope_query && as.shard)
         return fail(ctx, KVP_ERR_UNSUPPORTED, "query_prefill: KVP_ROPE_QUERY on an assembly made by kvp_assemble_at (the query's position is not prefix_len)");
     const bool skip_block = (flags & KVP_SKIP_QUERY_BLOCK) != 0;
-    const double *inv_freq_dev = reinterpret_cast<const double *>((char *)ctx->cfg.workspace + 256);
 
     int launches = 0;
     const bool fast = ctx->have_tma && !(flags & KVP_FORCE_SIMPLE);
@@ -1170,7 +1181,7 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
         return fail(ctx, KVP_ERR_UNSUPPORTED, "query_prefill_ragged: needs the tcgen05 kernel with its own append (bf16, head_dim 128, 16-byte aligned k_new / v_new)");
     if (!a.tail_direct && !skip_block) {
         KVP_CUDA(ctx, kvp_launch_append(sh, plan, as.batch, q_len, q_pos0, q, k_new, v_new, ctx->slot_k[slot], ctx->slot_v[slot],
-                                        layer, rope_query, inv_freq_dev, ctx->q_scratch, st));
+                                        layer, rope_query, ctx->half_turns, ctx->q_scratch, st));
         ++launches;
     }
     const void *q_used = rope_query ? (const void *)ctx->q_scratch : q;
@@ -1192,7 +1203,8 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
         const bool same_lens = q_lens ? (as.sched[li].q_lens.size() == (size_t)as.batch &&
                                           std::equal(q_lens, q_lens + as.batch, as.sched[li].q_lens.begin()))
                                        : as.sched[li].q_lens.empty();
-        if (as.sched[li].q_len != q_len || as.sched[li].q_pos0 != q_pos0 || as.sched[li].ctas == 0 || !same_lens ||
+        if (as.sched[li].q_len != q_len || as.sched[li].ctas == 0 || !same_lens ||
+            (as.sched[li].q_pos0 != q_pos0 && (q_lens || !same_causal_tiles(sh, q_len, as.sched[li].q_pos0, q_pos0))) ||
             as.sched[li].opts != part_opts) {
             const int32_t rc = build_schedule(ctx, as, slot, layer, q_len, q_pos0, q_lens, part_opts, st);
             if (rc != KVP_OK) return rc;
@@ -1210,7 +1222,7 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
         a.layer = layer;
         a.n_ctas = ss.ctas;
         a.cta_begin = reinterpret_cast<const int32_t *>(sd);
-        a.works = reinterpret_cast<const kvp_work *>(sd + ctx->sched_off_works);
+        a.works = reinterpret_cast<const kvp_work *>(sd + ss.off_works);
         a.q = q_used;
         a.out = out;
         a.lse = lse;
@@ -1227,7 +1239,7 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
             const bool partial = (flags & KVP_PARTIAL) != 0;
             const int64_t n_rt = ((int64_t)sh.group * q_len + KVP_TILE_ROWS - 1) / KVP_TILE_ROWS;
             KVP_CUDA(ctx, kvp_launch_merge_list(sh, q_len, ss.merges,
-                                                reinterpret_cast<const kvp_merge_item *>(sd + ctx->sched_off_merges),
+                                                reinterpret_cast<const kvp_merge_item *>(sd + ss.off_merges),
                                                 ctx->partial_o, ctx->partial_ml, out, lse, partial ? out : nullptr,
                                                 (int64_t)as.batch * sh.n_kv_heads * n_rt, st));
             ++launches;
@@ -1342,7 +1354,7 @@ int32_t kvp_export_schedule(kvp_ctx *ctx, int32_t assembly_id, int32_t q_len, in
     const int slot = find_slot(ctx, assembly_id);
     if (slot < 0) return fail(ctx, KVP_ERR_NOT_FOUND, "export_schedule: unknown assembly %d", assembly_id);
     if (q_len <= 0 || q_len > ctx->cfg.max_query_tokens) return fail(ctx, KVP_ERR_INVALID, "export_schedule: bad q_len");
-    schedule_t sc;
+    kvp_schedule &sc = ctx->plan;
     const int32_t rc = plan_schedule(ctx, ctx->slots[slot], 0, q_len, 0, nullptr, 0, sc);
     if (rc != KVP_OK) return rc;
     counts[0] = sc.n_ctas;

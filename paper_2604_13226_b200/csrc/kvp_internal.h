@@ -14,6 +14,7 @@
 #define KVP_TILE_ROWS 128      // packed query rows per CTA tile (MMA M)
 #define KVP_CHUNK_ROWS 32      // rows per gather work item
 #define KVP_MAX_SPLIT_UNITS 2048   // partial slots (128 query rows each) in the workspace
+#define KVP_SCHED_RING 8       // pinned staging buffers for work lists
 
 // ---- device-visible plan records (written by the host planner, uploaded once per assembly) -----
 
@@ -78,10 +79,16 @@ struct kvp_merge_item {        // 128 packed rows whose result is spread over n_
     int32_t pad[3];            // pad[0]: the request's own query length (0: the call's q_len)
 };
 
-// Offsets (bytes) of the arrays inside one plan blob; identical on host and device.
+// Capacity of one plan blob (entries per array, bytes in all).
 struct kvp_plan_layout {
-    uint64_t items, tiles, chunks, segs, rope, kept, total;
+    uint64_t total, upload;                // bytes on the device; bytes of the arrays that the host writes
     int32_t max_items, max_tiles, max_chunks, max_segs, max_rope;
+};
+
+// Offsets (bytes) of the arrays inside one plan blob, packed for the counts of the assembly it belongs to;
+// identical on host and device.  [0, upload) is copied to the device; the rope table is formed there.
+struct kvp_plan_offsets {
+    uint64_t items = 0, tiles = 0, chunks = 0, segs = 0, kept = 0, delta = 0, upload = 0, rope = 0;
 };
 
 // Pointers into a device-resident plan, passed to kernels by value.
@@ -91,6 +98,7 @@ struct kvp_plan_dev {
     const kvp_chunk *chunks;
     const kvp_seg *segs;
     const float2 *rope;        // [n_rope][head_dim/2] (cos, sin) of delta * theta_i
+    const int32_t *delta;      // [n_rope] the offsets of the rope table's rows (0 first)
     const int32_t *kept;       // [compressed packets of the assembly][n_layers * n_kv_heads] kept rows per plane
     int32_t item_stride;       // 0: one item / tile list for all planes; batch: items[(layer * n_kv_heads + kv head) * batch + b]
     int32_t n_planes;
@@ -117,7 +125,9 @@ struct kvp_assembly_host {
     std::vector<kvp_item> items;
     std::vector<kvp_seg> segs;
     std::vector<kvp_tile> tiles;
-    int32_t n_chunks = 0, n_rope = 0;
+    std::vector<kvp_chunk> chunks;         // gather work
+    std::vector<int32_t> delta;            // rope-table rows (row 0: no rotation)
+    kvp_plan_offsets off;
     int32_t item_stride = 0;               // batch when the assembly has a tile list per (layer, kv head) (compressed packets)
     int32_t last_q_len = 0;
     std::vector<int32_t> appended;         // per layer: query rows appended so far (KVP_CONTINUE)
@@ -126,8 +136,23 @@ struct kvp_assembly_host {
     bool waits_loads = false;              // uses packets that came from host memory: wait for the layer's load event
     // work lists of the two-stream kernel (one, or one per layer when the tile lists differ per layer), each
     // built for q_len query tokens at offset q_pos0 (q_len 0 = none yet)
-    struct sched_state { int32_t q_len = 0, q_pos0 = 0, ctas = 0, works = 0, merges = 0, slots = 0; uint32_t opts = 0; std::vector<int32_t> q_lens; };
+    struct sched_state { int32_t q_len = 0, q_pos0 = 0, ctas = 0, works = 0, merges = 0, slots = 0; uint32_t opts = 0, off_works = 0, off_merges = 0; std::vector<int32_t> q_lens; };
     std::vector<sched_state> sched;
+};
+
+// Work list of the two-stream kernel for one assembly and query length, with the scratch it is built in.
+struct kvp_schedule {
+    std::vector<int32_t> cta_begin;
+    std::vector<kvp_work> works;
+    std::vector<kvp_merge_item> merges;
+    int32_t n_ctas = 0, n_slots = 0, max_pieces = 1;
+    struct unit { int32_t b, hk, row_base, mode, n_all, n_pieces, q_len, t_first, tile_begin, tail_row0, n_tail, slot; };
+    struct cut { int32_t u, t; };
+    std::vector<unit> units;
+    std::vector<cut> cuts, model;
+    std::vector<int64_t> after;
+    std::vector<int32_t> order;            // emission order of the CTAs (indices into cuts)
+    std::vector<int32_t> work_unit;        // unit of every piece
 };
 
 struct kvp_ctx {
@@ -153,10 +178,18 @@ struct kvp_ctx {
     std::vector<char *> slot_plan_dev;     // per assembly slot
     std::vector<char *> slot_k, slot_v;    // per assembly slot: workspace rows
     std::vector<char *> slot_sched_dev;    // per assembly slot: cta ranges, work list, merge list
-    std::vector<char *> slot_sched_host;   // pinned staging of the same
-    std::vector<cudaEvent_t> sched_event;
-    uint64_t sched_off_works = 0, sched_off_merges = 0, sched_bytes = 0;
+    // pinned staging of the same: a ring, so that the layers of an assembly with a list each, or the steps of a
+    // decode, do not wait for one another's upload (which lies behind the attention kernels enqueued before it)
+    char *sched_ring[KVP_SCHED_RING] = {};
+    cudaEvent_t sched_event[KVP_SCHED_RING] = {};
+    int sched_next = 0;
+    const double *half_turns = nullptr;    // device [head_dim/2]: theta_i / pi (angles in half turns per position)
+    uint64_t sched_bytes = 0;
     int32_t sched_max_works = 0, sched_max_merges = 0;
+    // planning scratch, kept so that a call allocates nothing once the sizes have been seen
+    kvp_assembly_host build;
+    std::vector<int32_t> rope_hash, kept_row_of;
+    kvp_schedule plan;
     int32_t fused_append = 1;              // plain prefill: the attention kernel reads k_new / v_new itself and appends them
     void *encode_tiled = nullptr;          // cuTensorMapEncodeTiled
     float *partial_o = nullptr;            // [units][128][head_dim]
@@ -165,6 +198,7 @@ struct kvp_ctx {
     float2 *q_rope = nullptr;              // [max_batch*max_query][head_dim/2] for KVP_ROPE_QUERY
 
     // pinned host staging (one per slot) and the event guarding its reuse
+    char *staging = nullptr;               // the pinned block that all staging buffers lie in
     std::vector<char *> slot_plan_host;
     std::vector<cudaEvent_t> slot_event;
     std::vector<kvp_assembly_host> slots;
@@ -191,11 +225,13 @@ struct kvp_ctx {
 
 cudaError_t kvp_launch_store_rows(const kvp_shape &sh, const void *src, char *dst_plane0, int64_t plane_rows,
                                   int64_t dst_row0, int32_t n_tokens, cudaStream_t st);
-cudaError_t kvp_launch_gather(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t n_chunks,
-                              const char *pool_k, const char *pool_v, char *ws_k, char *ws_v, cudaStream_t st);
+// the rope table of an assembly and the gather of its chunks, one launch
+cudaError_t kvp_launch_gather(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t n_chunks, int32_t n_rope,
+                              const double *half_turns, const char *pool_k, const char *pool_v, char *ws_k, char *ws_v,
+                              cudaStream_t st);
 cudaError_t kvp_launch_append(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t batch, int32_t q_len,
                               int32_t q_pos0, const void *q, const void *k_new, const void *v_new, char *ws_k, char *ws_v,
-                              int32_t layer, int32_t rope_query, const double *inv_freq_dev, void *q_rot,
+                              int32_t layer, int32_t rope_query, const double *half_turns, void *q_rot,
                               cudaStream_t st);
 cudaError_t kvp_launch_export(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t b, int32_t layer,
                               int32_t prefix_len, int32_t n_query_rows, const char *pool_k, const char *pool_v,

@@ -86,33 +86,76 @@ __global__ void store_rows_kernel(const uint4 *__restrict__ src, char *__restric
     }
 }
 
-// ---- gather + re-base: pool rows -> workspace rows, all layers and kv heads ------------------------
-// grid (n_chunks, L*Hkv); one thread per (row, pair of 16-byte vectors); V is a byte copy, K is a byte
-// copy when the chunk's offset is 0 and an fp32 rotation otherwise.
-template <typename T>
-__global__ void gather_kernel(kvp_plan_dev plan, const char *__restrict__ pool_k, const char *__restrict__ pool_v,
-                              char *__restrict__ ws_k, char *__restrict__ ws_v, int64_t pool_rows, int64_t ws_rows,
-                              int vecs_per_row, int half_dim, int pairing)
+// (cos, sin) of offset x theta, narrowed to fp32 once: the angle is formed in double precision in half turns (offsets
+// reach 1e5 and more), which sincospi reduces exactly.
+__device__ __forceinline__ float2 offset_cos_sin(int32_t offset, double half_turn)
 {
-    const kvp_chunk ch = plan.chunks[blockIdx.x];
-    const int plane = blockIdx.y;
+    double s, c;
+    sincospi((double)offset * half_turn, &s, &c);
+    return make_float2((float)c, (float)s);
+}
+
+// ---- rope table + gather and re-base: pool rows -> workspace rows, all layers and kv heads -----------
+// The first n_table blocks form the assembly's (cos, sin) table, 256 entries each; attention reads it.  (On the host it
+// cost more than everything else in a call that composes many documents: 129 offsets x 64 angles, 0.2 ms.)  The other
+// blocks gather: `groups` of them share a 32-row chunk and take every groups-th plane.  A gather block forms the 64
+// angles of its chunk's offset itself, so it waits for no table block.  V is a byte copy, K is a byte copy when the
+// offset is 0 and an fp32 rotation otherwise.  Bound by DRAM for a whole cache (materialised), by latency for adapter
+// rows; a thread has the loads of two (row, plane) pairs in flight.
+template <typename T>
+__global__ void __launch_bounds__(256)
+gather_kernel(kvp_plan_dev plan, int n_table, int n_rope, int groups, const double *__restrict__ half_turns,
+              float2 *__restrict__ table, const char *__restrict__ pool_k, const char *__restrict__ pool_v,
+              char *__restrict__ ws_k, char *__restrict__ ws_v, int64_t pool_rows, int64_t ws_rows, int vecs_per_row,
+              int half_dim, int pairing)
+{
+    if ((int)blockIdx.x < n_table) {
+        const int e = blockIdx.x * 256 + threadIdx.x;
+        if (e < n_rope * half_dim) table[e] = offset_cos_sin(plan.delta[e / half_dim], half_turns[e % half_dim]);
+        return;
+    }
+    __shared__ float2 cs[64];
+    const int bi = blockIdx.x - n_table;
+    const kvp_chunk ch = plan.chunks[bi / groups];
     const int half_vecs = vecs_per_row / 2;
-    const float2 *cs = plan.rope + (size_t)ch.rope * half_dim;
-    const uint4 *sk = reinterpret_cast<const uint4 *>(pool_k) + ((int64_t)plane * pool_rows + ch.src_row0) * vecs_per_row;
-    const uint4 *sv = reinterpret_cast<const uint4 *>(pool_v) + ((int64_t)plane * pool_rows + ch.src_row0) * vecs_per_row;
-    uint4 *dk = reinterpret_cast<uint4 *>(ws_k) + ((int64_t)plane * ws_rows + ch.dst_row0) * vecs_per_row;
-    uint4 *dv = reinterpret_cast<uint4 *>(ws_v) + ((int64_t)plane * ws_rows + ch.dst_row0) * vecs_per_row;
-    for (int w = threadIdx.x; w < ch.n_rows * half_vecs; w += blockDim.x) {
-        const int row = w / half_vecs, c = w % half_vecs;
-        const int o = row * vecs_per_row + c;
-        Vec16<T> lo, hi;
-        lo.u = __ldg(sk + o);
-        hi.u = __ldg(sk + o + half_vecs);
-        if (ch.rope != 0) rotate_vec_pair<T>(lo, hi, cs, c, half_vecs, pairing);
-        dk[o] = lo.u;
-        dk[o + half_vecs] = hi.u;
-        dv[o] = __ldg(sv + o);
-        dv[o + half_vecs] = __ldg(sv + o + half_vecs);
+    if (ch.rope != 0) {
+        if ((int)threadIdx.x < half_dim) cs[threadIdx.x] = offset_cos_sin(plan.delta[ch.rope], half_turns[threadIdx.x]);
+        __syncthreads();
+    }
+    const int per_plane = ch.n_rows * half_vecs;
+    const int plane0 = bi % groups;
+    const int n_items = (plan.n_planes - plane0 + groups - 1) / groups * per_plane;
+    for (int w0 = threadIdx.x; w0 < n_items; w0 += 512) {
+        Vec16<T> lo[2], hi[2];
+        uint4 va[2], vb[2];
+        int64_t dst[2];
+        int c[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int w = w0 + 256 * u;
+            if (w >= n_items) break;
+            const int64_t plane = plane0 + (int64_t)(w / per_plane) * groups;
+            const int r = w % per_plane;
+            const int row = r / half_vecs;
+            c[u] = r % half_vecs;
+            const int64_t src = (plane * pool_rows + ch.src_row0 + row) * vecs_per_row + c[u];
+            dst[u] = (plane * ws_rows + ch.dst_row0 + row) * vecs_per_row + c[u];
+            const uint4 *sk = reinterpret_cast<const uint4 *>(pool_k) + src, *sv = reinterpret_cast<const uint4 *>(pool_v) + src;
+            lo[u].u = __ldg(sk);
+            hi[u].u = __ldg(sk + half_vecs);
+            va[u] = __ldg(sv);
+            vb[u] = __ldg(sv + half_vecs);
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            if (w0 + 256 * u >= n_items) break;
+            if (ch.rope != 0) rotate_vec_pair<T>(lo[u], hi[u], cs, c[u], half_vecs, pairing);
+            uint4 *dk = reinterpret_cast<uint4 *>(ws_k) + dst[u], *dv = reinterpret_cast<uint4 *>(ws_v) + dst[u];
+            dk[0] = lo[u].u;
+            dk[half_vecs] = hi[u].u;
+            dv[0] = va[u];
+            dv[half_vecs] = vb[u];
+        }
     }
 }
 
@@ -123,18 +166,14 @@ template <typename T>
 __global__ void append_kernel(kvp_plan_dev plan, int q_len, int q_pos0, const T *__restrict__ q, const T *__restrict__ k_new,
                               const T *__restrict__ v_new, char *__restrict__ ws_k, char *__restrict__ ws_v,
                               int64_t ws_rows, int layer, int n_q, int n_kv, int d, int pairing, int rope_query,
-                              const double *__restrict__ inv_freq, T *__restrict__ q_rot)
+                              const double *__restrict__ half_turns, T *__restrict__ q_rot)
 {
     __shared__ float2 cs[64];
     const int b = blockIdx.x / q_len, i = blockIdx.x % q_len;
     const kvp_item it = plan.items[b];
     const int half = d / 2;
     if (rope_query) {
-        for (int p = threadIdx.x; p < half; p += blockDim.x) {
-            double s, c;
-            sincos((double)(it.prefix_len + q_pos0 + i) * inv_freq[p], &s, &c);
-            cs[p] = make_float2((float)c, (float)s);
-        }
+        for (int p = threadIdx.x; p < half; p += blockDim.x) cs[p] = offset_cos_sin(it.prefix_len + q_pos0 + i, half_turns[p]);
         __syncthreads();
     }
     const int64_t tok = (int64_t)b * q_len + i;
@@ -460,37 +499,46 @@ cudaError_t kvp_launch_store_rows(const kvp_shape &sh, const void *src, char *ds
     return cudaGetLastError();
 }
 
-cudaError_t kvp_launch_gather(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t n_chunks, const char *pool_k,
-                              const char *pool_v, char *ws_k, char *ws_v, cudaStream_t st)
+cudaError_t kvp_launch_gather(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t n_chunks, int32_t n_rope,
+                              const double *half_turns, const char *pool_k, const char *pool_v, char *ws_k, char *ws_v,
+                              cudaStream_t st)
 {
-    if (n_chunks <= 0) return cudaSuccess;
-    const int vecs = sh.head_dim * sh.elem_bytes / 16;
-    const dim3 grid(n_chunks, sh.n_layers * sh.n_kv_heads);
-    const int threads = KVP_CHUNK_ROWS * (vecs / 2);
+    const int vecs = sh.head_dim * sh.elem_bytes / 16, half = sh.head_dim / 2;
+    const int planes = sh.n_layers * sh.n_kv_heads;
+    const int n_table = (n_rope * half + 255) / 256;
+    // Blocks per chunk: a block's angles cost about as much as moving one plane of its chunk, so a block takes several
+    // planes once there are blocks enough to fill the chip (8 x 148), at least two rounds of its 256 threads.
+    const int per_plane = KVP_CHUNK_ROWS * (vecs / 2);
+    int groups = n_chunks > 0 ? (1184 + n_chunks - 1) / n_chunks : 1;
+    const int most = (planes * per_plane + 511) / 512, least = (planes + 15) / 16;
+    groups = groups < least ? least : groups;
+    groups = groups > most ? most : groups;
+    const int grid = n_table + n_chunks * groups;
+    float2 *table = const_cast<float2 *>(plan.rope);
     if (sh.dtype == KVP_DTYPE_BF16)
-        gather_kernel<__nv_bfloat16><<<grid, threads, 0, st>>>(plan, pool_k, pool_v, ws_k, ws_v, sh.pool_rows,
-                                                              sh.ws_rows, vecs, sh.head_dim / 2, sh.pairing);
+        gather_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(plan, n_table, n_rope, groups, half_turns, table, pool_k, pool_v, ws_k,
+                                                          ws_v, sh.pool_rows, sh.ws_rows, vecs, half, sh.pairing);
     else
-        gather_kernel<float><<<grid, threads, 0, st>>>(plan, pool_k, pool_v, ws_k, ws_v, sh.pool_rows, sh.ws_rows,
-                                                      vecs, sh.head_dim / 2, sh.pairing);
+        gather_kernel<float><<<grid, 256, 0, st>>>(plan, n_table, n_rope, groups, half_turns, table, pool_k, pool_v, ws_k, ws_v,
+                                                  sh.pool_rows, sh.ws_rows, vecs, half, sh.pairing);
     return cudaGetLastError();
 }
 
 cudaError_t kvp_launch_append(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t batch, int32_t q_len,
                               int32_t q_pos0, const void *q, const void *k_new, const void *v_new, char *ws_k, char *ws_v,
-                              int32_t layer, int32_t rope_query, const double *inv_freq_dev, void *q_rot,
+                              int32_t layer, int32_t rope_query, const double *half_turns, void *q_rot,
                               cudaStream_t st)
 {
     const int grid = batch * q_len;
     if (sh.dtype == KVP_DTYPE_BF16)
         append_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(
             plan, q_len, q_pos0, (const __nv_bfloat16 *)q, (const __nv_bfloat16 *)k_new, (const __nv_bfloat16 *)v_new, ws_k,
-            ws_v, sh.ws_rows, layer, sh.n_q_heads, sh.n_kv_heads, sh.head_dim, sh.pairing, rope_query, inv_freq_dev,
+            ws_v, sh.ws_rows, layer, sh.n_q_heads, sh.n_kv_heads, sh.head_dim, sh.pairing, rope_query, half_turns,
             (__nv_bfloat16 *)q_rot);
     else
         append_kernel<float><<<grid, 256, 0, st>>>(plan, q_len, q_pos0, (const float *)q, (const float *)k_new,
                                                    (const float *)v_new, ws_k, ws_v, sh.ws_rows, layer, sh.n_q_heads,
-                                                   sh.n_kv_heads, sh.head_dim, sh.pairing, rope_query, inv_freq_dev,
+                                                   sh.n_kv_heads, sh.head_dim, sh.pairing, rope_query, half_turns,
                                                    (float *)q_rot);
     return cudaGetLastError();
 }
