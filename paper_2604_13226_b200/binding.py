@@ -9,6 +9,8 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
+from itertools import accumulate
 from typing import List, Optional, Sequence, Tuple
 
 from . import build as _build
@@ -68,12 +70,13 @@ def lib() -> ctypes.CDLL:
         "kvp_register_packet_host": (i32, [vp, vp, vp, i32, i32, pi32]),
         "kvp_evict_packet": (i32, [vp, i32]),
         "kvp_register_adapter": (i32, [vp, vp, vp, i32, i32, vp, vp, i32, i32, vp, pi32]),
-        "kvp_assemble": (i32, [vp, i32, pi32, pi32, pi32, u32, vp, pi32, pi32]),
-        "kvp_assemble_at": (i32, [vp, i32, pi32, pi32, pi32, pi32, u32, vp, pi32, pi32]),
+        # host index arrays go as addresses: assemble and the ragged call are on the path of every request
+        "kvp_assemble": (i32, [vp, i32, vp, vp, vp, u32, vp, pi32, pi32]),
+        "kvp_assemble_at": (i32, [vp, i32, vp, vp, vp, vp, u32, vp, pi32, pi32]),
         "kvp_partial_bytes": (u64, [vp, i32, i32]),
         "kvp_merge_partials": (i32, [vp, vp, i32, i32, i32, vp, vp, vp]),
         "kvp_query_prefill": (i32, [vp, i32, i32, vp, vp, vp, i32, u32, vp, vp, vp]),
-        "kvp_query_prefill_ragged": (i32, [vp, i32, i32, vp, vp, vp, i32, pi32, vp, vp, vp]),
+        "kvp_query_prefill_ragged": (i32, [vp, i32, i32, vp, vp, vp, i32, vp, vp, vp, vp]),
         "kvp_export_plan": (i32, [vp, i32, i32, pi32, pi32, pi32, pi32]),
         "kvp_export_cache": (i32, [vp, i32, i32, i32, i32, vp, vp, i32, vp]),
         "kvp_export_schedule": (i32, [vp, i32, i32, pi32, i32, pi32, i32, pi32, i32, pi32]),
@@ -153,6 +156,8 @@ class Context:
         if device >= 0:
             import torch
             self._torch = torch
+            self._raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (
+                lambda index: torch.cuda.current_stream(index).cuda_stream)
             dev = torch.device(f"cuda:{device}")
             ws_bytes = int(self._L.kvp_workspace_bytes(ctypes.byref(cfg)))
             self.pool = torch.empty(max(1, pool_tokens) * self.token_bytes + 1024, dtype=torch.uint8, device=dev)
@@ -173,11 +178,9 @@ class Context:
             raise KvpError(rc, (self._L.kvp_last_error(self._h) or b"").decode())
 
     def _stream(self, stream=None):
-        if self.device < 0:
-            return None
-        if stream is None:
-            stream = self._torch.cuda.current_stream(self.device)
-        return ctypes.c_void_p(stream.cuda_stream)
+        if stream is not None:
+            return stream.cuda_stream if self.device >= 0 else None
+        return self._raw_stream(self.device) if self.device >= 0 else None
 
     def close(self):
         if self._h:
@@ -226,22 +229,22 @@ class Context:
     def assemble(self, items: Sequence[Sequence[Tuple[int, int]]], flags: int = REBASE, stream=None, pos_base=None):
         """items[b] = [(packet_id, adapter_id), ...].  Returns (assembly_id, prefix_len list).
         pos_base (one position per request) -> ``kvp_assemble_at``: this rank's part of a sharded request."""
-        offs, pids, aids = [0], [], []
-        for it in items:
-            for pid, aid in it:
-                pids.append(pid)
-                aids.append(aid)
-            offs.append(len(pids))
         B = len(items)
+        pids = [p for it in items for p, _ in it]
+        aids = [a for it in items for _, a in it]
+        n = len(pids)
+        # packed ints: a ctypes array costs six times as much to fill
+        offs = struct.pack(f"{B + 1}i", 0, *accumulate(map(len, items)))
+        pids, aids = struct.pack(f"{n}i", *pids), struct.pack(f"{n}i", *aids)
         plen = (ctypes.c_int32 * max(1, B))()
         aid = ctypes.c_int32(-1)
         if pos_base is not None:
-            self._check(self._L.kvp_assemble_at(self._h, B, _i32_array(offs), _i32_array(pids), _i32_array(aids),
-                                                _i32_array(list(pos_base)), flags, self._stream(stream), plen, ctypes.byref(aid)))
+            self._check(self._L.kvp_assemble_at(self._h, B, offs, pids, aids, _i32_array(list(pos_base)), flags,
+                                                self._stream(stream), plen, ctypes.byref(aid)))
         else:
-            self._check(self._L.kvp_assemble(self._h, B, _i32_array(offs), _i32_array(pids), _i32_array(aids), flags,
-                                             self._stream(stream), plen, ctypes.byref(aid)))
-        return aid.value, [int(plen[b]) for b in range(B)]
+            self._check(self._L.kvp_assemble(self._h, B, offs, pids, aids, flags, self._stream(stream), plen,
+                                             ctypes.byref(aid)))
+        return aid.value, plen[:B]
 
     def partial_bytes(self, batch: int, q_len: int) -> int:
         return int(self._L.kvp_partial_bytes(self._h, batch, q_len))
