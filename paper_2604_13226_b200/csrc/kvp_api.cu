@@ -221,6 +221,8 @@ int find_slot(kvp_ctx *ctx, int32_t assembly_id)
 // fewer tiles.  Counted in single-stream tiles.
 constexpr int kPieceCost = 4;
 
+constexpr double kTcMinFlops64 = 4e8;
+
 // q_lens: nullptr, or one query length per request (<= q_len, the stride of the padded tensors); a request's
 // work records and merge items then carry its own length.
 // opts: KVP_PARTIAL - every unit writes partial slots and gets merge items (even with one piece or none);
@@ -649,7 +651,7 @@ int32_t kvp_create(const kvp_config *cfg, kvp_ctx **out)
         if (cudaEventCreateWithFlags(&ctx->load_done[l], cudaEventDisableTiming) != cudaSuccess)
             return bail(KVP_ERR_CUDA, "load event creation failed");
 
-    if (sh.dtype == KVP_DTYPE_BF16 && sh.head_dim == 128 && prop.major == 10) {
+    if (sh.dtype == KVP_DTYPE_BF16 && prop.major == 10) {
         void *fn = nullptr;
         cudaDriverEntryPointQueryResult qres;
         if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) == cudaSuccess && fn &&
@@ -665,7 +667,7 @@ int32_t kvp_create(const kvp_config *cfg, kvp_ctx **out)
                 ok = make_tensor_map(enc, &ctx->tm_ws_k[a], ctx->slot_k[a], sh.head_dim, sh.ws_rows, planes) &&
                      make_tensor_map(enc, &ctx->tm_ws_v[a], ctx->slot_v[a], sh.head_dim, sh.ws_rows, planes);
             if (!ok) return bail(KVP_ERR_CUDA, "cuTensorMapEncodeTiled failed");
-            if (kvp_attn_sm100_prepare() != cudaSuccess)
+            if (kvp_attn_sm100_prepare(sh.head_dim) != cudaSuccess)
                 return bail(KVP_ERR_CUDA, "tcgen05 kernel attribute setup failed");
             ctx->have_tma = true;
         }
@@ -1139,14 +1141,15 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
     const uint32_t part_opts = flags & (uint32_t)(KVP_PARTIAL | KVP_SKIP_QUERY_BLOCK);
     if ((flags & KVP_SKIP_QUERY_BLOCK) && !(flags & KVP_PARTIAL))
         return fail(ctx, KVP_ERR_INVALID, "query_prefill: KVP_SKIP_QUERY_BLOCK needs KVP_PARTIAL");
-    if (part_opts && ((flags & (KVP_CONTINUE | KVP_ROPE_QUERY | KVP_FORCE_SIMPLE)) || q_lens || !ctx->have_tma))
+    const bool tc128 = ctx->have_tma && ctx->shape.head_dim == 128;
+    if (part_opts && ((flags & (KVP_CONTINUE | KVP_ROPE_QUERY | KVP_FORCE_SIMPLE)) || q_lens || !tc128))
         return fail(ctx, KVP_ERR_UNSUPPORTED, "query_prefill: KVP_PARTIAL runs on the tcgen05 kernel only, without KVP_CONTINUE, KVP_ROPE_QUERY or per-request lengths");
     {
         // every kernel reads whole elements; the tcgen05 path moves q and out 16 bytes at a time
         const uintptr_t all = (uintptr_t)q | (uintptr_t)k_new | (uintptr_t)v_new | (uintptr_t)out;
         if ((all & (uintptr_t)(ctx->shape.elem_bytes - 1)) || ((uintptr_t)lse & 3))
             return fail(ctx, KVP_ERR_INVALID, "query_prefill: q / k_new / v_new / out / lse not aligned to their element size");
-        if (ctx->have_tma && !(flags & KVP_FORCE_SIMPLE) && ((((uintptr_t)q | (uintptr_t)out) & 15) != 0))
+        if (tc128 && !(flags & KVP_FORCE_SIMPLE) && ((((uintptr_t)q | (uintptr_t)out) & 15) != 0))
             return fail(ctx, KVP_ERR_INVALID, "query_prefill: q and out must be 16-byte aligned on the tcgen05 path (KVP_FORCE_SIMPLE takes any element-aligned pointer)");
     }
     if (q_len > ctx->cfg.max_query_tokens) return fail(ctx, KVP_ERR_CAPACITY, "query_prefill: q_len > max_query_tokens");
@@ -1166,8 +1169,15 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
     const bool skip_block = (flags & KVP_SKIP_QUERY_BLOCK) != 0;
 
     int launches = 0;
-    const bool fast = ctx->have_tma && !(flags & KVP_FORCE_SIMPLE);
-    if (q_lens && !fast) return fail(ctx, KVP_ERR_UNSUPPORTED, "query_prefill_ragged: needs the tcgen05 kernel (bf16, head_dim 128, sm_100)");
+    bool fast = ctx->have_tma && !(flags & KVP_FORCE_SIMPLE);
+    if (fast && sh.head_dim == 64) {
+        // The tcgen05 kernel has a start of several microseconds (tables, first Q tile, pipeline fill) and a merge launch
+        // behind it; below kTcMinFlops64 the CUDA-core kernel is done by then.  It also takes any alignment.
+        double keys = 0.0;
+        for (int b = 0; b < as.batch; ++b) keys += as.items[b].prefix_len + q_pos0 + q_len;
+        fast = 4.0 * sh.head_dim * sh.n_q_heads * q_len * keys >= kTcMinFlops64 && (((uintptr_t)q | (uintptr_t)out) & 15) == 0;
+    }
+    if (q_lens && !(tc128 && fast)) return fail(ctx, KVP_ERR_UNSUPPORTED, "query_prefill_ragged: needs the tcgen05 kernel (bf16, head_dim 128, sm_100)");
     // plain prefill on the two-stream kernel: it reads the query block's K/V from k_new / v_new and appends them itself
     kvp_attn2_args a;
     a.tail_direct = 0;
@@ -1289,7 +1299,7 @@ int32_t kvp_merge_partials(kvp_ctx *ctx, const void *parts, int32_t n_parts, int
     if (ctx->host_only) return fail(ctx, KVP_ERR_STATE, "merge_partials: host-only context");
     if (!parts || !out || n_parts <= 0 || batch <= 0 || q_len <= 0 || (((uintptr_t)parts | (uintptr_t)out) & 15) || ((uintptr_t)lse & 3))
         return fail(ctx, KVP_ERR_INVALID, "merge_partials: bad arguments (parts and out must be 16-byte aligned)");
-    if (!ctx->have_tma) return fail(ctx, KVP_ERR_UNSUPPORTED, "merge_partials: bf16, head_dim 128, sm_100 only");
+    if (!ctx->have_tma || ctx->shape.head_dim != 128) return fail(ctx, KVP_ERR_UNSUPPORTED, "merge_partials: bf16, head_dim 128, sm_100 only");
     if (batch > ctx->cfg.max_batch || q_len > ctx->cfg.max_query_tokens)
         return fail(ctx, KVP_ERR_CAPACITY, "merge_partials: batch or q_len beyond the context's maxima");
     KVP_CUDA(ctx, cudaSetDevice(ctx->cfg.device));

@@ -1,4 +1,4 @@
-// bf16 composed-cache attention for sm_100a: TMA-staged K/V tiles, tcgen05 MMA with TMEM accumulators,
+// bf16 composed-cache attention (head dimension 128, or 64) for sm_100a: TMA-staged K/V tiles, tcgen05 MMA with TMEM accumulators,
 // two query streams per CTA so that the tensor pipe works on one stream while the other is in softmax.
 //
 // A persistent CTA (one per SM) walks a host-built list of work pieces.  A piece is a contiguous range
@@ -36,24 +36,33 @@
 
 namespace {
 
-constexpr int kStages = 3;
-constexpr int kTileBytes = KVP_TILE_KEYS * 128 * 2;      // 32 KB: 128 rows x 128 bf16
-constexpr int kHalfBytes = kTileBytes / 2;               // one 64-column box
+constexpr int kHalfBytes = KVP_TILE_KEYS * 64 * 2;       // 16 KB: one 64-column box of 128 rows
+constexpr int kQBufBytes = 2 * kHalfBytes;               // a rotated-Q buffer
 constexpr int kThreads = 512;
 constexpr int kTmemCols = 512;
 constexpr uint32_t kColS = 0, kColO = 256;               // + 128 * stream
 
-constexpr int kOffQ = 0;                                  // two 32 KB rotated-Q buffers per stream: [stream][epoch & 1]
-constexpr int kOffRing = 4 * kTileBytes;                  // kStages x 32 KB
-constexpr int kOffBar = kOffRing + kStages * kTileBytes;
-constexpr int kOffMl = kOffBar + 256;                     // float2[128]: stream 1's (max, sum) in mode 1
-constexpr int kSmemBytes = kOffMl + 1024 + 1024;          // + alignment slack
-
-
-enum BarIdx { kKvFull = 0, kKvEmpty = kStages, kQFull = 2 * kStages, kQFree = kQFull + 4, kSFull = kQFree + 4,   // Q: [2 * stream + buffer]
-              kPFull = kSFull + 2, kOFull = kPFull + 2, kOFree = kOFull + 2, kMlFull = kOFree + 2, kDrain = kMlFull + 1,
-              kNumBars = kDrain + 1 };
-static_assert(8 * kNumBars + 8 <= 256, "barrier block");
+// Shared memory and barriers by head dimension D.  With D = 64 a tile is one box: the ring holds twice the stages, and
+// the Q buffer's second half takes the rounding remainders of the rotated Q.
+template <int D>
+struct Cfg {
+    static constexpr int kStages = D == 128 ? 3 : 6;
+    static constexpr int kTileBytes = KVP_TILE_KEYS * D * 2;
+    static constexpr int kOffQ = 0;                               // two rotated-Q buffers per stream: [stream][epoch & 1]
+    static constexpr int kOffRing = 4 * kQBufBytes;
+    static constexpr int kOffBar = kOffRing + kStages * kTileBytes;
+    static constexpr int kOffMl = kOffBar + 256;                  // float2[128]: stream 1's (max, sum) in mode 1
+    static constexpr int kSmemBytes = kOffMl + 1024 + 1024;       // + alignment slack
+    static constexpr int kVecs = D / 8;                           // 16-byte words of a row
+    static constexpr int kCols4 = D / 4;                          // float4 columns of a partial
+    // D = 64 carries the rotated Q and P in two bf16 numbers each: the fp32 results of the CUDA-core kernel, which
+    // serves this head dimension in small calls, hold for large ones too
+    static constexpr bool kSplit = D == 64;
+    enum BarIdx { kKvFull = 0, kKvEmpty = kStages, kQFull = 2 * kStages, kQFree = kQFull + 4, kSFull = kQFree + 4,   // Q: [2 * stream + buffer]
+                  kPFull = kSFull + 2, kOFull = kPFull + 2, kOFree = kOFull + 2, kMlFull = kOFree + 2, kDrain = kMlFull + 1,
+                  kNumBars = kDrain + 1 };
+    static_assert(8 * kNumBars + 8 <= 256, "barrier block");
+};
 
 struct Params {
     kvp_plan_dev plan;
@@ -354,29 +363,34 @@ __device__ __forceinline__ int load_seq(int mode, int n, int r, int kv)
 // its own chunks in place.
 // With `qrem` (precise mode) the remainders r - bf16(r) of the rotated values go, as bf16, to the same places of
 // a second tile: q' = hi + rem to about 2^-17, so that the rounding of the re-based operand leaves the scores.
+// With D = 64 a row is one 128-byte line of eight chunks: thread t owns chunks c = t & 3 and c + 4 of rows t >> 2, + 32, ...
+template <int D>
 __device__ __forceinline__ void produce_q_tile(const Params &p, char *qbuf, char *qrem, int t, const __nv_bfloat16 *q_b, int hk,
                                                int row_base, int n_rows, int rope)
 {
-    const int c = t & 7, r0 = t >> 3;
-    char *mine = qbuf + r0 * 128 + ((c ^ (r0 & 7)) << 4);                       // row & 7 == r0 & 7 for all of its rows
+    constexpr int kCh = D / 16, kRows = 128 / kCh;            // chunks to the rotation partner; rows per pass
+    const int c = t & (kCh - 1), r0 = t / kCh;
+    const int at = r0 * 128 + ((c ^ (r0 & 7)) << 4);          // row & 7 == r0 & 7 for all of its rows
+    char *mine = qbuf + at;
+    const int hi_off = D == 128 ? kHalfBytes : (at ^ 64) - at;            // from a chunk to its partner's place
     float4 w4[4];
     if (rope != 0) {
-        const float4 *cs = reinterpret_cast<const float4 *>(p.plan.rope + (size_t)rope * 64);   // (cos, sin) pairs
+        const float4 *cs = reinterpret_cast<const float4 *>(p.plan.rope + (size_t)rope * (D / 2));   // (cos, sin) pairs
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-            w4[j] = __ldg(p.pairing == 0 ? cs + c * 4 + j : cs + (c + 8 * (j >> 1)) * 2 + (j & 1));
+            w4[j] = __ldg(p.pairing == 0 ? cs + c * 4 + j : cs + (c + kCh * (j >> 1)) * 2 + (j & 1));
     }
 #pragma unroll 1
-    for (int i = 0; i < 8; ++i) {
-        const int r = row_base + r0 + 16 * i;
-        char *lo = mine + i * (16 * 128);
+    for (int i = 0; i < kCh; ++i) {
+        const int r = row_base + r0 + kRows * i;
+        char *lo = mine + i * (kRows * 128);
         if (r < n_rows) {
-            const uint4 *src = reinterpret_cast<const uint4 *>(q_b + ((long long)(r / p.group) * p.n_q + hk * p.group + r % p.group) * 128);
+            const uint4 *src = reinterpret_cast<const uint4 *>(q_b + ((long long)(r / p.group) * p.n_q + hk * p.group + r % p.group) * D);
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(lo)), "l"(src + c) : "memory");
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(lo + kHalfBytes)), "l"(src + c + 8) : "memory");
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(lo + hi_off)), "l"(src + c + kCh) : "memory");
         } else {
             *reinterpret_cast<uint4 *>(lo) = make_uint4(0, 0, 0, 0);
-            *reinterpret_cast<uint4 *>(lo + kHalfBytes) = make_uint4(0, 0, 0, 0);
+            *reinterpret_cast<uint4 *>(lo + hi_off) = make_uint4(0, 0, 0, 0);
         }
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
@@ -384,10 +398,10 @@ __device__ __forceinline__ void produce_q_tile(const Params &p, char *qbuf, char
     auto lo_f = [](uint32_t u) { return __uint_as_float(u << 16); };
     auto hi_f = [](uint32_t u) { return __uint_as_float(u & 0xffff0000u); };
 #pragma unroll 1
-    for (int i = 0; i < 8; ++i) {
-        if (row_base + r0 + 16 * i >= n_rows) break;
-        char *lo = mine + i * (16 * 128);
-        uint4 qa = *reinterpret_cast<uint4 *>(lo), qb = *reinterpret_cast<uint4 *>(lo + kHalfBytes);
+    for (int i = 0; i < kCh; ++i) {
+        if (row_base + r0 + kRows * i >= n_rows) break;
+        char *lo = mine + i * (kRows * 128);
+        uint4 qa = *reinterpret_cast<uint4 *>(lo), qb = *reinterpret_cast<uint4 *>(lo + hi_off);
         uint32_t *a = reinterpret_cast<uint32_t *>(&qa);
         uint32_t *b = reinterpret_cast<uint32_t *>(&qb);
         uint4 ra, rb;                                            // remainders (precise mode)
@@ -422,11 +436,11 @@ __device__ __forceinline__ void produce_q_tile(const Params &p, char *qbuf, char
             }
         }
         *reinterpret_cast<uint4 *>(lo) = qa;
-        *reinterpret_cast<uint4 *>(lo + kHalfBytes) = qb;
+        *reinterpret_cast<uint4 *>(lo + hi_off) = qb;
         if (qrem != nullptr) {
             char *rl = qrem + (lo - qbuf);
             *reinterpret_cast<uint4 *>(rl) = ra;
-            *reinterpret_cast<uint4 *>(rl + kHalfBytes) = rb;
+            *reinterpret_cast<uint4 *>(rl + hi_off) = rb;
         }
     }
 }
@@ -482,9 +496,11 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
     return d;
 }
 
-// p = exp2(s*c2 - mc) for 32 scores, packed as bf16 pairs into pk[16]; returns their fp32 sum.
+// p = exp2(s*c2 - mc) for 32 scores, packed as bf16 pairs into pk[0..15] (SPLIT: what that rounding dropped, as bf16
+// pairs, into pk[16..31]); returns their fp32 sum.
 // (Evaluating part of the exponentials by a polynomial on the FMA pipe was measured and lost: the
 // extra issue slots cost more than the special-function unit saves.)
+template <bool SPLIT>
 __device__ __forceinline__ float chunk_exp(const uint32_t *v, float c2, float mc, uint32_t *pk)
 {
     const uint64_t c2p = pair(c2, c2), nmc = pair(-mc, -mc);
@@ -496,6 +512,7 @@ __device__ __forceinline__ float chunk_exp(const uint32_t *v, float c2, float mc
         const float p0 = ex2(x0), p1 = ex2(x1);
         if (i & 2) lb = add2(lb, pair(p0, p1)); else la = add2(la, pair(p0, p1));
         pk[i >> 1] = pack_bf16(p0, p1);
+        if (SPLIT) pk[16 + (i >> 1)] = pack_bf16(p0 - __uint_as_float(pk[i >> 1] << 16), p1 - __uint_as_float(pk[i >> 1] & 0xffff0000u));
     }
     float s0, s1;
     unpair(add2(la, lb), s0, s1);
@@ -506,12 +523,13 @@ __device__ __forceinline__ float chunk_exp(const uint32_t *v, float c2, float mc
 // one shrinks by alpha = 2^(old - new): O in TMEM (when a P V product has been accumulated) and the P
 // chunks [0, n_chunks) of the current tile that were already written.  S of this step is complete, hence
 // so is the P V product of the previous step: O is quiet.
+template <int D>
 __device__ __forceinline__ void rescale_row(uint32_t s_addr, uint32_t o_addr, float alpha, int n_chunks, bool with_o)
 {
     uint32_t v[32];
     if (with_o) {
 #pragma unroll 1
-        for (int ch = 0; ch < 4; ++ch) {
+        for (int ch = 0; ch < D / 32; ++ch) {
             tmem_ld32(o_addr + ch * 32, v);
             tc_wait_ld();
 #pragma unroll
@@ -522,6 +540,20 @@ __device__ __forceinline__ void rescale_row(uint32_t s_addr, uint32_t o_addr, fl
     if (n_chunks > 0) tc_wait_st();                  // the P chunks this thread stored are read back below
 #pragma unroll 1
     for (int ch = 0; ch < n_chunks; ++ch) {          // 16 columns of packed bf16 pairs per chunk
+        if (Cfg<D>::kSplit) {                        // and 16 of remainders
+            tmem_ld32(s_addr + ch * 32, v);
+            tc_wait_ld();
+            landed32(v);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const float x = (__uint_as_float(v[i] << 16) + __uint_as_float(v[16 + i] << 16)) * alpha;
+                const float y = (__uint_as_float(v[i] & 0xffff0000u) + __uint_as_float(v[16 + i] & 0xffff0000u)) * alpha;
+                v[i] = pack_bf16(x, y);
+                v[16 + i] = pack_bf16(x - __uint_as_float(v[i] << 16), y - __uint_as_float(v[i] & 0xffff0000u));
+            }
+            tmem_st32(s_addr + ch * 32, v);
+            continue;
+        }
         asm volatile(
             "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
             "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
@@ -537,13 +569,15 @@ __device__ __forceinline__ void rescale_row(uint32_t s_addr, uint32_t o_addr, fl
     tc_wait_st();
 }
 
+template <int D>
 __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, const int S, const int t)
 {
+    using C = Cfg<D>;
     const uint32_t lane_base = (uint32_t)((t >> 5) * 32) << 16;
     const uint32_t s_addr = c.tmem + lane_base + kColS + S * 128;
     const uint32_t o_addr = c.tmem + lane_base + kColO + S * 128;
     const float c2 = p.scale_log2;
-    float2 *ml_smem = reinterpret_cast<float2 *>(c.smem + kOffMl);
+    float2 *ml_smem = reinterpret_cast<float2 *>(c.smem + C::kOffMl);
     uint32_t nS = 0, nO = 0, nMl = 0;
     bool ok = true;
 
@@ -563,7 +597,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
         for (int k = 0; k < steps; ++k) {
             const Tile tl = nxt;
             if (k + 1 < steps) nxt = get_tile(p, w, stream_tile(w, S, k + 1));
-            ok = mbar_wait(c.bar(kSFull + S), nS & 1, c.abort_flag, p.status, 30 + S);
+            ok = mbar_wait(c.bar(C::kSFull + S), nS & 1, c.abort_flag, p.status, 30 + S);
             ++nS;
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
@@ -580,23 +614,24 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
             // max is reduced alongside; the check comes last, so the two dependency chains overlap.
             auto process = [&](uint32_t *v, int ch) {
                 if (!full) chunk_mask(v, lim - ch * 32);
-                uint32_t pk[16];
+                uint32_t pk[C::kSplit ? 32 : 16];
                 const float cm = chunk_max(v, -INFINITY);
-                float ls = chunk_exp(v, c2, m_ref * c2, pk);
+                float ls = chunk_exp<C::kSplit>(v, c2, m_ref * c2, pk);
                 const bool need = (cm - m_ref) * c2 > 8.0f;
                 if (__any_sync(0xffffffffu, need)) {
                     const float m_new = need ? cm : m_ref;
                     const float alpha = need ? ex2((m_ref - m_new) * c2) : 1.f;
-                    rescale_row(s_addr, o_addr, alpha, ch, k > 0);
+                    rescale_row<D>(s_addr, o_addr, alpha, ch, k > 0);
                     l *= alpha;
                     m_ref = m_new;
                     tmem_ld32(s_addr + ch * 32, v);             // this chunk's scores again (P so far lies below them)
                     tc_wait_ld();
                     landed32(v);
                     if (!full) chunk_mask(v, lim - ch * 32);
-                    ls = chunk_exp(v, c2, m_ref * c2, pk);
+                    ls = chunk_exp<C::kSplit>(v, c2, m_ref * c2, pk);
                 }
-                tmem_st16(s_addr + ch * 16, pk);
+                if (C::kSplit) tmem_st32(s_addr + ch * 32, pk);         // over this chunk's own scores
+                else tmem_st16(s_addr + ch * 16, pk);
                 l += ls;
             };
             // a short tile (the end of a document, staged adapter rows) needs P only for the columns P V will read
@@ -610,12 +645,12 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
             }
             tc_wait_st();
             tc_fence_before();
-            mbar_arrive(c.bar(kPFull + S));
+            mbar_arrive(c.bar(C::kPFull + S));
         }
         if (!ok) break;
 
         // ---- end of the piece: O of this stream is complete once its last P V has landed ----------
-        ok = mbar_wait(c.bar(kOFull + S), nO & 1, c.abort_flag, p.status, 32 + S);
+        ok = mbar_wait(c.bar(C::kOFull + S), nO & 1, c.abort_flag, p.status, 32 + S);
         ++nO;
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
@@ -623,13 +658,13 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
 
         if (w.mode == 1 && S == 1) {
             ml_smem[t] = make_float2(m_ref, l);
-            mbar_arrive(c.bar(kMlFull));         // stream 0's warpgroup combines and writes
+            mbar_arrive(c.bar(C::kMlFull));         // stream 0's warpgroup combines and writes
             continue;
         }
         float w0 = 1.f, w1 = 0.f;
         const bool both = (w.mode == 1) && (w.steps1 > 0);
         if (both) {
-            ok = mbar_wait(c.bar(kMlFull), nMl & 1, c.abort_flag, p.status, 34);
+            ok = mbar_wait(c.bar(C::kMlFull), nMl & 1, c.abort_flag, p.status, 34);
             ++nMl;
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
@@ -649,11 +684,11 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
             w1 *= inv;
         }
         // un-normalised (partial slot) or normalised (output rows) O = w0 O_s (+ w1 O_1)
-        uint4 *orow_bf = (direct && valid) ? reinterpret_cast<uint4 *>(p.out + (((long long)w.b * p.q_len + qi) * p.n_q + h) * 128) : nullptr;
-        // partial slot layout: [32 float4 columns][128 rows], so that a warp's store covers 512 contiguous bytes
-        uint4 *orow_f = direct ? nullptr : reinterpret_cast<uint4 *>(p.partial_o) + (long long)slot * (32 * KVP_TILE_ROWS) + t;
+        uint4 *orow_bf = (direct && valid) ? reinterpret_cast<uint4 *>(p.out + (((long long)w.b * p.q_len + qi) * p.n_q + h) * D) : nullptr;
+        // partial slot layout: [D / 4 float4 columns][128 rows], so that a warp's store covers 512 contiguous bytes
+        uint4 *orow_f = direct ? nullptr : reinterpret_cast<uint4 *>(p.partial_o) + (long long)slot * (C::kCols4 * KVP_TILE_ROWS) + t;
 #pragma unroll 1
-        for (int ch = 0; ch < 4; ++ch) {
+        for (int ch = 0; ch < D / 32; ++ch) {
             uint32_t a[32];
             tmem_ld32(o_addr + ch * 32, a);
             tc_wait_ld();
@@ -689,14 +724,17 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
             p.partial_ml[(long long)slot * KVP_TILE_ROWS + t] = make_float2(m_ref, l);
         }
         tc_fence_before();
-        mbar_arrive(c.bar(kOFree + S));
-        if (both) mbar_arrive(c.bar(kOFree + 1));
+        mbar_arrive(c.bar(C::kOFree + S));
+        if (both) mbar_arrive(c.bar(C::kOFree + 1));
     }
 }
 
 // ---- Q producer -----------------------------------------------------------------------------------------
+template <int D>
 __device__ __forceinline__ void producer_role(const Params &p, const Cta &c, const int t)
 {
+    using C = Cfg<D>;
+    const bool one_buffer = !C::kSplit && p.precise;
     uint32_t nEp0 = 0, nEp1 = 0;
     bool ok = true;
     for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
@@ -707,19 +745,20 @@ __device__ __forceinline__ void producer_role(const Params &p, const Cta &c, con
         auto produce = [&](int s, int rope, uint32_t &nEp) {
             // two buffers per stream taken in turn; in precise mode one (value, remainder) pair, rewritten once
             // the last Q K^T of the epoch before has run
-            const int buf = p.precise ? 0 : (nEp & 1);
-            const uint32_t back = p.precise ? 1u : 2u;      // the epoch that used this buffer last
+            const int buf = one_buffer ? 0 : (nEp & 1);
+            const uint32_t back = one_buffer ? 1u : 2u;      // the epoch that used this buffer last
             if (nEp >= back) {
-                const uint32_t par = p.precise ? (nEp - 1) & 1 : ((nEp >> 1) - 1) & 1;
-                ok = mbar_wait(c.bar(kQFree + 2 * s + buf), par, c.abort_flag, p.status, 40 + s);
+                const uint32_t par = one_buffer ? (nEp - 1) & 1 : ((nEp >> 1) - 1) & 1;
+                ok = mbar_wait(c.bar(C::kQFree + 2 * s + buf), par, c.abort_flag, p.status, 40 + s);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) return;
             }
-            char *qb = c.smem + kOffQ + (2 * s + buf) * kTileBytes;
-            produce_q_tile(p, qb, p.precise ? qb + kTileBytes : nullptr, t, p.q + (long long)w.b * p.q_len * p.n_q * 128,
+            char *qb = c.smem + C::kOffQ + (2 * s + buf) * kQBufBytes;
+            char *qrem = C::kSplit ? qb + kHalfBytes : one_buffer ? qb + kQBufBytes : nullptr;
+            produce_q_tile<D>(p, qb, qrem, t, p.q + (long long)w.b * p.q_len * p.n_q * D,
                            w.hk, w.row_base + (w.mode == 0 ? s * KVP_TILE_ROWS : 0), n_rows, rope);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            mbar_arrive(c.bar(kQFull + 2 * s + buf));
+            mbar_arrive(c.bar(C::kQFull + 2 * s + buf));
             ++nEp;
         };
         for (int k = 0; k < max_steps && ok; ++k) {
@@ -742,8 +781,10 @@ __device__ __forceinline__ void producer_role(const Params &p, const Cta &c, con
 // behind the prefix in the workspace, for later calls.  Every unit copies the query tokens whose first packed row
 // it holds (for its kv head), in the piece that starts the unit, so the copy is spread over all CTAs; four
 // 16-byte words of K and of V are in flight per thread.  Nothing in this launch waits for the copy.
+template <int D>
 __device__ __forceinline__ void append_role(const Params &p, const Cta &c, const int t)
 {
+    constexpr int kVecs = Cfg<D>::kVecs;
     if (!p.tail_direct) return;
     for (int wi = c.item_begin; wi < c.item_end; ++wi) {
         const Work w = load_work(p, wi);
@@ -751,16 +792,16 @@ __device__ __forceinline__ void append_role(const Params &p, const Cta &c, const
         const int n_rows = p.group * w.q_len;
         const int row_end = min(n_rows, w.row_base + (w.mode ? KVP_TILE_ROWS : 2 * KVP_TILE_ROWS));
         const int i0 = (w.row_base + p.group - 1) / p.group, i1 = (row_end + p.group - 1) / p.group;   // tokens [i0, i1)
-        const long long src0 = (((long long)w.b * p.q_len + i0) * p.n_kv + w.hk) * 16;     // 16-byte words; a token's row is 16
-        const long long dst0 = ((long long)w.plane * p.ws_rows + w.tail_row0 + i0) * 16;
-        const int n_words = (i1 - i0) * 16;
+        const long long src0 = (((long long)w.b * p.q_len + i0) * p.n_kv + w.hk) * kVecs;     // 16-byte words
+        const long long dst0 = ((long long)w.plane * p.ws_rows + w.tail_row0 + i0) * kVecs;
+        const int n_words = (i1 - i0) * kVecs;
         for (int base = 0; base < n_words; base += 64 * 4) {
             uint4 k[4], v[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int i = base + j * 64 + t;
                 if (i < n_words) {
-                    const long long src = src0 + (long long)(i >> 4) * p.n_kv * 16 + (i & 15);
+                    const long long src = src0 + (long long)(i / kVecs) * p.n_kv * kVecs + i % kVecs;
                     k[j] = __ldg(p.k_new + src);
                     v[j] = __ldg(p.v_new + src);
                 }
@@ -778,11 +819,14 @@ __device__ __forceinline__ void append_role(const Params &p, const Cta &c, const
 }
 
 // ---- TMA producer (whole warp; lane 0 issues) ----------------------------------------------------------
+template <int D>
 __device__ __forceinline__ void tma_role(const Params &p, const Cta &c, const int lane, const CUtensorMap *tm_pool_k,
                                          const CUtensorMap *tm_pool_v, const CUtensorMap *tm_ws_k,
                                          const CUtensorMap *tm_ws_v, const CUtensorMap *tm_knew,
                                          const CUtensorMap *tm_vnew)
 {
+    using C = Cfg<D>;
+    constexpr int kStages = C::kStages, kTileBytes = C::kTileBytes;
     uint32_t ring_n = 0;                                   // loads issued before this piece
     bool ok = true;
     for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
@@ -817,24 +861,25 @@ __device__ __forceinline__ void tma_role(const Params &p, const Cta &c, const in
                     if (lane == 0 && i + KVP_L2_PREFETCH < cnt && src_j != 2) {
                         const CUtensorMap *tm = src_j == 0 ? (kv_j ? tm_pool_v : tm_pool_k) : (kv_j ? tm_ws_v : tm_ws_k);
                         asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(tm), "r"(0), "r"(row0_j), "r"(w.plane) : "memory");
-                        asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(tm), "r"(64), "r"(row0_j), "r"(w.plane) : "memory");
+                        if (D == 128)
+                            asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(tm), "r"(64), "r"(row0_j), "r"(w.plane) : "memory");
                     }
                 }
                 if (lane == 0) {
                     const uint32_t g = ring_n + (uint32_t)(q0 + i);
                     const uint32_t stage = g % kStages, use = g / kStages;
-                    if (use > 0) ok = mbar_wait(c.bar(kKvEmpty + stage), (use - 1) & 1, c.abort_flag, p.status, 10 + stage);
+                    if (use > 0) ok = mbar_wait(c.bar(C::kKvEmpty + stage), (use - 1) & 1, c.abort_flag, p.status, 10 + stage);
                     if (ok) {
-                        const uint32_t dst = c.smem_base + kOffRing + stage * kTileBytes;
-                        mbar_expect_tx(c.bar(kKvFull + stage), kTileBytes);
+                        const uint32_t dst = c.smem_base + C::kOffRing + stage * kTileBytes;
+                        mbar_expect_tx(c.bar(C::kKvFull + stage), kTileBytes);
                         if (src_i == 2) {
                             const CUtensorMap *tm = kv_i ? tm_vnew : tm_knew;
-                            tma_load_4d(dst, tm, 0, w.hk, row0_i, w.b, c.bar(kKvFull + stage));
-                            tma_load_4d(dst + kHalfBytes, tm, 64, w.hk, row0_i, w.b, c.bar(kKvFull + stage));
+                            tma_load_4d(dst, tm, 0, w.hk, row0_i, w.b, c.bar(C::kKvFull + stage));
+                            if (D == 128) tma_load_4d(dst + kHalfBytes, tm, 64, w.hk, row0_i, w.b, c.bar(C::kKvFull + stage));
                         } else {
                             const CUtensorMap *tm = src_i == 0 ? (kv_i ? tm_pool_v : tm_pool_k) : (kv_i ? tm_ws_v : tm_ws_k);
-                            tma_load_3d(dst, tm, 0, row0_i, w.plane, c.bar(kKvFull + stage));
-                            tma_load_3d(dst + kHalfBytes, tm, 64, row0_i, w.plane, c.bar(kKvFull + stage));
+                            tma_load_3d(dst, tm, 0, row0_i, w.plane, c.bar(C::kKvFull + stage));
+                            if (D == 128) tma_load_3d(dst + kHalfBytes, tm, 64, row0_i, w.plane, c.bar(C::kKvFull + stage));
                         }
                     }
                 }
@@ -852,9 +897,18 @@ struct MmaStream {
     Tile cur, nxt;
 };
 
+template <int D>
 __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
 {
-    const uint32_t idesc_pv = instr_desc(128, 1);
+    using C = Cfg<D>;
+    constexpr int kStages = C::kStages, kTileBytes = C::kTileBytes;
+    constexpr uint32_t kSteps = D / 16;                       // K-steps of Q K^T
+    constexpr uint32_t kRem16 = (C::kSplit ? kHalfBytes : kQBufBytes) >> 4;      // from the rotated Q to its remainders
+    const uint32_t idesc_pv = instr_desc(D, 1);
+    const bool one_buffer = !C::kSplit && p.precise, two_part = C::kSplit || p.precise;
+    // P of 16 keys (K-step kk) in the score columns: packed pairs one after the other, or per 32 keys 16 columns of
+    // pairs and 16 of remainders
+    auto p_col = [](int kk) { return C::kSplit ? (kk >> 1) * 32 + (kk & 1) * 8 : kk * 8; };
     MmaStream st[2];
     st[0].nP = st[0].nEpoch = st[0].nItems = st[0].qbuf = 0;
     st[1].nP = st[1].nEpoch = st[1].nItems = st[1].qbuf = 0;
@@ -874,42 +928,41 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
         }
         const Tile tl = ms.cur;
         if (k == 0 || tl.rope != ms.prev_rope) {                  // first tile of a document: its own Q buffer
-            ms.qbuf = p.precise ? 0 : (ms.nEpoch & 1);
-            ok = mbar_wait(c.bar(kQFull + 2 * s + ms.qbuf), (p.precise ? ms.nEpoch : ms.nEpoch >> 1) & 1, c.abort_flag, p.status, 20 + s);
+            ms.qbuf = one_buffer ? 0 : (ms.nEpoch & 1);
+            ok = mbar_wait(c.bar(C::kQFull + 2 * s + ms.qbuf), (one_buffer ? ms.nEpoch : ms.nEpoch >> 1) & 1, c.abort_flag, p.status, 20 + s);
             ++ms.nEpoch;
         }
         const int r = wq.mode ? 2 * k + s : k;
         const uint32_t g = base + (uint32_t)load_seq(wq.mode, wq.n, r, 0);
         const uint32_t stage = g % kStages, par = (g / kStages) & 1;
-        if (ok && !(shared_stage && s == 1)) ok = mbar_wait(c.bar(kKvFull + stage), par, c.abort_flag, p.status, 22);
+        if (ok && !(shared_stage && s == 1)) ok = mbar_wait(c.bar(C::kKvFull + stage), par, c.abort_flag, p.status, 22);
         ok = __all_sync(0xffffffffu, ok);                         // the lanes stay together
         if (!ok) return;
         tc_fence_after();
         const uint32_t n16 = max(16u, (uint32_t)(tl.n_keys + 15) & ~15u);
         const uint32_t idesc = instr_desc(n16, 0);
-        const uint32_t q_lo = desc_lo(c.smem_base + kOffQ + (2 * s + ms.qbuf) * kTileBytes, 16);
-        const uint32_t k_lo = desc_lo(c.smem_base + kOffRing + stage * kTileBytes, 16);
+        const uint32_t q_lo = desc_lo(c.smem_base + C::kOffQ + (2 * s + ms.qbuf) * kQBufBytes, 16);
+        const uint32_t k_lo = desc_lo(c.smem_base + C::kOffRing + stage * kTileBytes, 16);
         const uint32_t d = c.tmem + kColS + s * 128;
         mma_ss<0>(d, desc64(q_lo, kDescHi), desc64(k_lo, kDescHi), idesc);
 #pragma unroll
-        for (int kk = 1; kk < 8; ++kk) {                         // 16 columns per step: 32 bytes, second half 16 KB on
+        for (int kk = 1; kk < (int)kSteps; ++kk) {                         // 16 columns per step: 32 bytes, second half 16 KB on
             constexpr uint32_t kHalf16 = kHalfBytes >> 4;
             const uint32_t off = (kk >> 2) * kHalf16 + (kk & 3) * 2;
             mma_ss<1>(d, desc64(q_lo + off, kDescHi), desc64(k_lo + off, kDescHi), idesc);
         }
-        if (p.precise && tl.rope != 0) {                         // + (rounding remainder of the rotated Q) K^T
-            constexpr uint32_t kRem16 = kTileBytes >> 4;
+        if (two_part && tl.rope != 0) {                         // + (rounding remainder of the rotated Q) K^T
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk) {
+            for (int kk = 0; kk < (int)kSteps; ++kk) {
                 constexpr uint32_t kHalf16 = kHalfBytes >> 4;
                 const uint32_t off = (kk >> 2) * kHalf16 + (kk & 3) * 2;
                 mma_ss<1>(d, desc64(q_lo + kRem16 + off, kDescHi), desc64(k_lo + off, kDescHi), idesc);
             }
         }
-        tc_commit(c.bar(kSFull + s));
-        if (!shared_stage || s == 1) tc_commit(c.bar(kKvEmpty + stage));
+        tc_commit(c.bar(C::kSFull + s));
+        if (!shared_stage || s == 1) tc_commit(c.bar(C::kKvEmpty + stage));
         const bool last = (k + 1 == n_steps) || (ms.nxt.rope != tl.rope);
-        if (last) tc_commit(c.bar(kQFree + 2 * s + ms.qbuf));
+        if (last) tc_commit(c.bar(C::kQFree + 2 * s + ms.qbuf));
         ms.prev_rope = tl.rope;
         ms.prev_keys = tl.n_keys;
         ms.cur = ms.nxt;
@@ -927,7 +980,8 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
         uint32_t stK = ring_n % kStages, parK = (ring_n / kStages) & 1;                 // K(k), used at step k
         uint32_t stV = (ring_n + 1) % kStages, parV = ((ring_n + 1) / kStages) & 1;     // V(k - 1), used at step k
         auto advance = [](uint32_t &st_, uint32_t &par_) {                              // two loads further on
-            if (st_ == 0) st_ = 2; else { st_ -= 1; par_ ^= 1; }
+            st_ += 2;
+            if (st_ >= kStages) { st_ -= kStages; par_ ^= 1; }
         };
         int b0 = 0, nk_l = 0, rope_l = 0;
         auto refill = [&](int from) {
@@ -952,19 +1006,19 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
                 MmaStream &ms = st[s];
                 // ---- waits of the block ---------------------------------------------------------
                 if (s == 0) {                                 // the tiles first: they land while P is being formed
-                    if (k >= 1) ok = mbar_wait(c.bar(kKvFull + stV), parV, c.abort_flag, p.status, 23);
-                    if (k < n && ok) ok = mbar_wait(c.bar(kKvFull + stK), parK, c.abort_flag, p.status, 22);
+                    if (k >= 1) ok = mbar_wait(c.bar(C::kKvFull + stV), parV, c.abort_flag, p.status, 23);
+                    if (k < n && ok) ok = mbar_wait(c.bar(C::kKvFull + stK), parK, c.abort_flag, p.status, 22);
                 }
                 if (k >= 1) {
-                    if (ok) ok = mbar_wait(c.bar(kPFull + s), ms.nP & 1, c.abort_flag, p.status, 24 + s);
+                    if (ok) ok = mbar_wait(c.bar(C::kPFull + s), ms.nP & 1, c.abort_flag, p.status, 24 + s);
                     ++ms.nP;
                     if (ok && k == 1 && ms.nItems > 0)
-                        ok = mbar_wait(c.bar(kOFree + s), (ms.nItems - 1) & 1, c.abort_flag, p.status, 26 + s);
+                        ok = mbar_wait(c.bar(C::kOFree + s), (ms.nItems - 1) & 1, c.abort_flag, p.status, 26 + s);
                 }
                 if (k < n) {
                     if (newq) {
-                        ms.qbuf = p.precise ? 0 : (ms.nEpoch & 1);
-                        if (ok) ok = mbar_wait(c.bar(kQFull + 2 * s + ms.qbuf), (p.precise ? ms.nEpoch : ms.nEpoch >> 1) & 1, c.abort_flag, p.status, 20 + s);
+                        ms.qbuf = one_buffer ? 0 : (ms.nEpoch & 1);
+                        if (ok) ok = mbar_wait(c.bar(C::kQFull + 2 * s + ms.qbuf), (one_buffer ? ms.nEpoch : ms.nEpoch >> 1) & 1, c.abort_flag, p.status, 20 + s);
                         ++ms.nEpoch;
                     }
                 }
@@ -973,21 +1027,25 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
                 tc_fence_after();
                 if (k >= 1) {
                     // ---- O_s += P_s V of step k-1 ---------------------------------------------------
-                    const uint32_t v_lo = desc_lo(c.smem_base + kOffRing + stV * kTileBytes, kHalfBytes);
+                    const uint32_t v_lo = desc_lo(c.smem_base + C::kOffRing + stV * kTileBytes, kHalfBytes);
                     const uint32_t pa = c.tmem + kColS + s * 128;
                     const uint32_t oa = c.tmem + kColO + s * 128;
                     if (prev_nk == KVP_TILE_KEYS && k > 1) {
 #pragma unroll
-                        for (int kk = 0; kk < 8; ++kk)           // 16 keys per step: P advances 8 columns, V 2048 bytes
-                            mma_ts_c<1>(oa, pa + kk * 8, desc64(v_lo + kk * 128, kDescHi), idesc_pv);
+                        for (int kk = 0; kk < 8; ++kk) {         // 16 keys per step: V advances 2048 bytes
+                            mma_ts_c<1>(oa, pa + p_col(kk), desc64(v_lo + kk * 128, kDescHi), idesc_pv);
+                            if (C::kSplit) mma_ts_c<1>(oa, pa + p_col(kk) + 16, desc64(v_lo + kk * 128, kDescHi), idesc_pv);
+                        }
                     } else {
                         const int ksteps = max(1, (prev_nk + 15) >> 4);    // an empty tile still initialises O (P = 0)
-                        for (int kk = 0; kk < ksteps; ++kk)
-                            mma_ts(oa, pa + kk * 8, desc64(v_lo + kk * 128, kDescHi), idesc_pv, (k > 1 || kk > 0));
+                        for (int kk = 0; kk < ksteps; ++kk) {
+                            mma_ts(oa, pa + p_col(kk), desc64(v_lo + kk * 128, kDescHi), idesc_pv, (k > 1 || kk > 0));
+                            if (C::kSplit) mma_ts_c<1>(oa, pa + p_col(kk) + 16, desc64(v_lo + kk * 128, kDescHi), idesc_pv);
+                        }
                     }
-                    if (s == 1) tc_commit(c.bar(kKvEmpty + stV));
+                    if (s == 1) tc_commit(c.bar(C::kKvEmpty + stV));
                     if (k == n) {
-                        tc_commit(c.bar(kOFull + s));
+                        tc_commit(c.bar(C::kOFull + s));
                         ++ms.nItems;
                     }
                 }
@@ -995,28 +1053,27 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
                     // ---- S_s = Q_s K^T of step k ----------------------------------------------------
                     const uint32_t n16 = max(16u, (uint32_t)(nk + 15) & ~15u);   
                     const uint32_t idesc = instr_desc(n16, 0);
-                    const uint32_t q_lo = desc_lo(c.smem_base + kOffQ + (2 * s + ms.qbuf) * kTileBytes, 16);
-                    const uint32_t k_lo = desc_lo(c.smem_base + kOffRing + stK * kTileBytes, 16);
+                    const uint32_t q_lo = desc_lo(c.smem_base + C::kOffQ + (2 * s + ms.qbuf) * kQBufBytes, 16);
+                    const uint32_t k_lo = desc_lo(c.smem_base + C::kOffRing + stK * kTileBytes, 16);
                     const uint32_t d = c.tmem + kColS + s * 128;
                     mma_ss<0>(d, desc64(q_lo, kDescHi), desc64(k_lo, kDescHi), idesc);
 #pragma unroll
-                    for (int kk = 1; kk < 8; ++kk) {             // 16 columns per step: 32 bytes, second half 16 KB on
+                    for (int kk = 1; kk < (int)kSteps; ++kk) {             // 16 columns per step: 32 bytes, second half 16 KB on
                         constexpr uint32_t kHalf16 = kHalfBytes >> 4;
                         const uint32_t off = (kk >> 2) * kHalf16 + (kk & 3) * 2;
                         mma_ss<1>(d, desc64(q_lo + off, kDescHi), desc64(k_lo + off, kDescHi), idesc);
                     }
-                    if (p.precise && rope != 0) {                // + (rounding remainder of the rotated Q) K^T
-                        constexpr uint32_t kRem16 = kTileBytes >> 4;
+                    if (two_part && rope != 0) {                // + (rounding remainder of the rotated Q) K^T
 #pragma unroll
-                        for (int kk = 0; kk < 8; ++kk) {
+                        for (int kk = 0; kk < (int)kSteps; ++kk) {
                             constexpr uint32_t kHalf16 = kHalfBytes >> 4;
                             const uint32_t off = (kk >> 2) * kHalf16 + (kk & 3) * 2;
                             mma_ss<1>(d, desc64(q_lo + kRem16 + off, kDescHi), desc64(k_lo + off, kDescHi), idesc);
                         }
                     }
-                    tc_commit(c.bar(kSFull + s));
-                    if (s == 1) tc_commit(c.bar(kKvEmpty + stK));
-                    if (lastq) tc_commit(c.bar(kQFree + 2 * s + ms.qbuf));
+                    tc_commit(c.bar(C::kSFull + s));
+                    if (s == 1) tc_commit(c.bar(C::kKvEmpty + stK));
+                    if (lastq) tc_commit(c.bar(C::kQFree + 2 * s + ms.qbuf));
                 }
             };
             step(std::integral_constant<int, 0>{});
@@ -1046,29 +1103,33 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
                 const int r = w.mode ? 2 * (k - 1) + s : k - 1;
                 const uint32_t g = ring_n + (uint32_t)load_seq(w.mode, w.n, r, 1);
                 const uint32_t stage = g % kStages, par = (g / kStages) & 1;
-                if (!(shared_stage && s == 1)) ok = mbar_wait(c.bar(kKvFull + stage), par, c.abort_flag, p.status, 23);
-                if (ok) ok = mbar_wait(c.bar(kPFull + s), ms.nP & 1, c.abort_flag, p.status, 24 + s);
+                if (!(shared_stage && s == 1)) ok = mbar_wait(c.bar(C::kKvFull + stage), par, c.abort_flag, p.status, 23);
+                if (ok) ok = mbar_wait(c.bar(C::kPFull + s), ms.nP & 1, c.abort_flag, p.status, 24 + s);
                 ++ms.nP;
                 if (ok && k == 1 && ms.nItems > 0)
-                    ok = mbar_wait(c.bar(kOFree + s), (ms.nItems - 1) & 1, c.abort_flag, p.status, 26 + s);
+                    ok = mbar_wait(c.bar(C::kOFree + s), (ms.nItems - 1) & 1, c.abort_flag, p.status, 26 + s);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) return;
                 tc_fence_after();
-                const uint32_t v_lo = desc_lo(c.smem_base + kOffRing + stage * kTileBytes, kHalfBytes);
+                const uint32_t v_lo = desc_lo(c.smem_base + C::kOffRing + stage * kTileBytes, kHalfBytes);
                 const uint32_t pa = c.tmem + kColS + s * 128;
                 const uint32_t oa = c.tmem + kColO + s * 128;
                 if (ms.prev_keys == KVP_TILE_KEYS && k > 1) {
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk)               // 16 keys per step: P advances 8 columns, V 2048 bytes
-                        mma_ts_c<1>(oa, pa + kk * 8, desc64(v_lo + kk * 128, kDescHi), idesc_pv);
+                    for (int kk = 0; kk < 8; ++kk) {             // 16 keys per step: V advances 2048 bytes
+                        mma_ts_c<1>(oa, pa + p_col(kk), desc64(v_lo + kk * 128, kDescHi), idesc_pv);
+                        if (C::kSplit) mma_ts_c<1>(oa, pa + p_col(kk) + 16, desc64(v_lo + kk * 128, kDescHi), idesc_pv);
+                    }
                 } else {
                     const int ksteps = max(1, (ms.prev_keys + 15) >> 4);   // an empty tile still initialises O (P = 0)
-                    for (int kk = 0; kk < ksteps; ++kk)
-                        mma_ts(oa, pa + kk * 8, desc64(v_lo + kk * 128, kDescHi), idesc_pv, (k > 1 || kk > 0));
+                    for (int kk = 0; kk < ksteps; ++kk) {
+                        mma_ts(oa, pa + p_col(kk), desc64(v_lo + kk * 128, kDescHi), idesc_pv, (k > 1 || kk > 0));
+                        if (C::kSplit) mma_ts_c<1>(oa, pa + p_col(kk) + 16, desc64(v_lo + kk * 128, kDescHi), idesc_pv);
+                    }
                 }
-                if (!shared_stage || s == 1) tc_commit(c.bar(kKvEmpty + stage));
+                if (!shared_stage || s == 1) tc_commit(c.bar(C::kKvEmpty + stage));
                 if (k == steps[s]) {
-                    tc_commit(c.bar(kOFull + s));
+                    tc_commit(c.bar(C::kOFull + s));
                     ++ms.nItems;
                 }
             }
@@ -1082,24 +1143,26 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
     }
     __syncwarp();
     if (!ok) {                      // drain whatever was issued before giving TMEM back
-        tc_commit(c.bar(kDrain));
+        tc_commit(c.bar(C::kDrain));
         const uint64_t t0 = global_ns();
-        while (!mbar_try_wait(c.bar(kDrain), 0) && global_ns() - t0 < 100000000ull) {}
+        while (!mbar_try_wait(c.bar(C::kDrain), 0) && global_ns() - t0 < 100000000ull) {}
     }
 }
 
+template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_pool_k, const __grid_constant__ CUtensorMap tm_pool_v,
                   const __grid_constant__ CUtensorMap tm_ws_k, const __grid_constant__ CUtensorMap tm_ws_v,
                   const __grid_constant__ CUtensorMap tm_knew, const __grid_constant__ CUtensorMap tm_vnew,
                   const Params p)
 {
+    using C = Cfg<D>;
     extern __shared__ char smem_raw[];
     Cta c;
     c.smem = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     c.smem_base = smem_u32(c.smem);
-    c.bar0 = c.smem_base + kOffBar;
-    volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(c.smem + kOffBar + 8 * kNumBars);
+    c.bar0 = c.smem_base + C::kOffBar;
+    volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(c.smem + C::kOffBar + 8 * C::kNumBars);
     c.abort_flag = tmem_slot + 1;
     c.item_begin = __ldg(p.cta_begin + blockIdx.x);
     c.item_end = __ldg(p.cta_begin + blockIdx.x + 1);
@@ -1108,22 +1171,22 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_pool_k, const __grid_co
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     if (tid == 0) {
-        for (int s = 0; s < kStages; ++s) {
-            mbar_init(c.bar(kKvFull + s), 1);
-            mbar_init(c.bar(kKvEmpty + s), 1);
+        for (int s = 0; s < C::kStages; ++s) {
+            mbar_init(c.bar(C::kKvFull + s), 1);
+            mbar_init(c.bar(C::kKvEmpty + s), 1);
         }
         for (int s = 0; s < 4; ++s) {
-            mbar_init(c.bar(kQFull + s), 128);
-            mbar_init(c.bar(kQFree + s), 1);
+            mbar_init(c.bar(C::kQFull + s), 128);
+            mbar_init(c.bar(C::kQFree + s), 1);
         }
         for (int s = 0; s < 2; ++s) {
-            mbar_init(c.bar(kSFull + s), 1);
-            mbar_init(c.bar(kPFull + s), 128);
-            mbar_init(c.bar(kOFull + s), 1);
-            mbar_init(c.bar(kOFree + s), 128);
+            mbar_init(c.bar(C::kSFull + s), 1);
+            mbar_init(c.bar(C::kPFull + s), 128);
+            mbar_init(c.bar(C::kOFull + s), 1);
+            mbar_init(c.bar(C::kOFree + s), 128);
         }
-        mbar_init(c.bar(kMlFull), 128);
-        mbar_init(c.bar(kDrain), 1);
+        mbar_init(c.bar(C::kMlFull), 128);
+        mbar_init(c.bar(C::kDrain), 1);
         *c.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -1139,16 +1202,16 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_pool_k, const __grid_co
     c.tmem = *tmem_slot;
 
     if (warp < 8) {
-        softmax_role(p, c, warp >> 2, tid & 127);
+        softmax_role<D>(p, c, warp >> 2, tid & 127);
     } else if (warp < 12) {
-        producer_role(p, c, tid - 256);
+        producer_role<D>(p, c, tid - 256);
     } else {
         if (warp == 12) {
-            mma_role(p, c);
+            mma_role<D>(p, c);
         } else if (warp == 13) {
-            tma_role(p, c, lane, &tm_pool_k, &tm_pool_v, &tm_ws_k, &tm_ws_v, &tm_knew, &tm_vnew);
+            tma_role<D>(p, c, lane, &tm_pool_k, &tm_pool_v, &tm_ws_k, &tm_ws_v, &tm_knew, &tm_vnew);
         } else {
-            append_role(p, c, tid - 448);
+            append_role<D>(p, c, tid - 448);
         }
     }
 
@@ -1166,7 +1229,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_pool_k, const __grid_co
 }
 
 // ---- merge of partial results -------------------------------------------------------------------------------
-// A partial holds, per 128-row query tile: un-normalised O (fp32, stored [32 float4 columns][128 rows]), the
+// A partial holds, per 128-row query tile: un-normalised O (fp32, stored [D / 4 float4 columns][128 rows]), the
 // running max m of the raw scores and the sum l of exp2((s - m) * c).  Block = 32 rows of one query tile; lanes
 // run along rows while reading (coalesced).  The partials of a tile are `n` blocks `stride` apart (the slots of
 // a unit cut into pieces: consecutive; the same tile on every rank of a prefix-sharded request: one rank buffer
@@ -1174,26 +1237,28 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_pool_k, const __grid_co
 // written 256 contiguous bytes at a time - or again a partial, in the canonical order of a rank buffer
 // [request][kv head][row tile] (KVP_PARTIAL: what a rank hands to the exchange).
 struct MergeOut {
-    __nv_bfloat16 *out;         // final: [batch][q_len][n_q][128]
+    __nv_bfloat16 *out;         // final: [batch][q_len][n_q][D]
     float *lse;
-    float4 *part_o;             // or partial: [tiles][32][128] float4 ...
+    float4 *part_o;             // or partial: [tiles][D / 4][128] float4 ...
     float2 *part_ml;            // ... and [tiles][128] (m, l)
 };
 
+template <int D>
 __device__ __forceinline__ void merge_tile(int b, int hk, int row_base, int item_q_len, const float4 *po, const float2 *pml,
                                            int n, long long stride_o, long long stride_ml, int q_len, int n_q, int n_kv,
                                            int group, float scale, const MergeOut &mo)
 {
-    __shared__ uint2 tile[32][33];
+    constexpr int kC = D / 32;                                  // float4 columns per warp
+    __shared__ uint2 tile[32][D / 4 + 1];
     const int lane = threadIdx.x & 31, wv = threadIdx.x >> 5;
     const int row = blockIdx.y * 32 + lane;                     // row of the 128-row query tile
     const int n_rows = group * (item_q_len ? item_q_len : q_len);       // q_len stays the stride of the padded tensors
     const float c2 = scale * 1.4426950408889634f;
     float M = -INFINITY;
     float L = 0.f;
-    float4 o[4];
+    float4 o[kC];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) o[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int j = 0; j < kC; ++j) o[j] = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int s = 0; s < n; ++s) {
         const float2 ml = pml[s * stride_ml + row];
         if (ml.y > 0.f) M = fmaxf(M, ml.x);
@@ -1204,7 +1269,7 @@ __device__ __forceinline__ void merge_tile(int b, int hk, int row_base, int item
         const float w = exp2f((ml.x - M) * c2);
         L += w * ml.y;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < kC; ++j) {
             const float4 a = po[s * stride_o + (wv + 8 * j) * KVP_TILE_ROWS + row];
             o[j].x += w * a.x; o[j].y += w * a.y; o[j].z += w * a.z; o[j].w += w * a.w;
         }
@@ -1212,13 +1277,13 @@ __device__ __forceinline__ void merge_tile(int b, int hk, int row_base, int item
     if (mo.part_o != nullptr) {                                 // stays a partial: un-normalised, against the max M
         const long long c = ((long long)b * n_kv + hk) * ((group * q_len + KVP_TILE_ROWS - 1) / KVP_TILE_ROWS) + row_base / KVP_TILE_ROWS;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) mo.part_o[(c * 32 + wv + 8 * j) * KVP_TILE_ROWS + row] = o[j];
+        for (int j = 0; j < kC; ++j) mo.part_o[(c * (D / 4) + wv + 8 * j) * KVP_TILE_ROWS + row] = o[j];
         if (wv == 0) mo.part_ml[c * KVP_TILE_ROWS + row] = make_float2(L > 0.f ? M : -1e30f, L);
         return;
     }
     const float inv = L > 0.f ? 1.f / L : 0.f;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < kC; ++j) {
         uint2 u;
         u.x = pack_bf16(o[j].x * inv, o[j].y * inv);
         u.y = pack_bf16(o[j].z * inv, o[j].w * inv);
@@ -1228,26 +1293,29 @@ __device__ __forceinline__ void merge_tile(int b, int hk, int row_base, int item
     if (wv == 0 && r < n_rows && mo.lse != nullptr)
         mo.lse[((long long)b * n_q + hk * group + r % group) * q_len + r / group] = M * scale + logf(L);
     __syncthreads();
-    // 8 threads per output row, 32 bytes each
+    // 8 threads per output row, D / 4 bytes each
     const int orow = threadIdx.x >> 3, j8 = threadIdx.x & 7;
     const int r2 = row_base + blockIdx.y * 32 + orow;
     if (r2 < n_rows) {
         const int i = r2 / group, h = hk * group + r2 % group;
-        uint4 *dst = reinterpret_cast<uint4 *>(mo.out + (((long long)b * q_len + i) * n_q + h) * 128) + 2 * j8;
-        const uint2 a0 = tile[orow][4 * j8], a1 = tile[orow][4 * j8 + 1], a2 = tile[orow][4 * j8 + 2], a3 = tile[orow][4 * j8 + 3];
-        dst[0] = make_uint4(a0.x, a0.y, a1.x, a1.y);
-        dst[1] = make_uint4(a2.x, a2.y, a3.x, a3.y);
+        uint4 *dst = reinterpret_cast<uint4 *>(mo.out + (((long long)b * q_len + i) * n_q + h) * D) + (D / 64) * j8;
+#pragma unroll
+        for (int v = 0; v < D / 64; ++v) {
+            const uint2 a0 = tile[orow][2 * ((D / 64) * j8 + v)], a1 = tile[orow][2 * ((D / 64) * j8 + v) + 1];
+            dst[v] = make_uint4(a0.x, a0.y, a1.x, a1.y);
+        }
     }
 }
 
 // The partial slots of the units of one launch.  Grid (merge item, 4).
+template <int D>
 __global__ void __launch_bounds__(256)
 merge_list_kernel(const kvp_merge_item *__restrict__ merges, int q_len, int n_q, int n_kv, int group, float scale,
                   const float *__restrict__ part_o, const float2 *__restrict__ part_ml, MergeOut mo)
 {
     const kvp_merge_item mi = merges[blockIdx.x];
-    merge_tile(mi.b, mi.hk, mi.row_base, mi.pad[0], reinterpret_cast<const float4 *>(part_o) + (long long)mi.slot0 * (32 * KVP_TILE_ROWS),
-               part_ml + (long long)mi.slot0 * KVP_TILE_ROWS, mi.n_slots, 32 * KVP_TILE_ROWS, KVP_TILE_ROWS, q_len, n_q, n_kv,
+    merge_tile<D>(mi.b, mi.hk, mi.row_base, mi.pad[0], reinterpret_cast<const float4 *>(part_o) + (long long)mi.slot0 * (D / 4 * KVP_TILE_ROWS),
+               part_ml + (long long)mi.slot0 * KVP_TILE_ROWS, mi.n_slots, D / 4 * KVP_TILE_ROWS, KVP_TILE_ROWS, q_len, n_q, n_kv,
                group, scale, mo);
 }
 
@@ -1259,16 +1327,18 @@ merge_ranks_kernel(const char *__restrict__ parts, int n_parts, long long part_b
 {
     const int c = blockIdx.x;
     const int rt = c % n_rt, hk = (c / n_rt) % n_kv, b = c / (n_rt * n_kv);
-    merge_tile(b, hk, rt * KVP_TILE_ROWS, 0, reinterpret_cast<const float4 *>(parts) + (long long)c * (32 * KVP_TILE_ROWS),
+    merge_tile<128>(b, hk, rt * KVP_TILE_ROWS, 0, reinterpret_cast<const float4 *>(parts) + (long long)c * (32 * KVP_TILE_ROWS),
                reinterpret_cast<const float2 *>(parts + ml_offset) + (long long)c * KVP_TILE_ROWS, n_parts, part_bytes / 16,
                part_bytes / 8, q_len, n_q, n_kv, group, scale, mo);
 }
 
 }  // namespace
 
-cudaError_t kvp_attn_sm100_prepare(void)
+cudaError_t kvp_attn_sm100_prepare(int32_t head_dim)
 {
-    return cudaFuncSetAttribute(attn_sm100_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (head_dim == 64)
+        return cudaFuncSetAttribute(attn_sm100_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<64>::kSmemBytes);
+    return cudaFuncSetAttribute(attn_sm100_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<128>::kSmemBytes);
 }
 
 cudaError_t kvp_launch_attn_sm100(const kvp_shape &sh, const kvp_attn2_args &a, const CUtensorMap &tm_pool_k,
@@ -1303,9 +1373,11 @@ cudaError_t kvp_launch_attn_sm100(const kvp_shape &sh, const kvp_attn2_args &a, 
     p.ws_v = (uint4 *)a.ws_v;
     p.ws_rows = sh.ws_rows;
     // without tail_direct the two query maps are never dereferenced: any valid map will do
-    attn_sm100_kernel<<<a.n_ctas, kThreads, kSmemBytes, st>>>(tm_pool_k, tm_pool_v, tm_ws_k, tm_ws_v,
-                                                              a.tail_direct ? a.tm_knew : tm_ws_k,
-                                                              a.tail_direct ? a.tm_vnew : tm_ws_v, p);
+    const CUtensorMap &tk = a.tail_direct ? a.tm_knew : tm_ws_k, &tv = a.tail_direct ? a.tm_vnew : tm_ws_v;
+    if (sh.head_dim == 64)
+        attn_sm100_kernel<64><<<a.n_ctas, kThreads, Cfg<64>::kSmemBytes, st>>>(tm_pool_k, tm_pool_v, tm_ws_k, tm_ws_v, tk, tv, p);
+    else
+        attn_sm100_kernel<128><<<a.n_ctas, kThreads, Cfg<128>::kSmemBytes, st>>>(tm_pool_k, tm_pool_v, tm_ws_k, tm_ws_v, tk, tv, p);
     return cudaGetLastError();
 }
 
@@ -1323,8 +1395,11 @@ cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_
         mo.part_o = reinterpret_cast<float4 *>(part_out);
         mo.part_ml = reinterpret_cast<float2 *>((char *)part_out + (uint64_t)part_tiles * (32ull * KVP_TILE_ROWS * 16));
     }
-    merge_list_kernel<<<dim3(n_merges, KVP_TILE_ROWS / 32), 256, 0, st>>>(merges, q_len, sh.n_q_heads, sh.n_kv_heads, sh.group,
-                                                                        sh.scale, partial_o, partial_ml, mo);
+    const dim3 grid(n_merges, KVP_TILE_ROWS / 32);
+    if (sh.head_dim == 64)
+        merge_list_kernel<64><<<grid, 256, 0, st>>>(merges, q_len, sh.n_q_heads, sh.n_kv_heads, sh.group, sh.scale, partial_o, partial_ml, mo);
+    else
+        merge_list_kernel<128><<<grid, 256, 0, st>>>(merges, q_len, sh.n_q_heads, sh.n_kv_heads, sh.group, sh.scale, partial_o, partial_ml, mo);
     return cudaGetLastError();
 }
 

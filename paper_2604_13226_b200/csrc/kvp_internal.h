@@ -265,7 +265,7 @@ struct kvp_attn2_args {
     char *ws_k, *ws_v;
     CUtensorMap tm_knew, tm_vnew;
 };
-cudaError_t kvp_attn_sm100_prepare(void);
+cudaError_t kvp_attn_sm100_prepare(int32_t head_dim);
 cudaError_t kvp_launch_attn_sm100(const kvp_shape &sh, const kvp_attn2_args &a, const CUtensorMap &tm_pool_k,
                                   const CUtensorMap &tm_pool_v, const CUtensorMap &tm_ws_k,
                                   const CUtensorMap &tm_ws_v, cudaStream_t st);
