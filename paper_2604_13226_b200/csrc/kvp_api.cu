@@ -20,7 +20,7 @@ constexpr uint64_t kPlanAlign = 64;    // arrays of a plan blob
 inline uint64_t round_up(uint64_t x, uint64_t a) { return (x + a - 1) / a * a; }
 
 struct ws_layout {
-    uint64_t status, half_turns, slots, slot_stride, slot_plan, slot_sched, slot_k, slot_v, partial_o, partial_ml, q_scratch, total;
+    uint64_t status, half_turns, slots, slot_stride, slot_plan, slot_sched, slot_k, slot_v, partial_o, partial_ml, arrived, q_scratch, total;
     uint64_t rows_bytes;
 };
 
@@ -112,6 +112,7 @@ ws_layout workspace_layout(const kvp_config *c)
     w.slots = o;    o += w.slot_stride * c->max_assemblies;
     w.partial_o = o;  o = round_up(o + (uint64_t)KVP_MAX_SPLIT_UNITS * KVP_TILE_ROWS * c->head_dim * 4, kAlign);
     w.partial_ml = o; o = round_up(o + (uint64_t)KVP_MAX_SPLIT_UNITS * KVP_TILE_ROWS * 8, kAlign);
+    w.arrived = o;    o = round_up(o + 4ull * KVP_CORE_UNITS, kAlign);
     w.q_scratch = o;  o = round_up(o + (uint64_t)c->max_batch * c->max_query_tokens * c->n_q_heads * c->head_dim * e, kAlign);
     w.total = o;
     return w;
@@ -221,7 +222,8 @@ int find_slot(kvp_ctx *ctx, int32_t assembly_id)
 // fewer tiles.  Counted in single-stream tiles.
 constexpr int kPieceCost = 4;
 
-constexpr double kTcMinFlops64 = 4e8;
+// 0.08 Gflop: 11-17 us against 13-24; 0.12-0.15: 21 against 23; 0.23: 29 against 25; 2.3: 113 against 25.
+constexpr double kTcMinFlops64 = 1.5e8;
 
 // q_lens: nullptr, or one query length per request (<= q_len, the stride of the padded tensors); a request's
 // work records and merge items then carry its own length.
@@ -613,6 +615,7 @@ int32_t kvp_create(const kvp_config *cfg, kvp_ctx **out)
     }
     ctx->partial_o = (float *)(ws + w.partial_o);
     ctx->partial_ml = (float2 *)(ws + w.partial_ml);
+    ctx->arrived = (int32_t *)(ws + w.arrived);
     ctx->q_scratch = ws + w.q_scratch;
 
     // angles are formed on the device as (position offset) x (theta_i / pi), in half turns: sincospi reduces exactly
@@ -651,6 +654,7 @@ int32_t kvp_create(const kvp_config *cfg, kvp_ctx **out)
         if (cudaEventCreateWithFlags(&ctx->load_done[l], cudaEventDisableTiming) != cudaSuccess)
             return bail(KVP_ERR_CUDA, "load event creation failed");
 
+    if (kvp_attn_core_prepare(sh) != cudaSuccess) return bail(KVP_ERR_CUDA, "CUDA-core kernel attribute setup failed");
     if (sh.dtype == KVP_DTYPE_BF16 && prop.major == 10) {
         void *fn = nullptr;
         cudaDriverEntryPointQueryResult qres;
@@ -1171,11 +1175,13 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
     int launches = 0;
     bool fast = ctx->have_tma && !(flags & KVP_FORCE_SIMPLE);
     if (fast && sh.head_dim == 64) {
-        // The tcgen05 kernel has a start of several microseconds (tables, first Q tile, pipeline fill) and a merge launch
-        // behind it; below kTcMinFlops64 the CUDA-core kernel is done by then.  It also takes any alignment.
+        // Small calls stay on the CUDA cores: the tcgen05 kernel has a start of several microseconds (tables, first Q
+        // tile, pipeline fill) and a merge launch behind it, the CUDA-core kernel is one launch and done by then.  The
+        // work is counted as that kernel does it, in 16-row tiles.  It also takes any alignment.
         double keys = 0.0;
         for (int b = 0; b < as.batch; ++b) keys += as.items[b].prefix_len + q_pos0 + q_len;
-        fast = 4.0 * sh.head_dim * sh.n_q_heads * q_len * keys >= kTcMinFlops64 && (((uintptr_t)q | (uintptr_t)out) & 15) == 0;
+        const double rows = (double)(((int64_t)sh.group * q_len + 15) / 16 * 16);
+        fast = 4.0 * sh.head_dim * sh.n_kv_heads * rows * keys >= kTcMinFlops64 && (((uintptr_t)q | (uintptr_t)out) & 15) == 0;
     }
     if (q_lens && !(tc128 && fast)) return fail(ctx, KVP_ERR_UNSUPPORTED, "query_prefill_ragged: needs the tcgen05 kernel (bf16, head_dim 128, sm_100)");
     // plain prefill on the two-stream kernel: it reads the query block's K/V from k_new / v_new and appends them itself
@@ -1189,7 +1195,9 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
         a.tail_direct = 1;
     if (q_lens && !a.tail_direct)
         return fail(ctx, KVP_ERR_UNSUPPORTED, "query_prefill_ragged: needs the tcgen05 kernel with its own append (bf16, head_dim 128, 16-byte aligned k_new / v_new)");
-    if (!a.tail_direct && !skip_block) {
+    // the CUDA-core kernel does the same when nothing has to be rotated and no row was appended before
+    const bool core_append = !fast && ctx->fused_append && !rope_query && q_pos0 == 0 && (((uintptr_t)k_new | (uintptr_t)v_new) & 15) == 0;
+    if (!a.tail_direct && !skip_block && !core_append) {
         KVP_CUDA(ctx, kvp_launch_append(sh, plan, as.batch, q_len, q_pos0, q, k_new, v_new, ctx->slot_k[slot], ctx->slot_v[slot],
                                         layer, rope_query, ctx->half_turns, ctx->q_scratch, st));
         ++launches;
@@ -1202,8 +1210,14 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
     int32_t ctas = 0, splits = 1;
     if (!fast) {
         KVP_CUDA(ctx, time_edge(ctx, 0, 0, st));
-        KVP_CUDA(ctx, kvp_launch_attn_simple(sh, plan, as.batch, q_len, q_pos0, layer, q_used, ctx->pool_k, ctx->pool_v,
-                                             ctx->slot_k[slot], ctx->slot_v[slot], out, lse, &ctas, st));
+        int32_t n_tiles = 0;
+        for (const kvp_item &it : as.items) n_tiles = std::max(n_tiles, it.tile_end - it.tile_begin);
+        n_tiles += (q_pos0 + q_len - 1) / KVP_TILE_KEYS + 1;
+        const kvp_core_ws cw = {ctx->partial_o, ctx->partial_ml, ctx->arrived, (int64_t)KVP_MAX_SPLIT_UNITS * KVP_TILE_ROWS,
+                                KVP_CORE_UNITS, ctx->sm_count, core_append ? k_new : nullptr, core_append ? v_new : nullptr,
+                                ctx->slot_k[slot], ctx->slot_v[slot]};
+        KVP_CUDA(ctx, kvp_launch_attn_core(sh, plan, as.batch, q_len, q_pos0, layer, q_used, ctx->pool_k, ctx->pool_v,
+                                           ctx->slot_k[slot], ctx->slot_v[slot], n_tiles, cw, out, lse, &ctas, st));
         KVP_CUDA(ctx, time_edge(ctx, 0, 1, st));
         ++launches;
         ctx->last_kind = 0;

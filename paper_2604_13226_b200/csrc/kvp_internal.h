@@ -14,6 +14,7 @@
 #define KVP_TILE_ROWS 128      // packed query rows per CTA tile (MMA M)
 #define KVP_CHUNK_ROWS 32      // rows per gather work item
 #define KVP_MAX_SPLIT_UNITS 2048   // partial slots (128 query rows each) in the workspace
+#define KVP_CORE_UNITS 2048        // row tiles the CUDA-core kernel may split
 #define KVP_SCHED_RING 8       // pinned staging buffers for work lists
 
 // ---- device-visible plan records (written by the host planner, uploaded once per assembly) -----
@@ -194,6 +195,7 @@ struct kvp_ctx {
     void *encode_tiled = nullptr;          // cuTensorMapEncodeTiled
     float *partial_o = nullptr;            // [units][128][head_dim]
     float2 *partial_ml = nullptr;          // [units][128] (running max, running sum)
+    int32_t *arrived = nullptr;            // counters of the CUDA-core kernel's split row tiles
     char *q_scratch = nullptr;
     float2 *q_rope = nullptr;              // [max_batch*max_query][head_dim/2] for KVP_ROPE_QUERY
 
@@ -240,10 +242,24 @@ cudaError_t kvp_launch_export(const kvp_shape &sh, const kvp_plan_dev &plan, int
 cudaError_t kvp_launch_segment_mass(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t batch, int32_t q_len,
                                     int32_t q_pos0, int32_t layer, const void *q, const float *lse, const char *pool_k,
                                     const char *ws_k, float *mass, int32_t n_cols, cudaStream_t st);
-cudaError_t kvp_launch_attn_simple(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t batch, int32_t q_len,
-                                   int32_t q_pos0, int32_t layer, const void *q, const char *pool_k, const char *pool_v,
-                                   const char *ws_k, const char *ws_v, void *out, float *lse, int32_t *ctas,
-                                   cudaStream_t st);
+// Where the CUDA-core attention kernel leaves the rows of a split key range.
+struct kvp_core_ws {
+    float *partial_o;
+    float2 *partial_ml;
+    int32_t *arrived;          // max_units counters, zero between launches
+    int64_t max_rows, max_units;
+    int32_t sm_count;
+    // not null: the kernel reads the query block's rows from these ([batch][q_len][Hkv][d], 16-byte aligned) and copies
+    // them behind the prefix (ws_k, ws_v) itself; null: they are there already
+    const void *k_new, *v_new;
+    char *ws_k, *ws_v;
+};
+cudaError_t kvp_attn_core_prepare(const kvp_shape &sh);
+// n_tiles: most key tiles (causal and prefix) of any request
+cudaError_t kvp_launch_attn_core(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t batch, int32_t q_len, int32_t q_pos0,
+                                 int32_t layer, const void *q, const char *pool_k, const char *pool_v, const char *ws_k,
+                                 const char *ws_v, int32_t n_tiles, const kvp_core_ws &ws, void *out, float *lse, int32_t *ctas,
+                                 cudaStream_t st);
 
 struct kvp_attn2_args {
     kvp_plan_dev plan;

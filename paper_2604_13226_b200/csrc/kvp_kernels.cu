@@ -1,7 +1,9 @@
 // CUDA-core kernels of the composed-cache path: packet registration (layout change), gather with
-// RoPE re-basing (Eq. 1), query K/V append, cache export, a plain fp32 attention kernel that reads
-// packets in place through the tile list, and the split-KV merge.
+// RoPE re-basing (Eq. 1), query K/V append, cache export and an fp32 attention kernel that reads
+// packets in place through the tile list.
 #include <cuda_bf16.h>
+
+#include <algorithm>
 
 #include "kvp_internal.h"
 
@@ -275,50 +277,121 @@ __global__ void export_kernel(kvp_plan_dev plan, int b, int layer, int prefix_le
     }
 }
 
-// ---- plain fp32 attention over [tail tiles | prefix tiles] -----------------------------------------
-// 16 packed rows (query token i, head-in-group) per CTA, 32 keys per step, online softmax in fp32.
-// Keys still carrying an offset are rotated here as Eq. 1 states it (on K, in fp32).
-template <typename T, int D>
-__global__ void __launch_bounds__(128)
-attn_simple_kernel(kvp_plan_dev plan, int q_len, int q_pos0, int layer, const T *__restrict__ q, const char *__restrict__ pool_k,
-                   const char *__restrict__ pool_v, const char *__restrict__ ws_k, const char *__restrict__ ws_v,
-                   int64_t pool_rows, int64_t ws_rows, int n_q, int n_kv, int group, int pairing, float scale,
-                   T *__restrict__ out, float *__restrict__ lse)
+// ---- fp32 attention over [tail tiles | prefix tiles] on the CUDA cores ------------------------------
+// Any dtype and head dimension; every product, sum and exponential in fp32, keys still carrying an offset rotated here
+// as Eq. 1 states it (on K, in fp32).  A CTA takes BM = 4 TY packed rows (query token i, head-in-group) of one (request,
+// kv head) and a contiguous part of its 64-key blocks: split part `blockIdx.x % splits` of the range.  Thread (ty, tx)
+// holds rows 4 ty .. + 3: of S the keys tx + TX j, of O the columns tx * V .. in V-wide pieces - 4 x 4 products per pair
+// of 16-byte shared-memory words, so that the FMA pipe and not shared memory is the limit with BM = 64.  P takes the
+// place of K once the scores are formed.  When the range is split the parts leave un-normalised rows in global memory,
+// and the CTA that arrives last (a counter per row tile, which it clears again) combines them: one launch, no waiting.
+// Why: 16 CTAs of one row tile each walked all keys in a serial chain, 80 us for 3 x 128 documents and 32 tokens.
+struct CorePart {
+    float *o;                  // [row tile][split][BM][D]
+    float2 *ml;                // [row tile][split][BM]
+    int32_t *arrived;          // [row tile], zero between launches
+};
+
+// packed fp32 pairs: two products per instruction, so that the FMA pipe is not held back by instruction issue
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
 {
-    constexpr int RB = 16, KC = 32, HALF = D / 2;
-    __shared__ float Qs[RB][D];
-    __shared__ float Ks[KC][D + 1];
-    __shared__ float Vs[KC][D];
-    __shared__ float Ps[RB][KC];
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t both(float x)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float2 halves(uint64_t r)
+{
+    float2 f;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(r));
+    return f;
+}
 
-    const int hk = blockIdx.y, b = blockIdx.z;
+template <int N> struct VecOf;
+template <> struct VecOf<2> { typedef float2 type; };
+template <> struct VecOf<4> { typedef float4 type; };
+
+template <typename T, int D, int TY, int TX>
+__global__ void __launch_bounds__(TY *TX, 512 / (TY * TX))
+attn_core_kernel(kvp_plan_dev plan, int q_len, int q_pos0, int layer, const T *__restrict__ q, const char *__restrict__ pool_k,
+                 const char *__restrict__ pool_v, const char *__restrict__ ws_k, const char *__restrict__ ws_v,
+                 const uint4 *__restrict__ k_new, const uint4 *__restrict__ v_new, char *__restrict__ ws_k_out,
+                 char *__restrict__ ws_v_out, int64_t pool_rows, int64_t ws_rows, int n_q, int n_kv, int group, int pairing,
+                 float scale, int splits, CorePart part, T *__restrict__ out, float *__restrict__ lse)
+{
+    constexpr int BM = 4 * TY, BN = 64, NT = TY * TX, HALF = D / 2, LD = D + 4, LP = BN + 4;
+    constexpr int KN = BN / TX;                              // keys per thread
+    constexpr int V = D / TX < 4 ? D / TX : 4;               // width of a piece of O's columns
+    constexpr int PC = D / TX / V;                           // pieces per thread
+    constexpr int EV = Elem<T>::kPerVec;
+    typedef typename VecOf<V>::type VT;
+    extern __shared__ float sm[];
+    float *Qs = sm, *Ks = Qs + BM * LD, *Vs = Ks + BN * LD, *Ps = Ks;
+    __shared__ int last_in;
+
+    const int hk = blockIdx.y, b = blockIdx.z, rt = blockIdx.x / splits, sp = blockIdx.x % splits;
     const kvp_item it = plan.items[(layer * n_kv + hk) * plan.item_stride + b];
-    const int n_rows = group * q_len;
-    const int row = threadIdx.x / 8, sub = threadIdx.x % 8;
-    const int r = blockIdx.x * RB + row;
-    const bool valid = r < n_rows;
-    const int i = valid ? r / group : q_len - 1;
-    const int h = hk * group + (valid ? r % group : 0);
+    const int n_rows = group * q_len, row0 = rt * BM;
     const int plane = layer * n_kv + hk;
+    const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
 
-    for (int w = threadIdx.x; w < RB * D; w += blockDim.x) {
-        const int rr = blockIdx.x * RB + w / D, c = w % D;
-        float x = 0.f;
-        if (rr < n_rows) x = Elem<T>::to_f32(q[(((int64_t)b * q_len + rr / group) * n_q + hk * group + rr % group) * D + c]);
-        Qs[w / D][c] = x;
+    if (((uintptr_t)q & 15) == 0) {
+#pragma unroll
+        for (int u = 0; u < BM * D / EV / NT; ++u) {
+            const int w = threadIdx.x + u * NT, rr = row0 + w / (D / EV), c = w % (D / EV) * EV;
+            Vec16<T> x;
+            x.u = make_uint4(0, 0, 0, 0);
+            if (rr < n_rows)
+                x.u = __ldg(reinterpret_cast<const uint4 *>(q + (((int64_t)b * q_len + rr / group) * n_q + hk * group + rr % group) * D + c));
+#pragma unroll
+            for (int e = 0; e < EV; e += 4)
+                *reinterpret_cast<float4 *>(Qs + (w / (D / EV)) * LD + c + e) =
+                    make_float4(Elem<T>::to_f32(x.e[e]), Elem<T>::to_f32(x.e[e + 1]), Elem<T>::to_f32(x.e[e + 2]), Elem<T>::to_f32(x.e[e + 3]));
+        }
+    } else {                                                 // any element-aligned q is taken
+        for (int w = threadIdx.x; w < BM * D; w += NT) {
+            const int rr = row0 + w / D, c = w % D;
+            float x = 0.f;
+            if (rr < n_rows) x = Elem<T>::to_f32(q[(((int64_t)b * q_len + rr / group) * n_q + hk * group + rr % group) * D + c]);
+            Qs[(w / D) * LD + c] = x;
+        }
+    }
+    int lim[4];                                              // keys of the query block visible to row r: [0, lim)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) lim[r] = q_pos0 + min(row0 + 4 * ty + r, n_rows - 1) / group + 1;
+
+    // tail keys: rows appended earlier, then this call's, as far as this row tile sees them (the first one, which
+    // appends, walks them all)
+    const int i_max = k_new != nullptr && rt == 0 ? q_len - 1 : min(n_rows - 1, row0 + BM - 1) / group;
+    const int n_tail = (q_pos0 + i_max) / KVP_TILE_KEYS + 1;
+    const int n_blk = 2 * (n_tail + it.tile_end - it.tile_begin);
+    const int blk0 = (int)((int64_t)n_blk * sp / splits), blk1 = (int)((int64_t)n_blk * (sp + 1) / splits);
+
+    constexpr int AC = PC * V / 2;
+    float m[4], l[4];
+    uint64_t acc[4][AC];                                     // pairs of O's columns
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        m[r] = -1e30f;
+        l[r] = 0.f;
+#pragma unroll
+        for (int e = 0; e < AC; ++e) acc[r][e] = 0;
     }
 
-    const int last_row = min(n_rows - 1, blockIdx.x * RB + RB - 1);
-    const int i_max = last_row / group;
-    const int n_tail = (q_pos0 + i_max) / KVP_TILE_KEYS + 1;      // tail keys: rows appended earlier, then this call's
-    const int n_tiles = n_tail + (it.tile_end - it.tile_begin);
-
-    float m = -1e30f, l = 0.f;
-    float acc[D / 8];
-#pragma unroll
-    for (int e = 0; e < D / 8; ++e) acc[e] = 0.f;
-
-    for (int tt = 0; tt < n_tiles; ++tt) {
+#pragma unroll 1
+    for (int blk = blk0; blk < blk1; ++blk) {
+        const int tt = blk >> 1;
         kvp_tile tl;
         int qoff = -1;
         if (tt < n_tail) {
@@ -326,84 +399,254 @@ attn_simple_kernel(kvp_plan_dev plan, int q_len, int q_pos0, int layer, const T 
             tl.n_keys = (int16_t)min(KVP_TILE_KEYS, q_pos0 + q_len - tt * KVP_TILE_KEYS);
             tl.src = 1;
             tl.rope = 0;
-            qoff = tt * KVP_TILE_KEYS;
+            qoff = tt * KVP_TILE_KEYS + (blk & 1) * BN;
         } else {
             tl = plan.tiles[it.tile_begin + tt - n_tail];
         }
-        const int64_t prow = (tl.src == 0) ? (int64_t)plane * pool_rows : (int64_t)plane * ws_rows;
-        const T *kb = reinterpret_cast<const T *>(tl.src == 0 ? pool_k : ws_k) + (prow + tl.row0) * D;
-        const T *vb = reinterpret_cast<const T *>(tl.src == 0 ? pool_v : ws_v) + (prow + tl.row0) * D;
+        const int nk = min(BN, tl.n_keys - (blk & 1) * BN);
+        if (nk <= 0) continue;
+        const int64_t row = (tl.src == 0 ? (int64_t)plane * pool_rows : (int64_t)plane * ws_rows) + tl.row0 + (blk & 1) * BN;
+        const T *kb = reinterpret_cast<const T *>(tl.src == 0 ? pool_k : ws_k) + row * D;
+        const T *vb = reinterpret_cast<const T *>(tl.src == 0 ? pool_v : ws_v) + row * D;
         const float2 *cs = plan.rope + (size_t)tl.rope * HALF;
 
-        for (int k0 = 0; k0 < tl.n_keys; k0 += KC) {
-            const int nk = min(KC, tl.n_keys - k0);
-            __syncthreads();
-            for (int w = threadIdx.x; w < KC * HALF; w += blockDim.x) {
-                const int kk = w / HALF, p = w % HALF;
-                const int ia = pairing ? 2 * p : p, ib = pairing ? 2 * p + 1 : p + HALF;
-                float a = 0.f, bb = 0.f, va = 0.f, vb2 = 0.f;
-                if (kk < nk) {
-                    const T *kr = kb + (int64_t)(k0 + kk) * D;
-                    const T *vr = vb + (int64_t)(k0 + kk) * D;
-                    a = Elem<T>::to_f32(kr[ia]);
-                    bb = Elem<T>::to_f32(kr[ib]);
-                    va = Elem<T>::to_f32(vr[ia]);
-                    vb2 = Elem<T>::to_f32(vr[ib]);
-                    if (tl.rope != 0) rotate_pair(a, bb, cs[p].x, cs[p].y);
-                }
-                Ks[kk][ia] = a;
-                Ks[kk][ib] = bb;
-                Vs[kk][ia] = va;
-                Vs[kk][ib] = vb2;
-            }
-            __syncthreads();
+        // the query block's own rows: straight from the caller's tensors, and - by the first row tile - on to the cache
+        const bool fresh = qoff >= 0 && k_new != nullptr;
 
-            float s[4];
+        __syncthreads();                                     // the block before is done with K, P and V
+        constexpr int CP = HALF / EV;                        // pairs of 16-byte chunks per row
+        constexpr int PER = BN * CP / NT < 4 ? BN * CP / NT : 4;        // at most 16 words in flight per thread
+        static_assert(BN * CP % (NT * PER) == 0, "whole rounds");
+#pragma unroll 1
+        for (int w0 = threadIdx.x; w0 < BN * CP; w0 += NT * PER) {
+            Vec16<T> ka[PER], kc[PER], va[PER], vc[PER];
+#pragma unroll
+            for (int u = 0; u < PER; ++u) {
+                const int w = w0 + u * NT, kk = w / CP, c = w % CP;
+                ka[u].u = kc[u].u = va[u].u = vc[u].u = make_uint4(0, 0, 0, 0);
+                if (kk < nk) {
+                    const uint4 *kr = reinterpret_cast<const uint4 *>(kb + (int64_t)kk * D) + c;
+                    const uint4 *vr = reinterpret_cast<const uint4 *>(vb + (int64_t)kk * D) + c;
+                    if (fresh) {
+                        const int64_t src = (((int64_t)b * q_len + qoff + kk) * n_kv + hk) * (2 * CP) + c;
+                        kr = k_new + src;
+                        vr = v_new + src;
+                    }
+                    ka[u].u = __ldg(kr);
+                    kc[u].u = __ldg(kr + CP);
+                    va[u].u = __ldg(vr);
+                    vc[u].u = __ldg(vr + CP);
+                    if (fresh && rt == 0) {
+                        uint4 *kw = reinterpret_cast<uint4 *>(ws_k_out) + (row + kk) * (2 * CP) + c;
+                        uint4 *vw = reinterpret_cast<uint4 *>(ws_v_out) + (row + kk) * (2 * CP) + c;
+                        kw[0] = ka[u].u;
+                        kw[CP] = kc[u].u;
+                        vw[0] = va[u].u;
+                        vw[CP] = vc[u].u;
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < PER; ++u) {
+                const int w = w0 + u * NT, kk = w / CP, c = w % CP;
+                float a[EV], x[EV];
+#pragma unroll
+                for (int e = 0; e < EV; ++e) {
+                    a[e] = Elem<T>::to_f32(ka[u].e[e]);
+                    x[e] = Elem<T>::to_f32(kc[u].e[e]);
+                }
+                if (tl.rope != 0) {
+                    if (pairing == 0) {
+#pragma unroll
+                        for (int e = 0; e < EV; ++e) {
+                            const float2 r = __ldg(cs + c * EV + e);
+                            rotate_pair(a[e], x[e], r.x, r.y);
+                        }
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < EV; e += 2) {
+                            const float2 r = __ldg(cs + (c * EV + e) / 2), r2 = __ldg(cs + (c * EV + HALF + e) / 2);
+                            rotate_pair(a[e], a[e + 1], r.x, r.y);
+                            rotate_pair(x[e], x[e + 1], r2.x, r2.y);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int e = 0; e < EV; e += 4) {
+                    *reinterpret_cast<float4 *>(Ks + kk * LD + c * EV + e) = make_float4(a[e], a[e + 1], a[e + 2], a[e + 3]);
+                    *reinterpret_cast<float4 *>(Ks + kk * LD + HALF + c * EV + e) = make_float4(x[e], x[e + 1], x[e + 2], x[e + 3]);
+                    *reinterpret_cast<float4 *>(Vs + kk * D + c * EV + e) =
+                        make_float4(Elem<T>::to_f32(va[u].e[e]), Elem<T>::to_f32(va[u].e[e + 1]), Elem<T>::to_f32(va[u].e[e + 2]),
+                                    Elem<T>::to_f32(va[u].e[e + 3]));
+                    *reinterpret_cast<float4 *>(Vs + kk * D + HALF + c * EV + e) =
+                        make_float4(Elem<T>::to_f32(vc[u].e[e]), Elem<T>::to_f32(vc[u].e[e + 1]), Elem<T>::to_f32(vc[u].e[e + 2]),
+                                    Elem<T>::to_f32(vc[u].e[e + 3]));
+                }
+            }
+        }
+        __syncthreads();
+
+        uint64_t s2[4][KN];                                  // sums over even and odd columns, side by side
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int j = 0; j < KN; ++j) s2[r][j] = 0;
+#pragma unroll 4
+        for (int c = 0; c < D; c += 4) {
+            ulonglong2 qv[4], kv[KN];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) qv[r] = *reinterpret_cast<const ulonglong2 *>(Qs + (4 * ty + r) * LD + c);
+#pragma unroll
+            for (int j = 0; j < KN; ++j) kv[j] = *reinterpret_cast<const ulonglong2 *>(Ks + (tx + TX * j) * LD + c);
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int j = 0; j < KN; ++j) {
+                    s2[r][j] = fma2(qv[r].x, kv[j].x, s2[r][j]);
+                    s2[r][j] = fma2(qv[r].y, kv[j].y, s2[r][j]);
+                }
+        }
+        float s[4][KN];
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int j = 0; j < KN; ++j) {
+                const float2 h = halves(s2[r][j]);
+                s[r][j] = h.x + h.y;
+            }
+        __syncthreads();                                     // everyone has read K: P goes there
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
             float mx = -INFINITY;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int kk = sub + 8 * u;
-                float a = 0.f;
-#pragma unroll 8
-                for (int c = 0; c < D; ++c) a += Qs[row][c] * Ks[kk][c];
-                const bool vis = kk < nk && (qoff < 0 || qoff + k0 + kk <= q_pos0 + i);
-                s[u] = vis ? a * scale : -INFINITY;
-                mx = fmaxf(mx, s[u]);
+            for (int j = 0; j < KN; ++j) {
+                const int kk = tx + TX * j;
+                const bool vis = kk < nk && (qoff < 0 || qoff + kk < lim[r]);
+                s[r][j] = vis ? s[r][j] * scale : -INFINITY;
+                mx = fmaxf(mx, s[r][j]);
             }
-            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 4));
-            const float m_new = fmaxf(m, mx);
-            const float alpha = expf(m - m_new);
+#pragma unroll
+            for (int o = TX / 2; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            const float m_new = fmaxf(m[r], mx);
+            const float alpha = expf(m[r] - m_new);
             float ps = 0.f;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const float p = expf(s[u] - m_new);      // exp(-inf) = 0 for masked keys
-                Ps[row][sub + 8 * u] = p;
+            for (int j = 0; j < KN; ++j) {
+                const float p = expf(s[r][j] - m_new);       // exp(-inf) = 0 for masked keys
+                Ps[(4 * ty + r) * LP + tx + TX * j] = p;
                 ps += p;
             }
-            ps += __shfl_xor_sync(0xffffffffu, ps, 1);
-            ps += __shfl_xor_sync(0xffffffffu, ps, 2);
-            ps += __shfl_xor_sync(0xffffffffu, ps, 4);
-            l = l * alpha + ps;
-            m = m_new;
-            __syncwarp();
+            l[r] = l[r] * alpha + ps;                        // this thread's keys; added up over tx at the end
+            m[r] = m_new;
+            const uint64_t alpha2 = both(alpha);
 #pragma unroll
-            for (int e = 0; e < D / 8; ++e) acc[e] *= alpha;
-            for (int kk = 0; kk < KC; ++kk) {
-                const float p = Ps[row][kk];
+            for (int e = 0; e < AC; ++e) acc[r][e] = mul2(acc[r][e], alpha2);
+        }
+        __syncwarp();                                        // a row's P is written and read by one warp
+#pragma unroll 4
+        for (int kk = 0; kk < BN; kk += 4) {
+            float4 pv[4];
 #pragma unroll
-                for (int e = 0; e < D / 8; ++e) acc[e] += p * Vs[kk][sub + 8 * e];
+            for (int r = 0; r < 4; ++r) pv[r] = *reinterpret_cast<const float4 *>(Ps + (4 * ty + r) * LP + kk);
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                union { VT v[PC]; uint64_t p[AC]; } vv;
+#pragma unroll
+                for (int y = 0; y < PC; ++y)
+                    vv.v[y] = *reinterpret_cast<const VT *>(Vs + (kk + x) * D + y * (V * TX) + tx * V);
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const uint64_t p = both(x == 0 ? pv[r].x : x == 1 ? pv[r].y : x == 2 ? pv[r].z : pv[r].w);
+#pragma unroll
+                    for (int e = 0; e < AC; ++e) acc[r][e] = fma2(p, vv.p[e], acc[r][e]);
+                }
             }
-            __syncwarp();
         }
     }
-    if (valid) {
-        const float inv = 1.f / l;
-        T *o = out + (((int64_t)b * q_len + i) * n_q + h) * D;
 #pragma unroll
-        for (int e = 0; e < D / 8; ++e) o[sub + 8 * e] = Elem<T>::from_f32(acc[e] * inv);
-        if (lse != nullptr && sub == 0) lse[((int64_t)b * n_q + h) * q_len + i] = m + logf(l);
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int o = TX / 2; o > 0; o >>= 1) l[r] += __shfl_xor_sync(0xffffffffu, l[r], o);
+
+    if (splits == 1) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int row = row0 + 4 * ty + r;
+            if (row >= n_rows) break;
+            const float inv = 1.f / l[r];
+            const int i = row / group, h = hk * group + row % group;
+            T *dst = out + (((int64_t)b * q_len + i) * n_q + h) * D + tx * V;
+#pragma unroll
+            for (int e = 0; e < AC; ++e) {
+                const float2 o = halves(acc[r][e]);
+                dst[(2 * e / V) * (V * TX) + 2 * e % V] = Elem<T>::from_f32(o.x * inv);
+                dst[(2 * e / V) * (V * TX) + 2 * e % V + 1] = Elem<T>::from_f32(o.y * inv);
+            }
+            if (lse != nullptr && tx == 0) lse[((int64_t)b * n_q + h) * q_len + i] = m[r] + logf(l[r]);
+        }
+        return;
+    }
+    const int unit = (b * n_kv + hk) * (gridDim.x / splits) + rt;
+    const int64_t prow0 = (int64_t)unit * splits * BM;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int64_t pr = prow0 + sp * BM + 4 * ty + r;
+#pragma unroll
+        for (int y = 0; y < PC; ++y)
+            *reinterpret_cast<VT *>(part.o + pr * D + y * (V * TX) + tx * V) = *reinterpret_cast<VT *>(acc[r] + y * (V / 2));
+        if (tx == 0) part.ml[pr] = make_float2(m[r], l[r]);
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last_in = atomicAdd(part.arrived + unit, 1) == splits - 1;
+    __syncthreads();
+    if (!last_in) return;
+    __threadfence();
+    if (threadIdx.x == 0) part.arrived[unit] = 0;
+    // weights of the parts, per row, in shared memory (splits x BM pairs fit what K, V and Q took); then every thread
+    // takes float4 columns of rows, four parts' loads in flight
+    float2 *wl = reinterpret_cast<float2 *>(sm);
+    for (int w = threadIdx.x; w < splits * BM; w += NT) wl[w] = __ldcg(part.ml + prow0 + w);
+    __syncthreads();
+    if (threadIdx.x < BM) {
+        float M = -1e30f, L = 0.f;
+        for (int z = 0; z < splits; ++z) M = fmaxf(M, wl[z * BM + threadIdx.x].x);
+        for (int z = 0; z < splits; ++z) {
+            const float2 ml = wl[z * BM + threadIdx.x];
+            const float w = expf(ml.x - M);                  // a part without a visible key has l = 0 and O = 0
+            wl[z * BM + threadIdx.x].x = w;
+            L += w * ml.y;
+        }
+        const int row = row0 + threadIdx.x;
+        wl[threadIdx.x].y = 1.f / L;
+        if (lse != nullptr && row < n_rows)
+            lse[((int64_t)b * n_q + hk * group + row % group) * q_len + row / group] = M + logf(L);
+    }
+    __syncthreads();
+    constexpr int IT = BM * D / 4 / NT;                      // float4 columns per thread
+    float4 o[IT];
+#pragma unroll
+    for (int u = 0; u < IT; ++u) o[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+    for (int z = 0; z < splits; ++z) {
+#pragma unroll
+        for (int u = 0; u < IT; ++u) {
+            const int e = threadIdx.x + u * NT;
+            const float4 t = __ldcg(reinterpret_cast<const float4 *>(part.o + (prow0 + z * BM) * D) + e);
+            const float w = wl[z * BM + e / (D / 4)].x;
+            o[u].x += w * t.x; o[u].y += w * t.y; o[u].z += w * t.z; o[u].w += w * t.w;
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < IT; ++u) {
+        const int e = threadIdx.x + u * NT, row = row0 + e / (D / 4);
+        if (row >= n_rows) break;
+        const float inv = wl[e / (D / 4)].y;
+        T *dst = out + (((int64_t)b * q_len + row / group) * n_q + hk * group + row % group) * D + 4 * (e % (D / 4));
+        dst[0] = Elem<T>::from_f32(o[u].x * inv);
+        dst[1] = Elem<T>::from_f32(o[u].y * inv);
+        dst[2] = Elem<T>::from_f32(o[u].z * inv);
+        dst[3] = Elem<T>::from_f32(o[u].w * inv);
     }
 }
 
@@ -581,22 +824,69 @@ cudaError_t kvp_launch_segment_mass(const kvp_shape &sh, const kvp_plan_dev &pla
     return cudaGetLastError();
 }
 
-cudaError_t kvp_launch_attn_simple(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t batch, int32_t q_len,
-                                   int32_t q_pos0, int32_t layer, const void *q, const char *pool_k, const char *pool_v,
-                                   const char *ws_k, const char *ws_v, void *out, float *lse, int32_t *ctas,
-                                   cudaStream_t st)
+namespace {
+
+template <int D, int TY> constexpr int core_smem = 4 * (4 * TY * (D + 4) + 64 * (D + 4) + 64 * D);
+
+template <typename T, int D>
+cudaError_t prepare_core()
 {
-    const dim3 grid((sh.group * q_len + 15) / 16, sh.n_kv_heads, batch);
+    const cudaError_t rc = cudaFuncSetAttribute(attn_core_kernel<T, D, 16, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, core_smem<D, 16>);
+    if (rc != cudaSuccess) return rc;
+    return cudaFuncSetAttribute(attn_core_kernel<T, D, 4, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, core_smem<D, 4>);
+}
+
+template <typename T, int D, int TY, int TX>
+cudaError_t launch_core(const kvp_shape &sh, const kvp_plan_dev &plan, int batch, int q_len, int q_pos0, int layer, const void *q,
+                        const char *pool_k, const char *pool_v, const char *ws_k, const char *ws_v, int n_tiles,
+                        const kvp_core_ws &ws, void *out, float *lse, int32_t *ctas, cudaStream_t st)
+{
+    constexpr int BM = 4 * TY;
+    static_assert(8 * 64 * BM <= core_smem<D, TY>, "the parts' weights fit");
+    // Split the keys until the chip is full (two CTAs of 256 threads or four of 128 per SM), but never below one 64-key
+    // block per part, and only as far as the partial rows and the counters reach.
+    const int64_t row_tiles = (sh.group * (int64_t)q_len + BM - 1) / BM, units = row_tiles * sh.n_kv_heads * batch;
+    const int64_t slots = (int64_t)ws.sm_count * (512 / (TY * TX));
+    int64_t splits = (slots + units - 1) / units;
+    splits = std::min<int64_t>(std::min<int64_t>(splits, 2 * n_tiles), 64);
+    splits = std::min<int64_t>(splits, ws.max_rows / (units * BM));
+    if (units > ws.max_units || splits < 1) splits = 1;
+    const dim3 grid((unsigned)(row_tiles * splits), sh.n_kv_heads, batch);
     if (ctas) *ctas = (int32_t)(grid.x * grid.y * grid.z);
-#define KVP_SIMPLE(T, D)                                                                                             \
-    attn_simple_kernel<T, D><<<grid, 128, 0, st>>>(plan, q_len, q_pos0, layer, (const T *)q, pool_k, pool_v, ws_k, ws_v,     \
-                                                   sh.pool_rows, sh.ws_rows, sh.n_q_heads, sh.n_kv_heads, sh.group,  \
-                                                   sh.pairing, sh.scale, (T *)out, lse)
-    if (sh.dtype == KVP_DTYPE_BF16) {
-        if (sh.head_dim == 128) KVP_SIMPLE(__nv_bfloat16, 128); else KVP_SIMPLE(__nv_bfloat16, 64);
-    } else {
-        if (sh.head_dim == 128) KVP_SIMPLE(float, 128); else KVP_SIMPLE(float, 64);
-    }
-#undef KVP_SIMPLE
+    const CorePart part = {ws.partial_o, ws.partial_ml, ws.arrived};
+    attn_core_kernel<T, D, TY, TX><<<grid, TY * TX, core_smem<D, TY>, st>>>(plan, q_len, q_pos0, layer, (const T *)q, pool_k, pool_v, ws_k, ws_v,
+                                    (const uint4 *)ws.k_new, (const uint4 *)ws.v_new, ws.ws_k, ws.ws_v, sh.pool_rows, sh.ws_rows,
+                                    sh.n_q_heads, sh.n_kv_heads, sh.group, sh.pairing, sh.scale, (int)splits, part, (T *)out, lse);
     return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t kvp_attn_core_prepare(const kvp_shape &sh)
+{
+    if (sh.dtype == KVP_DTYPE_BF16) return sh.head_dim == 128 ? prepare_core<__nv_bfloat16, 128>() : prepare_core<__nv_bfloat16, 64>();
+    return sh.head_dim == 128 ? prepare_core<float, 128>() : prepare_core<float, 64>();
+}
+
+cudaError_t kvp_launch_attn_core(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t batch, int32_t q_len, int32_t q_pos0,
+                                 int32_t layer, const void *q, const char *pool_k, const char *pool_v, const char *ws_k,
+                                 const char *ws_v, int32_t n_tiles, const kvp_core_ws &ws, void *out, float *lse, int32_t *ctas,
+                                 cudaStream_t st)
+{
+    // 64-row tiles use the FMA pipe twice as well as 16-row ones (a shared-memory word feeds twice the products); 16-row
+    // tiles when the rows would leave the larger ones half empty, or when even fully split 64-row tiles are fewer than SMs.
+    const int64_t rows = sh.group * (int64_t)q_len;
+    const int64_t most = (rows + 63) / 64 * sh.n_kv_heads * batch * 2 * n_tiles;
+    const bool big = rows > 32 && most >= ws.sm_count;
+#define KVP_CORE(T, D)                                                                                                   \
+    return big ? launch_core<T, D, 16, 16>(sh, plan, batch, q_len, q_pos0, layer, q, pool_k, pool_v, ws_k, ws_v, n_tiles, \
+                                           ws, out, lse, ctas, st)                                                      \
+               : launch_core<T, D, 4, 32>(sh, plan, batch, q_len, q_pos0, layer, q, pool_k, pool_v, ws_k, ws_v, n_tiles,  \
+                                          ws, out, lse, ctas, st)
+    if (sh.dtype == KVP_DTYPE_BF16) {
+        if (sh.head_dim == 128) KVP_CORE(__nv_bfloat16, 128); else KVP_CORE(__nv_bfloat16, 64);
+    } else {
+        if (sh.head_dim == 128) KVP_CORE(float, 128); else KVP_CORE(float, 64);
+    }
+#undef KVP_CORE
 }
