@@ -597,9 +597,10 @@ int32_t kvp_create(const kvp_config *cfg, kvp_ctx **out)
     if (sh.pool_rows <= 0) return bail(KVP_ERR_CAPACITY, "pool smaller than one token");
     if (cfg->workspace_bytes < w.total) return bail(KVP_ERR_CAPACITY, "workspace too small");
     if (cudaSetDevice(cfg->device) != cudaSuccess) return bail(KVP_ERR_CUDA, "cudaSetDevice failed");
-    cudaDeviceProp prop;
-    if (cudaGetDeviceProperties(&prop, cfg->device) != cudaSuccess) return bail(KVP_ERR_CUDA, "no device properties");
-    ctx->sm_count = prop.multiProcessorCount;
+    int cc_major = 0;                          // (all properties at once take milliseconds)
+    if (cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, cfg->device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&cc_major, cudaDevAttrComputeCapabilityMajor, cfg->device) != cudaSuccess)
+        return bail(KVP_ERR_CUDA, "no device attributes");
 
     const uint64_t plane_bytes = (uint64_t)sh.n_layers * sh.n_kv_heads * sh.pool_rows * sh.head_dim * sh.elem_bytes;
     ctx->pool_k = (char *)cfg->pool;
@@ -655,7 +656,7 @@ int32_t kvp_create(const kvp_config *cfg, kvp_ctx **out)
             return bail(KVP_ERR_CUDA, "load event creation failed");
 
     if (kvp_attn_core_prepare(sh) != cudaSuccess) return bail(KVP_ERR_CUDA, "CUDA-core kernel attribute setup failed");
-    if (sh.dtype == KVP_DTYPE_BF16 && prop.major == 10) {
+    if (sh.dtype == KVP_DTYPE_BF16 && cc_major == 10) {
         void *fn = nullptr;
         cudaDriverEntryPointQueryResult qres;
         if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) == cudaSuccess && fn &&
