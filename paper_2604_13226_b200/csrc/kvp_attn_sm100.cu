@@ -378,7 +378,7 @@ __device__ __forceinline__ void produce_q_tile(const Params &p, char *qbuf, char
         const float4 *cs = reinterpret_cast<const float4 *>(p.plan.rope + (size_t)rope * (D / 2));   // (cos, sin) pairs
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-            w4[j] = __ldg(p.pairing == 0 ? cs + c * 4 + j : cs + (c + kCh * (j >> 1)) * 2 + (j & 1));
+            w4[j] = *(p.pairing == 0 ? cs + c * 4 + j : cs + (c + kCh * (j >> 1)) * 2 + (j & 1));
     }
 #pragma unroll 1
     for (int i = 0; i < kCh; ++i) {
@@ -686,7 +686,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
         // un-normalised (partial slot) or normalised (output rows) O = w0 O_s (+ w1 O_1)
         uint4 *orow_bf = (direct && valid) ? reinterpret_cast<uint4 *>(p.out + (((long long)w.b * p.q_len + qi) * p.n_q + h) * D) : nullptr;
         // partial slot layout: [D / 4 float4 columns][128 rows], so that a warp's store covers 512 contiguous bytes
-        uint4 *orow_f = direct ? nullptr : reinterpret_cast<uint4 *>(p.partial_o) + (long long)slot * (C::kCols4 * KVP_TILE_ROWS) + t;
+        uint4 *orow_f = direct || !valid ? nullptr : reinterpret_cast<uint4 *>(p.partial_o) + (long long)slot * (C::kCols4 * KVP_TILE_ROWS) + t;
 #pragma unroll 1
         for (int ch = 0; ch < D / 32; ++ch) {
             uint32_t a[32];
@@ -720,7 +720,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
         if (direct) {
             if (valid && p.lse != nullptr)
                 p.lse[((long long)w.b * p.n_q + h) * p.q_len + qi] = m_ref * p.scale + logf(l);
-        } else {
+        } else if (valid) {
             p.partial_ml[(long long)slot * KVP_TILE_ROWS + t] = make_float2(m_ref, l);
         }
         tc_fence_before();
@@ -737,6 +737,7 @@ __device__ __forceinline__ void producer_role(const Params &p, const Cta &c, con
     const bool one_buffer = !C::kSplit && p.precise;
     uint32_t nEp0 = 0, nEp1 = 0;
     bool ok = true;
+    pdl_wait();
     for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
         const Work w = load_work(p, wi);
         const int n_rows = p.group * w.q_len;
@@ -786,6 +787,7 @@ __device__ __forceinline__ void append_role(const Params &p, const Cta &c, const
 {
     constexpr int kVecs = Cfg<D>::kVecs;
     if (!p.tail_direct) return;
+    pdl_wait();
     for (int wi = c.item_begin; wi < c.item_end; ++wi) {
         const Work w = load_work(p, wi);
         if (w.lo != 0) continue;
@@ -802,8 +804,8 @@ __device__ __forceinline__ void append_role(const Params &p, const Cta &c, const
                 const int i = base + j * 64 + t;
                 if (i < n_words) {
                     const long long src = src0 + (long long)(i / kVecs) * p.n_kv * kVecs + i % kVecs;
-                    k[j] = __ldg(p.k_new + src);
-                    v[j] = __ldg(p.v_new + src);
+                    k[j] = p.k_new[src];
+                    v[j] = p.v_new[src];
                 }
             }
 #pragma unroll
@@ -828,7 +830,7 @@ __device__ __forceinline__ void tma_role(const Params &p, const Cta &c, const in
     using C = Cfg<D>;
     constexpr int kStages = C::kStages, kTileBytes = C::kTileBytes;
     uint32_t ring_n = 0;                                   // loads issued before this piece
-    bool ok = true;
+    bool ok = true, waited = false;
     for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
         const Work w = load_work(p, wi);
         const int n_loads = 2 * w.n;
@@ -872,6 +874,10 @@ __device__ __forceinline__ void tma_role(const Params &p, const Cta &c, const in
                     if (ok) {
                         const uint32_t dst = c.smem_base + C::kOffRing + stage * kTileBytes;
                         mbar_expect_tx(c.bar(C::kKvFull + stage), kTileBytes);
+                        if (src_i != 0 && !waited) {       // staged or appended rows: a kernel in front may have written them
+                            pdl_wait();
+                            waited = true;
+                        }
                         if (src_i == 2) {
                             const CUtensorMap *tm = kv_i ? tm_vnew : tm_knew;
                             tma_load_4d(dst, tm, 0, w.hk, row0_i, w.b, c.bar(C::kKvFull + stage));
@@ -1164,9 +1170,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_pool_k, const __grid_co
     c.bar0 = c.smem_base + C::kOffBar;
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(c.smem + C::kOffBar + 8 * C::kNumBars);
     c.abort_flag = tmem_slot + 1;
-    c.item_begin = __ldg(p.cta_begin + blockIdx.x);
-    c.item_end = __ldg(p.cta_begin + blockIdx.x + 1);
-    if (c.item_begin >= c.item_end) return;
+    pdl_launch_dependents();
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -1196,6 +1200,10 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_pool_k, const __grid_co
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    // from here on: the Q producer, the append and the TMA warp (for anything but pool tiles) wait for the kernel in front;
+    // everything else follows from what they deliver
+    c.item_begin = __ldg(p.cta_begin + blockIdx.x);           // (the work list gives every CTA at least one piece)
+    c.item_end = __ldg(p.cta_begin + blockIdx.x + 1);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -1254,6 +1262,10 @@ __device__ __forceinline__ void merge_tile(int b, int hk, int row_base, int item
     const int row = blockIdx.y * 32 + lane;                     // row of the 128-row query tile
     const int n_rows = group * (item_q_len ? item_q_len : q_len);       // q_len stays the stride of the padded tensors
     const float c2 = scale * 1.4426950408889634f;
+    // rows behind the request's last one exist in no partial (a decode step fills 4 of 128): nothing to read or write
+    if (row_base + (int)blockIdx.y * 32 >= n_rows) return;
+    const bool valid = row_base + row < n_rows;
+    if (!valid) n = 0;
     float M = -INFINITY;
     float L = 0.f;
     float4 o[kC];
@@ -1275,6 +1287,7 @@ __device__ __forceinline__ void merge_tile(int b, int hk, int row_base, int item
         }
     }
     if (mo.part_o != nullptr) {                                 // stays a partial: un-normalised, against the max M
+        if (!valid) return;
         const long long c = ((long long)b * n_kv + hk) * ((group * q_len + KVP_TILE_ROWS - 1) / KVP_TILE_ROWS) + row_base / KVP_TILE_ROWS;
 #pragma unroll
         for (int j = 0; j < kC; ++j) mo.part_o[(c * (D / 4) + wv + 8 * j) * KVP_TILE_ROWS + row] = o[j];
@@ -1313,6 +1326,9 @@ __global__ void __launch_bounds__(256)
 merge_list_kernel(const kvp_merge_item *__restrict__ merges, int q_len, int n_q, int n_kv, int group, float scale,
                   const float *__restrict__ part_o, const float2 *__restrict__ part_ml, MergeOut mo)
 {
+    pdl_launch_dependents();
+    pdl_wait();
+    PDL_AFTER(part_o); PDL_AFTER(part_ml);
     const kvp_merge_item mi = merges[blockIdx.x];
     merge_tile<D>(mi.b, mi.hk, mi.row_base, mi.pad[0], reinterpret_cast<const float4 *>(part_o) + (long long)mi.slot0 * (D / 4 * KVP_TILE_ROWS),
                part_ml + (long long)mi.slot0 * KVP_TILE_ROWS, mi.n_slots, D / 4 * KVP_TILE_ROWS, KVP_TILE_ROWS, q_len, n_q, n_kv,
@@ -1375,10 +1391,8 @@ cudaError_t kvp_launch_attn_sm100(const kvp_shape &sh, const kvp_attn2_args &a, 
     // without tail_direct the two query maps are never dereferenced: any valid map will do
     const CUtensorMap &tk = a.tail_direct ? a.tm_knew : tm_ws_k, &tv = a.tail_direct ? a.tm_vnew : tm_ws_v;
     if (sh.head_dim == 64)
-        attn_sm100_kernel<64><<<a.n_ctas, kThreads, Cfg<64>::kSmemBytes, st>>>(tm_pool_k, tm_pool_v, tm_ws_k, tm_ws_v, tk, tv, p);
-    else
-        attn_sm100_kernel<128><<<a.n_ctas, kThreads, Cfg<128>::kSmemBytes, st>>>(tm_pool_k, tm_pool_v, tm_ws_k, tm_ws_v, tk, tv, p);
-    return cudaGetLastError();
+        return launch_pdl(attn_sm100_kernel<64>, a.n_ctas, kThreads, Cfg<64>::kSmemBytes, st, tm_pool_k, tm_pool_v, tm_ws_k, tm_ws_v, tk, tv, p);
+    return launch_pdl(attn_sm100_kernel<128>, a.n_ctas, kThreads, Cfg<128>::kSmemBytes, st, tm_pool_k, tm_pool_v, tm_ws_k, tm_ws_v, tk, tv, p);
 }
 
 cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_merges, const kvp_merge_item *merges,
@@ -1397,10 +1411,8 @@ cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_
     }
     const dim3 grid(n_merges, KVP_TILE_ROWS / 32);
     if (sh.head_dim == 64)
-        merge_list_kernel<64><<<grid, 256, 0, st>>>(merges, q_len, sh.n_q_heads, sh.n_kv_heads, sh.group, sh.scale, partial_o, partial_ml, mo);
-    else
-        merge_list_kernel<128><<<grid, 256, 0, st>>>(merges, q_len, sh.n_q_heads, sh.n_kv_heads, sh.group, sh.scale, partial_o, partial_ml, mo);
-    return cudaGetLastError();
+        return launch_pdl(merge_list_kernel<64>, grid, 256, 0, st, merges, q_len, sh.n_q_heads, sh.n_kv_heads, sh.group, sh.scale, partial_o, partial_ml, mo);
+    return launch_pdl(merge_list_kernel<128>, grid, 256, 0, st, merges, q_len, sh.n_q_heads, sh.n_kv_heads, sh.group, sh.scale, partial_o, partial_ml, mo);
 }
 
 cudaError_t kvp_launch_merge_ranks(const kvp_shape &sh, int32_t batch, int32_t q_len, const void *parts, int32_t n_parts,

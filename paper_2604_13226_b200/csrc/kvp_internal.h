@@ -223,6 +223,37 @@ struct kvp_ctx {
     std::string err;
 };
 
+// ---- launches that may begin before the kernel in front of them has ended ------------------------
+// Every kernel of a call releases its successor at once and waits for its predecessor (griddepcontrol) before it reads what
+// a kernel may have written just before or writes anything, so that launch latency and set-up - barriers, TMEM, filling
+// the grid - lie under the predecessor's tail.  Some thread of every block waits before the block can end, so a grid that
+// has ended implies that its predecessors have: later work in the stream needs no more than that.
+// Readable without waiting: what only copies write (plans, work lists), and the pool - its writers (registration, host
+// copies) never release a successor early, so whatever starts after them finds it complete.
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Loads the compiler may take for invariant (const __restrict__ parameters) could be moved in front of the wait; a pointer
+// that passes through here cannot be used before this point.
+#define PDL_AFTER(p) asm volatile("" : "+l"(p)::"memory")
+
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+#endif
+
 // ---- kernel launchers (kvp_kernels.cu, kvp_attn_sm100.cu) ---------------------------------------
 
 cudaError_t kvp_launch_store_rows(const kvp_shape &sh, const void *src, char *dst_plane0, int64_t plane_rows,

@@ -111,6 +111,9 @@ gather_kernel(kvp_plan_dev plan, int n_table, int n_rope, int groups, const doub
               char *__restrict__ ws_k, char *__restrict__ ws_v, int64_t pool_rows, int64_t ws_rows, int vecs_per_row,
               int half_dim, int pairing)
 {
+    pdl_launch_dependents();
+    pdl_wait();
+    PDL_AFTER(pool_k); PDL_AFTER(pool_v);
     if ((int)blockIdx.x < n_table) {
         const int e = blockIdx.x * 256 + threadIdx.x;
         if (e < n_rope * half_dim) table[e] = offset_cos_sin(plan.delta[e / half_dim], half_turns[e % half_dim]);
@@ -164,116 +167,192 @@ gather_kernel(kvp_plan_dev plan, int n_table, int n_rope, int groups, const doub
 // ---- append: the query chunk's own K/V rows go behind the prefix (Section 3.2 step 4) --------------
 // grid (batch*q_len); the rows go behind the q_pos0 rows appended earlier; with rope_query the raw
 // k_new and q are first rotated to positions prefix_len + q_pos0 + i, angles formed in double precision.
+// Latency is all there is (a decode step moves a few KB): a thread takes a pair of 16-byte words - the rotation partners -
+// of K and V or of Q, and every load is issued before the angles are formed.  One element at a time with the angles first
+// it took 9.4 us of a 75 us decode layer.
 template <typename T>
-__global__ void append_kernel(kvp_plan_dev plan, int q_len, int q_pos0, const T *__restrict__ q, const T *__restrict__ k_new,
-                              const T *__restrict__ v_new, char *__restrict__ ws_k, char *__restrict__ ws_v,
-                              int64_t ws_rows, int layer, int n_q, int n_kv, int d, int pairing, int rope_query,
-                              const double *__restrict__ half_turns, T *__restrict__ q_rot)
+__device__ __forceinline__ Vec16<T> load_vec(const T *p, bool aligned)
 {
+    Vec16<T> v;
+    if (aligned) {
+        v.u = __ldg(reinterpret_cast<const uint4 *>(p));
+    } else {
+#pragma unroll
+        for (int e = 0; e < Elem<T>::kPerVec; ++e) v.e[e] = p[e];
+    }
+    return v;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256)
+append_kernel(kvp_plan_dev plan, int q_len, int q_pos0, const T *__restrict__ q, const T *__restrict__ k_new,
+              const T *__restrict__ v_new, char *__restrict__ ws_k, char *__restrict__ ws_v,
+              int64_t ws_rows, int layer, int n_q, int n_kv, int d, int pairing, int rope_query,
+              const double *__restrict__ half_turns, T *__restrict__ q_rot)
+{
+    constexpr int EV = Elem<T>::kPerVec;
     __shared__ float2 cs[64];
+    pdl_launch_dependents();
+    pdl_wait();
+    PDL_AFTER(q); PDL_AFTER(k_new); PDL_AFTER(v_new);
     const int b = blockIdx.x / q_len, i = blockIdx.x % q_len;
     const kvp_item it = plan.items[b];
-    const int half = d / 2;
-    if (rope_query) {
-        for (int p = threadIdx.x; p < half; p += blockDim.x) cs[p] = offset_cos_sin(it.prefix_len + q_pos0 + i, half_turns[p]);
-        __syncthreads();
-    }
+    const int half = d / 2, half_vecs = half / EV, vecs = 2 * half_vecs;
     const int64_t tok = (int64_t)b * q_len + i;
-    // keys and values: one thread per (kv head, pair)
-    for (int w = threadIdx.x; w < n_kv * half; w += blockDim.x) {
-        const int hk = w / half, p = w % half;
-        const int ia = pairing ? 2 * p : p, ib = pairing ? 2 * p + 1 : p + half;
-        const T *ks = k_new + (tok * n_kv + hk) * d;
-        const T *vs = v_new + (tok * n_kv + hk) * d;
-        const int64_t drow = ((int64_t)(layer * n_kv + hk)) * ws_rows + it.tail_row0 + q_pos0 + i;
-        T *kd = reinterpret_cast<T *>(ws_k) + drow * d;
-        T *vd = reinterpret_cast<T *>(ws_v) + drow * d;
-        float a = Elem<T>::to_f32(ks[ia]), bb = Elem<T>::to_f32(ks[ib]);
-        if (rope_query) {
-            rotate_pair(a, bb, cs[p].x, cs[p].y);
-            kd[ia] = Elem<T>::from_f32(a);
-            kd[ib] = Elem<T>::from_f32(bb);
-        } else {
-            kd[ia] = ks[ia];
-            kd[ib] = ks[ib];
+    const bool al_q = ((uintptr_t)q & 15) == 0, al_k = ((uintptr_t)k_new & 15) == 0, al_v = ((uintptr_t)v_new & 15) == 0;
+    // keys and values: items [0, n_kv half_vecs); with rope_query the query rows behind them
+    const int n_items = (n_kv + (rope_query ? n_q : 0)) * half_vecs;
+    bool first = rope_query != 0;
+    for (int w = threadIdx.x; w < n_items || first; w += 256) {
+        Vec16<T> lo, hi, va, vb;
+        const bool kv = w < n_kv * half_vecs;
+        const int head = kv ? w / half_vecs : w / half_vecs - n_kv, c = w % half_vecs;
+        if (w < n_items) {
+            const T *src = (kv ? k_new + (tok * n_kv + head) * d : q + (tok * n_q + head) * d) + c * EV;
+            lo = load_vec<T>(src, kv ? al_k : al_q);
+            hi = load_vec<T>(src + half, kv ? al_k : al_q);
+            if (kv) {
+                const T *vs = v_new + (tok * n_kv + head) * d + c * EV;
+                va = load_vec<T>(vs, al_v);
+                vb = load_vec<T>(vs + half, al_v);
+            }
         }
-        vd[ia] = vs[ia];
-        vd[ib] = vs[ib];
-    }
-    if (rope_query) {
-        for (int w = threadIdx.x; w < n_q * half; w += blockDim.x) {
-            const int h = w / half, p = w % half;
-            const int ia = pairing ? 2 * p : p, ib = pairing ? 2 * p + 1 : p + half;
-            const T *qs = q + (tok * n_q + h) * d;
-            T *qd = q_rot + (tok * n_q + h) * d;
-            float a = Elem<T>::to_f32(qs[ia]), bb = Elem<T>::to_f32(qs[ib]);
-            rotate_pair(a, bb, cs[p].x, cs[p].y);
-            qd[ia] = Elem<T>::from_f32(a);
-            qd[ib] = Elem<T>::from_f32(bb);
+        if (first) {
+            if ((int)threadIdx.x < half) cs[threadIdx.x] = offset_cos_sin(it.prefix_len + q_pos0 + i, half_turns[threadIdx.x]);
+            __syncthreads();
+            first = false;
+        }
+        if (w >= n_items) break;
+        if (rope_query) rotate_vec_pair<T>(lo, hi, cs, c, half_vecs, pairing);
+        if (kv) {
+            const int64_t drow = ((int64_t)(layer * n_kv + head)) * ws_rows + it.tail_row0 + q_pos0 + i;
+            uint4 *dk = reinterpret_cast<uint4 *>(ws_k) + drow * vecs + c, *dv = reinterpret_cast<uint4 *>(ws_v) + drow * vecs + c;
+            dk[0] = lo.u;
+            dk[half_vecs] = hi.u;
+            dv[0] = va.u;
+            dv[half_vecs] = vb.u;
+        } else {
+            uint4 *dq = reinterpret_cast<uint4 *>(q_rot) + (tok * n_q + head) * vecs + c;
+            dq[0] = lo.u;
+            dq[half_vecs] = hi.u;
         }
     }
 }
 
 // ---- export of the logical composed cache of one (layer, request) ---------------------------------
-// grid (n_rows, Hkv), one thread per pair.  Prefix rows come from where attention reads them: the
-// materialised cache or the staged adapter rows (already re-based), else the pool (rotated here).
+// A block takes kExportRows rows of all kv heads: where each row lies is looked up once (prefix rows come from where
+// attention reads them: the materialised cache or the staged adapter rows, already re-based, else the pool, rotated
+// here), then every thread moves pairs of 16-byte words, two in flight.  Bound by DRAM: one element per thread and one
+// row and head per block took 39 us for 9,000 rows of 8 heads of 128 (73 MB), 1.9 TB/s.
+constexpr int kExportRows = 16;
+
 template <typename T>
-__global__ void export_kernel(kvp_plan_dev plan, int b, int layer, int prefix_len, const char *__restrict__ pool_k,
-                              const char *__restrict__ pool_v, const char *__restrict__ ws_k,
-                              const char *__restrict__ ws_v, int64_t pool_rows, int64_t ws_rows, int n_kv, int d,
-                              int pairing, void *__restrict__ k_out, T *__restrict__ v_out, int k_as_f32)
+__device__ __forceinline__ void store_vec(T *p, const Vec16<T> &v, bool aligned)
 {
-    const int t = blockIdx.x, hk = blockIdx.y;
-    const kvp_item it = plan.items[b];
-    const int half = d / 2;
-    const int plane = layer * n_kv + hk;
-    const T *ks, *vs;
-    int rope = 0;
-    if (t >= prefix_len) {
-        const int64_t r = (int64_t)plane * ws_rows + it.tail_row0 + (t - prefix_len);
-        ks = reinterpret_cast<const T *>(ws_k) + r * d;
-        vs = reinterpret_cast<const T *>(ws_v) + r * d;
-    } else if (it.cache_row0 >= 0) {
-        const int64_t r = (int64_t)plane * ws_rows + it.cache_row0 + t;
-        ks = reinterpret_cast<const T *>(ws_k) + r * d;
-        vs = reinterpret_cast<const T *>(ws_v) + r * d;
+    if (aligned) {
+        *reinterpret_cast<uint4 *>(p) = v.u;
     } else {
-        int lo = it.seg_begin, hi = it.seg_end - 1;      // last segment with dst_pos0 <= t
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) / 2;
-            if (plan.segs[mid].dst_pos0 <= t) lo = mid; else hi = mid - 1;
-        }
-        const kvp_seg sg = plan.segs[lo];
-        const int off = t - sg.dst_pos0;
-        if (sg.pad[0] >= 0) {                            // staged in the workspace, already re-based
-            const int64_t r = (int64_t)plane * ws_rows + sg.pad[0] + off;
-            ks = reinterpret_cast<const T *>(ws_k) + r * d;
-            vs = reinterpret_cast<const T *>(ws_v) + r * d;
-        } else {
-            const int64_t r = (int64_t)plane * pool_rows + sg.src_row0 + off;
-            ks = reinterpret_cast<const T *>(pool_k) + r * d;
-            vs = reinterpret_cast<const T *>(pool_v) + r * d;
-            rope = sg.rope;
-        }
+#pragma unroll
+        for (int e = 0; e < Elem<T>::kPerVec; ++e) p[e] = v.e[e];
     }
-    const float2 *cs = plan.rope + (size_t)rope * half;
-    const int64_t orow = ((int64_t)t * n_kv + hk) * d;
-    for (int p = threadIdx.x; p < half; p += blockDim.x) {
-        const int ia = pairing ? 2 * p : p, ib = pairing ? 2 * p + 1 : p + half;
-        float a = Elem<T>::to_f32(ks[ia]), bb = Elem<T>::to_f32(ks[ib]);
-        if (rope != 0) rotate_pair(a, bb, cs[p].x, cs[p].y);
-        if (k_as_f32) {
-            reinterpret_cast<float *>(k_out)[orow + ia] = a;
-            reinterpret_cast<float *>(k_out)[orow + ib] = bb;
-        } else if (rope != 0) {
-            reinterpret_cast<T *>(k_out)[orow + ia] = Elem<T>::from_f32(a);
-            reinterpret_cast<T *>(k_out)[orow + ib] = Elem<T>::from_f32(bb);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256)
+export_kernel(kvp_plan_dev plan, int b, int layer, int prefix_len, int n_rows, const char *__restrict__ pool_k,
+              const char *__restrict__ pool_v, const char *__restrict__ ws_k,
+              const char *__restrict__ ws_v, int64_t pool_rows, int64_t ws_rows, int n_kv, int d,
+              int pairing, void *__restrict__ k_out, T *__restrict__ v_out, int k_as_f32)
+{
+    constexpr int EV = Elem<T>::kPerVec;
+    __shared__ int s_row[kExportRows], s_rope[kExportRows], s_pool[kExportRows];
+    pdl_launch_dependents();
+    pdl_wait();
+    PDL_AFTER(pool_k); PDL_AFTER(pool_v); PDL_AFTER(ws_k); PDL_AFTER(ws_v); PDL_AFTER(plan.rope);
+    const int t0 = blockIdx.x * kExportRows;
+    if (threadIdx.x < kExportRows && t0 + (int)threadIdx.x < n_rows) {
+        const int t = t0 + threadIdx.x;
+        const kvp_item it = plan.items[b];
+        int row, rope = 0, pool = 0;
+        if (t >= prefix_len) {
+            row = it.tail_row0 + (t - prefix_len);
+        } else if (it.cache_row0 >= 0) {
+            row = it.cache_row0 + t;
         } else {
-            reinterpret_cast<T *>(k_out)[orow + ia] = ks[ia];
-            reinterpret_cast<T *>(k_out)[orow + ib] = ks[ib];
+            int lo = it.seg_begin, hi = it.seg_end - 1;      // last segment with dst_pos0 <= t
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) / 2;
+                if (plan.segs[mid].dst_pos0 <= t) lo = mid; else hi = mid - 1;
+            }
+            const kvp_seg sg = plan.segs[lo];
+            const int off = t - sg.dst_pos0;
+            pool = sg.pad[0] < 0;                            // else staged in the workspace, already re-based
+            row = (pool ? sg.src_row0 : sg.pad[0]) + off;
+            if (pool) rope = sg.rope;
         }
-        v_out[orow + ia] = vs[ia];
-        v_out[orow + ib] = vs[ib];
+        s_row[threadIdx.x] = row;
+        s_rope[threadIdx.x] = rope;
+        s_pool[threadIdx.x] = pool;
+    }
+    __syncthreads();
+    const int half = d / 2, half_vecs = half / EV, vecs = 2 * half_vecs;
+    const int n_items = min(kExportRows, n_rows - t0) * n_kv * half_vecs;
+    const bool al_k = ((uintptr_t)k_out & 15) == 0, al_v = ((uintptr_t)v_out & 15) == 0;
+    for (int w0 = threadIdx.x; w0 < n_items; w0 += 512) {
+        Vec16<T> lo[2], hi[2], va[2], vb[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int w = w0 + 256 * u;
+            if (w >= n_items) break;
+            const int c = w % half_vecs, hk = w / half_vecs % n_kv, r = w / (half_vecs * n_kv);
+            const int64_t src = ((int64_t)(layer * n_kv + hk) * (s_pool[r] ? pool_rows : ws_rows) + s_row[r]) * vecs + c;
+            const uint4 *ks = reinterpret_cast<const uint4 *>(s_pool[r] ? pool_k : ws_k) + src;
+            const uint4 *vs = reinterpret_cast<const uint4 *>(s_pool[r] ? pool_v : ws_v) + src;
+            lo[u].u = __ldg(ks);
+            hi[u].u = __ldg(ks + half_vecs);
+            va[u].u = __ldg(vs);
+            vb[u].u = __ldg(vs + half_vecs);
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int w = w0 + 256 * u;
+            if (w >= n_items) break;
+            const int c = w % half_vecs, hk = w / half_vecs % n_kv, r = w / (half_vecs * n_kv);
+            const int64_t o = ((int64_t)(t0 + r) * n_kv + hk) * d + c * EV;
+            const float2 *cs = plan.rope + (size_t)s_rope[r] * half;
+            if (k_as_f32) {                                  // the rotation's fp32 result, before narrowing
+                float a[EV], x[EV];
+#pragma unroll
+                for (int e = 0; e < EV; ++e) {
+                    a[e] = Elem<T>::to_f32(lo[u].e[e]);
+                    x[e] = Elem<T>::to_f32(hi[u].e[e]);
+                }
+                if (s_rope[r] != 0) {
+#pragma unroll
+                    for (int e = 0; e < EV; ++e) {
+                        if (pairing == 0) {
+                            rotate_pair(a[e], x[e], cs[c * EV + e].x, cs[c * EV + e].y);
+                        } else if (e % 2 == 0) {
+                            const float2 p = cs[(c * EV + e) / 2], p2 = cs[(half + c * EV + e) / 2];
+                            rotate_pair(a[e], a[e + 1], p.x, p.y);
+                            rotate_pair(x[e], x[e + 1], p2.x, p2.y);
+                        }
+                    }
+                }
+                float *ko = reinterpret_cast<float *>(k_out) + o;
+#pragma unroll
+                for (int e = 0; e < EV; ++e) {
+                    ko[e] = a[e];
+                    ko[half + e] = x[e];
+                }
+            } else {
+                if (s_rope[r] != 0) rotate_vec_pair<T>(lo[u], hi[u], cs, c, half_vecs, pairing);
+                store_vec<T>(reinterpret_cast<T *>(k_out) + o, lo[u], al_k);
+                store_vec<T>(reinterpret_cast<T *>(k_out) + o + half, hi[u], al_k);
+            }
+            store_vec<T>(v_out + o, va[u], al_v);
+            store_vec<T>(v_out + o + half, vb[u], al_v);
+        }
     }
 }
 
@@ -339,6 +418,10 @@ attn_core_kernel(kvp_plan_dev plan, int q_len, int q_pos0, int layer, const T *_
     extern __shared__ float sm[];
     float *Qs = sm, *Ks = Qs + BM * LD, *Vs = Ks + BN * LD, *Ps = Ks;
     __shared__ int last_in;
+    pdl_launch_dependents();
+    pdl_wait();
+    PDL_AFTER(q); PDL_AFTER(pool_k); PDL_AFTER(pool_v); PDL_AFTER(ws_k); PDL_AFTER(ws_v); PDL_AFTER(plan.rope);
+    PDL_AFTER(k_new); PDL_AFTER(v_new);
 
     const int hk = blockIdx.y, b = blockIdx.z, rt = blockIdx.x / splits, sp = blockIdx.x % splits;
     const kvp_item it = plan.items[(layer * n_kv + hk) * plan.item_stride + b];
@@ -774,16 +857,12 @@ cudaError_t kvp_launch_append(const kvp_shape &sh, const kvp_plan_dev &plan, int
 {
     const int grid = batch * q_len;
     if (sh.dtype == KVP_DTYPE_BF16)
-        append_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(
-            plan, q_len, q_pos0, (const __nv_bfloat16 *)q, (const __nv_bfloat16 *)k_new, (const __nv_bfloat16 *)v_new, ws_k,
-            ws_v, sh.ws_rows, layer, sh.n_q_heads, sh.n_kv_heads, sh.head_dim, sh.pairing, rope_query, half_turns,
-            (__nv_bfloat16 *)q_rot);
-    else
-        append_kernel<float><<<grid, 256, 0, st>>>(plan, q_len, q_pos0, (const float *)q, (const float *)k_new,
-                                                   (const float *)v_new, ws_k, ws_v, sh.ws_rows, layer, sh.n_q_heads,
-                                                   sh.n_kv_heads, sh.head_dim, sh.pairing, rope_query, half_turns,
-                                                   (float *)q_rot);
-    return cudaGetLastError();
+        return launch_pdl(append_kernel<__nv_bfloat16>, grid, 256, 0, st, plan, q_len, q_pos0, (const __nv_bfloat16 *)q,
+                          (const __nv_bfloat16 *)k_new, (const __nv_bfloat16 *)v_new, ws_k, ws_v, sh.ws_rows, layer, sh.n_q_heads,
+                          sh.n_kv_heads, sh.head_dim, sh.pairing, rope_query, half_turns, (__nv_bfloat16 *)q_rot);
+    return launch_pdl(append_kernel<float>, grid, 256, 0, st, plan, q_len, q_pos0, (const float *)q, (const float *)k_new,
+                      (const float *)v_new, ws_k, ws_v, sh.ws_rows, layer, sh.n_q_heads, sh.n_kv_heads, sh.head_dim, sh.pairing,
+                      rope_query, half_turns, (float *)q_rot);
 }
 
 cudaError_t kvp_launch_export(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t b, int32_t layer,
@@ -793,16 +872,13 @@ cudaError_t kvp_launch_export(const kvp_shape &sh, const kvp_plan_dev &plan, int
 {
     const int n_rows = prefix_len + n_query_rows;
     if (n_rows <= 0) return cudaSuccess;
-    const dim3 grid(n_rows, sh.n_kv_heads);
+    const int grid = (n_rows + kExportRows - 1) / kExportRows;
     if (sh.dtype == KVP_DTYPE_BF16)
-        export_kernel<__nv_bfloat16><<<grid, 64, 0, st>>>(plan, b, layer, prefix_len, pool_k, pool_v, ws_k, ws_v,
-                                                         sh.pool_rows, sh.ws_rows, sh.n_kv_heads, sh.head_dim,
-                                                         sh.pairing, k_out, (__nv_bfloat16 *)v_out, k_as_f32);
-    else
-        export_kernel<float><<<grid, 64, 0, st>>>(plan, b, layer, prefix_len, pool_k, pool_v, ws_k, ws_v, sh.pool_rows,
-                                                 sh.ws_rows, sh.n_kv_heads, sh.head_dim, sh.pairing, k_out,
-                                                 (float *)v_out, k_as_f32);
-    return cudaGetLastError();
+        return launch_pdl(export_kernel<__nv_bfloat16>, grid, 256, 0, st, plan, b, layer, prefix_len, n_rows, pool_k, pool_v, ws_k,
+                          ws_v, sh.pool_rows, sh.ws_rows, sh.n_kv_heads, sh.head_dim, sh.pairing, k_out, (__nv_bfloat16 *)v_out,
+                          k_as_f32);
+    return launch_pdl(export_kernel<float>, grid, 256, 0, st, plan, b, layer, prefix_len, n_rows, pool_k, pool_v, ws_k, ws_v,
+                      sh.pool_rows, sh.ws_rows, sh.n_kv_heads, sh.head_dim, sh.pairing, k_out, (float *)v_out, k_as_f32);
 }
 
 cudaError_t kvp_launch_segment_mass(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t batch, int32_t q_len,
@@ -854,10 +930,9 @@ cudaError_t launch_core(const kvp_shape &sh, const kvp_plan_dev &plan, int batch
     const dim3 grid((unsigned)(row_tiles * splits), sh.n_kv_heads, batch);
     if (ctas) *ctas = (int32_t)(grid.x * grid.y * grid.z);
     const CorePart part = {ws.partial_o, ws.partial_ml, ws.arrived};
-    attn_core_kernel<T, D, TY, TX><<<grid, TY * TX, core_smem<D, TY>, st>>>(plan, q_len, q_pos0, layer, (const T *)q, pool_k, pool_v, ws_k, ws_v,
+    return launch_pdl(attn_core_kernel<T, D, TY, TX>, grid, TY * TX, core_smem<D, TY>, st, plan, q_len, q_pos0, layer, (const T *)q, pool_k, pool_v, ws_k, ws_v,
                                     (const uint4 *)ws.k_new, (const uint4 *)ws.v_new, ws.ws_k, ws.ws_v, sh.pool_rows, sh.ws_rows,
                                     sh.n_q_heads, sh.n_kv_heads, sh.group, sh.pairing, sh.scale, (int)splits, part, (T *)out, lse);
-    return cudaGetLastError();
 }
 
 }  // namespace
