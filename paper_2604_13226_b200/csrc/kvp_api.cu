@@ -212,6 +212,34 @@ int find_slot(kvp_ctx *ctx, int32_t assembly_id)
     return ctx->slots[slot].id == assembly_id ? slot : -1;
 }
 
+// Waits until the last upload from a staging buffer has read it.  That is nearly always so already; otherwise the flags
+// are polled, and after a while the stream is asked as well, so that an upload that never ran (an error on the device, a
+// stream that is being captured) ends the wait with an error.
+int32_t stage_wait(kvp_ctx *ctx, kvp_stage &sg)
+{
+    for (int b = 0; b < sg.blocks; ++b)
+        for (uint32_t polls = 1; sg.flags[b] != sg.seq; ++polls) {
+            if (polls % 4096) continue;
+            const cudaError_t rc = cudaStreamQuery(sg.stream);
+            if (rc == cudaErrorNotReady) continue;
+            if (rc != cudaSuccess) return fail(ctx, KVP_ERR_CUDA, "waiting for an upload: %s", cudaGetErrorString(rc));
+            if (sg.flags[b] != sg.seq) return fail(ctx, KVP_ERR_CUDA, "waiting for an upload: it was never run");
+        }
+    return KVP_OK;
+}
+
+cudaError_t stage_upload(kvp_stage &sg, char *dst, uint64_t bytes, cudaStream_t st)
+{
+    sg.blocks = 0;
+    int32_t blocks = 0;
+    const cudaError_t rc = kvp_launch_upload(sg.host, dst, bytes, sg.flags, sg.seq + 1, &blocks, st);
+    if (rc != cudaSuccess) return rc;
+    ++sg.seq;
+    sg.blocks = blocks;
+    sg.stream = st;
+    return cudaSuccess;
+}
+
 // Work list of the two-stream kernel for one assembly and query length.  Units (<= 256 packed query
 // rows of one request and kv head) are laid end to end, each weighted by the tensor-core work of its
 // key tiles, and the line is cut into equal shares, one per CTA; a cut closer than two tiles to a unit
@@ -489,14 +517,14 @@ int32_t build_schedule(kvp_ctx *ctx, kvp_assembly_host &as, int slot, int layer,
     const size_t used = off_merges + sizeof(kvp_merge_item) * sc.merges.size();
     const int ring = ctx->sched_next;
     ctx->sched_next = (ring + 1) % KVP_SCHED_RING;
-    KVP_CUDA(ctx, cudaEventSynchronize(ctx->sched_event[ring]));          // staging buffer free again?
-    char *h = ctx->sched_ring[ring];
+    const int32_t rs = stage_wait(ctx, ctx->sched_ring[ring]);
+    if (rs != KVP_OK) return rs;
+    char *h = ctx->sched_ring[ring].host;
     memcpy(h, sc.cta_begin.data(), 4 * sc.cta_begin.size());
     memcpy(h + off_works, sc.works.data(), sizeof(kvp_work) * sc.works.size());
     memcpy(h + off_merges, sc.merges.data(), sizeof(kvp_merge_item) * sc.merges.size());
     const int li = as.item_stride ? layer : 0;                   // which of the assembly's work lists
-    KVP_CUDA(ctx, cudaMemcpyAsync(ctx->slot_sched_dev[slot] + ctx->sched_bytes * li, h, used, cudaMemcpyHostToDevice, st));
-    KVP_CUDA(ctx, cudaEventRecord(ctx->sched_event[ring], st));
+    KVP_CUDA(ctx, stage_upload(ctx->sched_ring[ring], ctx->slot_sched_dev[slot] + ctx->sched_bytes * li, used, st));
     kvp_assembly_host::sched_state &ss = as.sched[li];
     ss.q_len = q_len;
     ss.q_lens.assign(q_lens ? q_lens : nullptr, q_lens ? q_lens + as.batch : nullptr);
@@ -629,22 +657,19 @@ int32_t kvp_create(const kvp_config *cfg, kvp_ctx **out)
         cudaDeviceSynchronize() != cudaSuccess)
         return bail(KVP_ERR_CUDA, "clearing pool/workspace failed");
 
-    // one pinned block for all staging buffers: a cudaHostAlloc takes a millisecond or two
-    const uint64_t plan_stage = round_up(ctx->pl.upload, 256);
-    if (cudaHostAlloc((void **)&ctx->staging, plan_stage * cfg->max_assemblies + ctx->sched_bytes * KVP_SCHED_RING,
-                      cudaHostAllocDefault) != cudaSuccess)
+    // one pinned block for all staging buffers and their flags: a cudaHostAlloc takes a millisecond or two
+    const int n_plan = cfg->max_assemblies + 1;
+    const uint64_t plan_stage = round_up(ctx->pl.upload, 256), flag_bytes = 4 * KVP_UPLOAD_BLOCKS;
+    const uint64_t stage_flags = plan_stage * n_plan + ctx->sched_bytes * KVP_SCHED_RING;
+    const uint64_t stage_total = stage_flags + flag_bytes * (n_plan + KVP_SCHED_RING);
+    if (cudaHostAlloc((void **)&ctx->staging, stage_total, cudaHostAllocDefault) != cudaSuccess)
         return bail(KVP_ERR_CUDA, "pinned staging allocation failed");
-    for (int a = 0; a < cfg->max_assemblies; ++a) {
-        cudaEvent_t ev;
-        if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess)
-            return bail(KVP_ERR_CUDA, "staging event creation failed");
-        ctx->slot_plan_host.push_back(ctx->staging + plan_stage * a);
-        ctx->slot_event.push_back(ev);
-    }
-    for (int r = 0; r < KVP_SCHED_RING; ++r) {
-        ctx->sched_ring[r] = ctx->staging + plan_stage * cfg->max_assemblies + ctx->sched_bytes * r;
-        if (cudaEventCreateWithFlags(&ctx->sched_event[r], cudaEventDisableTiming) != cudaSuccess)
-            return bail(KVP_ERR_CUDA, "staging event creation failed");
+    memset(ctx->staging + stage_flags, 0, stage_total - stage_flags);
+    ctx->plan_ring.resize(n_plan);
+    for (int r = 0; r < n_plan + KVP_SCHED_RING; ++r) {
+        kvp_stage &sg = r < n_plan ? ctx->plan_ring[r] : ctx->sched_ring[r - n_plan];
+        sg.host = ctx->staging + (r < n_plan ? plan_stage * r : plan_stage * n_plan + ctx->sched_bytes * (r - n_plan));
+        sg.flags = reinterpret_cast<volatile uint32_t *>(ctx->staging + stage_flags + flag_bytes * r);
     }
 
     if (cudaStreamCreateWithFlags(&ctx->load_stream, cudaStreamNonBlocking) != cudaSuccess ||
@@ -687,8 +712,6 @@ int32_t kvp_destroy(kvp_ctx *ctx)
         cudaSetDevice(ctx->cfg.device);
         cudaDeviceSynchronize();
         if (ctx->staging) cudaFreeHost(ctx->staging);
-        for (cudaEvent_t e : ctx->slot_event) cudaEventDestroy(e);
-        for (cudaEvent_t e : ctx->sched_event) if (e) cudaEventDestroy(e);
         for (auto &w : ctx->tev) for (auto &v : w) for (cudaEvent_t e : v) cudaEventDestroy(e);
         for (cudaEvent_t e : ctx->load_done) cudaEventDestroy(e);
         if (ctx->load_fence) cudaEventDestroy(ctx->load_fence);
@@ -1036,8 +1059,11 @@ static int32_t assemble_impl(kvp_ctx *ctx, int32_t batch, const int32_t *slot_of
     if (!ctx->host_only) {
         cudaStream_t st = (cudaStream_t)stream;
         KVP_CUDA(ctx, cudaSetDevice(cfg.device));
-        KVP_CUDA(ctx, cudaEventSynchronize(ctx->slot_event[slot]));      // staging buffer free again?
-        char *h = ctx->slot_plan_host[slot];
+        kvp_stage &sg = ctx->plan_ring[ctx->plan_next];
+        ctx->plan_next = (ctx->plan_next + 1) % (int)ctx->plan_ring.size();
+        const int32_t rs = stage_wait(ctx, sg);
+        if (rs != KVP_OK) return rs;
+        char *h = sg.host;
         memcpy(h + as.off.items, as.items.data(), sizeof(kvp_item) * as.items.size());
         memcpy(h + as.off.tiles, as.tiles.data(), sizeof(kvp_tile) * as.tiles.size());
         memcpy(h + as.off.chunks, as.chunks.data(), sizeof(kvp_chunk) * as.chunks.size());
@@ -1045,8 +1071,7 @@ static int32_t assemble_impl(kvp_ctx *ctx, int32_t batch, const int32_t *slot_of
         memcpy(h + as.off.delta, as.delta.data(), 4 * as.delta.size());
         for (size_t r = 0; r < kept_packets.size(); ++r)
             memcpy(h + as.off.kept + 4 * r * planes, ctx->packets[kept_packets[r]].kept.data(), 4 * (size_t)planes);
-        KVP_CUDA(ctx, cudaMemcpyAsync(ctx->slot_plan_dev[slot], h, as.off.upload, cudaMemcpyHostToDevice, st));
-        KVP_CUDA(ctx, cudaEventRecord(ctx->slot_event[slot], st));
+        KVP_CUDA(ctx, stage_upload(sg, ctx->slot_plan_dev[slot], as.off.upload, st));
     }
     const int32_t n_chunks = (int32_t)as.chunks.size(), n_rope = (int32_t)as.delta.size();
     std::swap(ctx->slots[slot], ctx->build);
@@ -1228,11 +1253,13 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
         const bool same_lens = q_lens ? (as.sched[li].q_lens.size() == (size_t)as.batch &&
                                           std::equal(q_lens, q_lens + as.batch, as.sched[li].q_lens.begin()))
                                        : as.sched[li].q_lens.empty();
+        a.fresh = 0;
         if (as.sched[li].q_len != q_len || as.sched[li].ctas == 0 || !same_lens ||
             (as.sched[li].q_pos0 != q_pos0 && (q_lens || !same_causal_tiles(sh, q_len, as.sched[li].q_pos0, q_pos0))) ||
             as.sched[li].opts != part_opts) {
             const int32_t rc = build_schedule(ctx, as, slot, layer, q_len, q_pos0, q_lens, part_opts, st);
             if (rc != KVP_OK) return rc;
+            a.fresh = 1;
         }
         const kvp_assembly_host::sched_state &ss = as.sched[li];
         const char *sd = ctx->slot_sched_dev[slot] + ctx->sched_bytes * li;

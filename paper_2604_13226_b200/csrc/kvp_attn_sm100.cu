@@ -82,6 +82,7 @@ struct Params {
     // precise: the counter-rotated query is kept as value + rounding remainder (two bf16 tiles per stream, one
     // epoch buffer instead of two) and Q K^T of a rotated tile takes both
     int precise;
+    int fresh;                 // the work list was uploaded by the kernel in front
     // l2_prefetch: the K/V tiles of a unit are read by at most two units of the launch, i.e. they come from DRAM
     // rather than from L2: the TMA warp then asks L2 for each tile a few loads before it fetches it
     int l2_prefetch;
@@ -302,7 +303,7 @@ struct Work {
 __device__ __forceinline__ Work load_work(const Params &p, int wi)
 {
     const int4 *w4 = reinterpret_cast<const int4 *>(p.works + wi);
-    const int4 a = __ldg(w4), c = __ldg(w4 + 1), e = __ldg(w4 + 2);
+    const int4 a = w4[0], c = w4[1], e = w4[2];
     Work w;
     w.b = a.x; w.hk = a.y; w.row_base = a.z; w.mode = a.w & 0xff;
     w.q_len = (a.w >> 8) ? (a.w >> 8) : p.q_len;
@@ -333,7 +334,7 @@ __device__ __forceinline__ Tile get_tile(const Params &p, const Work &w, int j)
         t.rope = 0;
         t.qoff = j * KVP_TILE_KEYS;
     } else {
-        const int4 g = __ldg(reinterpret_cast<const int4 *>(p.plan.tiles + w.tile_begin + (j - w.n_tail)));
+        const int4 g = *reinterpret_cast<const int4 *>(p.plan.tiles + w.tile_begin + (j - w.n_tail));
         t.row0 = g.x;
         t.n_keys = g.y & 0xFFFF;
         t.src = g.y >> 16;
@@ -1170,7 +1171,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_pool_k, const __grid_co
     c.bar0 = c.smem_base + C::kOffBar;
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(c.smem + C::kOffBar + 8 * C::kNumBars);
     c.abort_flag = tmem_slot + 1;
-    pdl_launch_dependents();
+    if (!p.fresh) pdl_launch_dependents();
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -1200,10 +1201,14 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_pool_k, const __grid_co
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    if (p.fresh) {
+        pdl_wait();
+        pdl_launch_dependents();
+    }
     // from here on: the Q producer, the append and the TMA warp (for anything but pool tiles) wait for the kernel in front;
     // everything else follows from what they deliver
-    c.item_begin = __ldg(p.cta_begin + blockIdx.x);           // (the work list gives every CTA at least one piece)
-    c.item_end = __ldg(p.cta_begin + blockIdx.x + 1);
+    c.item_begin = p.cta_begin[blockIdx.x];                   // (the work list gives every CTA at least one piece)
+    c.item_end = p.cta_begin[blockIdx.x + 1];
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -1251,15 +1256,22 @@ struct MergeOut {
     float2 *part_ml;            // ... and [tiles][128] (m, l)
 };
 
-template <int D>
+// A block takes 32 rows and one of CS column parts of the tile; the parts of a tile are read U at a time, their O and
+// (m, l) together, and folded in by the online rule, so that a tile of up to U parts costs one memory round trip.  CS > 1
+// when a launch has few tiles (a short query over a long context: 8 tiles of 19 parts each took 22 us with 32 blocks that
+// walked the parts one by one, twice).
+template <int D, int CS>
 __device__ __forceinline__ void merge_tile(int b, int hk, int row_base, int item_q_len, const float4 *po, const float2 *pml,
                                            int n, long long stride_o, long long stride_ml, int q_len, int n_q, int n_kv,
                                            int group, float scale, const MergeOut &mo)
 {
-    constexpr int kC = D / 32;                                  // float4 columns per warp
-    __shared__ uint2 tile[32][D / 4 + 1];
+    constexpr int kC = D / 32 / CS;                             // float4 columns per warp
+    constexpr int U = kC == 1 ? 8 : 4;
+    constexpr int kV = D / 64 / CS > 0 ? D / 64 / CS : 1;       // 16-byte words of a row this block writes per thread
+    __shared__ uint2 tile[32][D / 4 / CS + 1];
     const int lane = threadIdx.x & 31, wv = threadIdx.x >> 5;
     const int row = blockIdx.y * 32 + lane;                     // row of the 128-row query tile
+    const int col0 = CS > 1 ? blockIdx.z * (D / 4 / CS) : 0;    // first float4 column of this block
     const int n_rows = group * (item_q_len ? item_q_len : q_len);       // q_len stays the stride of the padded tensors
     const float c2 = scale * 1.4426950408889634f;
     // rows behind the request's last one exist in no partial (a decode step fills 4 of 128): nothing to read or write
@@ -1271,27 +1283,47 @@ __device__ __forceinline__ void merge_tile(int b, int hk, int row_base, int item
     float4 o[kC];
 #pragma unroll
     for (int j = 0; j < kC; ++j) o[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int s = 0; s < n; ++s) {
-        const float2 ml = pml[s * stride_ml + row];
-        if (ml.y > 0.f) M = fmaxf(M, ml.x);
-    }
-    for (int s = 0; s < n; ++s) {
-        const float2 ml = pml[s * stride_ml + row];
-        if (!(ml.y > 0.f)) continue;                        // an empty partial: nothing was visible to this row
-        const float w = exp2f((ml.x - M) * c2);
-        L += w * ml.y;
+#pragma unroll 1
+    for (int s0 = 0; s0 < n; s0 += U) {
+        float2 ml[U];
+        float4 a[U][kC];
 #pragma unroll
-        for (int j = 0; j < kC; ++j) {
-            const float4 a = po[s * stride_o + (wv + 8 * j) * KVP_TILE_ROWS + row];
-            o[j].x += w * a.x; o[j].y += w * a.y; o[j].z += w * a.z; o[j].w += w * a.w;
+        for (int u = 0; u < U; ++u) {
+            ml[u] = make_float2(0.f, 0.f);
+            if (s0 + u < n) {
+                ml[u] = pml[(s0 + u) * stride_ml + row];
+#pragma unroll
+                for (int j = 0; j < kC; ++j) a[u][j] = po[(s0 + u) * stride_o + (col0 + wv + 8 * j) * KVP_TILE_ROWS + row];
+            }
+        }
+        float m_new = M;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (ml[u].y > 0.f) m_new = fmaxf(m_new, ml[u].x);
+        if (m_new > M) {
+            const float alpha = exp2f((M - m_new) * c2);        // (0 while nothing has been added)
+            L *= alpha;
+#pragma unroll
+            for (int j = 0; j < kC; ++j) { o[j].x *= alpha; o[j].y *= alpha; o[j].z *= alpha; o[j].w *= alpha; }
+            M = m_new;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (!(ml[u].y > 0.f)) continue;                     // an empty partial: nothing was visible to this row
+            const float w = exp2f((ml[u].x - M) * c2);
+            L += w * ml[u].y;
+#pragma unroll
+            for (int j = 0; j < kC; ++j) {
+                o[j].x += w * a[u][j].x; o[j].y += w * a[u][j].y; o[j].z += w * a[u][j].z; o[j].w += w * a[u][j].w;
+            }
         }
     }
     if (mo.part_o != nullptr) {                                 // stays a partial: un-normalised, against the max M
         if (!valid) return;
         const long long c = ((long long)b * n_kv + hk) * ((group * q_len + KVP_TILE_ROWS - 1) / KVP_TILE_ROWS) + row_base / KVP_TILE_ROWS;
 #pragma unroll
-        for (int j = 0; j < kC; ++j) mo.part_o[(c * (D / 4) + wv + 8 * j) * KVP_TILE_ROWS + row] = o[j];
-        if (wv == 0) mo.part_ml[c * KVP_TILE_ROWS + row] = make_float2(L > 0.f ? M : -1e30f, L);
+        for (int j = 0; j < kC; ++j) mo.part_o[(c * (D / 4) + col0 + wv + 8 * j) * KVP_TILE_ROWS + row] = o[j];
+        if (wv == 0 && col0 == 0) mo.part_ml[c * KVP_TILE_ROWS + row] = make_float2(L > 0.f ? M : -1e30f, L);
         return;
     }
     const float inv = L > 0.f ? 1.f / L : 0.f;
@@ -1303,34 +1335,35 @@ __device__ __forceinline__ void merge_tile(int b, int hk, int row_base, int item
         tile[lane][wv + 8 * j] = u;
     }
     const int r = row_base + row;
-    if (wv == 0 && r < n_rows && mo.lse != nullptr)
+    if (wv == 0 && col0 == 0 && r < n_rows && mo.lse != nullptr)
         mo.lse[((long long)b * n_q + hk * group + r % group) * q_len + r / group] = M * scale + logf(L);
     __syncthreads();
-    // 8 threads per output row, D / 4 bytes each
-    const int orow = threadIdx.x >> 3, j8 = threadIdx.x & 7;
+    // 8 threads per output row (4 when the block's part of a row is 64 bytes)
+    constexpr int kT = D / 8 / CS / kV;
+    const int orow = threadIdx.x / kT, jt = threadIdx.x % kT;
     const int r2 = row_base + blockIdx.y * 32 + orow;
-    if (r2 < n_rows) {
+    if (orow < 32 && r2 < n_rows) {
         const int i = r2 / group, h = hk * group + r2 % group;
-        uint4 *dst = reinterpret_cast<uint4 *>(mo.out + (((long long)b * q_len + i) * n_q + h) * D) + (D / 64) * j8;
+        uint4 *dst = reinterpret_cast<uint4 *>(mo.out + (((long long)b * q_len + i) * n_q + h) * D) + col0 / 2 + kV * jt;
 #pragma unroll
-        for (int v = 0; v < D / 64; ++v) {
-            const uint2 a0 = tile[orow][2 * ((D / 64) * j8 + v)], a1 = tile[orow][2 * ((D / 64) * j8 + v) + 1];
+        for (int v = 0; v < kV; ++v) {
+            const uint2 a0 = tile[orow][2 * (kV * jt + v)], a1 = tile[orow][2 * (kV * jt + v) + 1];
             dst[v] = make_uint4(a0.x, a0.y, a1.x, a1.y);
         }
     }
 }
 
-// The partial slots of the units of one launch.  Grid (merge item, 4).
-template <int D>
+// The partial slots of the units of one launch.  Grid (merge item, 4, CS).
+template <int D, int CS>
 __global__ void __launch_bounds__(256)
 merge_list_kernel(const kvp_merge_item *__restrict__ merges, int q_len, int n_q, int n_kv, int group, float scale,
                   const float *__restrict__ part_o, const float2 *__restrict__ part_ml, MergeOut mo)
 {
     pdl_launch_dependents();
     pdl_wait();
-    PDL_AFTER(part_o); PDL_AFTER(part_ml);
+    PDL_AFTER(part_o); PDL_AFTER(part_ml); PDL_AFTER(merges);
     const kvp_merge_item mi = merges[blockIdx.x];
-    merge_tile<D>(mi.b, mi.hk, mi.row_base, mi.pad[0], reinterpret_cast<const float4 *>(part_o) + (long long)mi.slot0 * (D / 4 * KVP_TILE_ROWS),
+    merge_tile<D, CS>(mi.b, mi.hk, mi.row_base, mi.pad[0], reinterpret_cast<const float4 *>(part_o) + (long long)mi.slot0 * (D / 4 * KVP_TILE_ROWS),
                part_ml + (long long)mi.slot0 * KVP_TILE_ROWS, mi.n_slots, D / 4 * KVP_TILE_ROWS, KVP_TILE_ROWS, q_len, n_q, n_kv,
                group, scale, mo);
 }
@@ -1343,7 +1376,7 @@ merge_ranks_kernel(const char *__restrict__ parts, int n_parts, long long part_b
 {
     const int c = blockIdx.x;
     const int rt = c % n_rt, hk = (c / n_rt) % n_kv, b = c / (n_rt * n_kv);
-    merge_tile<128>(b, hk, rt * KVP_TILE_ROWS, 0, reinterpret_cast<const float4 *>(parts) + (long long)c * (32 * KVP_TILE_ROWS),
+    merge_tile<128, 1>(b, hk, rt * KVP_TILE_ROWS, 0, reinterpret_cast<const float4 *>(parts) + (long long)c * (32 * KVP_TILE_ROWS),
                reinterpret_cast<const float2 *>(parts + ml_offset) + (long long)c * KVP_TILE_ROWS, n_parts, part_bytes / 16,
                part_bytes / 8, q_len, n_q, n_kv, group, scale, mo);
 }
@@ -1382,6 +1415,7 @@ cudaError_t kvp_launch_attn_sm100(const kvp_shape &sh, const kvp_attn2_args &a, 
     p.status = a.status;
     p.tail_direct = a.tail_direct;
     p.precise = a.precise;
+    p.fresh = a.fresh;
     p.l2_prefetch = a.l2_prefetch;
     p.k_new = (const uint4 *)a.k_new;
     p.v_new = (const uint4 *)a.v_new;
@@ -1409,10 +1443,14 @@ cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_
         mo.part_o = reinterpret_cast<float4 *>(part_out);
         mo.part_ml = reinterpret_cast<float2 *>((char *)part_out + (uint64_t)part_tiles * (32ull * KVP_TILE_ROWS * 16));
     }
-    const dim3 grid(n_merges, KVP_TILE_ROWS / 32);
-    if (sh.head_dim == 64)
-        return launch_pdl(merge_list_kernel<64>, grid, 256, 0, st, merges, q_len, sh.n_q_heads, sh.n_kv_heads, sh.group, sh.scale, partial_o, partial_ml, mo);
-    return launch_pdl(merge_list_kernel<128>, grid, 256, 0, st, merges, q_len, sh.n_q_heads, sh.n_kv_heads, sh.group, sh.scale, partial_o, partial_ml, mo);
+    // whole rows per block when that gives two blocks per SM, else quarter rows (halves with head dimension 64)
+    const bool few = n_merges * (KVP_TILE_ROWS / 32) < 2 * 148;
+    auto go = [&](auto *kernel, int cs) {
+        return launch_pdl(kernel, dim3(n_merges, KVP_TILE_ROWS / 32, cs), 256, 0, st, merges, q_len, sh.n_q_heads, sh.n_kv_heads,
+                          sh.group, sh.scale, partial_o, partial_ml, mo);
+    };
+    if (sh.head_dim == 64) return few ? go(merge_list_kernel<64, 2>, 2) : go(merge_list_kernel<64, 1>, 1);
+    return few ? go(merge_list_kernel<128, 4>, 4) : go(merge_list_kernel<128, 1>, 1);
 }
 
 cudaError_t kvp_launch_merge_ranks(const kvp_shape &sh, int32_t batch, int32_t q_len, const void *parts, int32_t n_parts,

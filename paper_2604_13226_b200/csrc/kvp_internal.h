@@ -16,6 +16,7 @@
 #define KVP_MAX_SPLIT_UNITS 2048   // partial slots (128 query rows each) in the workspace
 #define KVP_CORE_UNITS 2048        // row tiles the CUDA-core kernel may split
 #define KVP_SCHED_RING 8       // pinned staging buffers for work lists
+#define KVP_UPLOAD_BLOCKS 16   // blocks of an upload, each with a completion flag of its own
 
 // ---- device-visible plan records (written by the host planner, uploaded once per assembly) -----
 
@@ -112,6 +113,17 @@ struct kvp_shape {
     int64_t ws_rows;           // rows per plane in one assembly's workspace rows
 };
 
+// One pinned staging buffer of the tables a call sends to the device.  The upload kernel reads it over the host link and
+// then writes the number of the upload into its blocks' flags, which lie in the same pinned memory: whether the buffer is
+// free again is a plain read for the host.
+struct kvp_stage {
+    char *host = nullptr;
+    volatile uint32_t *flags = nullptr;    // [KVP_UPLOAD_BLOCKS]
+    uint32_t seq = 0;                      // number of the last upload from here
+    int32_t blocks = 0;                    // and its blocks
+    cudaStream_t stream = nullptr;         // and its stream
+};
+
 // ---- host-side context -----------------------------------------------------------------------
 
 struct kvp_segment_host {
@@ -181,8 +193,7 @@ struct kvp_ctx {
     std::vector<char *> slot_sched_dev;    // per assembly slot: cta ranges, work list, merge list
     // pinned staging of the same: a ring, so that the layers of an assembly with a list each, or the steps of a
     // decode, do not wait for one another's upload (which lies behind the attention kernels enqueued before it)
-    char *sched_ring[KVP_SCHED_RING] = {};
-    cudaEvent_t sched_event[KVP_SCHED_RING] = {};
+    kvp_stage sched_ring[KVP_SCHED_RING];
     int sched_next = 0;
     const double *half_turns = nullptr;    // device [head_dim/2]: theta_i / pi (angles in half turns per position)
     uint64_t sched_bytes = 0;
@@ -199,10 +210,9 @@ struct kvp_ctx {
     char *q_scratch = nullptr;
     float2 *q_rope = nullptr;              // [max_batch*max_query][head_dim/2] for KVP_ROPE_QUERY
 
-    // pinned host staging (one per slot) and the event guarding its reuse
-    char *staging = nullptr;               // the pinned block that all staging buffers lie in
-    std::vector<char *> slot_plan_host;
-    std::vector<cudaEvent_t> slot_event;
+    char *staging = nullptr;               // the pinned block that all staging buffers and their flags lie in
+    std::vector<kvp_stage> plan_ring;      // staging of plans: one more than assemblies alive
+    int plan_next = 0;
     std::vector<kvp_assembly_host> slots;
     int32_t next_assembly = 0;
 
@@ -228,8 +238,10 @@ struct kvp_ctx {
 // a kernel may have written just before or writes anything, so that launch latency and set-up - barriers, TMEM, filling
 // the grid - lie under the predecessor's tail.  Some thread of every block waits before the block can end, so a grid that
 // has ended implies that its predecessors have: later work in the stream needs no more than that.
-// Readable without waiting: what only copies write (plans, work lists), and the pool - its writers (registration, host
-// copies) never release a successor early, so whatever starts after them finds it complete.
+// Readable without waiting: the pool - its writers (registration, host copies) never release a successor early, so
+// whatever starts after them finds it complete - and tables that a kernel further in front has waited for before it
+// released anyone: the attention kernel behind a fresh work list waits first and releases then, so that the launches
+// behind it find that list and the plan complete.
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -258,6 +270,10 @@ cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
 
 cudaError_t kvp_launch_store_rows(const kvp_shape &sh, const void *src, char *dst_plane0, int64_t plane_rows,
                                   int64_t dst_row0, int32_t n_tokens, cudaStream_t st);
+// `bytes` (rounded up to 16) from pinned host memory to the device; the blocks' flags receive `seq` once they have read
+// their part.  Returns through *blocks how many there are.
+cudaError_t kvp_launch_upload(const void *host, void *dst, uint64_t bytes, volatile uint32_t *flags, uint32_t seq,
+                              int32_t *blocks, cudaStream_t st);
 // the rope table of an assembly and the gather of its chunks, one launch
 cudaError_t kvp_launch_gather(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t n_chunks, int32_t n_rope,
                               const double *half_turns, const char *pool_k, const char *pool_v, char *ws_k, char *ws_v,
@@ -307,6 +323,7 @@ struct kvp_attn2_args {
     // tm_knew / tm_vnew and the kernel copies those rows into the workspace rows itself
     int32_t tail_direct;
     int32_t precise;               // KVP_PRECISE_QK
+    int32_t fresh;                 // the work list was uploaded just before, by a kernel this launch has to wait for
     int32_t l2_prefetch;           // the launch has at most two 256-row units per (request, kv head)
     const void *k_new, *v_new;
     char *ws_k, *ws_v;

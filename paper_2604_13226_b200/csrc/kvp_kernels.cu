@@ -88,6 +88,37 @@ __global__ void store_rows_kernel(const uint4 *__restrict__ src, char *__restric
     }
 }
 
+// ---- upload of a plan or work list -------------------------------------------------------------------
+// A copy engine's transfer of a few KB takes 3.5 us and leaves 2-3 us on either side of it in a stream of kernels; this
+// kernel reads the pinned buffer (up to four 16-byte words per thread in flight) while its predecessor still runs and
+// only the stores come after the wait.  5 x 512 tokens, one layer: two uploads, 47 -> 35 us per pass.
+__global__ void __launch_bounds__(1024)
+upload_kernel(const uint4 *__restrict__ host, uint4 *__restrict__ dst, int n_words, volatile uint32_t *flags, uint32_t seq)
+{
+    pdl_launch_dependents();
+    const int per = (n_words + gridDim.x - 1) / gridDim.x;
+    const int end = min(n_words, ((int)blockIdx.x + 1) * per);
+    bool waited = false;
+    for (int i0 = blockIdx.x * per; i0 < end; i0 += 4096) {
+        uint4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = i0 + u * 1024 + threadIdx.x;
+            if (i < end) v[u] = __ldcv(host + i);
+        }
+        if (!waited) pdl_wait();
+        waited = true;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = i0 + u * 1024 + threadIdx.x;
+            if (i < end) dst[i] = v[u];
+        }
+    }
+    if (!waited) pdl_wait();
+    __syncthreads();                             // every word of this block has been read
+    if (threadIdx.x == 0) flags[blockIdx.x] = seq;
+}
+
 // (cos, sin) of offset x theta, narrowed to fp32 once: the angle is formed in double precision in half turns (offsets
 // reach 1e5 and more), which sincospi reduces exactly.
 __device__ __forceinline__ float2 offset_cos_sin(int32_t offset, double half_turn)
@@ -113,7 +144,7 @@ gather_kernel(kvp_plan_dev plan, int n_table, int n_rope, int groups, const doub
 {
     pdl_launch_dependents();
     pdl_wait();
-    PDL_AFTER(pool_k); PDL_AFTER(pool_v);
+    PDL_AFTER(pool_k); PDL_AFTER(pool_v); PDL_AFTER(plan.chunks); PDL_AFTER(plan.delta);
     if ((int)blockIdx.x < n_table) {
         const int e = blockIdx.x * 256 + threadIdx.x;
         if (e < n_rope * half_dim) table[e] = offset_cos_sin(plan.delta[e / half_dim], half_turns[e % half_dim]);
@@ -825,6 +856,15 @@ cudaError_t kvp_launch_store_rows(const kvp_shape &sh, const void *src, char *ds
     return cudaGetLastError();
 }
 
+cudaError_t kvp_launch_upload(const void *host, void *dst, uint64_t bytes, volatile uint32_t *flags, uint32_t seq,
+                              int32_t *blocks, cudaStream_t st)
+{
+    const int n_words = (int)((bytes + 15) / 16);
+    const int n = std::min(KVP_UPLOAD_BLOCKS, (n_words + 1023) / 1024);
+    *blocks = n;
+    return launch_pdl(upload_kernel, n, 1024, 0, st, (const uint4 *)host, (uint4 *)dst, n_words, flags, seq);
+}
+
 cudaError_t kvp_launch_gather(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t n_chunks, int32_t n_rope,
                               const double *half_turns, const char *pool_k, const char *pool_v, char *ws_k, char *ws_v,
                               cudaStream_t st)
@@ -842,12 +882,10 @@ cudaError_t kvp_launch_gather(const kvp_shape &sh, const kvp_plan_dev &plan, int
     const int grid = n_table + n_chunks * groups;
     float2 *table = const_cast<float2 *>(plan.rope);
     if (sh.dtype == KVP_DTYPE_BF16)
-        gather_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(plan, n_table, n_rope, groups, half_turns, table, pool_k, pool_v, ws_k,
-                                                          ws_v, sh.pool_rows, sh.ws_rows, vecs, half, sh.pairing);
-    else
-        gather_kernel<float><<<grid, 256, 0, st>>>(plan, n_table, n_rope, groups, half_turns, table, pool_k, pool_v, ws_k, ws_v,
-                                                  sh.pool_rows, sh.ws_rows, vecs, half, sh.pairing);
-    return cudaGetLastError();
+        return launch_pdl(gather_kernel<__nv_bfloat16>, grid, 256, 0, st, plan, n_table, n_rope, groups, half_turns, table, pool_k,
+                          pool_v, ws_k, ws_v, sh.pool_rows, sh.ws_rows, vecs, half, sh.pairing);
+    return launch_pdl(gather_kernel<float>, grid, 256, 0, st, plan, n_table, n_rope, groups, half_turns, table, pool_k, pool_v, ws_k,
+                      ws_v, sh.pool_rows, sh.ws_rows, vecs, half, sh.pairing);
 }
 
 cudaError_t kvp_launch_append(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t batch, int32_t q_len,
