@@ -61,11 +61,12 @@ struct Cfg {
     enum BarIdx { kKvFull = 0, kKvEmpty = kStages, kQFull = 2 * kStages, kQFree = kQFull + 4, kSFull = kQFree + 4,   // Q: [2 * stream + buffer]
                   kPFull = kSFull + 2, kOFull = kPFull + 2, kOFree = kOFull + 2, kMlFull = kOFree + 2, kDrain = kMlFull + 1,
                   kNumBars = kDrain + 1 };
-    static_assert(8 * kNumBars + 8 <= 256, "barrier block");
+    static_assert(8 * kNumBars <= 248, "barrier block");
 };
 
 struct Params {
     kvp_plan_dev plan;
+    uint32_t group_magic;                                     // ceil(2^32 / group): r / group = high word of r * magic
     int q_len, q_pos0, layer, n_q, n_kv, group, pairing;      // q_pos0: tail rows appended by earlier calls
     float scale, scale_log2;
     const int32_t *cta_begin;
@@ -119,6 +120,17 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
         : "memory");
     return ok != 0;
 }
+// words of shared memory that several roles look at, by 32-bit address (a generic pointer costs two registers)
+__device__ __forceinline__ uint32_t ld_shared(uint32_t a)
+{
+    uint32_t x;
+    asm volatile("ld.volatile.shared.u32 %0, [%1];" : "=r"(x) : "r"(a) : "memory");
+    return x;
+}
+__device__ __forceinline__ void st_shared(uint32_t a, uint32_t x)
+{
+    asm volatile("st.volatile.shared.u32 [%0], %1;" ::"r"(a), "r"(x) : "memory");
+}
 __device__ __forceinline__ uint64_t global_ns()
 {
     uint64_t t;
@@ -128,7 +140,7 @@ __device__ __forceinline__ uint64_t global_ns()
 
 // Bounded wait.  Returns false when another role has aborted or after ~2 s (then the status word and
 // the CTA's abort flag are set).  `code` identifies the wait.
-__device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag,
+__device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, uint32_t abort_flag,
                                             int32_t *status, int code)
 {
     const uint64_t t0 = global_ns();
@@ -136,16 +148,16 @@ __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volat
     while (true) {
         if (mbar_try_wait(bar, parity)) return true;
         if ((++it & 63u) == 0) {
-            if (*abort_flag) return false;
+            if (ld_shared(abort_flag)) return false;
             if (global_ns() - t0 > 2000000000ull) {
                 atomicCAS(status, 0, code);
-                *abort_flag = 1;
+                st_shared(abort_flag, 1);
                 return false;
             }
         }
     }
 }
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag,
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_t abort_flag,
                                           int32_t *status, int code)
 {
     if (mbar_try_wait(bar, parity)) return true;
@@ -170,12 +182,17 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *tm,
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-// The MMA warp runs convergently; one elected lane issues each tcgen05.mma / tcgen05.commit.
+// The MMA warp runs convergently and one lane, elected once, issues every tcgen05.mma and tcgen05.commit (electing for each
+// of them cost the warp issue slots that it shares with softmax warps).
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+    return e != 0;
+}
 __device__ __forceinline__ void tc_commit(uint32_t bar)
 {
-    asm volatile(
-        "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
-        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar) : "memory");
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
@@ -193,8 +210,8 @@ template <int ACC>
 __device__ __forceinline__ void mma_ss(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc)
 {
     asm volatile(
-        "{\n\t.reg .pred p, e;\n\telect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(d), "l"(a), "l"(b), "r"(idesc), "n"(ACC)
         : "memory");
 }
@@ -202,8 +219,8 @@ __device__ __forceinline__ void mma_ss(uint32_t d, uint64_t a, uint64_t b, uint3
 __device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t acc)
 {
     asm volatile(
-        "{\n\t.reg .pred p, e;\n\telect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
         ::"r"(d), "r"(a), "l"(b), "r"(idesc), "r"(acc)
         : "memory");
 }
@@ -211,8 +228,8 @@ template <int ACC>
 __device__ __forceinline__ void mma_ts_c(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc)
 {
     asm volatile(
-        "{\n\t.reg .pred p, e;\n\telect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
         ::"r"(d), "r"(a), "l"(b), "r"(idesc), "n"(ACC)
         : "memory");
 }
@@ -228,6 +245,15 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t *r)
         "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
         "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
         : KVP_R8(r, 0), KVP_R8(r, 8), KVP_R8(r, 16), KVP_R8(r, 24)
+        : "r"(taddr)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t *r)
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : KVP_R8(r, 0), KVP_R8(r, 8)
         : "r"(taddr)
         : "memory");
 }
@@ -256,6 +282,11 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t *r)
 __device__ __forceinline__ void landed32(uint32_t *r)
 {
     asm volatile("" : KVP_RW8(r, 0), KVP_RW8(r, 8), KVP_RW8(r, 16), KVP_RW8(r, 24)::"memory");
+}
+
+__device__ __forceinline__ void landed16(uint32_t *r)
+{
+    asm volatile("" : KVP_RW8(r, 0), KVP_RW8(r, 8)::"memory");
 }
 
 __device__ __forceinline__ float ex2(float x)
@@ -346,6 +377,9 @@ __device__ __forceinline__ Tile get_tile(const Params &p, const Work &w, int j)
 // unit tile number of step k of stream s
 __device__ __forceinline__ int stream_tile(const Work &w, int s, int k) { return w.lo + (w.mode ? 2 * k + s : k); }
 
+// query token of packed row r
+__device__ __forceinline__ int row_token(const Params &p, int r) { return p.group == 1 ? r : (int)__umulhi((uint32_t)r, p.group_magic); }
+
 // Position of a K (kv = 0) or V (kv = 1) tile, r-th of the piece, in the piece's load order.
 //   mode 0: K0 V0 K1 V1 ...        mode 1: K0 K1 V0 K2 V1 K3 V2 ... V(n-1)
 __device__ __forceinline__ int load_seq(int mode, int n, int r, int kv)
@@ -353,6 +387,36 @@ __device__ __forceinline__ int load_seq(int mode, int n, int r, int kv)
     if (mode == 0) return 2 * r + kv;
     if (kv == 0) return r == 0 ? 0 : 2 * r - 1;
     return r <= n - 2 ? 2 * r + 2 : 2 * n - 1;
+}
+
+// ---- packed fp32 pairs (two lanes of the FMA pipe per instruction) --------------------------------------
+__device__ __forceinline__ uint64_t pair(float lo, float hi)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpair(uint64_t r, float &lo, float &hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(r));
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
 }
 
 // The Q producer (128 threads) writes one 128-row query tile, counter-rotated by the offset of rope-table row
@@ -386,7 +450,7 @@ __device__ __forceinline__ void produce_q_tile(const Params &p, char *qbuf, char
         const int r = row_base + r0 + kRows * i;
         char *lo = mine + i * (kRows * 128);
         if (r < n_rows) {
-            const uint4 *src = reinterpret_cast<const uint4 *>(q_b + ((long long)(r / p.group) * p.n_q + hk * p.group + r % p.group) * D);
+            const uint4 *src = reinterpret_cast<const uint4 *>(q_b) + ((long long)row_token(p, r) * (p.n_q - p.group) + hk * p.group + r) * (D / 8);
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(lo)), "l"(src + c) : "memory");
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(lo + hi_off)), "l"(src + c + kCh) : "memory");
         } else {
@@ -398,60 +462,71 @@ __device__ __forceinline__ void produce_q_tile(const Params &p, char *qbuf, char
     if (rope == 0) return;
     auto lo_f = [](uint32_t u) { return __uint_as_float(u << 16); };
     auto hi_f = [](uint32_t u) { return __uint_as_float(u & 0xffff0000u); };
-#pragma unroll 1
-    for (int i = 0; i < kCh; ++i) {
-        if (row_base + r0 + kRows * i >= n_rows) break;
-        char *lo = mine + i * (kRows * 128);
-        uint4 qa = *reinterpret_cast<uint4 *>(lo), qb = *reinterpret_cast<uint4 *>(lo + hi_off);
-        uint32_t *a = reinterpret_cast<uint32_t *>(&qa);
-        uint32_t *b = reinterpret_cast<uint32_t *>(&qb);
-        uint4 ra, rb;                                            // remainders (precise mode)
-        uint32_t *ar = reinterpret_cast<uint32_t *>(&ra);
-        uint32_t *br = reinterpret_cast<uint32_t *>(&rb);
-        // word = bf16 pair of (x, y); rem = bf16 pair of what the rounding of the word dropped
+    // word = bf16 pair of (x, y); rem = bf16 pair of what the rounding of the word dropped
+    auto rotate = [&](auto rem_c) {
+        constexpr bool kRem = decltype(rem_c)::value;
         auto put = [&](uint32_t &word, uint32_t &rem, float x, float y) {
             word = pack_bf16(x, y);
-            rem = pack_bf16(x - lo_f(word), y - hi_f(word));
+            if (kRem) rem = pack_bf16(x - lo_f(word), y - hi_f(word));
         };
-        if (p.pairing == 0) {
-            // pairs (i, i + 64): word j of chunk c holds elements 8c+2j, 8c+2j+1; partners in chunk c+8
+#pragma unroll 2
+        for (int i = 0; i < kCh; ++i) {
+            if (row_base + r0 + kRows * i >= n_rows) break;
+            char *lo = mine + i * (kRows * 128);
+            uint4 qa = *reinterpret_cast<uint4 *>(lo), qb = *reinterpret_cast<uint4 *>(lo + hi_off);
+            uint32_t *a = reinterpret_cast<uint32_t *>(&qa);
+            uint32_t *b = reinterpret_cast<uint32_t *>(&qb);
+            uint4 ra, rb;                                        // remainders
+            uint32_t *ar = reinterpret_cast<uint32_t *>(&ra);
+            uint32_t *br = reinterpret_cast<uint32_t *>(&rb);
+            if (p.pairing == 0) {
+                // pairs (i, i + D/2): word j of chunk c holds elements 8c+2j, 8c+2j+1; partners in chunk c + kCh
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float4 w = w4[j];                          // cos, sin of pair 8c+2j; cos, sin of pair 8c+2j+1
-                const float a0 = lo_f(a[j]), a1 = hi_f(a[j]), b0 = lo_f(b[j]), b1 = hi_f(b[j]);
-                put(a[j], ar[j], a0 * w.x + b0 * w.y, a1 * w.z + b1 * w.w);     // R(-Delta): cos same, sin negated
-                put(b[j], br[j], b0 * w.x - a0 * w.y, b1 * w.z - a1 * w.w);
+                for (int j = 0; j < 4; ++j) {
+                    const float4 w = w4[j];                      // cos, sin of pair 8c+2j; cos, sin of pair 8c+2j+1
+                    const uint64_t va = pair(lo_f(a[j]), hi_f(a[j])), vb = pair(lo_f(b[j]), hi_f(b[j]));
+                    const uint64_t cc = pair(w.x, w.z), ss = pair(w.y, w.w), ns = pair(-w.y, -w.w);
+                    float x, y;
+                    unpair(fma2(vb, ss, mul2(va, cc)), x, y);    // R(-Delta): cos same, sin negated
+                    put(a[j], ar[j], x, y);
+                    unpair(fma2(va, ns, mul2(vb, cc)), x, y);
+                    put(b[j], br[j], x, y);
+                }
+            } else {
+                // pairs (2i, 2i+1): one word each; chunk c holds pairs 4c..4c+3 (w4[0], w4[1]), its partner w4[2], w4[3]
+#pragma unroll
+                for (int j = 0; j < 4; j += 2) {
+                    float4 w = w4[j >> 1];
+                    float x0 = lo_f(a[j]), y0 = hi_f(a[j]), x1 = lo_f(a[j + 1]), y1 = hi_f(a[j + 1]);
+                    put(a[j], ar[j], x0 * w.x + y0 * w.y, y0 * w.x - x0 * w.y);
+                    put(a[j + 1], ar[j + 1], x1 * w.z + y1 * w.w, y1 * w.z - x1 * w.w);
+                    w = w4[2 + (j >> 1)];
+                    x0 = lo_f(b[j]); y0 = hi_f(b[j]); x1 = lo_f(b[j + 1]); y1 = hi_f(b[j + 1]);
+                    put(b[j], br[j], x0 * w.x + y0 * w.y, y0 * w.x - x0 * w.y);
+                    put(b[j + 1], br[j + 1], x1 * w.z + y1 * w.w, y1 * w.z - x1 * w.w);
+                }
             }
-        } else {
-            // pairs (2i, 2i+1): one word each; chunk c holds pairs 4c..4c+3 (w4[0], w4[1]), chunk c+8 w4[2], w4[3]
-#pragma unroll
-            for (int j = 0; j < 4; j += 2) {
-                float4 w = w4[j >> 1];
-                float x0 = lo_f(a[j]), y0 = hi_f(a[j]), x1 = lo_f(a[j + 1]), y1 = hi_f(a[j + 1]);
-                put(a[j], ar[j], x0 * w.x + y0 * w.y, y0 * w.x - x0 * w.y);
-                put(a[j + 1], ar[j + 1], x1 * w.z + y1 * w.w, y1 * w.z - x1 * w.w);
-                w = w4[2 + (j >> 1)];
-                x0 = lo_f(b[j]); y0 = hi_f(b[j]); x1 = lo_f(b[j + 1]); y1 = hi_f(b[j + 1]);
-                put(b[j], br[j], x0 * w.x + y0 * w.y, y0 * w.x - x0 * w.y);
-                put(b[j + 1], br[j + 1], x1 * w.z + y1 * w.w, y1 * w.z - x1 * w.w);
+            *reinterpret_cast<uint4 *>(lo) = qa;
+            *reinterpret_cast<uint4 *>(lo + hi_off) = qb;
+            if (kRem) {
+                char *rl = qrem + (lo - qbuf);
+                *reinterpret_cast<uint4 *>(rl) = ra;
+                *reinterpret_cast<uint4 *>(rl + hi_off) = rb;
             }
         }
-        *reinterpret_cast<uint4 *>(lo) = qa;
-        *reinterpret_cast<uint4 *>(lo + hi_off) = qb;
-        if (qrem != nullptr) {
-            char *rl = qrem + (lo - qbuf);
-            *reinterpret_cast<uint4 *>(rl) = ra;
-            *reinterpret_cast<uint4 *>(rl + hi_off) = rb;
-        }
-    }
+    };
+    if (qrem != nullptr) rotate(std::integral_constant<bool, true>{});
+    else rotate(std::integral_constant<bool, false>{});
 }
 
 struct Cta {
-    char *smem;
     uint32_t smem_base, bar0, tmem;
-    volatile uint32_t *abort_flag;
     int item_begin, item_end;
     __device__ __forceinline__ uint32_t bar(int i) const { return bar0 + 8u * i; }
+    // behind the barriers: TMEM address and abort flag
+    __device__ __forceinline__ uint32_t tmem_slot() const { return bar0 + 248; }
+    __device__ __forceinline__ uint32_t abort_flag() const { return bar0 + 252; }
+    __device__ __forceinline__ char *smem() const { return reinterpret_cast<char *>(__cvta_shared_to_generic(smem_base)); }
 };
 
 // ---- softmax / correction / epilogue of stream S -------------------------------------------------------
@@ -473,30 +548,6 @@ __device__ __forceinline__ void chunk_mask(uint32_t *v, int lim)
     for (int i = 0; i < 32; ++i)
         if (i >= lim) v[i] = 0xff800000u;                  // -inf
 }
-// ---- packed fp32 pairs (two lanes of the FMA pipe per instruction) --------------------------------------
-__device__ __forceinline__ uint64_t pair(float lo, float hi)
-{
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpair(uint64_t r, float &lo, float &hi)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(r));
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
-{
-    uint64_t d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
-{
-    uint64_t d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
 // p = exp2(s*c2 - mc) for 32 scores, packed as bf16 pairs into pk[0..15] (SPLIT: what that rounding dropped, as bf16
 // pairs, into pk[16..31]); returns their fp32 sum.
 // (Evaluating part of the exponentials by a polynomial on the FMA pipe was measured and lost: the
@@ -533,6 +584,7 @@ __device__ __forceinline__ void rescale_row(uint32_t s_addr, uint32_t o_addr, fl
         for (int ch = 0; ch < D / 32; ++ch) {
             tmem_ld32(o_addr + ch * 32, v);
             tc_wait_ld();
+            landed32(v);
 #pragma unroll
             for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) * alpha);
             tmem_st32(o_addr + ch * 32, v);
@@ -555,13 +607,9 @@ __device__ __forceinline__ void rescale_row(uint32_t s_addr, uint32_t o_addr, fl
             tmem_st32(s_addr + ch * 32, v);
             continue;
         }
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-            "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-            : KVP_R8(v, 0), KVP_R8(v, 8)
-            : "r"(s_addr + ch * 16)
-            : "memory");
+        tmem_ld16(s_addr + ch * 16, v);
         tc_wait_ld();
+        landed16(v);
 #pragma unroll
         for (int i = 0; i < 16; ++i)
             v[i] = pack_bf16(__uint_as_float(v[i] << 16) * alpha, __uint_as_float(v[i] & 0xffff0000u) * alpha);
@@ -578,44 +626,60 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
     const uint32_t s_addr = c.tmem + lane_base + kColS + S * 128;
     const uint32_t o_addr = c.tmem + lane_base + kColO + S * 128;
     const float c2 = p.scale_log2;
-    float2 *ml_smem = reinterpret_cast<float2 *>(c.smem + C::kOffMl);
-    uint32_t nS = 0, nO = 0, nMl = 0;
+    uint32_t ph = 0;                                            // parities: bit 0 S full, bit 1 O full, bit 2 (m, l) full
     bool ok = true;
 
     for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
-        const Work w = load_work(p, wi);
-        const int steps = S == 0 ? w.steps0 : w.steps1;
+        // what the loop needs of the piece; the rest is read again at its end (registers are short here)
+        int steps, first, stride, n_tail, n_total, limit;
+        const kvp_tile *tiles;
+        {
+            const Work w = load_work(p, wi);
+            steps = S == 0 ? w.steps0 : w.steps1;
+            first = stream_tile(w, S, 0);
+            stride = w.mode ? 2 : 1;
+            n_tail = w.n_tail;
+            tiles = p.plan.tiles + w.tile_begin - n_tail;
+            n_total = p.q_pos0 + w.q_len;
+            const int r = w.row_base + (w.mode == 0 ? S * KVP_TILE_ROWS : 0) + t;
+            limit = p.q_pos0 + (r < p.group * w.q_len ? row_token(p, r) : w.q_len - 1) + 1;     // causal keys this row sees
+        }
         if (steps == 0) continue;
-        const int n_rows = p.group * w.q_len;
-        const int r = w.row_base + (w.mode == 0 ? S * KVP_TILE_ROWS : 0) + t;
-        const bool valid = r < n_rows;
-        const int qi = valid ? r / p.group : w.q_len - 1;
-        const int h = w.hk * p.group + (valid ? r % p.group : 0);
 
         float m_ref = -1e30f, l = 0.f;
-        Tile nxt = get_tile(p, w, stream_tile(w, S, 0));
+        auto keys_of = [&](int j) {                             // keys of tile j
+            return j < n_tail ? min(KVP_TILE_KEYS, n_total - j * KVP_TILE_KEYS) : (int)tiles[j].n_keys;
+        };
+        int nk_next = keys_of(first);
 #pragma unroll 1
         for (int k = 0; k < steps; ++k) {
-            const Tile tl = nxt;
-            if (k + 1 < steps) nxt = get_tile(p, w, stream_tile(w, S, k + 1));
-            ok = mbar_wait(c.bar(C::kSFull + S), nS & 1, c.abort_flag, p.status, 30 + S);
-            ++nS;
+            const int j = first + k * stride, n_keys = nk_next;
+            if (k + 1 < steps) nk_next = keys_of(j + stride);
+            ok = mbar_wait(c.bar(C::kSFull + S), ph & 1, c.abort_flag(), p.status, 30 + S);
+            ph ^= 1;
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
 
-            const bool full = (tl.n_keys == KVP_TILE_KEYS) && (tl.qoff < 0);
-            const int lim = tl.qoff < 0 ? tl.n_keys : min(tl.n_keys, p.q_pos0 + qi - tl.qoff + 1);       // visible keys: [0, lim)
-            uint32_t va[32];
+            const bool full = n_keys == KVP_TILE_KEYS && j >= n_tail;
+            const int lim = j >= n_tail ? n_keys : min(n_keys, limit - j * KVP_TILE_KEYS);       // visible keys: [0, lim)
 
-            // One pass over S: the exponentials use the reference max carried over from earlier tiles; each
-            // 32-column chunk's own max is checked first, and only if it exceeds the reference by more than
-            // 2^8 (first tile of a piece, or a rare jump) are l, O and the P chunks already written rescaled.
-            // The exponentials of a chunk are formed optimistically against the current reference while its
-            // max is reduced alongside; the check comes last, so the two dependency chains overlap.
-            auto process = [&](uint32_t *v, int ch) {
-                if (!full) chunk_mask(v, lim - ch * 32);
-                uint32_t pk[C::kSplit ? 32 : 16];
+            // One pass over S, 32 columns at a time: the exponentials use the reference max carried over from earlier tiles;
+            // a chunk's own max is reduced alongside and checked last, so that the two dependency chains overlap.  Only if it
+            // exceeds the reference by more than 2^8 (first tile of a piece, or a rare jump) are l, O and the P chunks
+            // already written rescaled.
+            // a short tile (the end of a document, staged adapter rows) needs P only for the columns P V will read
+            const int n_ch = full ? 4 : max(1, (n_keys + 31) >> 5);
+#pragma unroll 1
+            for (int ch = 0; ch < n_ch; ++ch) {
+                uint32_t v[32], pk[C::kSplit ? 32 : 16];
+                auto load = [&] {
+                    tmem_ld32(s_addr + ch * 32, v);
+                    tc_wait_ld();
+                    landed32(v);
+                    if (!full) chunk_mask(v, lim - ch * 32);
+                };
+                load();
                 const float cm = chunk_max(v, -INFINITY);
                 float ls = chunk_exp<C::kSplit>(v, c2, m_ref * c2, pk);
                 const bool need = (cm - m_ref) * c2 > 8.0f;
@@ -625,24 +689,12 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
                     rescale_row<D>(s_addr, o_addr, alpha, ch, k > 0);
                     l *= alpha;
                     m_ref = m_new;
-                    tmem_ld32(s_addr + ch * 32, v);             // this chunk's scores again (P so far lies below them)
-                    tc_wait_ld();
-                    landed32(v);
-                    if (!full) chunk_mask(v, lim - ch * 32);
+                    load();                                     // this chunk's scores again (P so far lies below them)
                     ls = chunk_exp<C::kSplit>(v, c2, m_ref * c2, pk);
                 }
                 if (C::kSplit) tmem_st32(s_addr + ch * 32, pk);         // over this chunk's own scores
                 else tmem_st16(s_addr + ch * 16, pk);
                 l += ls;
-            };
-            // a short tile (the end of a document, staged adapter rows) needs P only for the columns P V will read
-            const int n_ch = full ? 4 : max(1, (tl.n_keys + 31) >> 5);
-#pragma unroll 1
-            for (int ch = 0; ch < n_ch; ++ch) {
-                tmem_ld32(s_addr + ch * 32, va);
-                tc_wait_ld();
-                landed32(va);
-                process(va, ch);
             }
             tc_wait_st();
             tc_fence_before();
@@ -651,8 +703,15 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
         if (!ok) break;
 
         // ---- end of the piece: O of this stream is complete once its last P V has landed ----------
-        ok = mbar_wait(c.bar(C::kOFull + S), nO & 1, c.abort_flag, p.status, 32 + S);
-        ++nO;
+        const Work w = load_work(p, wi);
+        const int n_rows = p.group * w.q_len;
+        const int r = w.row_base + (w.mode == 0 ? S * KVP_TILE_ROWS : 0) + t;
+        const bool valid = r < n_rows;
+        const int qi = valid ? row_token(p, r) : w.q_len - 1;
+        const int h = w.hk * p.group + (valid ? r - qi * p.group : 0);
+        float2 *ml_smem = reinterpret_cast<float2 *>(c.smem() + C::kOffMl);
+        ok = mbar_wait(c.bar(C::kOFull + S), (ph >> 1) & 1, c.abort_flag(), p.status, 32 + S);
+        ph ^= 2;
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         tc_fence_after();
@@ -665,8 +724,8 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
         float w0 = 1.f, w1 = 0.f;
         const bool both = (w.mode == 1) && (w.steps1 > 0);
         if (both) {
-            ok = mbar_wait(c.bar(C::kMlFull), nMl & 1, c.abort_flag, p.status, 34);
-            ++nMl;
+            ok = mbar_wait(c.bar(C::kMlFull), (ph >> 2) & 1, c.abort_flag(), p.status, 34);
+            ph ^= 4;
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
@@ -693,12 +752,14 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
             uint32_t a[32];
             tmem_ld32(o_addr + ch * 32, a);
             tc_wait_ld();
+            landed32(a);
 #pragma unroll
             for (int i = 0; i < 32; ++i) a[i] = __float_as_uint(__uint_as_float(a[i]) * w0);
             if (both) {
                 uint32_t b2[32];
                 tmem_ld32(o_addr + 128 + ch * 32, b2);
                 tc_wait_ld();
+                landed32(b2);
 #pragma unroll
                 for (int i = 0; i < 32; ++i) a[i] = __float_as_uint(fmaf(__uint_as_float(b2[i]), w1, __uint_as_float(a[i])));
             }
@@ -751,11 +812,11 @@ __device__ __forceinline__ void producer_role(const Params &p, const Cta &c, con
             const uint32_t back = one_buffer ? 1u : 2u;      // the epoch that used this buffer last
             if (nEp >= back) {
                 const uint32_t par = one_buffer ? (nEp - 1) & 1 : ((nEp >> 1) - 1) & 1;
-                ok = mbar_wait(c.bar(C::kQFree + 2 * s + buf), par, c.abort_flag, p.status, 40 + s);
+                ok = mbar_wait(c.bar(C::kQFree + 2 * s + buf), par, c.abort_flag(), p.status, 40 + s);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) return;
             }
-            char *qb = c.smem + C::kOffQ + (2 * s + buf) * kQBufBytes;
+            char *qb = c.smem() + C::kOffQ + (2 * s + buf) * kQBufBytes;
             char *qrem = C::kSplit ? qb + kHalfBytes : one_buffer ? qb + kQBufBytes : nullptr;
             produce_q_tile<D>(p, qb, qrem, t, p.q + (long long)w.b * p.q_len * p.n_q * D,
                            w.hk, w.row_base + (w.mode == 0 ? s * KVP_TILE_ROWS : 0), n_rows, rope);
@@ -831,7 +892,7 @@ __device__ __forceinline__ void tma_role(const Params &p, const Cta &c, const in
     using C = Cfg<D>;
     constexpr int kStages = C::kStages, kTileBytes = C::kTileBytes;
     uint32_t ring_n = 0;                                   // loads issued before this piece
-    bool ok = true, waited = false;
+    bool ok = true;
     for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
         const Work w = load_work(p, wi);
         const int n_loads = 2 * w.n;
@@ -850,47 +911,36 @@ __device__ __forceinline__ void tma_role(const Params &p, const Cta &c, const in
                 row0 = tl.row0;
                 src = tl.src;
             }
+            // its lane issues each load when its turn comes (nothing is handed round: this warp shares its sub-partition's
+            // issue slots with softmax warps)
+            const CUtensorMap *tm = src == 2 ? (kv ? tm_vnew : tm_knew) : src == 0 ? (kv ? tm_pool_v : tm_pool_k) : (kv ? tm_ws_v : tm_ws_k);
             const int cnt = min(32, n_loads - q0);
+            const bool ahead = p.l2_prefetch && w.mode == 0 && lane < cnt && src != 2;
+            uint32_t stage = (ring_n + (uint32_t)q0) % kStages, use = (ring_n + (uint32_t)q0) / kStages;
+#pragma unroll 1
             for (int i = 0; i < cnt && ok; ++i) {
-                const int row0_i = __shfl_sync(0xffffffffu, row0, i);
-                const int src_i = __shfl_sync(0xffffffffu, src, i);
-                const int kv_i = __shfl_sync(0xffffffffu, kv, i);
-                if (p.l2_prefetch && w.mode == 0) {      // tiles that come from DRAM: ask L2 for the one four loads ahead
-                    constexpr int KVP_L2_PREFETCH = 4;
-                    const int j = min(i + KVP_L2_PREFETCH, 31);
-                    const int row0_j = __shfl_sync(0xffffffffu, row0, j);
-                    const int src_j = __shfl_sync(0xffffffffu, src, j);
-                    const int kv_j = __shfl_sync(0xffffffffu, kv, j);
-                    if (lane == 0 && i + KVP_L2_PREFETCH < cnt && src_j != 2) {
-                        const CUtensorMap *tm = src_j == 0 ? (kv_j ? tm_pool_v : tm_pool_k) : (kv_j ? tm_ws_v : tm_ws_k);
-                        asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(tm), "r"(0), "r"(row0_j), "r"(w.plane) : "memory");
-                        if (D == 128)
-                            asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(tm), "r"(64), "r"(row0_j), "r"(w.plane) : "memory");
-                    }
+                if (ahead && lane == i + 4) {              // tiles that come from DRAM: L2 is asked for the one four loads ahead
+                    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(tm), "r"(0), "r"(row0), "r"(w.plane) : "memory");
+                    if (D == 128)
+                        asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(tm), "r"(64), "r"(row0), "r"(w.plane) : "memory");
                 }
-                if (lane == 0) {
-                    const uint32_t g = ring_n + (uint32_t)(q0 + i);
-                    const uint32_t stage = g % kStages, use = g / kStages;
-                    if (use > 0) ok = mbar_wait(c.bar(C::kKvEmpty + stage), (use - 1) & 1, c.abort_flag, p.status, 10 + stage);
+                if (lane == i) {
+                    if (use > 0) ok = mbar_wait(c.bar(C::kKvEmpty + stage), (use - 1) & 1, c.abort_flag(), p.status, 10 + stage);
                     if (ok) {
-                        const uint32_t dst = c.smem_base + C::kOffRing + stage * kTileBytes;
-                        mbar_expect_tx(c.bar(C::kKvFull + stage), kTileBytes);
-                        if (src_i != 0 && !waited) {       // staged or appended rows: a kernel in front may have written them
-                            pdl_wait();
-                            waited = true;
-                        }
-                        if (src_i == 2) {
-                            const CUtensorMap *tm = kv_i ? tm_vnew : tm_knew;
-                            tma_load_4d(dst, tm, 0, w.hk, row0_i, w.b, c.bar(C::kKvFull + stage));
-                            if (D == 128) tma_load_4d(dst + kHalfBytes, tm, 64, w.hk, row0_i, w.b, c.bar(C::kKvFull + stage));
+                        const uint32_t dst = c.smem_base + C::kOffRing + stage * kTileBytes, full = c.bar(C::kKvFull + stage);
+                        mbar_expect_tx(full, kTileBytes);
+                        if (src != 0) pdl_wait();          // staged or appended rows: a kernel in front may have written them
+                        if (src == 2) {
+                            tma_load_4d(dst, tm, 0, w.hk, row0, w.b, full);
+                            if (D == 128) tma_load_4d(dst + kHalfBytes, tm, 64, w.hk, row0, w.b, full);
                         } else {
-                            const CUtensorMap *tm = src_i == 0 ? (kv_i ? tm_pool_v : tm_pool_k) : (kv_i ? tm_ws_v : tm_ws_k);
-                            tma_load_3d(dst, tm, 0, row0_i, w.plane, c.bar(C::kKvFull + stage));
-                            if (D == 128) tma_load_3d(dst + kHalfBytes, tm, 64, row0_i, w.plane, c.bar(C::kKvFull + stage));
+                            tma_load_3d(dst, tm, 0, row0, w.plane, full);
+                            if (D == 128) tma_load_3d(dst + kHalfBytes, tm, 64, row0, w.plane, full);
                         }
                     }
                 }
-                ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+                ok = __all_sync(0xffffffffu, ok);
+                if (++stage == kStages) { stage = 0; ++use; }
             }
         }
         ring_n += (uint32_t)n_loads;
@@ -912,6 +962,7 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
     constexpr uint32_t kSteps = D / 16;                       // K-steps of Q K^T
     constexpr uint32_t kRem16 = (C::kSplit ? kHalfBytes : kQBufBytes) >> 4;      // from the rotated Q to its remainders
     const uint32_t idesc_pv = instr_desc(D, 1);
+    const bool lead = elect_one();
     const bool one_buffer = !C::kSplit && p.precise, two_part = C::kSplit || p.precise;
     // P of 16 keys (K-step kk) in the score columns: packed pairs one after the other, or per 32 keys 16 columns of
     // pairs and 16 of remainders
@@ -936,40 +987,43 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
         const Tile tl = ms.cur;
         if (k == 0 || tl.rope != ms.prev_rope) {                  // first tile of a document: its own Q buffer
             ms.qbuf = one_buffer ? 0 : (ms.nEpoch & 1);
-            ok = mbar_wait(c.bar(C::kQFull + 2 * s + ms.qbuf), (one_buffer ? ms.nEpoch : ms.nEpoch >> 1) & 1, c.abort_flag, p.status, 20 + s);
+            ok = mbar_wait(c.bar(C::kQFull + 2 * s + ms.qbuf), (one_buffer ? ms.nEpoch : ms.nEpoch >> 1) & 1, c.abort_flag(), p.status, 20 + s);
             ++ms.nEpoch;
         }
         const int r = wq.mode ? 2 * k + s : k;
         const uint32_t g = base + (uint32_t)load_seq(wq.mode, wq.n, r, 0);
         const uint32_t stage = g % kStages, par = (g / kStages) & 1;
-        if (ok && !(shared_stage && s == 1)) ok = mbar_wait(c.bar(C::kKvFull + stage), par, c.abort_flag, p.status, 22);
+        if (ok && !(shared_stage && s == 1)) ok = mbar_wait(c.bar(C::kKvFull + stage), par, c.abort_flag(), p.status, 22);
         ok = __all_sync(0xffffffffu, ok);                         // the lanes stay together
         if (!ok) return;
         tc_fence_after();
-        const uint32_t n16 = max(16u, (uint32_t)(tl.n_keys + 15) & ~15u);
-        const uint32_t idesc = instr_desc(n16, 0);
-        const uint32_t q_lo = desc_lo(c.smem_base + C::kOffQ + (2 * s + ms.qbuf) * kQBufBytes, 16);
-        const uint32_t k_lo = desc_lo(c.smem_base + C::kOffRing + stage * kTileBytes, 16);
-        const uint32_t d = c.tmem + kColS + s * 128;
-        mma_ss<0>(d, desc64(q_lo, kDescHi), desc64(k_lo, kDescHi), idesc);
+        const bool last = (k + 1 == n_steps) || (ms.nxt.rope != tl.rope);
+        if (lead) {
+            const uint32_t n16 = max(16u, (uint32_t)(tl.n_keys + 15) & ~15u);
+            const uint32_t idesc = instr_desc(n16, 0);
+            const uint32_t q_lo = desc_lo(c.smem_base + C::kOffQ + (2 * s + ms.qbuf) * kQBufBytes, 16);
+            const uint32_t k_lo = desc_lo(c.smem_base + C::kOffRing + stage * kTileBytes, 16);
+            const uint32_t d = c.tmem + kColS + s * 128;
+            mma_ss<0>(d, desc64(q_lo, kDescHi), desc64(k_lo, kDescHi), idesc);
 #pragma unroll
-        for (int kk = 1; kk < (int)kSteps; ++kk) {                         // 16 columns per step: 32 bytes, second half 16 KB on
-            constexpr uint32_t kHalf16 = kHalfBytes >> 4;
-            const uint32_t off = (kk >> 2) * kHalf16 + (kk & 3) * 2;
-            mma_ss<1>(d, desc64(q_lo + off, kDescHi), desc64(k_lo + off, kDescHi), idesc);
-        }
-        if (two_part && tl.rope != 0) {                         // + (rounding remainder of the rotated Q) K^T
-#pragma unroll
-            for (int kk = 0; kk < (int)kSteps; ++kk) {
+            for (int kk = 1; kk < (int)kSteps; ++kk) {                         // 16 columns per step: 32 bytes, second half 16 KB on
                 constexpr uint32_t kHalf16 = kHalfBytes >> 4;
                 const uint32_t off = (kk >> 2) * kHalf16 + (kk & 3) * 2;
-                mma_ss<1>(d, desc64(q_lo + kRem16 + off, kDescHi), desc64(k_lo + off, kDescHi), idesc);
+                mma_ss<1>(d, desc64(q_lo + off, kDescHi), desc64(k_lo + off, kDescHi), idesc);
             }
+            if (two_part && tl.rope != 0) {                         // + (rounding remainder of the rotated Q) K^T
+#pragma unroll
+                for (int kk = 0; kk < (int)kSteps; ++kk) {
+                    constexpr uint32_t kHalf16 = kHalfBytes >> 4;
+                    const uint32_t off = (kk >> 2) * kHalf16 + (kk & 3) * 2;
+                    mma_ss<1>(d, desc64(q_lo + kRem16 + off, kDescHi), desc64(k_lo + off, kDescHi), idesc);
+                }
+            }
+            tc_commit(c.bar(C::kSFull + s));
+            if (!shared_stage || s == 1) tc_commit(c.bar(C::kKvEmpty + stage));
+            if (last) tc_commit(c.bar(C::kQFree + 2 * s + ms.qbuf));
         }
-        tc_commit(c.bar(C::kSFull + s));
-        if (!shared_stage || s == 1) tc_commit(c.bar(C::kKvEmpty + stage));
-        const bool last = (k + 1 == n_steps) || (ms.nxt.rope != tl.rope);
-        if (last) tc_commit(c.bar(C::kQFree + 2 * s + ms.qbuf));
+        __syncwarp();
         ms.prev_rope = tl.rope;
         ms.prev_keys = tl.n_keys;
         ms.cur = ms.nxt;
@@ -1013,75 +1067,78 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
                 MmaStream &ms = st[s];
                 // ---- waits of the block ---------------------------------------------------------
                 if (s == 0) {                                 // the tiles first: they land while P is being formed
-                    if (k >= 1) ok = mbar_wait(c.bar(C::kKvFull + stV), parV, c.abort_flag, p.status, 23);
-                    if (k < n && ok) ok = mbar_wait(c.bar(C::kKvFull + stK), parK, c.abort_flag, p.status, 22);
+                    if (k >= 1) ok = mbar_wait(c.bar(C::kKvFull + stV), parV, c.abort_flag(), p.status, 23);
+                    if (k < n && ok) ok = mbar_wait(c.bar(C::kKvFull + stK), parK, c.abort_flag(), p.status, 22);
                 }
                 if (k >= 1) {
-                    if (ok) ok = mbar_wait(c.bar(C::kPFull + s), ms.nP & 1, c.abort_flag, p.status, 24 + s);
+                    if (ok) ok = mbar_wait(c.bar(C::kPFull + s), ms.nP & 1, c.abort_flag(), p.status, 24 + s);
                     ++ms.nP;
                     if (ok && k == 1 && ms.nItems > 0)
-                        ok = mbar_wait(c.bar(C::kOFree + s), (ms.nItems - 1) & 1, c.abort_flag, p.status, 26 + s);
+                        ok = mbar_wait(c.bar(C::kOFree + s), (ms.nItems - 1) & 1, c.abort_flag(), p.status, 26 + s);
                 }
                 if (k < n) {
                     if (newq) {
                         ms.qbuf = one_buffer ? 0 : (ms.nEpoch & 1);
-                        if (ok) ok = mbar_wait(c.bar(C::kQFull + 2 * s + ms.qbuf), (one_buffer ? ms.nEpoch : ms.nEpoch >> 1) & 1, c.abort_flag, p.status, 20 + s);
+                        if (ok) ok = mbar_wait(c.bar(C::kQFull + 2 * s + ms.qbuf), (one_buffer ? ms.nEpoch : ms.nEpoch >> 1) & 1, c.abort_flag(), p.status, 20 + s);
                         ++ms.nEpoch;
                     }
                 }
                 ok = __all_sync(0xffffffffu, ok);                 // the lanes stay together
                 if (!ok) return;
                 tc_fence_after();
-                if (k >= 1) {
-                    // ---- O_s += P_s V of step k-1 ---------------------------------------------------
-                    const uint32_t v_lo = desc_lo(c.smem_base + C::kOffRing + stV * kTileBytes, kHalfBytes);
-                    const uint32_t pa = c.tmem + kColS + s * 128;
-                    const uint32_t oa = c.tmem + kColO + s * 128;
-                    if (prev_nk == KVP_TILE_KEYS && k > 1) {
+                if (lead) {
+                    if (k >= 1) {
+                        // ---- O_s += P_s V of step k-1 ---------------------------------------------------
+                        const uint32_t v_lo = desc_lo(c.smem_base + C::kOffRing + stV * kTileBytes, kHalfBytes);
+                        const uint32_t pa = c.tmem + kColS + s * 128;
+                        const uint32_t oa = c.tmem + kColO + s * 128;
+                        if (prev_nk == KVP_TILE_KEYS && k > 1) {
 #pragma unroll
-                        for (int kk = 0; kk < 8; ++kk) {         // 16 keys per step: V advances 2048 bytes
-                            mma_ts_c<1>(oa, pa + p_col(kk), desc64(v_lo + kk * 128, kDescHi), idesc_pv);
-                            if (C::kSplit) mma_ts_c<1>(oa, pa + p_col(kk) + 16, desc64(v_lo + kk * 128, kDescHi), idesc_pv);
+                            for (int kk = 0; kk < 8; ++kk) {         // 16 keys per step: V advances 2048 bytes
+                                mma_ts_c<1>(oa, pa + p_col(kk), desc64(v_lo + kk * 128, kDescHi), idesc_pv);
+                                if (C::kSplit) mma_ts_c<1>(oa, pa + p_col(kk) + 16, desc64(v_lo + kk * 128, kDescHi), idesc_pv);
+                            }
+                        } else {
+                            const int ksteps = max(1, (prev_nk + 15) >> 4);    // an empty tile still initialises O (P = 0)
+                            for (int kk = 0; kk < ksteps; ++kk) {
+                                mma_ts(oa, pa + p_col(kk), desc64(v_lo + kk * 128, kDescHi), idesc_pv, (k > 1 || kk > 0));
+                                if (C::kSplit) mma_ts_c<1>(oa, pa + p_col(kk) + 16, desc64(v_lo + kk * 128, kDescHi), idesc_pv);
+                            }
                         }
-                    } else {
-                        const int ksteps = max(1, (prev_nk + 15) >> 4);    // an empty tile still initialises O (P = 0)
-                        for (int kk = 0; kk < ksteps; ++kk) {
-                            mma_ts(oa, pa + p_col(kk), desc64(v_lo + kk * 128, kDescHi), idesc_pv, (k > 1 || kk > 0));
-                            if (C::kSplit) mma_ts_c<1>(oa, pa + p_col(kk) + 16, desc64(v_lo + kk * 128, kDescHi), idesc_pv);
+                        if (s == 1) tc_commit(c.bar(C::kKvEmpty + stV));
+                        if (k == n) {
+                            tc_commit(c.bar(C::kOFull + s));
                         }
                     }
-                    if (s == 1) tc_commit(c.bar(C::kKvEmpty + stV));
-                    if (k == n) {
-                        tc_commit(c.bar(C::kOFull + s));
-                        ++ms.nItems;
-                    }
-                }
-                if (k < n) {
-                    // ---- S_s = Q_s K^T of step k ----------------------------------------------------
-                    const uint32_t n16 = max(16u, (uint32_t)(nk + 15) & ~15u);   
-                    const uint32_t idesc = instr_desc(n16, 0);
-                    const uint32_t q_lo = desc_lo(c.smem_base + C::kOffQ + (2 * s + ms.qbuf) * kQBufBytes, 16);
-                    const uint32_t k_lo = desc_lo(c.smem_base + C::kOffRing + stK * kTileBytes, 16);
-                    const uint32_t d = c.tmem + kColS + s * 128;
-                    mma_ss<0>(d, desc64(q_lo, kDescHi), desc64(k_lo, kDescHi), idesc);
+                    if (k < n) {
+                        // ---- S_s = Q_s K^T of step k ----------------------------------------------------
+                        const uint32_t n16 = max(16u, (uint32_t)(nk + 15) & ~15u);   
+                        const uint32_t idesc = instr_desc(n16, 0);
+                        const uint32_t q_lo = desc_lo(c.smem_base + C::kOffQ + (2 * s + ms.qbuf) * kQBufBytes, 16);
+                        const uint32_t k_lo = desc_lo(c.smem_base + C::kOffRing + stK * kTileBytes, 16);
+                        const uint32_t d = c.tmem + kColS + s * 128;
+                        mma_ss<0>(d, desc64(q_lo, kDescHi), desc64(k_lo, kDescHi), idesc);
 #pragma unroll
-                    for (int kk = 1; kk < (int)kSteps; ++kk) {             // 16 columns per step: 32 bytes, second half 16 KB on
-                        constexpr uint32_t kHalf16 = kHalfBytes >> 4;
-                        const uint32_t off = (kk >> 2) * kHalf16 + (kk & 3) * 2;
-                        mma_ss<1>(d, desc64(q_lo + off, kDescHi), desc64(k_lo + off, kDescHi), idesc);
-                    }
-                    if (two_part && rope != 0) {                // + (rounding remainder of the rotated Q) K^T
-#pragma unroll
-                        for (int kk = 0; kk < (int)kSteps; ++kk) {
+                        for (int kk = 1; kk < (int)kSteps; ++kk) {             // 16 columns per step: 32 bytes, second half 16 KB on
                             constexpr uint32_t kHalf16 = kHalfBytes >> 4;
                             const uint32_t off = (kk >> 2) * kHalf16 + (kk & 3) * 2;
-                            mma_ss<1>(d, desc64(q_lo + kRem16 + off, kDescHi), desc64(k_lo + off, kDescHi), idesc);
+                            mma_ss<1>(d, desc64(q_lo + off, kDescHi), desc64(k_lo + off, kDescHi), idesc);
                         }
+                        if (two_part && rope != 0) {                // + (rounding remainder of the rotated Q) K^T
+#pragma unroll
+                            for (int kk = 0; kk < (int)kSteps; ++kk) {
+                                constexpr uint32_t kHalf16 = kHalfBytes >> 4;
+                                const uint32_t off = (kk >> 2) * kHalf16 + (kk & 3) * 2;
+                                mma_ss<1>(d, desc64(q_lo + kRem16 + off, kDescHi), desc64(k_lo + off, kDescHi), idesc);
+                            }
+                        }
+                        tc_commit(c.bar(C::kSFull + s));
+                        if (s == 1) tc_commit(c.bar(C::kKvEmpty + stK));
+                        if (lastq) tc_commit(c.bar(C::kQFree + 2 * s + ms.qbuf));
                     }
-                    tc_commit(c.bar(C::kSFull + s));
-                    if (s == 1) tc_commit(c.bar(C::kKvEmpty + stK));
-                    if (lastq) tc_commit(c.bar(C::kQFree + 2 * s + ms.qbuf));
                 }
+                __syncwarp();
+                if (k == n) ++ms.nItems;
             };
             step(std::integral_constant<int, 0>{});
             if (ok) step(std::integral_constant<int, 1>{});
@@ -1110,35 +1167,38 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
                 const int r = w.mode ? 2 * (k - 1) + s : k - 1;
                 const uint32_t g = ring_n + (uint32_t)load_seq(w.mode, w.n, r, 1);
                 const uint32_t stage = g % kStages, par = (g / kStages) & 1;
-                if (!(shared_stage && s == 1)) ok = mbar_wait(c.bar(C::kKvFull + stage), par, c.abort_flag, p.status, 23);
-                if (ok) ok = mbar_wait(c.bar(C::kPFull + s), ms.nP & 1, c.abort_flag, p.status, 24 + s);
+                if (!(shared_stage && s == 1)) ok = mbar_wait(c.bar(C::kKvFull + stage), par, c.abort_flag(), p.status, 23);
+                if (ok) ok = mbar_wait(c.bar(C::kPFull + s), ms.nP & 1, c.abort_flag(), p.status, 24 + s);
                 ++ms.nP;
                 if (ok && k == 1 && ms.nItems > 0)
-                    ok = mbar_wait(c.bar(C::kOFree + s), (ms.nItems - 1) & 1, c.abort_flag, p.status, 26 + s);
+                    ok = mbar_wait(c.bar(C::kOFree + s), (ms.nItems - 1) & 1, c.abort_flag(), p.status, 26 + s);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) return;
                 tc_fence_after();
-                const uint32_t v_lo = desc_lo(c.smem_base + C::kOffRing + stage * kTileBytes, kHalfBytes);
-                const uint32_t pa = c.tmem + kColS + s * 128;
-                const uint32_t oa = c.tmem + kColO + s * 128;
-                if (ms.prev_keys == KVP_TILE_KEYS && k > 1) {
+                if (lead) {
+                    const uint32_t v_lo = desc_lo(c.smem_base + C::kOffRing + stage * kTileBytes, kHalfBytes);
+                    const uint32_t pa = c.tmem + kColS + s * 128;
+                    const uint32_t oa = c.tmem + kColO + s * 128;
+                    if (ms.prev_keys == KVP_TILE_KEYS && k > 1) {
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk) {             // 16 keys per step: V advances 2048 bytes
-                        mma_ts_c<1>(oa, pa + p_col(kk), desc64(v_lo + kk * 128, kDescHi), idesc_pv);
-                        if (C::kSplit) mma_ts_c<1>(oa, pa + p_col(kk) + 16, desc64(v_lo + kk * 128, kDescHi), idesc_pv);
+                        for (int kk = 0; kk < 8; ++kk) {             // 16 keys per step: V advances 2048 bytes
+                            mma_ts_c<1>(oa, pa + p_col(kk), desc64(v_lo + kk * 128, kDescHi), idesc_pv);
+                            if (C::kSplit) mma_ts_c<1>(oa, pa + p_col(kk) + 16, desc64(v_lo + kk * 128, kDescHi), idesc_pv);
+                        }
+                    } else {
+                        const int ksteps = max(1, (ms.prev_keys + 15) >> 4);   // an empty tile still initialises O (P = 0)
+                        for (int kk = 0; kk < ksteps; ++kk) {
+                            mma_ts(oa, pa + p_col(kk), desc64(v_lo + kk * 128, kDescHi), idesc_pv, (k > 1 || kk > 0));
+                            if (C::kSplit) mma_ts_c<1>(oa, pa + p_col(kk) + 16, desc64(v_lo + kk * 128, kDescHi), idesc_pv);
+                        }
                     }
-                } else {
-                    const int ksteps = max(1, (ms.prev_keys + 15) >> 4);   // an empty tile still initialises O (P = 0)
-                    for (int kk = 0; kk < ksteps; ++kk) {
-                        mma_ts(oa, pa + p_col(kk), desc64(v_lo + kk * 128, kDescHi), idesc_pv, (k > 1 || kk > 0));
-                        if (C::kSplit) mma_ts_c<1>(oa, pa + p_col(kk) + 16, desc64(v_lo + kk * 128, kDescHi), idesc_pv);
+                    if (!shared_stage || s == 1) tc_commit(c.bar(C::kKvEmpty + stage));
+                    if (k == steps[s]) {
+                        tc_commit(c.bar(C::kOFull + s));
                     }
                 }
-                if (!shared_stage || s == 1) tc_commit(c.bar(C::kKvEmpty + stage));
-                if (k == steps[s]) {
-                    tc_commit(c.bar(C::kOFull + s));
-                    ++ms.nItems;
-                }
+                __syncwarp();
+                if (k == steps[s]) ++ms.nItems;
             }
             if (k < steps[s]) issue_qk(s_c, w, ring_n, k);
         };
@@ -1150,7 +1210,7 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
     }
     __syncwarp();
     if (!ok) {                      // drain whatever was issued before giving TMEM back
-        tc_commit(c.bar(C::kDrain));
+        if (lead) tc_commit(c.bar(C::kDrain));
         const uint64_t t0 = global_ns();
         while (!mbar_try_wait(c.bar(C::kDrain), 0) && global_ns() - t0 < 100000000ull) {}
     }
@@ -1166,11 +1226,8 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_pool_k, const __grid_co
     using C = Cfg<D>;
     extern __shared__ char smem_raw[];
     Cta c;
-    c.smem = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    c.smem_base = smem_u32(c.smem);
+    c.smem_base = (smem_u32(smem_raw) + 1023) & ~1023u;
     c.bar0 = c.smem_base + C::kOffBar;
-    volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(c.smem + C::kOffBar + 8 * C::kNumBars);
-    c.abort_flag = tmem_slot + 1;
     if (!p.fresh) pdl_launch_dependents();
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -1192,11 +1249,11 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_pool_k, const __grid_co
         }
         mbar_init(c.bar(C::kMlFull), 128);
         mbar_init(c.bar(C::kDrain), 1);
-        *c.abort_flag = 0;
+        st_shared(c.abort_flag(), 0);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 12) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32((const void *)tmem_slot)),
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(c.tmem_slot()),
                      "r"(kTmemCols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -1212,7 +1269,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_pool_k, const __grid_co
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    c.tmem = *tmem_slot;
+    c.tmem = ld_shared(c.tmem_slot());
 
     if (warp < 8) {
         softmax_role<D>(p, c, warp >> 2, tid & 127);
@@ -1229,7 +1286,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_pool_k, const __grid_co
     }
 
     // ---- teardown ------------------------------------------------------------------------------
-    if (*c.abort_flag) {                    // let copies still in flight land before the CTA goes away
+    if (ld_shared(c.abort_flag())) {                    // let copies still in flight land before the CTA goes away
         const uint64_t t0 = global_ns();
         while (global_ns() - t0 < 200000ull) __nanosleep(1000);
     }
@@ -1402,6 +1459,7 @@ cudaError_t kvp_launch_attn_sm100(const kvp_shape &sh, const kvp_attn2_args &a, 
     p.n_q = sh.n_q_heads;
     p.n_kv = sh.n_kv_heads;
     p.group = sh.group;
+    p.group_magic = (uint32_t)((0x100000000ull + sh.group - 1) / sh.group);
     p.pairing = sh.pairing;
     p.scale = sh.scale;
     p.scale_log2 = sh.scale * 1.4426950408889634f;
