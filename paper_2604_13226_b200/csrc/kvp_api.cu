@@ -140,13 +140,13 @@ typedef CUresult (*encode_tiled_fn)(CUtensorMap *, CUtensorMapDataType, cuuint32
                                     const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
                                     CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// One K or V plane set as a 3-D bf16 tensor (head_dim, rows, layer*kv_head); box = 64 columns x 128
-// rows with the 128-byte swizzle the MMA descriptors expect; out-of-range rows read as zero.
-bool make_tensor_map(encode_tiled_fn enc, CUtensorMap *tm, void *base, int head_dim, int64_t rows, int planes)
+// One K or V plane set as a 3-D bf16 tensor (head_dim, rows, layer*kv_head); box = 64 columns x 128 rows
+// (64 for the half K tile of a CTA of a pair) with the 128-byte swizzle the MMA descriptors expect; out-of-range rows read as zero.
+bool make_tensor_map(encode_tiled_fn enc, CUtensorMap *tm, void *base, int head_dim, int64_t rows, int planes, int box_rows)
 {
     const cuuint64_t dims[3] = {(cuuint64_t)head_dim, (cuuint64_t)rows, (cuuint64_t)planes};
     const cuuint64_t strides[2] = {(cuuint64_t)head_dim * 2, (cuuint64_t)rows * head_dim * 2};
-    const cuuint32_t box[3] = {64, KVP_TILE_KEYS, 1};
+    const cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1};
     const cuuint32_t estr[3] = {1, 1, 1};
     return enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -155,11 +155,12 @@ bool make_tensor_map(encode_tiled_fn enc, CUtensorMap *tm, void *base, int head_
 
 // The caller's k_new or v_new, [batch][q_len][Hkv][d] bf16, as a 4-D tensor (d, Hkv, q_len, batch); box = 64
 // columns x 1 head x 128 tokens, the same shared-memory tile as a pool box.  Tokens past q_len read as zero.
-bool make_query_tensor_map(encode_tiled_fn enc, CUtensorMap *tm, const void *base, int head_dim, int n_kv, int q_len, int batch)
+bool make_query_tensor_map(encode_tiled_fn enc, CUtensorMap *tm, const void *base, int head_dim, int n_kv, int q_len, int batch,
+                           int box_rows)
 {
     const cuuint64_t dims[4] = {(cuuint64_t)head_dim, (cuuint64_t)n_kv, (cuuint64_t)q_len, (cuuint64_t)batch};
     const cuuint64_t strides[3] = {(cuuint64_t)head_dim * 2, (cuuint64_t)n_kv * head_dim * 2, (cuuint64_t)q_len * n_kv * head_dim * 2};
-    const cuuint32_t box[4] = {64, 1, KVP_TILE_KEYS, 1};
+    const cuuint32_t box[4] = {64, 1, (cuuint32_t)box_rows, 1};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     return enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(base), dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -248,10 +249,27 @@ cudaError_t stage_upload(kvp_stage &sg, char *dst, uint64_t bytes, cudaStream_t 
 // two-stream key tiles (measured: 7,000 cycles per piece against 3,500-4,000 per tile pair, from the
 // per-CTA durations of a config-3 launch); the unit weights carry it so that CTAs with more pieces get
 // fewer tiles.  Counted in single-stream tiles.
-constexpr int kPieceCost = 4;
+constexpr int kPieceCostOne = 4, kPieceCostPair = 8;
 
 // 0.08 Gflop: 11-17 us against 13-24; 0.12-0.15: 21 against 23; 0.23: 29 against 25; 2.3: 113 against 25.
 constexpr double kTcMinFlops64 = 1.5e8;
+
+// Whether a call runs on CTA pairs (kvp_attn_pair.cu): units of up to 256 rows, of which the one-CTA kernel keeps the
+// calls whose units mostly hold no more than 128.  Per key tile a pair takes about 2 x 1,400 cycles for 256 rows and for
+// 128 rows alike, the one-CTA kernel 3,900 and 1,950.
+bool use_pairs(const kvp_ctx *ctx, const kvp_assembly_host &as, int q_len, const int32_t *q_lens)
+{
+    const kvp_shape &sh = ctx->shape;
+    if (!ctx->have_tma || sh.head_dim != 128 || ctx->split_target_ctas == 1) return false;
+    int64_t wide = 0, narrow = 0;                                 // units, weighted by their request's prefix
+    for (int b = 0; b < as.batch; ++b) {
+        const int64_t rows = (int64_t)sh.group * (q_lens ? q_lens[b] : q_len), rest = rows % (2 * KVP_TILE_ROWS);
+        const int64_t keys = as.items[b].prefix_len + q_len;
+        wide += keys * (rows / (2 * KVP_TILE_ROWS) + (rest > KVP_TILE_ROWS ? 1 : 0));
+        narrow += keys * (rest > 0 && rest <= KVP_TILE_ROWS ? 1 : 0);
+    }
+    return 2 * wide >= narrow;
+}
 
 // q_lens: nullptr, or one query length per request (<= q_len, the stride of the padded tensors); a request's
 // work records and merge items then carry its own length.
@@ -261,6 +279,8 @@ int32_t plan_schedule(kvp_ctx *ctx, const kvp_assembly_host &as, int layer, int 
                       uint32_t opts, kvp_schedule &out)
 {
     const kvp_shape &sh = ctx->shape;
+    out.pair = use_pairs(ctx, as, q_len, q_lens);
+    const int kPieceCost = out.pair ? kPieceCostPair : kPieceCostOne;
     const bool force_partial = (opts & KVP_PARTIAL) != 0, skip_tail = (opts & KVP_SKIP_QUERY_BLOCK) != 0;
     typedef kvp_schedule::unit unit_t;
     typedef kvp_schedule::cut cut_t;
@@ -281,7 +301,7 @@ int32_t plan_schedule(kvp_ctx *ctx, const kvp_assembly_host &as, int layer, int 
                 unit_t u;
                 u.q_len = q_lens ? q_lens[b] : 0;
                 u.b = b; u.hk = hk; u.row_base = row_base;
-                u.mode = (n_rows - row_base <= KVP_TILE_ROWS) ? 1 : 0;
+                u.mode = (!out.pair && n_rows - row_base <= KVP_TILE_ROWS) ? 1 : 0;
                 const int last = std::min(n_rows - 1, row_base + (u.mode ? 1 : 2) * KVP_TILE_ROWS - 1);
                 const int n_tail = (q_pos0 + last / sh.group) / KVP_TILE_KEYS + 1;
                 u.n_all = n_tail + n_prefix;
@@ -297,6 +317,7 @@ int32_t plan_schedule(kvp_ctx *ctx, const kvp_assembly_host &as, int layer, int 
         }
     int G = std::min(ctx->sm_count, kMaxCtas);
     if (ctx->split_target_ctas > 0) G = std::min(ctx->split_target_ctas, kMaxCtas);
+    if (out.pair) G /= 2;                                         // entries of cta_begin are pairs
     const bool no_split = ctx->force_splits == 1;               // cuts only between units
 
     // Cut positions (unit, tile), non-decreasing.  A run of units is dealt out to g CTAs one after the other, each
@@ -689,15 +710,19 @@ int32_t kvp_create(const kvp_config *cfg, kvp_ctx **out)
             encode_tiled_fn enc = (encode_tiled_fn)fn;
             ctx->encode_tiled = fn;
             const int planes = sh.n_layers * sh.n_kv_heads;
-            bool ok = make_tensor_map(enc, &ctx->tm_pool_k, ctx->pool_k, sh.head_dim, sh.pool_rows, planes) &&
-                      make_tensor_map(enc, &ctx->tm_pool_v, ctx->pool_v, sh.head_dim, sh.pool_rows, planes);
-            ctx->tm_ws_k.resize(cfg->max_assemblies);
-            ctx->tm_ws_v.resize(cfg->max_assemblies);
-            for (int a = 0; ok && a < cfg->max_assemblies; ++a)
-                ok = make_tensor_map(enc, &ctx->tm_ws_k[a], ctx->slot_k[a], sh.head_dim, sh.ws_rows, planes) &&
-                     make_tensor_map(enc, &ctx->tm_ws_v[a], ctx->slot_v[a], sh.head_dim, sh.ws_rows, planes);
+            const int d = sh.head_dim, na = cfg->max_assemblies;
+            bool ok = make_tensor_map(enc, &ctx->tm_pool_k, ctx->pool_k, d, sh.pool_rows, planes, KVP_TILE_KEYS) &&
+                      make_tensor_map(enc, &ctx->tm_pool_v, ctx->pool_v, d, sh.pool_rows, planes, KVP_TILE_KEYS) &&
+                      make_tensor_map(enc, &ctx->tm_pool_k_half, ctx->pool_k, d, sh.pool_rows, planes, KVP_TILE_KEYS / 2);
+            ctx->tm_ws_k.resize(na);
+            ctx->tm_ws_v.resize(na);
+            ctx->tm_ws_k_half.resize(na);
+            for (int a = 0; ok && a < na; ++a)
+                ok = make_tensor_map(enc, &ctx->tm_ws_k[a], ctx->slot_k[a], d, sh.ws_rows, planes, KVP_TILE_KEYS) &&
+                     make_tensor_map(enc, &ctx->tm_ws_v[a], ctx->slot_v[a], d, sh.ws_rows, planes, KVP_TILE_KEYS) &&
+                     make_tensor_map(enc, &ctx->tm_ws_k_half[a], ctx->slot_k[a], d, sh.ws_rows, planes, KVP_TILE_KEYS / 2);
             if (!ok) return bail(KVP_ERR_CUDA, "cuTensorMapEncodeTiled failed");
-            if (kvp_attn_sm100_prepare(sh.head_dim) != cudaSuccess)
+            if (kvp_attn_sm100_prepare(sh.head_dim) != cudaSuccess || (sh.head_dim == 128 && kvp_attn_pair_prepare() != cudaSuccess))
                 return bail(KVP_ERR_CUDA, "tcgen05 kernel attribute setup failed");
             ctx->have_tma = true;
         }
@@ -1214,10 +1239,13 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
     kvp_attn2_args a;
     a.tail_direct = 0;
     a.precise = (flags & KVP_PRECISE_QK) ? 1 : 0;
+    const bool pairs = fast && use_pairs(ctx, as, q_len, q_lens);
     if (fast && ctx->fused_append && !rope_query && q_pos0 == 0 && !skip_block &&
         (((uintptr_t)k_new | (uintptr_t)v_new) & 15) == 0 &&
-        make_query_tensor_map((encode_tiled_fn)ctx->encode_tiled, &a.tm_knew, k_new, sh.head_dim, sh.n_kv_heads, q_len, as.batch) &&
-        make_query_tensor_map((encode_tiled_fn)ctx->encode_tiled, &a.tm_vnew, v_new, sh.head_dim, sh.n_kv_heads, q_len, as.batch))
+        make_query_tensor_map((encode_tiled_fn)ctx->encode_tiled, &a.tm_knew, k_new, sh.head_dim, sh.n_kv_heads, q_len, as.batch,
+                              pairs ? KVP_TILE_KEYS / 2 : KVP_TILE_KEYS) &&
+        make_query_tensor_map((encode_tiled_fn)ctx->encode_tiled, &a.tm_vnew, v_new, sh.head_dim, sh.n_kv_heads, q_len, as.batch,
+                              KVP_TILE_KEYS))
         a.tail_direct = 1;
     if (q_lens && !a.tail_direct)
         return fail(ctx, KVP_ERR_UNSUPPORTED, "query_prefill_ragged: needs the tcgen05 kernel with its own append (bf16, head_dim 128, 16-byte aligned k_new / v_new)");
@@ -1283,7 +1311,10 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
         a.status = ctx->status_dev;
         if (ss.ctas > 0) {                                         // (a rank may hold no key of any request)
             KVP_CUDA(ctx, time_edge(ctx, 0, 0, st));
-            KVP_CUDA(ctx, kvp_launch_attn_sm100(sh, a, ctx->tm_pool_k, ctx->tm_pool_v, ctx->tm_ws_k[slot], ctx->tm_ws_v[slot], st));
+            if (pairs)
+                KVP_CUDA(ctx, kvp_launch_attn_pair(sh, a, ctx->tm_pool_k_half, ctx->tm_pool_v, ctx->tm_ws_k_half[slot], ctx->tm_ws_v[slot], st));
+            else
+                KVP_CUDA(ctx, kvp_launch_attn_sm100(sh, a, ctx->tm_pool_k, ctx->tm_pool_v, ctx->tm_ws_k[slot], ctx->tm_ws_v[slot], st));
             KVP_CUDA(ctx, time_edge(ctx, 0, 1, st));
             ++launches;
         }
@@ -1296,7 +1327,7 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
                                                 (int64_t)as.batch * sh.n_kv_heads * n_rt, st));
             ++launches;
         }
-        ctas = ss.ctas;
+        ctas = pairs ? 2 * ss.ctas : ss.ctas;
         splits = ss.slots;
         ctx->last_kind = 1;
     }

@@ -1,0 +1,653 @@
+// bf16 composed-cache attention for sm_100a, head dimension 128, more than 128 packed query rows per (request, kv head):
+// a pair of CTAs works on one unit of 256 rows, CTA r on rows [128 r, 128 r + 128), with tcgen05.mma over both
+// (cta_group::2, M = 256).  Each CTA holds its own Q, S, P and O; of every K tile it loads half the keys, of every V tile
+// half the columns, and the tensor cores of both read both halves.
+//
+// Why a pair: with both 128-row tiles of a unit in one CTA, TMEM (512 columns) is full with S and O of two streams, P lies
+// over S, and per stream the steps form one chain - Q K^T, softmax, P V, and the next Q K^T only behind that P V - of
+// about 3,900 cycles, in which tensor cores and special-function units are busy 2,048 each.  One tile per CTA leaves room
+// for three S buffers beside O: Q K^T runs up to three tiles ahead, and the two softmax warpgroups take alternate tiles,
+// so that the special-function unit's own 1,024 cycles per tile are what is left in the chain.  K and V traffic per SM
+// stays what it was, because the pair shares every tile.
+//
+//   warps 0-3 / 4-7   softmax of the even / odd tiles of a piece: one thread per query row, exponentials against a
+//                     reference maximum m, P as bf16 over S.  O is shared by both warpgroups, so tile k's P has to be
+//                     relative to the reference that is in force after tile k - 1: the two warps of a row quadrant hand it
+//                     over (mref, an mbarrier per warp).  It rarely changes (only by more than 2^8); then this tile's P
+//                     or, once P V of tile k - 1 has landed, O is rescaled.
+//   warps 8-11        Q producer: counter-rotates this CTA's rows once per document (as in the one-CTA kernel), and appends
+//                     the query block's K/V rows
+//   warps 12-14       CTA 0 of the pair: MMA issuers for both, step by step in turn.  Warp 12 owns TMEM in each.
+//   warp 15           TMA producer of this CTA's halves; its bytes are counted on CTA 0's barriers
+//
+// Barriers that CTA 0's MMA warps wait for live in CTA 0 and are arrived at from both CTAs; those they signal
+// (tcgen05.commit, multicast) exist in both.  Every wait is bounded: when it runs out the status word gets a code, both
+// CTAs' abort flags are set and every role leaves.
+#include "kvp_attn_common.cuh"
+
+namespace {
+
+constexpr int kThreads = 512;
+constexpr int kStageBytes = 16384;                       // half a K or V tile
+// Ring and Q buffers share 208 KB: two buffers of 32 KB (value) or 64 KB (value and remainder) and 9 or 5 stages.
+constexpr int kMaxStages = 9;
+constexpr int kOffBar = 208 * 1024;
+constexpr int kOffMref = kOffBar + 512;                   // float[128]
+constexpr int kOffMl = kOffMref + 512;                    // float2[2][128]: (m, l) of both warpgroups at the end of a piece
+constexpr int kSmemBytes = kOffMl + 2048 + 1024;          // + alignment slack
+constexpr uint32_t kColO = 384;                           // S buffer b: columns [128 b, 128 b + 128)
+constexpr uint16_t kBoth = 3;
+
+enum BarIdx { kKvFull = 0, kKvEmpty = kMaxStages, kQFull = 2 * kMaxStages, kQFree = kQFull + 2, kSFull = kQFree + 2, kPFull = kSFull + 3,
+              kPvDone = kPFull + 3, kOFull = kPvDone + 2, kOFree, kMref, kEnd = kMref + 8, kTurn = kEnd + 8,       // Mref, End: [4 * warpgroup + quadrant]
+              kDrain = kTurn + 3, kNumBars = kDrain + 3 };
+static_assert(8 * kNumBars <= 504, "barrier block");
+
+struct Cta {
+    uint32_t smem_base, bar0, lead0, tmem;                // lead0: CTA 0's barriers, as an address of the cluster's shared memory
+    int rank, item_begin, item_end;
+    __device__ __forceinline__ uint32_t bar(int i) const { return bar0 + 8u * i; }
+    __device__ __forceinline__ uint32_t lead(int i) const { return lead0 + 8u * i; }
+    __device__ __forceinline__ uint32_t tmem_slot() const { return bar0 + 504; }
+    __device__ __forceinline__ uint32_t abort_flag() const { return bar0 + 508; }
+    __device__ __forceinline__ char *smem() const { return reinterpret_cast<char *>(__cvta_shared_to_generic(smem_base)); }
+};
+
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t a, uint32_t rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Shared memory written before it (the rotated Q) is released to the cluster.
+__device__ __forceinline__ void remote_arrive_release(uint32_t cluster_bar)
+{
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
+}
+// For what lies in TMEM, which tcgen05.fence::before_thread_sync orders: a release to the cluster waits for everything the
+// SM has in flight, 1,000 cycles and more per tile (it took half of the softmax warps' time).
+__device__ __forceinline__ void remote_arrive(uint32_t cluster_bar)
+{
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
+}
+
+// the waits of this kernel; one that runs out also raises the other CTA's abort flag
+__device__ __noinline__ bool wait_slow(uint32_t bar, uint32_t parity, uint32_t abort_flag, int rank, int32_t *status, int code)
+{
+    if (mbar_wait_slow(bar, parity, abort_flag, status, code)) return true;
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr(abort_flag, (uint32_t)(rank ^ 1))), "r"(1u) : "memory");
+    return false;
+}
+__device__ __forceinline__ bool wait(const Params &p, const Cta &c, int i, uint32_t parity, int code)
+{
+    if (mbar_try_wait(c.bar(i), parity)) return true;
+    return wait_slow(c.bar(i), parity, c.abort_flag(), c.rank, p.status, code);
+}
+
+__device__ __forceinline__ void load_3d(uint32_t dst, const CUtensorMap *tm, int x, int y, int z, uint32_t cluster_bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%2, %3, %4}], [%5];"
+        ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(z), "r"(cluster_bar)
+        : "memory");
+}
+__device__ __forceinline__ void load_4d(uint32_t dst, const CUtensorMap *tm, int x, int y, int z, int w, uint32_t cluster_bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%2, %3, %4, %5}], [%6];"
+        ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(z), "r"(w), "r"(cluster_bar)
+        : "memory");
+}
+
+// arrives at the barrier of this place in both CTAs once the MMAs this thread has issued so far have run
+__device__ __forceinline__ void commit_both(uint32_t bar)
+{
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar), "h"(kBoth)
+                 : "memory");
+}
+template <int ACC>
+__device__ __forceinline__ void mma_ss(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d), "l"(a), "l"(b), "r"(idesc), "n"(ACC)
+        : "memory");
+}
+__device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t acc)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        ::"r"(d), "r"(a), "l"(b), "r"(idesc), "r"(acc)
+        : "memory");
+}
+// bf16 x bf16 -> fp32, M = 256 over the pair, N = n, A K-major, B K-major or MN-major
+__device__ __forceinline__ uint32_t instr_desc(uint32_t n, uint32_t b_mn_major)
+{
+    return (1u << 4) | (1u << 7) | (1u << 10) | (b_mn_major << 16) | ((n >> 3) << 17) | ((256u >> 4) << 24);
+}
+// N of a tile's Q K^T: its keys rounded up to what M = 256 takes; CTA r holds keys [r N / 2, (r + 1) N / 2)
+__device__ __forceinline__ int qk_n(int n_keys) { return max(32, (n_keys + 31) & ~31); }
+
+// ---- softmax / epilogue of warpgroup G (tiles G, G + 2, ... of a piece) ------------------------------------
+// Scales P of a tile (n_chunks x 16 columns of packed pairs) by alpha.
+__device__ __forceinline__ void scale_p(uint32_t s_addr, float alpha, int n_chunks)
+{
+    tc_wait_st();                                         // the P chunks this thread stored are read back
+#pragma unroll 1
+    for (int ch = 0; ch < n_chunks; ++ch) {
+        uint32_t v[16];
+        tmem_ld16(s_addr + ch * 16, v);
+        tc_wait_ld();
+        landed16(v);
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+            v[i] = pack_bf16(__uint_as_float(v[i] << 16) * alpha, __uint_as_float(v[i] & 0xffff0000u) * alpha);
+        tmem_st16(s_addr + ch * 16, v);
+    }
+    tc_wait_st();
+}
+__device__ __forceinline__ void scale_o(uint32_t o_addr, float alpha)
+{
+#pragma unroll 1
+    for (int ch = 0; ch < 4; ++ch) {
+        uint32_t v[32];
+        tmem_ld32(o_addr + ch * 32, v);
+        tc_wait_ld();
+        landed32(v);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) * alpha);
+        tmem_st32(o_addr + ch * 32, v);
+    }
+    tc_wait_st();
+}
+
+__device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, const int G, const int t)
+{
+    const int quad = t >> 5;
+    const bool lead_lane = (t & 31) == 0;
+    const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
+    const uint32_t o_addr = c.tmem + lane_base + kColO;
+    const float c2 = p.scale_log2;
+    const uint32_t mref = c.smem_base + kOffMref + 4 * t;
+    const int own = 4 * G + quad, other = 4 * (G ^ 1) + quad;         // hand-over barriers of this row quadrant's two warps
+    uint32_t T0 = 0;                                      // tiles of the pieces before this one
+    uint32_t seen = 0;                                    // the other warp's tiles up to the last one looked at
+    uint32_t phO = 0;                                     // pieces
+    bool ok = true;
+
+    for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
+        int n, lo, n_tail, n_total, limit;
+        const kvp_tile *tiles;
+        {
+            const Work w = load_work(p, wi);
+            n = w.n;
+            lo = w.lo;
+            n_tail = w.n_tail;
+            tiles = p.plan.tiles + w.tile_begin - n_tail;
+            n_total = p.q_pos0 + w.q_len;
+            const int r = w.row_base + c.rank * KVP_TILE_ROWS + t;
+            limit = p.q_pos0 + (r < p.group * w.q_len ? row_token(p, r) : w.q_len - 1) + 1;     // causal keys this row sees
+        }
+        float m = -1e30f, l = 0.f;
+        auto keys_of = [&](int j) {                       // keys of tile j
+            return j < n_tail ? min(KVP_TILE_KEYS, n_total - j * KVP_TILE_KEYS) : (int)tiles[j].n_keys;
+        };
+        int nk_next = G < n ? keys_of(lo + G) : 0;
+#pragma unroll 1
+        for (int k = G; k < n; k += 2) {
+            const int j = lo + k, n_keys = nk_next;
+            if (k + 2 < n) nk_next = keys_of(j + 2);
+            const uint32_t T = T0 + (uint32_t)k, use = T / 3, buf = T - 3 * use;
+            const uint32_t s_addr = c.tmem + lane_base + buf * 128;
+            ok = wait(p, c, kSFull + buf, use & 1, 30 + G);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            tc_fence_after();
+
+            const bool full = n_keys == KVP_TILE_KEYS && j >= n_tail;
+            const int lim = j >= n_tail ? n_keys : min(n_keys, limit - j * KVP_TILE_KEYS);       // visible keys: [0, lim)
+            // a short tile (the end of a document, staged adapter rows) needs P only for the columns P V will read
+            const int n_ch = full ? 4 : max(1, (n_keys + 31) >> 5);
+            // One pass over S, 32 columns at a time, against the reference max this warpgroup knows; a chunk's own max is
+            // reduced alongside and checked last.  Only if it exceeds the reference by more than 2^8 (first tile, or a
+            // rare jump) does the reference move and the P written so far with it.
+#pragma unroll 1
+            for (int ch = 0; ch < n_ch; ++ch) {
+                uint32_t v[32], pk[16];
+                auto load = [&] {
+                    tmem_ld32(s_addr + ch * 32, v);
+                    tc_wait_ld();
+                    landed32(v);
+                    if (!full) chunk_mask(v, lim - ch * 32);
+                };
+                load();
+                const float cm = chunk_max(v, -INFINITY);
+                float ls = chunk_exp<false>(v, c2, m * c2, pk);
+                const bool need = (cm - m) * c2 > 8.0f;
+                if (__any_sync(0xffffffffu, need)) {
+                    const float m_new = need ? cm : m;
+                    const float alpha = need ? ex2((m - m_new) * c2) : 1.f;
+                    scale_p(s_addr, alpha, ch);
+                    l *= alpha;
+                    m = m_new;
+                    load();                               // this chunk's scores again (P so far lies below them)
+                    ls = chunk_exp<false>(v, c2, m * c2, pk);
+                }
+                tmem_st16(s_addr + ch * 16, pk);
+                l += ls;
+            }
+            // the reference in force after tile k - 1
+            if (k > 0) {
+                ok = wait(p, c, kMref + other, seen & 1, 36);
+                ++seen;
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                const float mp = __uint_as_float(ld_shared(mref));
+                if (__any_sync(0xffffffffu, mp != m)) {
+                    const bool raise = (m - mp) * c2 > 8.0f;              // O follows this tile; else this tile follows O
+                    const float ap = raise ? 1.f : ex2((m - mp) * c2), ao = raise ? ex2((mp - m) * c2) : 1.f;
+                    scale_p(s_addr, ap, n_ch);
+                    l *= ap;
+                    if (!raise) m = mp;
+                    if (__any_sync(0xffffffffu, raise)) {
+                        // O is quiet then: P V of tile k waits for this warp (tiles take two barriers in turn: S of this
+                        // tile shows that P V of tile k - 3 is done, so the phase meant here is the next or the last one)
+                        ok = wait(p, c, kPvDone + ((T - 1) & 1), ((T - 1) >> 1) & 1, 37);
+                        ok = __all_sync(0xffffffffu, ok);
+                        if (!ok) break;
+                        tc_fence_after();
+                        scale_o(o_addr, ao);
+                    }
+                }
+            }
+            st_shared(mref, __float_as_uint(m));
+            tc_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lead_lane) {
+                mbar_arrive(c.bar(kMref + own));
+                remote_arrive(c.lead(kPFull + buf));
+            }
+        }
+        T0 += (uint32_t)n;
+        if (!ok) break;
+
+        // ---- end of the piece: O is complete once its last P V has landed ----------
+        ok = wait(p, c, kOFull, phO & 1, 32);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        tc_fence_after();
+        float2 *ml = reinterpret_cast<float2 *>(c.smem() + kOffMl) + t;
+        ml[128 * G] = make_float2(m, l);
+        __syncwarp();
+        if (lead_lane) mbar_arrive(c.bar(kEnd + own));
+        seen += G == 0 ? n / 2 - (n - 1) / 2 : (n + 1) / 2 - n / 2;       // a last tile of the other warp that was not waited for
+        ok = wait(p, c, kEnd + other, phO & 1, 34);
+        ++phO;
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        const float2 o = ml[128 * (G ^ 1)];
+        const float M = ((n - 1) & 1) == G ? m : o.x;     // O is relative to the last tile's reference
+        l = l * ex2((m - M) * c2) + o.y * ex2((o.x - M) * c2);
+
+        const Work w = load_work(p, wi);
+        const int r = w.row_base + c.rank * KVP_TILE_ROWS + t;
+        const bool valid = r < p.group * w.q_len;
+        const int qi = valid ? row_token(p, r) : w.q_len - 1;
+        const int h = w.hk * p.group + (valid ? r - qi * p.group : 0);
+        const int slot = c.rank == 0 ? w.slot0 : w.slot1;
+        const bool direct = slot < 0;
+        const float w0 = direct ? 1.f / l : 1.f;
+        // un-normalised (partial slot) or normalised (output rows) O, this warpgroup's half of the columns
+        uint4 *orow_bf = (direct && valid) ? reinterpret_cast<uint4 *>(p.out + (((long long)w.b * p.q_len + qi) * p.n_q + h) * 128 + G * 64) : nullptr;
+        // partial slot layout: [32 float4 columns][128 rows], so that a warp's store covers 512 contiguous bytes
+        uint4 *orow_f = direct || !valid ? nullptr : reinterpret_cast<uint4 *>(p.partial_o) + ((long long)slot * 32 + G * 16) * KVP_TILE_ROWS + t;
+#pragma unroll 1
+        for (int ch = 0; ch < 2; ++ch) {
+            uint32_t a[32];
+            tmem_ld32(o_addr + G * 64 + ch * 32, a);
+            tc_wait_ld();
+            landed32(a);
+#pragma unroll
+            for (int i = 0; i < 32; ++i) a[i] = __float_as_uint(__uint_as_float(a[i]) * w0);
+            if (orow_bf != nullptr) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    uint4 u;
+                    u.x = pack_bf16(__uint_as_float(a[8 * i + 0]), __uint_as_float(a[8 * i + 1]));
+                    u.y = pack_bf16(__uint_as_float(a[8 * i + 2]), __uint_as_float(a[8 * i + 3]));
+                    u.z = pack_bf16(__uint_as_float(a[8 * i + 4]), __uint_as_float(a[8 * i + 5]));
+                    u.w = pack_bf16(__uint_as_float(a[8 * i + 6]), __uint_as_float(a[8 * i + 7]));
+                    orow_bf[ch * 4 + i] = u;
+                }
+            } else if (orow_f != nullptr) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    orow_f[(ch * 8 + i) * KVP_TILE_ROWS] = make_uint4(a[4 * i], a[4 * i + 1], a[4 * i + 2], a[4 * i + 3]);
+            }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lead_lane) remote_arrive(c.lead(kOFree));
+        if (G == 0) {
+            if (direct) {
+                if (valid && p.lse != nullptr) p.lse[((long long)w.b * p.n_q + h) * p.q_len + qi] = M * p.scale + logf(l);
+            } else if (valid) {
+                p.partial_ml[(long long)slot * KVP_TILE_ROWS + t] = make_float2(M, l);
+            }
+        }
+    }
+}
+
+// ---- Q producer: this CTA's 128 rows, once per document; append ------------------------------------------------
+__device__ __forceinline__ void producer_role(const Params &p, const Cta &c, const int t)
+{
+    const uint32_t stride = p.precise ? 2 * kQBufBytes : kQBufBytes;
+    uint32_t ep = 0;
+    bool ok = true;
+    pdl_wait();
+    for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
+        const Work w = load_work(p, wi);
+        const int n_rows = p.group * w.q_len;
+        int prev = 0;
+        for (int k = 0; k < w.n && ok; ++k) {
+            const int rope = get_tile(p, w, w.lo + k).rope;
+            if (k > 0 && rope == prev) continue;
+            prev = rope;
+            const uint32_t buf = ep & 1;
+            if (ep >= 2) {
+                ok = wait(p, c, kQFree + buf, ((ep >> 1) - 1) & 1, 40);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+            }
+            char *qb = c.smem() + buf * stride;
+            produce_q_tile<128>(p, qb, p.precise ? qb + kQBufBytes : nullptr, t, p.q + (long long)w.b * p.q_len * p.n_q * 128, w.hk,
+                                w.row_base + c.rank * KVP_TILE_ROWS, n_rows, rope);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if ((t & 31) == 0) remote_arrive_release(c.lead(kQFull + buf));
+            ++ep;
+            // the append (as in the one-CTA kernel): the tokens whose first packed row lies in this CTA's rows, behind the
+            // piece's first Q tile
+            if (k == 0 && w.lo == 0 && p.tail_direct) append_rows<16, 128>(p, w, w.row_base + c.rank * KVP_TILE_ROWS, KVP_TILE_ROWS, t);
+        }
+    }
+}
+
+// Loads of a piece with n tiles in the order the MMA warps take them: Q K^T runs three tiles ahead of P V, so
+// K0 K1 K2 V0 K3 V1 K4 ... V(n-1).  Load q is tile r's K (kv = 0) or V (kv = 1).
+__device__ __forceinline__ void load_at(int n, int q, int &r, int &kv)
+{
+    if (q < min(n, 3)) { r = q; kv = 0; }
+    else if (q >= n + max(n - 3, 0)) { r = q - n; kv = 1; }
+    else { kv = (q - 3) & 1 ? 0 : 1; r = (q - 3) / 2 + (kv ? 0 : 3); }
+}
+
+// ---- TMA producer (whole warp): this CTA's half of every tile ---------------------------------------------------
+__device__ __forceinline__ void tma_role(const Params &p, const Cta &c, const int lane, const CUtensorMap *k_pool,
+                                         const CUtensorMap *v_pool, const CUtensorMap *k_ws, const CUtensorMap *v_ws,
+                                         const CUtensorMap *k_new, const CUtensorMap *v_new)
+{
+    const uint32_t n_stages = p.precise ? 5 : 9;
+    const uint32_t ring = c.smem_base + (p.precise ? 4 : 2) * kQBufBytes;
+    uint32_t stage = 0, use = 0;
+    bool ok = true;
+    for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
+        const Work w = load_work(p, wi);
+        const int n_loads = 2 * w.n;
+        for (int q0 = 0; q0 < n_loads && ok; q0 += 32) {
+            // lane i looks up the tile of load q0 + i and issues it when its turn comes
+            const int q = q0 + lane;
+            int row0 = 0, src = 0, kv = 0, n_keys = 0;
+            if (q < n_loads) {
+                int r;
+                load_at(w.n, q, r, kv);
+                const Tile tl = get_tile(p, w, w.lo + r);
+                row0 = tl.row0;
+                src = tl.src;
+                n_keys = tl.n_keys;
+            }
+            const CUtensorMap *tm = src == 2 ? (kv ? v_new : k_new) : src == 0 ? (kv ? v_pool : k_pool) : (kv ? v_ws : k_ws);
+            const int x = kv ? 64 * c.rank : 0, y = kv ? row0 : row0 + c.rank * (qk_n(n_keys) / 2);
+            const int cnt = min(32, n_loads - q0);
+            const bool ahead = p.l2_prefetch && lane < cnt && src != 2;
+#pragma unroll 1
+            for (int i = 0; i < cnt && ok; ++i) {
+                if (ahead && lane == i + 4) {             // tiles that come from DRAM: L2 is asked for the one four loads ahead
+                    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(tm), "r"(x), "r"(y), "r"(w.plane) : "memory");
+                    if (!kv)
+                        asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(tm), "r"(64), "r"(y), "r"(w.plane) : "memory");
+                }
+                if (lane == i) {
+                    if (use > 0) ok = wait(p, c, kKvEmpty + stage, (use - 1) & 1, 10);
+                    if (ok) {
+                        const uint32_t dst = ring + stage * kStageBytes, full = c.lead(kKvFull + stage);
+                        if (c.rank == 0) mbar_expect_tx(c.bar(kKvFull + stage), 2 * kStageBytes);
+                        if (src != 0) pdl_wait();         // staged or appended rows: a kernel in front may have written them
+                        if (src == 2) {
+                            load_4d(dst, tm, x, w.hk, y, w.b, full);
+                            if (!kv) load_4d(dst + kStageBytes / 2, tm, 64, w.hk, y, w.b, full);
+                        } else {
+                            load_3d(dst, tm, x, y, w.plane, full);
+                            if (!kv) load_3d(dst + kStageBytes / 2, tm, 64, y, w.plane, full);
+                        }
+                    }
+                }
+                ok = __all_sync(0xffffffffu, ok);
+                if (++stage == n_stages) { stage = 0; ++use; }
+            }
+        }
+    }
+}
+
+// ---- MMA issuers (one thread of each of three warps of CTA 0) --------------------------------------------------------
+// Step k of a piece is O += P V of tile k - 3 and S = Q K^T of tile k, which takes over that tile's S buffer: warp I takes
+// the steps of S buffer I, each in its turn.  The MMAs of a step wait in a queue that the sub-partition's special-function
+// instructions go through too: with one issuing warp its two softmax warps took 3,200 cycles per tile against 2,400 of the
+// others; three warps on three sub-partitions share that out.  What a step waits for is waited for before its turn.
+__device__ __forceinline__ void mma_role(const Params &p, const Cta &c, const uint32_t I)
+{
+    const uint32_t q_stride = (p.precise ? 2 * kQBufBytes : kQBufBytes) >> 4;
+    const uint32_t ring = c.smem_base + (p.precise ? 4 : 2) * kQBufBytes;
+    const uint32_t idesc_pv = instr_desc(128, 1);
+    const uint32_t v_desc = desc_lo(ring, kHalfBytes), k_desc = desc_lo(ring, 16), q_desc = desc_lo(c.smem_base, 16);
+    const uint32_t sp = c.tmem + I * 128, oa = c.tmem + kColO;
+    uint32_t g0 = 0;                                      // steps of the pieces before this one, mod 3
+    uint32_t T0 = 0, R0 = 0;                              // their tiles and loads
+    uint32_t parP = 0;
+    int turn = I == 0 ? -1 : 0;                           // phase of the turn barrier (warp 0 begins without one)
+    int ep = -1, ep_ready = -1, pieces = 0;               // Q epoch of the last tile looked at; last one waited for
+    bool ok = true;
+    auto stage_of = [&](uint32_t load, uint32_t &par) {
+        const uint32_t use = p.precise ? load / 5 : load / 9;
+        par = use & 1;
+        return load - use * (p.precise ? 5 : 9);
+    };
+
+    for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
+        const Work w = load_work(p, wi);
+        const int n = w.n;
+        int nk3 = 0, last_rope = -1;                      // key count of tile k - 3; document of the last tile looked at
+        int seen = 0;                                     // tiles looked at
+#pragma unroll 1
+        for (int k = (int)((I + 3 - g0) % 3); k < n + 3; k += 3) {
+            // the Q epoch of tile k: a new one at each change of document
+            int nk = 0;
+            bool lastq = true;
+            if (k < n) {
+                for (; seen <= k; ++seen) {
+                    const Tile t = get_tile(p, w, w.lo + seen);
+                    if (t.rope != last_rope) ++ep;
+                    last_rope = t.rope;
+                    nk = t.n_keys;
+                }
+                lastq = k + 1 >= n || get_tile(p, w, w.lo + k + 1).rope != last_rope;
+            }
+            const uint32_t qbuf = ep & 1;
+            uint32_t pv_par = 0, pk_par = 0, sv = 0, sk = 0;
+            if (k >= 3) {
+                sv = stage_of(R0 + (uint32_t)(k - 3 + min(n, k)), pv_par);
+                ok = wait(p, c, kKvFull + sv, pv_par, 23);
+                if (ok && k == 3 && pieces > 0) ok = wait(p, c, kOFree, (pieces - 1) & 1, 26);
+                ok = ok && wait(p, c, kPFull + I, parP, 24);
+                parP ^= 1;
+            }
+            if (k < n) {
+                sk = stage_of(R0 + (uint32_t)(k + max(0, k - 2)), pk_par);
+                if (!p.precise) ok = ok && wait(p, c, kKvFull + sk, pk_par, 22);      // (with 5 stages the phase is known in turn only)
+            }
+            // ---- this warp's turn -----------------------------------------------------------------
+            if (turn >= 0) ok = ok && wait(p, c, kTurn + I, (uint32_t)turn & 1, 25);
+            if (p.precise && k < n) ok = ok && wait(p, c, kKvFull + sk, pk_par, 22);
+            if (k < n && ep != ep_ready) {                 // (in turn only: documents may be of one tile)
+                ok = ok && wait(p, c, kQFull + qbuf, ((uint32_t)ep >> 1) & 1, 20);
+                ep_ready = ep;
+            }
+            if (!ok) break;
+            tc_fence_after();
+            if (k >= 3) {                                  // O += P V
+                const uint32_t v_lo = v_desc + sv * (kStageBytes >> 4);
+                if (nk3 == KVP_TILE_KEYS && k > 3) {
+#pragma unroll
+                    for (int kk = 0; kk < 8; ++kk)               // 16 keys per step: P advances 8 columns, V 2048 bytes
+                        mma_ts(oa, sp + kk * 8, desc64(v_lo + kk * 128, kDescHi), idesc_pv, 1);
+                } else {
+                    const int ksteps = max(1, (nk3 + 15) >> 4);
+                    for (int kk = 0; kk < ksteps; ++kk)
+                        mma_ts(oa, sp + kk * 8, desc64(v_lo + kk * 128, kDescHi), idesc_pv, (k > 3 || kk > 0));
+                }
+                commit_both(c.bar(kKvEmpty + sv));
+                commit_both(c.bar(kPvDone + ((T0 + (uint32_t)k - 3) & 1)));
+                if (k == n + 2) commit_both(c.bar(kOFull));
+            }
+            if (k < n) {                                   // S = Q K^T
+                const uint32_t idesc = instr_desc((uint32_t)qk_n(nk), 0);
+                const uint32_t q_lo = q_desc + qbuf * q_stride, k_lo = k_desc + sk * (kStageBytes >> 4);
+                // 16 columns per step: 32 bytes; the second 64 columns lie 16 KB (Q) and 8 KB (K) on
+                mma_ss<0>(sp, desc64(q_lo, kDescHi), desc64(k_lo, kDescHi), idesc);
+#pragma unroll
+                for (int kk = 1; kk < 8; ++kk)
+                    mma_ss<1>(sp, desc64(q_lo + (kk >> 2) * (kHalfBytes >> 4) + (kk & 3) * 2, kDescHi),
+                              desc64(k_lo + (kk >> 2) * (kStageBytes >> 5) + (kk & 3) * 2, kDescHi), idesc);
+                if (p.precise && last_rope != 0) {               // + (rounding remainder of the rotated Q) K^T
+#pragma unroll
+                    for (int kk = 0; kk < 8; ++kk)
+                        mma_ss<1>(sp, desc64(q_lo + (kQBufBytes >> 4) + (kk >> 2) * (kHalfBytes >> 4) + (kk & 3) * 2, kDescHi),
+                                  desc64(k_lo + (kk >> 2) * (kStageBytes >> 5) + (kk & 3) * 2, kDescHi), idesc);
+                }
+            }
+            tc_fence_before();
+            mbar_arrive(c.bar(kTurn + (I == 2 ? 0 : I + 1)));
+            ++turn;
+            if (k < n) {
+                commit_both(c.bar(kSFull + I));
+                commit_both(c.bar(kKvEmpty + sk));
+                if (lastq) commit_both(c.bar(kQFree + qbuf));
+            }
+            nk3 = nk;
+        }
+        for (; seen < n; ++seen) {                         // tiles behind this warp's last step
+            const int r = get_tile(p, w, w.lo + seen).rope;
+            if (r != last_rope) ++ep;
+            last_rope = r;
+        }
+        g0 = (g0 + (uint32_t)n) % 3;
+        T0 += (uint32_t)n;
+        R0 += 2u * (uint32_t)n;
+        ++pieces;
+    }
+    if (!ok) {                      // drain whatever was issued before giving TMEM back
+        asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(c.bar(kDrain + I)) : "memory");
+        const uint64_t t0 = global_ns();
+        while (!mbar_try_wait(c.bar(kDrain + I), 0) && global_ns() - t0 < 100000000ull) {}
+    }
+}
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+attn_pair_kernel(const __grid_constant__ CUtensorMap k_pool, const __grid_constant__ CUtensorMap v_pool,
+                 const __grid_constant__ CUtensorMap k_ws, const __grid_constant__ CUtensorMap v_ws,
+                 const __grid_constant__ CUtensorMap k_new, const __grid_constant__ CUtensorMap v_new, const Params p)
+{
+    extern __shared__ char smem_raw[];
+    Cta c;
+    c.smem_base = (smem_u32(smem_raw) + 1023) & ~1023u;
+    c.bar0 = c.smem_base + kOffBar;
+    c.lead0 = cluster_addr(c.bar0, 0);
+    c.rank = (int)(blockIdx.x & 1);
+    if (!p.fresh) pdl_launch_dependents();
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+
+    if (tid == 0) {
+        for (int i = 0; i < kNumBars; ++i) {
+            uint32_t count = 1;
+            if (i >= kQFull && i < kQFree) count = 8;                   // four producer warps of both CTAs
+            else if (i >= kPFull && i < kPvDone) count = 8;             // four softmax warps of both CTAs
+            else if (i == kOFree) count = 16;                           // eight softmax warps of both CTAs
+            mbar_init(c.bar(i), count);
+        }
+        st_shared(c.abort_flag(), 0);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 12) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(c.tmem_slot()) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    if (p.fresh) {
+        pdl_wait();
+        pdl_launch_dependents();
+    }
+    // from here on: the Q producer, the append and the TMA warp (for anything but pool tiles) wait for the kernel in front;
+    // everything else follows from what they deliver
+    c.item_begin = p.cta_begin[blockIdx.x >> 1];              // (the work list gives every pair at least one piece)
+    c.item_end = p.cta_begin[(blockIdx.x >> 1) + 1];
+    __syncwarp();
+    tc_fence_before();
+    cluster_sync();                                           // both CTAs' barriers and TMEM are there
+    tc_fence_after();
+    c.tmem = ld_shared(c.tmem_slot());
+
+    if (warp < 8) {
+        softmax_role(p, c, warp >> 2, tid & 127);
+    } else if (warp < 12) {
+        producer_role(p, c, tid - 256);
+    } else if (warp < 15) {
+        if (c.rank == 0 && elect_one()) mma_role(p, c, (uint32_t)warp - 12);
+        __syncwarp();
+    } else {
+        tma_role(p, c, lane, &k_pool, &v_pool, &k_ws, &v_ws, &k_new, &v_new);
+    }
+
+    // ---- teardown: neither CTA leaves while the other may still reach into it -------------------------------
+    if (ld_shared(c.abort_flag())) {        // let copies still in flight land
+        const uint64_t t0 = global_ns();
+        while (global_ns() - t0 < 200000ull) __nanosleep(1000);
+    }
+    __syncwarp();
+    tc_fence_before();
+    cluster_sync();
+    if (warp == 12) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(c.tmem) : "memory");
+    }
+}
+
+}  // namespace
+
+cudaError_t kvp_attn_pair_prepare(void)
+{
+    return cudaFuncSetAttribute(attn_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+}
+
+cudaError_t kvp_launch_attn_pair(const kvp_shape &sh, const kvp_attn2_args &a, const CUtensorMap &k_pool, const CUtensorMap &v_pool,
+                                 const CUtensorMap &k_ws, const CUtensorMap &v_ws, cudaStream_t st)
+{
+    // without tail_direct the two query maps are never dereferenced: any valid map will do
+    return launch_pdl(attn_pair_kernel, 2 * a.n_ctas, kThreads, kSmemBytes, st, k_pool, v_pool, k_ws, v_ws,
+                      a.tail_direct ? a.tm_knew : k_ws, a.tail_direct ? a.tm_vnew : v_ws, make_params(sh, a));
+}

@@ -159,6 +159,7 @@ struct kvp_schedule {
     std::vector<kvp_work> works;
     std::vector<kvp_merge_item> merges;
     int32_t n_ctas = 0, n_slots = 0, max_pieces = 1;
+    bool pair = false;                     // for CTA pairs: every unit in mode 0, n_ctas counts pairs
     struct unit { int32_t b, hk, row_base, mode, n_all, n_pieces, q_len, t_first, tile_begin, tail_row0, n_tail, slot; };
     struct cut { int32_t u, t; };
     std::vector<unit> units;
@@ -218,8 +219,8 @@ struct kvp_ctx {
 
     // TMA descriptors (bf16, head_dim 128 only)
     bool have_tma = false;
-    CUtensorMap tm_pool_k, tm_pool_v;
-    std::vector<CUtensorMap> tm_ws_k, tm_ws_v;
+    CUtensorMap tm_pool_k, tm_pool_v, tm_pool_k_half;       // _half: boxes of 64 rows, a CTA's part of a K tile in a pair
+    std::vector<CUtensorMap> tm_ws_k, tm_ws_v, tm_ws_k_half;
 
     int32_t sm_count = 148;
     int32_t split_target_ctas = 0, force_splits = 0;
@@ -330,6 +331,10 @@ struct kvp_attn2_args {
     CUtensorMap tm_knew, tm_vnew;
 };
 cudaError_t kvp_attn_sm100_prepare(int32_t head_dim);
+cudaError_t kvp_attn_pair_prepare(void);
+// a.n_ctas counts CTA pairs; the K maps have boxes of 64 rows
+cudaError_t kvp_launch_attn_pair(const kvp_shape &sh, const kvp_attn2_args &a, const CUtensorMap &k_pool, const CUtensorMap &v_pool,
+                                 const CUtensorMap &k_ws, const CUtensorMap &v_ws, cudaStream_t st);
 cudaError_t kvp_launch_attn_sm100(const kvp_shape &sh, const kvp_attn2_args &a, const CUtensorMap &tm_pool_k,
                                   const CUtensorMap &tm_pool_v, const CUtensorMap &tm_ws_k,
                                   const CUtensorMap &tm_ws_v, cudaStream_t st);
