@@ -254,9 +254,10 @@ constexpr int kPieceCostOne = 4, kPieceCostPair = 8;
 // 0.08 Gflop: 11-17 us against 13-24; 0.12-0.15: 21 against 23; 0.23: 29 against 25; 2.3: 113 against 25.
 constexpr double kTcMinFlops64 = 1.5e8;
 
-// Whether a call runs on CTA pairs (kvp_attn_pair.cu): units of up to 256 rows, of which the one-CTA kernel keeps the
-// calls whose units mostly hold no more than 128.  Per key tile a pair takes about 2 x 1,400 cycles for 256 rows and for
-// 128 rows alike, the one-CTA kernel 3,900 and 1,950.
+// Whether a call runs on CTA pairs (kvp_attn_pair.cu), whose units are 256 rows: a unit that holds no more than 128 costs
+// a pair as much as a full one (2 x 1,600 cycles per key tile; the one-CTA kernel 3,900, and 1,950 for a narrow unit).
+// With three narrow units to two wide ones pairs were 4 % slower, with one to four 1 % (ragged batches), without any
+// 2-10 % faster.
 bool use_pairs(const kvp_ctx *ctx, const kvp_assembly_host &as, int q_len, const int32_t *q_lens)
 {
     const kvp_shape &sh = ctx->shape;
@@ -268,7 +269,7 @@ bool use_pairs(const kvp_ctx *ctx, const kvp_assembly_host &as, int q_len, const
         wide += keys * (rows / (2 * KVP_TILE_ROWS) + (rest > KVP_TILE_ROWS ? 1 : 0));
         narrow += keys * (rest > 0 && rest <= KVP_TILE_ROWS ? 1 : 0);
     }
-    return 2 * wide >= narrow;
+    return wide >= 6 * narrow;
 }
 
 // q_lens: nullptr, or one query length per request (<= q_len, the stride of the padded tensors); a request's

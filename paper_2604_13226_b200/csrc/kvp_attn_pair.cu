@@ -17,17 +17,17 @@
 //                     or, once P V of tile k - 1 has landed, O is rescaled.
 //   warps 8-11        Q producer: counter-rotates this CTA's rows once per document (as in the one-CTA kernel), and appends
 //                     the query block's K/V rows
-//   warps 12-14       CTA 0 of the pair: MMA issuers for both, step by step in turn.  Warp 12 owns TMEM in each.
-//   warp 15           TMA producer of this CTA's halves; its bytes are counted on CTA 0's barriers
+//   warp 12           CTA 0 of the pair: MMA issuer for both.  TMEM owner in each.
+//   warp 13           TMA producer of this CTA's halves; its bytes are counted on CTA 0's barriers
 //
-// Barriers that CTA 0's MMA warps wait for live in CTA 0 and are arrived at from both CTAs; those they signal
+// Barriers that CTA 0's MMA warp waits for live in CTA 0 and are arrived at from both CTAs; those they signal
 // (tcgen05.commit, multicast) exist in both.  Every wait is bounded: when it runs out the status word gets a code, both
 // CTAs' abort flags are set and every role leaves.
 #include "kvp_attn_common.cuh"
 
 namespace {
 
-constexpr int kThreads = 512;
+constexpr int kThreads = 448;
 constexpr int kStageBytes = 16384;                       // half a K or V tile
 // Ring and Q buffers share 208 KB: two buffers of 32 KB (value) or 64 KB (value and remainder) and 9 or 5 stages.
 constexpr int kMaxStages = 9;
@@ -39,8 +39,8 @@ constexpr uint32_t kColO = 384;                           // S buffer b: columns
 constexpr uint16_t kBoth = 3;
 
 enum BarIdx { kKvFull = 0, kKvEmpty = kMaxStages, kQFull = 2 * kMaxStages, kQFree = kQFull + 2, kSFull = kQFree + 2, kPFull = kSFull + 3,
-              kPvDone = kPFull + 3, kOFull = kPvDone + 2, kOFree, kMref, kEnd = kMref + 8, kTurn = kEnd + 8,       // Mref, End: [4 * warpgroup + quadrant]
-              kDrain = kTurn + 3, kNumBars = kDrain + 3 };
+              kPvDone = kPFull + 3, kOFull = kPvDone + 2, kOFree, kMref, kEnd = kMref + 8, kDrain = kEnd + 8,      // Mref, End: [4 * warpgroup + quadrant]
+              kNumBars };
 static_assert(8 * kNumBars <= 504, "barrier block");
 
 struct Cta {
@@ -380,7 +380,7 @@ __device__ __forceinline__ void producer_role(const Params &p, const Cta &c, con
     }
 }
 
-// Loads of a piece with n tiles in the order the MMA warps take them: Q K^T runs three tiles ahead of P V, so
+// Loads of a piece with n tiles in the order the MMA warp takes them: Q K^T runs three tiles ahead of P V, so
 // K0 K1 K2 V0 K3 V1 K4 ... V(n-1).  Load q is tile r's K (kv = 0) or V (kv = 1).
 __device__ __forceinline__ void load_at(int n, int q, int &r, int &kv)
 {
@@ -446,126 +446,137 @@ __device__ __forceinline__ void tma_role(const Params &p, const Cta &c, const in
     }
 }
 
-// ---- MMA issuers (one thread of each of three warps of CTA 0) --------------------------------------------------------
-// Step k of a piece is O += P V of tile k - 3 and S = Q K^T of tile k, which takes over that tile's S buffer: warp I takes
-// the steps of S buffer I, each in its turn.  The MMAs of a step wait in a queue that the sub-partition's special-function
-// instructions go through too: with one issuing warp its two softmax warps took 3,200 cycles per tile against 2,400 of the
-// others; three warps on three sub-partitions share that out.  What a step waits for is waited for before its turn.
-__device__ __forceinline__ void mma_role(const Params &p, const Cta &c, const uint32_t I)
+// ---- MMA issuer (one warp of CTA 0, convergent; one elected lane issues) ----------------------------------------
+// Step k of a piece is O += P V of tile k - 3 and S = Q K^T of tile k, which takes over that tile's S buffer.  The MMAs
+// wait in a queue that the sub-partition's special-function instructions go through too, so this warp's two softmax
+// neighbours are slower than the others (3,000 cycles per tile against 2,400); three issuing warps on three sub-partitions
+// in turn evened that out and did not help: the launch is then bound by power (1,000 W) or by the hand-over between them.
+__device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
 {
-    const uint32_t q_stride = (p.precise ? 2 * kQBufBytes : kQBufBytes) >> 4;
+    const uint32_t n_stages = p.precise ? 5 : 9;
+    const uint32_t q_stride = p.precise ? 2 * kQBufBytes : kQBufBytes;
     const uint32_t ring = c.smem_base + (p.precise ? 4 : 2) * kQBufBytes;
     const uint32_t idesc_pv = instr_desc(128, 1);
-    const uint32_t v_desc = desc_lo(ring, kHalfBytes), k_desc = desc_lo(ring, 16), q_desc = desc_lo(c.smem_base, 16);
-    const uint32_t sp = c.tmem + I * 128, oa = c.tmem + kColO;
-    uint32_t g0 = 0;                                      // steps of the pieces before this one, mod 3
-    uint32_t T0 = 0, R0 = 0;                              // their tiles and loads
-    uint32_t parP = 0;
-    int turn = I == 0 ? -1 : 0;                           // phase of the turn barrier (warp 0 begins without one)
-    int ep = -1, ep_ready = -1, pieces = 0;               // Q epoch of the last tile looked at; last one waited for
+    const bool lead = elect_one();
+    const int lane = threadIdx.x & 31;
+    uint32_t stage = 0, par = 0;                          // ring position of the next load to be used
+    uint32_t bufS = 0;                                    // S buffer of the next Q K^T
+    uint32_t bufP = 0, parP = 0;                          // of the next P V
+    uint32_t T = 0;                                       // its running number
+    uint32_t ep = 0, pieces = 0;
     bool ok = true;
-    auto stage_of = [&](uint32_t load, uint32_t &par) {
-        const uint32_t use = p.precise ? load / 5 : load / 9;
-        par = use & 1;
-        return load - use * (p.precise ? 5 : 9);
-    };
+    auto advance = [&] { if (++stage == n_stages) { stage = 0; par ^= 1; } };
 
     for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
         const Work w = load_work(p, wi);
         const int n = w.n;
-        int nk3 = 0, last_rope = -1;                      // key count of tile k - 3; document of the last tile looked at
-        int seen = 0;                                     // tiles looked at
+        // tile facts are fetched 32 at a time, one per lane, and handed round by shuffle
+        int b0 = 0, nk_l = 0, rope_l = 0;
+        auto refill = [&](int from) {
+            b0 = from;
+            if (from + lane < n) {
+                const Tile t = get_tile(p, w, w.lo + from + lane);
+                nk_l = t.n_keys;
+                rope_l = t.rope;
+            }
+        };
+        refill(0);
+        int nk1 = 0, nk2 = 0, nk3 = 0;                    // key counts of the last three tiles
+        int prev_rope = 0;
+        uint32_t qbuf = 0;
 #pragma unroll 1
-        for (int k = (int)((I + 3 - g0) % 3); k < n + 3; k += 3) {
-            // the Q epoch of tile k: a new one at each change of document
-            int nk = 0;
-            bool lastq = true;
-            if (k < n) {
-                for (; seen <= k; ++seen) {
-                    const Tile t = get_tile(p, w, w.lo + seen);
-                    if (t.rope != last_rope) ++ep;
-                    last_rope = t.rope;
-                    nk = t.n_keys;
-                }
-                lastq = k + 1 >= n || get_tile(p, w, w.lo + k + 1).rope != last_rope;
-            }
-            const uint32_t qbuf = ep & 1;
-            uint32_t pv_par = 0, pk_par = 0, sv = 0, sk = 0;
+        for (int k = 0; k < n + 3; ++k) {
+            // ---- waits: the tiles first, which land while P is being formed ------------------------------
+            int nk = 0, rope = 0;
+            bool lastq = false;
+            uint32_t stK = stage;                         // K(k) lies behind V(k - 3) in the ring
             if (k >= 3) {
-                sv = stage_of(R0 + (uint32_t)(k - 3 + min(n, k)), pv_par);
-                ok = wait(p, c, kKvFull + sv, pv_par, 23);
-                if (ok && k == 3 && pieces > 0) ok = wait(p, c, kOFree, (pieces - 1) & 1, 26);
-                ok = ok && wait(p, c, kPFull + I, parP, 24);
-                parP ^= 1;
+                ok = wait(p, c, kKvFull + stage, par, 23);
+                if (++stK == n_stages) stK = 0;
             }
             if (k < n) {
-                sk = stage_of(R0 + (uint32_t)(k + max(0, k - 2)), pk_par);
-                if (!p.precise) ok = ok && wait(p, c, kKvFull + sk, pk_par, 22);      // (with 5 stages the phase is known in turn only)
+                if (k - b0 == 31) refill(k);              // tile k + 1 stays inside the batch
+                nk = __shfl_sync(0xffffffffu, nk_l, k - b0);
+                rope = __shfl_sync(0xffffffffu, rope_l, k - b0);
+                const int rope_n = __shfl_sync(0xffffffffu, rope_l, (k + 1 - b0) & 31);
+                const bool newq = k == 0 || rope != prev_rope;   // first tile of a document: its own Q buffer
+                lastq = k + 1 >= n || rope_n != rope;
+                prev_rope = rope;
+                if (ok) ok = wait(p, c, kKvFull + stK, stK < stage ? par ^ 1 : par, 22);
+                if (newq) {
+                    qbuf = ep & 1;
+                    if (ok) ok = wait(p, c, kQFull + qbuf, (ep >> 1) & 1, 20);
+                    ++ep;
+                }
             }
-            // ---- this warp's turn -----------------------------------------------------------------
-            if (turn >= 0) ok = ok && wait(p, c, kTurn + I, (uint32_t)turn & 1, 25);
-            if (p.precise && k < n) ok = ok && wait(p, c, kKvFull + sk, pk_par, 22);
-            if (k < n && ep != ep_ready) {                 // (in turn only: documents may be of one tile)
-                ok = ok && wait(p, c, kQFull + qbuf, ((uint32_t)ep >> 1) & 1, 20);
-                ep_ready = ep;
+            if (k >= 3) {
+                if (ok) ok = wait(p, c, kPFull + bufP, parP, 24);
+                if (ok && k == 3 && pieces > 0) ok = wait(p, c, kOFree, (pieces - 1) & 1, 26);
             }
+            ok = __all_sync(0xffffffffu, ok);             // the lanes stay together
             if (!ok) break;
             tc_fence_after();
-            if (k >= 3) {                                  // O += P V
-                const uint32_t v_lo = v_desc + sv * (kStageBytes >> 4);
-                if (nk3 == KVP_TILE_KEYS && k > 3) {
+            if (k >= 3) {
+                // ---- O += P V of tile k - 3 ---------------------------------------------------------
+                if (lead) {
+                    const uint32_t v_lo = desc_lo(ring + stage * kStageBytes, kHalfBytes);
+                    const uint32_t pa = c.tmem + bufP * 128, oa = c.tmem + kColO;
+                    if (nk3 == KVP_TILE_KEYS && k > 3) {
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk)               // 16 keys per step: P advances 8 columns, V 2048 bytes
-                        mma_ts(oa, sp + kk * 8, desc64(v_lo + kk * 128, kDescHi), idesc_pv, 1);
-                } else {
-                    const int ksteps = max(1, (nk3 + 15) >> 4);
-                    for (int kk = 0; kk < ksteps; ++kk)
-                        mma_ts(oa, sp + kk * 8, desc64(v_lo + kk * 128, kDescHi), idesc_pv, (k > 3 || kk > 0));
+                        for (int kk = 0; kk < 8; ++kk)           // 16 keys per step: P advances 8 columns, V 2048 bytes
+                            mma_ts(oa, pa + kk * 8, desc64(v_lo + kk * 128, kDescHi), idesc_pv, 1);
+                    } else {
+                        const int ksteps = max(1, (nk3 + 15) >> 4);
+                        for (int kk = 0; kk < ksteps; ++kk)
+                            mma_ts(oa, pa + kk * 8, desc64(v_lo + kk * 128, kDescHi), idesc_pv, (k > 3 || kk > 0));
+                    }
+                    commit_both(c.bar(kKvEmpty + stage));
+                    commit_both(c.bar(kPvDone + (T & 1)));
+                    if (k == n + 2) commit_both(c.bar(kOFull));
                 }
-                commit_both(c.bar(kKvEmpty + sv));
-                commit_both(c.bar(kPvDone + ((T0 + (uint32_t)k - 3) & 1)));
-                if (k == n + 2) commit_both(c.bar(kOFull));
+                __syncwarp();
+                advance();
+                ++T;
+                if (++bufP == 3) { bufP = 0; parP ^= 1; }
             }
-            if (k < n) {                                   // S = Q K^T
-                const uint32_t idesc = instr_desc((uint32_t)qk_n(nk), 0);
-                const uint32_t q_lo = q_desc + qbuf * q_stride, k_lo = k_desc + sk * (kStageBytes >> 4);
-                // 16 columns per step: 32 bytes; the second 64 columns lie 16 KB (Q) and 8 KB (K) on
-                mma_ss<0>(sp, desc64(q_lo, kDescHi), desc64(k_lo, kDescHi), idesc);
-#pragma unroll
-                for (int kk = 1; kk < 8; ++kk)
-                    mma_ss<1>(sp, desc64(q_lo + (kk >> 2) * (kHalfBytes >> 4) + (kk & 3) * 2, kDescHi),
-                              desc64(k_lo + (kk >> 2) * (kStageBytes >> 5) + (kk & 3) * 2, kDescHi), idesc);
-                if (p.precise && last_rope != 0) {               // + (rounding remainder of the rotated Q) K^T
-#pragma unroll
-                    for (int kk = 0; kk < 8; ++kk)
-                        mma_ss<1>(sp, desc64(q_lo + (kQBufBytes >> 4) + (kk >> 2) * (kHalfBytes >> 4) + (kk & 3) * 2, kDescHi),
-                                  desc64(k_lo + (kk >> 2) * (kStageBytes >> 5) + (kk & 3) * 2, kDescHi), idesc);
-                }
-            }
-            tc_fence_before();
-            mbar_arrive(c.bar(kTurn + (I == 2 ? 0 : I + 1)));
-            ++turn;
             if (k < n) {
-                commit_both(c.bar(kSFull + I));
-                commit_both(c.bar(kKvEmpty + sk));
-                if (lastq) commit_both(c.bar(kQFree + qbuf));
+                // ---- S = Q K^T of tile k ----------------------------------------------------------
+                if (lead) {
+                    const uint32_t idesc = instr_desc((uint32_t)qk_n(nk), 0);
+                    const uint32_t q_lo = desc_lo(c.smem_base + qbuf * q_stride, 16);
+                    const uint32_t k_lo = desc_lo(ring + stage * kStageBytes, 16);
+                    const uint32_t d = c.tmem + bufS * 128;
+                    // 16 columns per step: 32 bytes; the second 64 columns lie 16 KB (Q) and 8 KB (K) on
+                    mma_ss<0>(d, desc64(q_lo, kDescHi), desc64(k_lo, kDescHi), idesc);
+#pragma unroll
+                    for (int kk = 1; kk < 8; ++kk)
+                        mma_ss<1>(d, desc64(q_lo + (kk >> 2) * (kHalfBytes >> 4) + (kk & 3) * 2, kDescHi),
+                                  desc64(k_lo + (kk >> 2) * (kStageBytes >> 5) + (kk & 3) * 2, kDescHi), idesc);
+                    if (p.precise && rope != 0) {                // + (rounding remainder of the rotated Q) K^T
+#pragma unroll
+                        for (int kk = 0; kk < 8; ++kk)
+                            mma_ss<1>(d, desc64(q_lo + (kQBufBytes >> 4) + (kk >> 2) * (kHalfBytes >> 4) + (kk & 3) * 2, kDescHi),
+                                      desc64(k_lo + (kk >> 2) * (kStageBytes >> 5) + (kk & 3) * 2, kDescHi), idesc);
+                    }
+                    commit_both(c.bar(kSFull + bufS));
+                    commit_both(c.bar(kKvEmpty + stage));
+                    if (lastq) commit_both(c.bar(kQFree + qbuf));
+                }
+                __syncwarp();
+                advance();
+                if (++bufS == 3) bufS = 0;
             }
-            nk3 = nk;
+            nk3 = nk2;
+            nk2 = nk1;
+            nk1 = nk;
         }
-        for (; seen < n; ++seen) {                         // tiles behind this warp's last step
-            const int r = get_tile(p, w, w.lo + seen).rope;
-            if (r != last_rope) ++ep;
-            last_rope = r;
-        }
-        g0 = (g0 + (uint32_t)n) % 3;
-        T0 += (uint32_t)n;
-        R0 += 2u * (uint32_t)n;
         ++pieces;
     }
+    __syncwarp();
     if (!ok) {                      // drain whatever was issued before giving TMEM back
-        asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(c.bar(kDrain + I)) : "memory");
+        if (lead) asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(c.bar(kDrain)) : "memory");
         const uint64_t t0 = global_ns();
-        while (!mbar_try_wait(c.bar(kDrain + I), 0) && global_ns() - t0 < 100000000ull) {}
+        while (!mbar_try_wait(c.bar(kDrain), 0) && global_ns() - t0 < 100000000ull) {}
     }
 }
 
@@ -616,10 +627,9 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap k_pool, const __grid_consta
         softmax_role(p, c, warp >> 2, tid & 127);
     } else if (warp < 12) {
         producer_role(p, c, tid - 256);
-    } else if (warp < 15) {
-        if (c.rank == 0 && elect_one()) mma_role(p, c, (uint32_t)warp - 12);
-        __syncwarp();
-    } else {
+    } else if (warp == 12) {
+        if (c.rank == 0) mma_role(p, c);
+    } else if (warp == 13) {
         tma_role(p, c, lane, &k_pool, &v_pool, &k_ws, &v_ws, &k_new, &v_new);
     }
 

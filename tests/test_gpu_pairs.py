@@ -1,0 +1,54 @@
+"""The attention kernel on CTA pairs at the edges of its pipeline: pieces of one to four tiles (three S buffers), documents
+of a single tile (a new Q buffer at every step), short tiles, remainders of rows in the second CTA, outliers that move the
+reference maximum late in a piece - every row against the oracle, and the same bits when run again."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2604_13226_b200 import binding as kvp
+from paper_2604_13226_b200 import inputs as gen
+from paper_2604_13226_b200.session import Session
+from test_gpu_parity import check_attention
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("lens,q_len,ctas,flags", [
+    ([1], 64, 0, 0),                                   # two or three tiles in all
+    ([128], 33, 2, 0),                                 # 132 rows: four in the second CTA; one pair walks everything
+    ([100, 1, 128, 127, 31, 33, 64], 64, 0, 0),        # a document per tile
+    ([100, 1, 128, 127, 31, 33, 64], 64, 4, kvp.PRECISE_QK),
+    ([129, 257, 385, 513], 70, 148, 0),                # many pieces of two tiles
+    ([640, 1024], 150, 6, kvp.PRECISE_QK),             # two causal tiles, several pieces per pair
+])
+def test_pipeline_edges(lens, q_len, ctas, flags):
+    shape = gen.ModelShape(1, 32, 8, 128, "bf16", 500000.0, 0)
+    wl = gen.make_workload(shape, lens, [[(p, 0) for p in range(len(lens))]], q_len=q_len, seed=91 + q_len)
+    sess = Session(wl)
+    sess.assemble()
+    if ctas:
+        sess.ctx.tune(kvp.TUNE_SPLIT_TARGET_CTAS, ctas)
+    check_attention(wl, sess, flags=flags)
+    assert sess.ctx.last_launch()["kind"] == 1 and sess.ctx.last_launch()["ctas"] % 2 == 0
+    qkv = sess.query_tensors(0)
+    first, _ = sess.prefill(0, flags, qkv=qkv)
+    for _ in range(20):
+        assert torch.equal(first, sess.prefill(0, flags, qkv=qkv)[0])
+    sess.close()
+
+
+def test_reference_maximum_moves_late_in_a_piece():
+    # keys grow from document to document, so that scores rise by more than 2^8 at tiles of both warpgroups: O and the
+    # tile at hand are rescaled.  Scores reach +-40, so the rounding of the rotated Q (2^-9 relative per term) shows in the
+    # probabilities: KVP_PRECISE_QK, whose outputs the shared bounds hold for
+    shape = gen.ModelShape(1, 32, 8, 128, "bf16", 500000.0, 0)
+    wl = gen.make_workload(shape, [300, 200, 130, 500, 90], [[(p, 0) for p in range(5)]], q_len=64, seed=7)
+    for i, pk in enumerate(wl.packets):
+        pk.k[:] = gen.to_stored(gen.bf16_bits_to_f32(pk.k) * np.float32(0.2 * 2.2 ** i), "bf16")
+    for ctas in (2, 0):
+        sess = Session(wl)
+        sess.assemble()
+        if ctas:
+            sess.ctx.tune(kvp.TUNE_SPLIT_TARGET_CTAS, ctas)
+        check_attention(wl, sess, flags=kvp.PRECISE_QK)
+        sess.close()
