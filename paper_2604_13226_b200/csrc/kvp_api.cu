@@ -773,6 +773,19 @@ int32_t kvp_register_packet(kvp_ctx *ctx, const void *k, const void *v, int32_t 
     return KVP_OK;
 }
 
+// The device address of a host buffer that is pinned from its first to its last byte and 16-byte aligned; else nullptr.
+static const char *pinned_address(const void *host, size_t bytes)
+{
+    cudaPointerAttributes first, last;
+    if (((uintptr_t)host & 15) == 0 && cudaPointerGetAttributes(&first, host) == cudaSuccess && first.type == cudaMemoryTypeHost &&
+        first.devicePointer && cudaPointerGetAttributes(&last, (const char *)host + bytes - 1) == cudaSuccess &&
+        last.type == cudaMemoryTypeHost && (char *)last.devicePointer == (char *)first.devicePointer + bytes - 1 &&
+        ((uintptr_t)first.devicePointer & 15) == 0)
+        return (const char *)first.devicePointer;
+    (void)cudaGetLastError();
+    return nullptr;
+}
+
 int32_t kvp_register_packet_host(kvp_ctx *ctx, const void *k_host, const void *v_host, int32_t n_tokens,
                                  int32_t cache_pos0, int32_t *packet_id)
 {
@@ -789,6 +802,12 @@ int32_t kvp_register_packet_host(kvp_ctx *ctx, const void *k_host, const void *v
     src.v = (const char *)v_host;
     src.from_host = true;
     src.resident = false;
+    if (!ctx->host_only) {
+        // what kernels may read themselves: pinned buffers, aligned for bulk copies
+        const size_t bytes = (size_t)ctx->shape.n_layers * ctx->shape.n_kv_heads * n_tokens * ctx->shape.head_dim * ctx->shape.elem_bytes;
+        src.dev_k = pinned_address(k_host, bytes);
+        src.dev_v = pinned_address(v_host, bytes);
+    }
     *packet_id = (int32_t)ctx->packets.size() - 1;
     return KVP_OK;
 }
@@ -805,7 +824,8 @@ int32_t kvp_evict_packet(kvp_ctx *ctx, int32_t packet_id)
 
 // Host -> pool copies of the packets of an assembly that are not on the device yet, one layer after the other
 // on the context's own stream, an event per layer.  Host layout [n_layers][n_kv_heads][n_tokens][head_dim]: a
-// layer of a packet is n_kv_heads runs of n_tokens rows, one per plane, i.e. one 2-D copy for K and one for V.
+// layer of a packet is n_kv_heads runs of n_tokens rows, one per plane.  Pinned buffers: one launch for all packets of
+// a layer, which reads them over the host link; others: one 2-D copy for K and one for V of each packet.
 static int32_t load_host_packets(kvp_ctx *ctx, const std::vector<int32_t> &ids, cudaStream_t st)
 {
     const kvp_shape &sh = ctx->shape;
@@ -815,9 +835,19 @@ static int32_t load_host_packets(kvp_ctx *ctx, const std::vector<int32_t> &ids, 
     KVP_CUDA(ctx, cudaEventRecord(ctx->load_fence, st));
     KVP_CUDA(ctx, cudaStreamWaitEvent(ctx->load_stream, ctx->load_fence, 0));
     for (int l = 0; l < sh.n_layers; ++l) {
+        kvp_load_list list;
+        list.n_items = 0;
         for (int32_t id : ids) {
             const kvp_segment_host &pk = ctx->packets[id];
             const kvp_ctx::host_src &src = ctx->packet_src[id];
+            if (src.dev_k && src.dev_v) {
+                list.item[list.n_items++] = {src.dev_k, src.dev_v, pk.n, pk.row0, 0, 0};
+                if (list.n_items == KVP_LOAD_ITEMS) {
+                    KVP_CUDA(ctx, kvp_launch_load(sh, list, l, ctx->pool_k, ctx->pool_v, ctx->status_dev, ctx->load_stream));
+                    list.n_items = 0;
+                }
+                continue;
+            }
             const size_t run = (size_t)pk.n * row_bytes;
             const size_t dst = ((size_t)l * sh.n_kv_heads * sh.pool_rows + pk.row0) * row_bytes;
             const size_t from = (size_t)l * sh.n_kv_heads * run;
@@ -826,6 +856,7 @@ static int32_t load_host_packets(kvp_ctx *ctx, const std::vector<int32_t> &ids, 
             KVP_CUDA(ctx, cudaMemcpy2DAsync(ctx->pool_v + dst, (size_t)sh.pool_rows * row_bytes, src.v + from, run, run,
                                             sh.n_kv_heads, cudaMemcpyHostToDevice, ctx->load_stream));
         }
+        if (list.n_items) KVP_CUDA(ctx, kvp_launch_load(sh, list, l, ctx->pool_k, ctx->pool_v, ctx->status_dev, ctx->load_stream));
         KVP_CUDA(ctx, cudaEventRecord(ctx->load_done[l], ctx->load_stream));
     }
     for (int32_t id : ids) ctx->packet_src[id].resident = true;

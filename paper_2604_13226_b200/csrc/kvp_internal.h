@@ -176,7 +176,8 @@ struct kvp_ctx {
     std::vector<double> inv_freq;
     std::vector<kvp_segment_host> packets;
     // packets whose K/V wait in host memory until a request uses them (parallel to `packets`, grown on demand)
-    struct host_src { const char *k = nullptr, *v = nullptr; bool from_host = false, resident = true; };
+    // (dev_k, dev_v: the same buffers as kernels see them, if they are pinned)
+    struct host_src { const char *k = nullptr, *v = nullptr, *dev_k = nullptr, *dev_v = nullptr; bool from_host = false, resident = true; };
     std::vector<host_src> packet_src;
     cudaStream_t load_stream = nullptr;             // host -> pool copies, layer by layer
     cudaEvent_t load_fence = nullptr;               // the caller's stream at the assemble that starts a load
@@ -271,6 +272,21 @@ cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
 
 cudaError_t kvp_launch_store_rows(const kvp_shape &sh, const void *src, char *dst_plane0, int64_t plane_rows,
                                   int64_t dst_row0, int32_t n_tokens, cudaStream_t st);
+// One layer of packets that wait in pinned host memory, into the pool.
+struct kvp_load_item {
+    const char *k, *v;         // device addresses of the host buffers, [n_layers][n_kv_heads][n][head_dim]
+    int32_t n, row0;           // tokens; first pool row
+    int32_t piece0;            // first of its pieces in the launch
+    int32_t pad;
+};
+#define KVP_LOAD_ITEMS 48
+struct kvp_load_list {
+    int32_t n_items, n_pieces;
+    kvp_load_item item[KVP_LOAD_ITEMS];
+};
+// fills in piece0 and n_pieces
+cudaError_t kvp_launch_load(const kvp_shape &sh, kvp_load_list &list, int32_t layer, char *pool_k, char *pool_v, int32_t *status,
+                            cudaStream_t st);
 // `bytes` (rounded up to 16) from pinned host memory to the device; the blocks' flags receive `seq` once they have read
 // their part.  Returns through *blocks how many there are.
 cudaError_t kvp_launch_upload(const void *host, void *dst, uint64_t bytes, volatile uint32_t *flags, uint32_t seq,

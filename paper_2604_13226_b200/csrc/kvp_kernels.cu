@@ -119,6 +119,91 @@ upload_kernel(const uint4 *__restrict__ host, uint4 *__restrict__ dst, int n_wor
     if (threadIdx.x == 0) flags[blockIdx.x] = seq;
 }
 
+// ---- packets from pinned host memory into the pool, one layer ---------------------------------------------
+// A run - one kv head of K or V of a packet - is contiguous on both sides; runs are cut into pieces of 4 KB and the blocks
+// take pieces in turn, one thread each, with bulk copies host -> shared memory -> pool in a ring of three.  Bound by the
+// host link: reads from the SMs reach 51.2 GB/s whatever the sizes, where a copy per packet, layer and K/V costs 4 us
+// beside its transfer (1 MB each: 45.7 GB/s, 256 KB: 28.8; one copy of 128 MB: 55.2).  A block is one warp with 12 KB, so
+// that the attention kernel on CTA pairs fits beside it.
+constexpr int kLoadPiece = 4096, kLoadStages = 3;
+
+__device__ __forceinline__ uint32_t shared_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ uint64_t now_ns()
+{
+    uint64_t t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
+__global__ void __launch_bounds__(32)
+load_kernel(const __grid_constant__ kvp_load_list list, int layer, int n_kv, int row_bytes, int64_t pool_rows,
+            char *__restrict__ pool_k, char *__restrict__ pool_v, int32_t *status)
+{
+    __shared__ __align__(128) char buf[kLoadStages][kLoadPiece];
+    __shared__ uint64_t bars[kLoadStages];
+    if (threadIdx.x != 0) return;
+    for (int i = 0; i < kLoadStages; ++i)
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(shared_addr(&bars[i])) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    const int mine = (list.n_pieces - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+    int it = 0;                                              // packet of the next piece to fetch
+    char *dst[kLoadStages];
+    uint32_t size[kLoadStages];
+    auto fetch = [&](int k, int stage) {
+        const int piece = blockIdx.x + k * gridDim.x;
+        while (it + 1 < list.n_items && piece >= list.item[it + 1].piece0) ++it;
+        const kvp_load_item &x = list.item[it];
+        const int64_t run = (int64_t)x.n * row_bytes;
+        const int per_run = (int)((run + kLoadPiece - 1) / kLoadPiece);
+        const int r = (piece - x.piece0) / per_run;
+        const int64_t off = (int64_t)((piece - x.piece0) % per_run) * kLoadPiece;
+        const int head = r % n_kv;
+        const bool is_v = r >= n_kv;
+        const char *src = (is_v ? x.v : x.k) + ((int64_t)layer * n_kv + head) * run + off;
+        dst[stage] = (is_v ? pool_v : pool_k) + (((int64_t)layer * n_kv + head) * pool_rows + x.row0) * row_bytes + off;
+        size[stage] = (uint32_t)min((int64_t)kLoadPiece, run - off);
+        const uint32_t bar = shared_addr(&bars[stage]);
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(size[stage]) : "memory");
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(shared_addr(buf[stage])),
+                     "l"(src), "r"(size[stage]), "r"(bar)
+                     : "memory");
+    };
+#pragma unroll
+    for (int k = 0; k < kLoadStages; ++k)
+        if (k < mine) fetch(k, k);
+    bool ok = true;
+    for (int k0 = 0; k0 < mine && ok; k0 += kLoadStages) {
+#pragma unroll
+        for (int s = 0; s < kLoadStages; ++s) {
+            const int k = k0 + s;
+            if (k >= mine || !ok) break;
+            const uint64_t t0 = now_ns();
+            uint32_t done = 0;
+            while (!done && now_ns() - t0 < 2000000000ull)  // bounded: 2 s
+                asm volatile(
+                    "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                    : "=r"(done)
+                    : "r"(shared_addr(&bars[s])), "r"((uint32_t)(k / kLoadStages) & 1u)
+                    : "memory");
+            if (!done) {
+                atomicCAS(status, 0, 50);
+                ok = false;
+                break;
+            }
+            asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst[s]), "r"(shared_addr(buf[s])), "r"(size[s])
+                         : "memory");
+            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+            if (k + kLoadStages < mine) {
+                asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");      // the buffer has been read
+                fetch(k + kLoadStages, s);
+            }
+        }
+    }
+    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    if (!ok)                                                 // let loads still in flight land before the block goes away
+        for (const uint64_t t0 = now_ns(); now_ns() - t0 < 200000ull;) {}
+}
+
 // (cos, sin) of offset x theta, narrowed to fp32 once: the angle is formed in double precision in half turns (offsets
 // reach 1e5 and more), which sincospi reduces exactly.
 __device__ __forceinline__ float2 offset_cos_sin(int32_t offset, double half_turn)
@@ -853,6 +938,21 @@ cudaError_t kvp_launch_store_rows(const kvp_shape &sh, const void *src, char *ds
     const int grid = (int)((total + 255) / 256 > 65535 * 8 ? 65535 * 8 : (total + 255) / 256);
     store_rows_kernel<<<grid, 256, 0, st>>>(reinterpret_cast<const uint4 *>(src), dst_plane0, plane_rows, dst_row0,
                                             n_tokens, sh.n_layers, sh.n_kv_heads, vecs);
+    return cudaGetLastError();
+}
+
+cudaError_t kvp_launch_load(const kvp_shape &sh, kvp_load_list &list, int32_t layer, char *pool_k, char *pool_v, int32_t *status,
+                            cudaStream_t st)
+{
+    const int row_bytes = sh.head_dim * sh.elem_bytes;
+    int64_t pieces = 0;
+    for (int i = 0; i < list.n_items; ++i) {
+        list.item[i].piece0 = (int32_t)pieces;
+        pieces += 2ll * sh.n_kv_heads * (((int64_t)list.item[i].n * row_bytes + kLoadPiece - 1) / kLoadPiece);
+    }
+    list.n_pieces = (int32_t)pieces;
+    // 64 blocks have 768 KB in flight, several times what the link's latency takes
+    load_kernel<<<(int)std::min<int64_t>(64, pieces), 32, 0, st>>>(list, layer, sh.n_kv_heads, row_bytes, sh.pool_rows, pool_k, pool_v, status);
     return cudaGetLastError();
 }
 
