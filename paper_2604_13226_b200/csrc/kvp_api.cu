@@ -529,7 +529,7 @@ int32_t plan_schedule(kvp_ctx *ctx, const kvp_assembly_host &as, int layer, int 
 }
 
 int32_t build_schedule(kvp_ctx *ctx, kvp_assembly_host &as, int slot, int layer, int q_len, int q_pos0, const int32_t *q_lens,
-                       uint32_t opts, cudaStream_t st)
+                       uint32_t opts, kvp_attn2_args &a, cudaStream_t st)
 {
     kvp_schedule &sc = ctx->plan;
     const int32_t rc = plan_schedule(ctx, as, layer, q_len, q_pos0, q_lens, opts, sc);
@@ -537,16 +537,27 @@ int32_t build_schedule(kvp_ctx *ctx, kvp_assembly_host &as, int slot, int layer,
     const uint32_t off_works = (uint32_t)round_up(4 * sc.cta_begin.size(), kPlanAlign);
     const uint32_t off_merges = (uint32_t)round_up(off_works + sizeof(kvp_work) * sc.works.size(), kPlanAlign);
     const size_t used = off_merges + sizeof(kvp_merge_item) * sc.merges.size();
-    const int ring = ctx->sched_next;
-    ctx->sched_next = (ring + 1) % KVP_SCHED_RING;
-    const int32_t rs = stage_wait(ctx, ctx->sched_ring[ring]);
-    if (rs != KVP_OK) return rs;
-    char *h = ctx->sched_ring[ring].host;
-    memcpy(h, sc.cta_begin.data(), 4 * sc.cta_begin.size());
-    memcpy(h + off_works, sc.works.data(), sizeof(kvp_work) * sc.works.size());
-    memcpy(h + off_merges, sc.merges.data(), sizeof(kvp_merge_item) * sc.merges.size());
     const int li = as.item_stride ? layer : 0;                   // which of the assembly's work lists
-    KVP_CUDA(ctx, stage_upload(ctx->sched_ring[ring], ctx->slot_sched_dev[slot] + ctx->sched_bytes * li, used, st));
+    auto pack = [&](char *h) {
+        memcpy(h, sc.cta_begin.data(), 4 * sc.cta_begin.size());
+        memcpy(h + off_works, sc.works.data(), sizeof(kvp_work) * sc.works.size());
+        memcpy(h + off_merges, sc.merges.data(), sizeof(kvp_merge_item) * sc.merges.size());
+    };
+    a.list_dev = ctx->slot_sched_dev[slot] + ctx->sched_bytes * li;
+    if (sc.n_ctas > 0 && used <= KVP_INLINE_LARGE) {               // comes along with the attention launch
+        pack(ctx->list_inline);
+        a.list = ctx->list_inline;
+        a.list_bytes = (uint32_t)round_up(used, 16);
+        a.list_works = off_works;
+    } else {
+        const int ring = ctx->sched_next;
+        ctx->sched_next = (ring + 1) % KVP_SCHED_RING;
+        const int32_t rs = stage_wait(ctx, ctx->sched_ring[ring]);
+        if (rs != KVP_OK) return rs;
+        pack(ctx->sched_ring[ring].host);
+        KVP_CUDA(ctx, stage_upload(ctx->sched_ring[ring], a.list_dev, used, st));
+    }
+    a.fresh = 1;
     kvp_assembly_host::sched_state &ss = as.sched[li];
     ss.q_len = q_len;
     ss.q_lens.assign(q_lens ? q_lens : nullptr, q_lens ? q_lens + as.batch : nullptr);
@@ -1113,14 +1124,21 @@ static int32_t assemble_impl(kvp_ctx *ctx, int32_t batch, const int32_t *slot_of
     const int32_t id = ctx->next_assembly++;
     const int slot = id % cfg.max_assemblies;
     as.id = id;
+    const char *blob = nullptr;
     if (!ctx->host_only) {
         cudaStream_t st = (cudaStream_t)stream;
         KVP_CUDA(ctx, cudaSetDevice(cfg.device));
-        kvp_stage &sg = ctx->plan_ring[ctx->plan_next];
-        ctx->plan_next = (ctx->plan_next + 1) % (int)ctx->plan_ring.size();
-        const int32_t rs = stage_wait(ctx, sg);
-        if (rs != KVP_OK) return rs;
-        char *h = sg.host;
+        char *h = ctx->plan_inline;
+        kvp_stage *sg = nullptr;
+        if (as.off.upload > KVP_INLINE_SMALL) {
+            sg = &ctx->plan_ring[ctx->plan_next];
+            ctx->plan_next = (ctx->plan_next + 1) % (int)ctx->plan_ring.size();
+            const int32_t rs = stage_wait(ctx, *sg);
+            if (rs != KVP_OK) return rs;
+            h = sg->host;
+        } else {
+            blob = h;                                              // comes along with the gather launch
+        }
         memcpy(h + as.off.items, as.items.data(), sizeof(kvp_item) * as.items.size());
         memcpy(h + as.off.tiles, as.tiles.data(), sizeof(kvp_tile) * as.tiles.size());
         memcpy(h + as.off.chunks, as.chunks.data(), sizeof(kvp_chunk) * as.chunks.size());
@@ -1128,10 +1146,12 @@ static int32_t assemble_impl(kvp_ctx *ctx, int32_t batch, const int32_t *slot_of
         memcpy(h + as.off.delta, as.delta.data(), 4 * as.delta.size());
         for (size_t r = 0; r < kept_packets.size(); ++r)
             memcpy(h + as.off.kept + 4 * r * planes, ctx->packets[kept_packets[r]].kept.data(), 4 * (size_t)planes);
-        KVP_CUDA(ctx, stage_upload(sg, ctx->slot_plan_dev[slot], as.off.upload, st));
+        if (sg) KVP_CUDA(ctx, stage_upload(*sg, ctx->slot_plan_dev[slot], as.off.upload, st));
     }
     const int32_t n_chunks = (int32_t)as.chunks.size(), n_rope = (int32_t)as.delta.size();
+    const uint32_t blob_bytes = (uint32_t)as.off.upload;
     std::swap(ctx->slots[slot], ctx->build);
+    if (!ctx->host_only) ctx->slots[slot].id = -1;
     *assembly_id = id;
     if (ctx->host_only) {
         for (int32_t id : to_load) ctx->packet_src[id].resident = true;
@@ -1145,7 +1165,9 @@ static int32_t assemble_impl(kvp_ctx *ctx, int32_t batch, const int32_t *slot_of
             KVP_CUDA(ctx, cudaStreamWaitEvent(st, ctx->load_done[ctx->shape.n_layers - 1], 0));
         KVP_CUDA(ctx, time_edge(ctx, 1, 0, st));
         KVP_CUDA(ctx, kvp_launch_gather(ctx->shape, plan_dev(ctx, slot), n_chunks, n_rope, ctx->half_turns, ctx->pool_k,
-                                        ctx->pool_v, ctx->slot_k[slot], ctx->slot_v[slot], st));
+                                        ctx->pool_v, ctx->slot_k[slot], ctx->slot_v[slot], blob, blob_bytes,
+                                        ctx->slot_plan_dev[slot], st));
+        ctx->slots[slot].id = id;                                 // from here on the device has the plan
         KVP_CUDA(ctx, time_edge(ctx, 1, 1, st));
     }
     return KVP_OK;
@@ -1314,12 +1336,14 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
                                           std::equal(q_lens, q_lens + as.batch, as.sched[li].q_lens.begin()))
                                        : as.sched[li].q_lens.empty();
         a.fresh = 0;
+        a.list = nullptr;
+        a.list_bytes = a.list_works = 0;
+        a.list_dev = nullptr;
         if (as.sched[li].q_len != q_len || as.sched[li].ctas == 0 || !same_lens ||
             (as.sched[li].q_pos0 != q_pos0 && (q_lens || !same_causal_tiles(sh, q_len, as.sched[li].q_pos0, q_pos0))) ||
             as.sched[li].opts != part_opts) {
-            const int32_t rc = build_schedule(ctx, as, slot, layer, q_len, q_pos0, q_lens, part_opts, st);
+            const int32_t rc = build_schedule(ctx, as, slot, layer, q_len, q_pos0, q_lens, part_opts, a, st);
             if (rc != KVP_OK) return rc;
-            a.fresh = 1;
         }
         const kvp_assembly_host::sched_state &ss = as.sched[li];
         const char *sd = ctx->slot_sched_dev[slot] + ctx->sched_bytes * li;
@@ -1343,10 +1367,11 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
         a.status = ctx->status_dev;
         if (ss.ctas > 0) {                                         // (a rank may hold no key of any request)
             KVP_CUDA(ctx, time_edge(ctx, 0, 0, st));
-            if (pairs)
-                KVP_CUDA(ctx, kvp_launch_attn_pair(sh, a, ctx->tm_pool_k_half, ctx->tm_pool_v, ctx->tm_ws_k_half[slot], ctx->tm_ws_v[slot], st));
-            else
-                KVP_CUDA(ctx, kvp_launch_attn_sm100(sh, a, ctx->tm_pool_k, ctx->tm_pool_v, ctx->tm_ws_k[slot], ctx->tm_ws_v[slot], st));
+            const cudaError_t launched =
+                pairs ? kvp_launch_attn_pair(sh, a, ctx->tm_pool_k_half, ctx->tm_pool_v, ctx->tm_ws_k_half[slot], ctx->tm_ws_v[slot], st)
+                      : kvp_launch_attn_sm100(sh, a, ctx->tm_pool_k, ctx->tm_pool_v, ctx->tm_ws_k[slot], ctx->tm_ws_v[slot], st);
+            if (launched != cudaSuccess) as.sched[li].q_len = 0;   // its work list never reached the device
+            KVP_CUDA(ctx, launched);
             KVP_CUDA(ctx, time_edge(ctx, 0, 1, st));
             ++launches;
         }

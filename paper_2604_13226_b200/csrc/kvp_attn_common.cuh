@@ -32,7 +32,9 @@ struct Params {
     // precise: the counter-rotated query is kept as value + rounding remainder (two bf16 tiles per stream, one
     // epoch buffer instead of two) and Q K^T of a rotated tile takes both
     int precise;
-    int fresh;                 // the work list was uploaded by the kernel in front
+    int fresh;                 // the work list was uploaded by the kernel in front, or comes along with this launch
+    uint32_t list_bytes, list_works;           // in the latter case: its size, where the pieces begin, and where it is stored for
+    uint4 *list_dev;                           // the launches behind this one
     // l2_prefetch: the K/V tiles of a unit are read by at most two units of the launch, i.e. they come from DRAM
     // rather than from L2: the TMA warp then asks L2 for each tile a few loads before it fetches it
     int l2_prefetch;
@@ -242,9 +244,9 @@ struct Work {
     int q_len;                 // query tokens of this request (the call's q_len unless the work record carries its own)
 };
 
-__device__ __forceinline__ Work load_work(const Params &p, int wi)
+__device__ __forceinline__ Work load_work(const Params &p, const kvp_work *works, int wi)
 {
-    const int4 *w4 = reinterpret_cast<const int4 *>(p.works + wi);
+    const int4 *w4 = reinterpret_cast<const int4 *>(works + wi);
     const int4 a = w4[0], c = w4[1], e = w4[2];
     Work w;
     w.b = a.x; w.hk = a.y; w.row_base = a.z; w.mode = a.w & 0xff;
@@ -493,6 +495,16 @@ __device__ __forceinline__ void append_rows(const Params &p, const Work &w, int 
     }
 }
 
+// Start of a kernel whose work list comes along with the launch (a list in device memory costs a kernel of its own in front,
+// 4 us on the way to the first tile): CTA 0 stores it for the launches behind, before any of them is released.
+template <int LB>
+__device__ __forceinline__ void store_list(const Params &p, const kvp_blob<LB> &list, int tid, int n_threads)
+{
+    if (blockIdx.x != 0) return;
+    for (uint32_t i = tid; i < p.list_bytes / 16; i += n_threads) p.list_dev[i] = list.w[i];
+    __threadfence();
+}
+
 inline Params make_params(const kvp_shape &sh, const kvp_attn2_args &a)
 {
     Params p;
@@ -518,6 +530,9 @@ inline Params make_params(const kvp_shape &sh, const kvp_attn2_args &a)
     p.tail_direct = a.tail_direct;
     p.precise = a.precise;
     p.fresh = a.fresh;
+    p.list_bytes = a.list_bytes;
+    p.list_works = a.list_works;
+    p.list_dev = (uint4 *)a.list_dev;
     p.l2_prefetch = a.l2_prefetch;
     p.k_new = (const uint4 *)a.k_new;
     p.v_new = (const uint4 *)a.v_new;

@@ -46,6 +46,7 @@ static_assert(8 * kNumBars <= 504, "barrier block");
 struct Cta {
     uint32_t smem_base, bar0, lead0, tmem;                // lead0: CTA 0's barriers, as an address of the cluster's shared memory
     int rank, item_begin, item_end;
+    const kvp_work *works;
     __device__ __forceinline__ uint32_t bar(int i) const { return bar0 + 8u * i; }
     __device__ __forceinline__ uint32_t lead(int i) const { return lead0 + 8u * i; }
     __device__ __forceinline__ uint32_t tmem_slot() const { return bar0 + 504; }
@@ -185,7 +186,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
         int n, lo, n_tail, n_total, limit;
         const kvp_tile *tiles;
         {
-            const Work w = load_work(p, wi);
+            const Work w = load_work(p, c.works, wi);
             n = w.n;
             lo = w.lo;
             n_tail = w.n_tail;
@@ -296,7 +297,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
         const float M = ((n - 1) & 1) == G ? m : o.x;     // O is relative to the last tile's reference
         l = l * ex2((m - M) * c2) + o.y * ex2((o.x - M) * c2);
 
-        const Work w = load_work(p, wi);
+        const Work w = load_work(p, c.works, wi);
         const int r = w.row_base + c.rank * KVP_TILE_ROWS + t;
         const bool valid = r < p.group * w.q_len;
         const int qi = valid ? row_token(p, r) : w.q_len - 1;
@@ -353,7 +354,7 @@ __device__ __forceinline__ void producer_role(const Params &p, const Cta &c, con
     bool ok = true;
     pdl_wait();
     for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
-        const Work w = load_work(p, wi);
+        const Work w = load_work(p, c.works, wi);
         const int n_rows = p.group * w.q_len;
         int prev = 0;
         for (int k = 0; k < w.n && ok; ++k) {
@@ -399,7 +400,7 @@ __device__ __forceinline__ void tma_role(const Params &p, const Cta &c, const in
     uint32_t stage = 0, use = 0;
     bool ok = true;
     for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
-        const Work w = load_work(p, wi);
+        const Work w = load_work(p, c.works, wi);
         const int n_loads = 2 * w.n;
         for (int q0 = 0; q0 < n_loads && ok; q0 += 32) {
             // lane i looks up the tile of load q0 + i and issues it when its turn comes
@@ -468,7 +469,7 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
     auto advance = [&] { if (++stage == n_stages) { stage = 0; par ^= 1; } };
 
     for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
-        const Work w = load_work(p, wi);
+        const Work w = load_work(p, c.works, wi);
         const int n = w.n;
         // tile facts are fetched 32 at a time, one per lane, and handed round by shuffle
         int b0 = 0, nk_l = 0, rope_l = 0;
@@ -580,10 +581,12 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
     }
 }
 
+template <int LB>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 attn_pair_kernel(const __grid_constant__ CUtensorMap k_pool, const __grid_constant__ CUtensorMap v_pool,
                  const __grid_constant__ CUtensorMap k_ws, const __grid_constant__ CUtensorMap v_ws,
-                 const __grid_constant__ CUtensorMap k_new, const __grid_constant__ CUtensorMap v_new, const Params p)
+                 const __grid_constant__ CUtensorMap k_new, const __grid_constant__ CUtensorMap v_new, const Params p,
+                 const __grid_constant__ kvp_blob<LB> list)
 {
     extern __shared__ char smem_raw[];
     Cta c;
@@ -609,17 +612,25 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap k_pool, const __grid_consta
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(c.tmem_slot()) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
-    if (p.fresh) {
+    const int32_t *cta_begin = p.cta_begin;
+    c.works = p.works;
+    if (LB > 0) {
+        pdl_wait();
+        store_list<LB>(p, list, tid, kThreads);
+        cta_begin = reinterpret_cast<const int32_t *>(&list);
+        c.works = reinterpret_cast<const kvp_work *>(reinterpret_cast<const char *>(&list) + p.list_works);
+    } else if (p.fresh) {
         pdl_wait();
         pdl_launch_dependents();
     }
     // from here on: the Q producer, the append and the TMA warp (for anything but pool tiles) wait for the kernel in front;
     // everything else follows from what they deliver
-    c.item_begin = p.cta_begin[blockIdx.x >> 1];              // (the work list gives every pair at least one piece)
-    c.item_end = p.cta_begin[(blockIdx.x >> 1) + 1];
+    c.item_begin = cta_begin[blockIdx.x >> 1];   // (the work list gives every pair at least one piece)
+    c.item_end = cta_begin[(blockIdx.x >> 1) + 1];
     __syncwarp();
     tc_fence_before();
     cluster_sync();                                           // both CTAs' barriers and TMEM are there
+    if (LB > 0) pdl_launch_dependents();
     tc_fence_after();
     c.tmem = ld_shared(c.tmem_slot());
 
@@ -651,13 +662,24 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap k_pool, const __grid_consta
 
 cudaError_t kvp_attn_pair_prepare(void)
 {
-    return cudaFuncSetAttribute(attn_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    const cudaFuncAttribute what = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaError_t rc = cudaFuncSetAttribute(attn_pair_kernel<0>, what, kSmemBytes);
+    if (rc == cudaSuccess) rc = cudaFuncSetAttribute(attn_pair_kernel<KVP_INLINE_SMALL>, what, kSmemBytes);
+    if (rc == cudaSuccess) rc = cudaFuncSetAttribute(attn_pair_kernel<KVP_INLINE_LARGE>, what, kSmemBytes);
+    return rc;
 }
 
 cudaError_t kvp_launch_attn_pair(const kvp_shape &sh, const kvp_attn2_args &a, const CUtensorMap &k_pool, const CUtensorMap &v_pool,
                                  const CUtensorMap &k_ws, const CUtensorMap &v_ws, cudaStream_t st)
 {
     // without tail_direct the two query maps are never dereferenced: any valid map will do
-    return launch_pdl(attn_pair_kernel, 2 * a.n_ctas, kThreads, kSmemBytes, st, k_pool, v_pool, k_ws, v_ws,
-                      a.tail_direct ? a.tm_knew : k_ws, a.tail_direct ? a.tm_vnew : v_ws, make_params(sh, a));
+    const Params p = make_params(sh, a);
+    auto go = [&](auto *kernel, const auto &list) {
+        return launch_pdl(kernel, 2 * a.n_ctas, kThreads, kSmemBytes, st, k_pool, v_pool, k_ws, v_ws, a.tail_direct ? a.tm_knew : k_ws,
+                          a.tail_direct ? a.tm_vnew : v_ws, p, list);
+    };
+    if (!a.list) return go(attn_pair_kernel<0>, kvp_blob<0>());
+    if (a.list_bytes <= KVP_INLINE_SMALL)
+        return go(attn_pair_kernel<KVP_INLINE_SMALL>, *reinterpret_cast<const kvp_blob<KVP_INLINE_SMALL> *>(a.list));
+    return go(attn_pair_kernel<KVP_INLINE_LARGE>, *reinterpret_cast<const kvp_blob<KVP_INLINE_LARGE> *>(a.list));
 }

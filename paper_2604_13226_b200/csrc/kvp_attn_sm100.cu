@@ -112,6 +112,7 @@ __device__ __forceinline__ int load_seq(int mode, int n, int r, int kv)
 struct Cta {
     uint32_t smem_base, bar0, tmem;
     int item_begin, item_end;
+    const kvp_work *works;
     __device__ __forceinline__ uint32_t bar(int i) const { return bar0 + 8u * i; }
     // behind the barriers: TMEM address and abort flag
     __device__ __forceinline__ uint32_t tmem_slot() const { return bar0 + 248; }
@@ -185,7 +186,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
         int steps, first, stride, n_tail, n_total, limit;
         const kvp_tile *tiles;
         {
-            const Work w = load_work(p, wi);
+            const Work w = load_work(p, c.works, wi);
             steps = S == 0 ? w.steps0 : w.steps1;
             first = stream_tile(w, S, 0);
             stride = w.mode ? 2 : 1;
@@ -254,7 +255,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
         if (!ok) break;
 
         // ---- end of the piece: O of this stream is complete once its last P V has landed ----------
-        const Work w = load_work(p, wi);
+        const Work w = load_work(p, c.works, wi);
         const int n_rows = p.group * w.q_len;
         const int r = w.row_base + (w.mode == 0 ? S * KVP_TILE_ROWS : 0) + t;
         const bool valid = r < n_rows;
@@ -352,7 +353,7 @@ __device__ __forceinline__ void producer_role(const Params &p, const Cta &c, con
     bool ok = true;
     pdl_wait();
     for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
-        const Work w = load_work(p, wi);
+        const Work w = load_work(p, c.works, wi);
         const int n_rows = p.group * w.q_len;
         const int max_steps = max(w.steps0, w.steps1);
         int prev0 = 0, prev1 = 0;
@@ -401,7 +402,7 @@ __device__ __forceinline__ void append_role(const Params &p, const Cta &c, const
     if (!p.tail_direct) return;
     pdl_wait();
     for (int wi = c.item_begin; wi < c.item_end; ++wi) {
-        const Work w = load_work(p, wi);
+        const Work w = load_work(p, c.works, wi);
         if (w.lo == 0) append_rows<Cfg<D>::kVecs, 64>(p, w, w.row_base, w.mode ? KVP_TILE_ROWS : 2 * KVP_TILE_ROWS, t);
     }
 }
@@ -418,7 +419,7 @@ __device__ __forceinline__ void tma_role(const Params &p, const Cta &c, const in
     uint32_t ring_n = 0;                                   // loads issued before this piece
     bool ok = true;
     for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
-        const Work w = load_work(p, wi);
+        const Work w = load_work(p, c.works, wi);
         const int n_loads = 2 * w.n;
         for (int q0 = 0; q0 < n_loads && ok; q0 += 32) {
             // lane i looks up the tile of load q0 + i
@@ -674,7 +675,7 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
     };
 
     for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
-        const Work w = load_work(p, wi);
+        const Work w = load_work(p, c.works, wi);
         if (w.mode == 0) {
             piece_mode0(w);
             ring_n += 2u * (uint32_t)w.n;
@@ -740,12 +741,12 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
     }
 }
 
-template <int D>
+template <int D, int LB>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_pool_k, const __grid_constant__ CUtensorMap tm_pool_v,
                   const __grid_constant__ CUtensorMap tm_ws_k, const __grid_constant__ CUtensorMap tm_ws_v,
                   const __grid_constant__ CUtensorMap tm_knew, const __grid_constant__ CUtensorMap tm_vnew,
-                  const Params p)
+                  const Params p, const __grid_constant__ kvp_blob<LB> list)
 {
     using C = Cfg<D>;
     extern __shared__ char smem_raw[];
@@ -782,16 +783,24 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_pool_k, const __grid_co
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    if (p.fresh) {
+    const int32_t *cta_begin = p.cta_begin;
+    c.works = p.works;
+    if (LB > 0) {
+        pdl_wait();
+        store_list<LB>(p, list, tid, kThreads);
+        cta_begin = reinterpret_cast<const int32_t *>(&list);
+        c.works = reinterpret_cast<const kvp_work *>(reinterpret_cast<const char *>(&list) + p.list_works);
+    } else if (p.fresh) {
         pdl_wait();
         pdl_launch_dependents();
     }
     // from here on: the Q producer, the append and the TMA warp (for anything but pool tiles) wait for the kernel in front;
     // everything else follows from what they deliver
-    c.item_begin = p.cta_begin[blockIdx.x];                   // (the work list gives every CTA at least one piece)
-    c.item_end = p.cta_begin[blockIdx.x + 1];
+    c.item_begin = cta_begin[blockIdx.x];   // (the work list gives every CTA at least one piece)
+    c.item_end = cta_begin[(blockIdx.x) + 1];
     tc_fence_before();
     __syncthreads();
+    if (LB > 0) pdl_launch_dependents();
     tc_fence_after();
     c.tmem = ld_shared(c.tmem_slot());
 
@@ -964,12 +973,16 @@ merge_ranks_kernel(const char *__restrict__ parts, int n_parts, long long part_b
 
 }  // namespace
 
-cudaError_t kvp_attn_sm100_prepare(int32_t head_dim)
+template <int D>
+static cudaError_t prepare()
 {
-    if (head_dim == 64)
-        return cudaFuncSetAttribute(attn_sm100_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<64>::kSmemBytes);
-    return cudaFuncSetAttribute(attn_sm100_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<128>::kSmemBytes);
+    const cudaFuncAttribute what = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaError_t rc = cudaFuncSetAttribute(attn_sm100_kernel<D, 0>, what, Cfg<D>::kSmemBytes);
+    if (rc == cudaSuccess) rc = cudaFuncSetAttribute(attn_sm100_kernel<D, KVP_INLINE_SMALL>, what, Cfg<D>::kSmemBytes);
+    if (rc == cudaSuccess) rc = cudaFuncSetAttribute(attn_sm100_kernel<D, KVP_INLINE_LARGE>, what, Cfg<D>::kSmemBytes);
+    return rc;
 }
+cudaError_t kvp_attn_sm100_prepare(int32_t head_dim) { return head_dim == 64 ? prepare<64>() : prepare<128>(); }
 
 cudaError_t kvp_launch_attn_sm100(const kvp_shape &sh, const kvp_attn2_args &a, const CUtensorMap &tm_pool_k,
                                   const CUtensorMap &tm_pool_v, const CUtensorMap &tm_ws_k,
@@ -978,9 +991,19 @@ cudaError_t kvp_launch_attn_sm100(const kvp_shape &sh, const kvp_attn2_args &a, 
     const Params p = make_params(sh, a);
     // without tail_direct the two query maps are never dereferenced: any valid map will do
     const CUtensorMap &tk = a.tail_direct ? a.tm_knew : tm_ws_k, &tv = a.tail_direct ? a.tm_vnew : tm_ws_v;
+    auto go = [&](auto *kernel, int smem, const auto &list) {
+        return launch_pdl(kernel, a.n_ctas, kThreads, smem, st, tm_pool_k, tm_pool_v, tm_ws_k, tm_ws_v, tk, tv, p, list);
+    };
+    const auto *small = reinterpret_cast<const kvp_blob<KVP_INLINE_SMALL> *>(a.list);
+    const auto *large = reinterpret_cast<const kvp_blob<KVP_INLINE_LARGE> *>(a.list);
+    const int size = !a.list ? 0 : a.list_bytes <= KVP_INLINE_SMALL ? 1 : 2;
     if (sh.head_dim == 64)
-        return launch_pdl(attn_sm100_kernel<64>, a.n_ctas, kThreads, Cfg<64>::kSmemBytes, st, tm_pool_k, tm_pool_v, tm_ws_k, tm_ws_v, tk, tv, p);
-    return launch_pdl(attn_sm100_kernel<128>, a.n_ctas, kThreads, Cfg<128>::kSmemBytes, st, tm_pool_k, tm_pool_v, tm_ws_k, tm_ws_v, tk, tv, p);
+        return size == 0   ? go(attn_sm100_kernel<64, 0>, Cfg<64>::kSmemBytes, kvp_blob<0>())
+               : size == 1 ? go(attn_sm100_kernel<64, KVP_INLINE_SMALL>, Cfg<64>::kSmemBytes, *small)
+                           : go(attn_sm100_kernel<64, KVP_INLINE_LARGE>, Cfg<64>::kSmemBytes, *large);
+    return size == 0   ? go(attn_sm100_kernel<128, 0>, Cfg<128>::kSmemBytes, kvp_blob<0>())
+           : size == 1 ? go(attn_sm100_kernel<128, KVP_INLINE_SMALL>, Cfg<128>::kSmemBytes, *small)
+                       : go(attn_sm100_kernel<128, KVP_INLINE_LARGE>, Cfg<128>::kSmemBytes, *large);
 }
 
 cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_merges, const kvp_merge_item *merges,

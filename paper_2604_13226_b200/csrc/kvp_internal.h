@@ -16,6 +16,11 @@
 #define KVP_MAX_SPLIT_UNITS 2048   // partial slots (128 query rows each) in the workspace
 #define KVP_CORE_UNITS 2048        // row tiles the CUDA-core kernel may split
 #define KVP_SCHED_RING 8       // pinned staging buffers for work lists
+// Plans up to the first size and work lists up to the second travel as parameters of the kernel that needs them first.  An
+// upload kernel in front costs 4 us on the way to the first tile; a launch costs 2.1 us with up to 4 KB of parameters,
+// 2.7 with 12 KB, 4.5 with 30 KB.
+#define KVP_INLINE_SMALL 4096
+#define KVP_INLINE_LARGE 16384
 #define KVP_UPLOAD_BLOCKS 16   // blocks of an upload, each with a completion flag of its own
 
 // ---- device-visible plan records (written by the host planner, uploaded once per assembly) -----
@@ -203,6 +208,7 @@ struct kvp_ctx {
     // planning scratch, kept so that a call allocates nothing once the sizes have been seen
     kvp_assembly_host build;
     std::vector<int32_t> rope_hash, kept_row_of;
+    alignas(16) char list_inline[KVP_INLINE_LARGE], plan_inline[KVP_INLINE_SMALL];
     kvp_schedule plan;
     int32_t fused_append = 1;              // plain prefill: the attention kernel reads k_new / v_new itself and appends them
     void *encode_tiled = nullptr;          // cuTensorMapEncodeTiled
@@ -251,8 +257,9 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // that passes through here cannot be used before this point.
 #define PDL_AFTER(p) asm volatile("" : "+l"(p)::"memory")
 
-template <typename... P, typename... A>
-cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args)
+template <typename T> struct as_given { typedef T type; };
+template <typename... P>
+cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, const typename as_given<P>::type &...args)
 {
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -264,8 +271,12 @@ cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
     cfg.stream = st;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    void *ptrs[] = {(void *)&args...};
+    return cudaLaunchKernelExC(&cfg, (const void *)kernel, ptrs);
 }
+
+// Tables that travel as a kernel's own parameters.  N = 0: none.
+template <int N> struct kvp_blob { uint4 w[N ? N / 16 : 1]; };
 #endif
 
 // ---- kernel launchers (kvp_kernels.cu, kvp_attn_sm100.cu) ---------------------------------------
@@ -291,10 +302,11 @@ cudaError_t kvp_launch_load(const kvp_shape &sh, kvp_load_list &list, int32_t la
 // their part.  Returns through *blocks how many there are.
 cudaError_t kvp_launch_upload(const void *host, void *dst, uint64_t bytes, volatile uint32_t *flags, uint32_t seq,
                               int32_t *blocks, cudaStream_t st);
-// the rope table of an assembly and the gather of its chunks, one launch
+// the rope table of an assembly and the gather of its chunks, one launch; blob not null: the plan (blob_bytes) comes along and
+// the launch stores it at blob_dev, where `plan` points
 cudaError_t kvp_launch_gather(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t n_chunks, int32_t n_rope,
                               const double *half_turns, const char *pool_k, const char *pool_v, char *ws_k, char *ws_v,
-                              cudaStream_t st);
+                              const void *blob, uint32_t blob_bytes, char *blob_dev, cudaStream_t st);
 cudaError_t kvp_launch_append(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t batch, int32_t q_len,
                               int32_t q_pos0, const void *q, const void *k_new, const void *v_new, char *ws_k, char *ws_v,
                               int32_t layer, int32_t rope_query, const double *half_turns, void *q_rot,
@@ -341,6 +353,10 @@ struct kvp_attn2_args {
     int32_t tail_direct;
     int32_t precise;               // KVP_PRECISE_QK
     int32_t fresh;                 // the work list was uploaded just before, by a kernel this launch has to wait for
+    // not null: the work list (list_bytes, padded to 16) comes along, works at list_works; the launch stores it at list_dev
+    const void *list;
+    uint32_t list_bytes, list_works;
+    char *list_dev;
     int32_t l2_prefetch;           // the launch has at most two 256-row units per (request, kv head)
     const void *k_new, *v_new;
     char *ws_k, *ws_v;

@@ -220,9 +220,10 @@ __device__ __forceinline__ float2 offset_cos_sin(int32_t offset, double half_tur
 // angles of its chunk's offset itself, so it waits for no table block.  V is a byte copy, K is a byte copy when the
 // offset is 0 and an fp32 rotation otherwise.  Bound by DRAM for a whole cache (materialised), by latency for adapter
 // rows; a thread has the loads of two (row, plane) pairs in flight.
-template <typename T>
+// With LB > 0 the plan comes along as a parameter: it is read from there, and block 0 stores it for everyone behind.
+template <typename T, int LB>
 __global__ void __launch_bounds__(256)
-gather_kernel(kvp_plan_dev plan, int n_table, int n_rope, int groups, const double *__restrict__ half_turns,
+gather_kernel(kvp_plan_dev plan, const __grid_constant__ kvp_blob<LB> blob, int blob_words, uint4 *blob_dev, int n_table, int n_rope, int groups, const double *__restrict__ half_turns,
               float2 *__restrict__ table, const char *__restrict__ pool_k, const char *__restrict__ pool_v,
               char *__restrict__ ws_k, char *__restrict__ ws_v, int64_t pool_rows, int64_t ws_rows, int vecs_per_row,
               int half_dim, int pairing)
@@ -230,6 +231,12 @@ gather_kernel(kvp_plan_dev plan, int n_table, int n_rope, int groups, const doub
     pdl_launch_dependents();
     pdl_wait();
     PDL_AFTER(pool_k); PDL_AFTER(pool_v); PDL_AFTER(plan.chunks); PDL_AFTER(plan.delta);
+    if (LB > 0) {
+        if (blockIdx.x == 0 && (int)threadIdx.x < blob_words) blob_dev[threadIdx.x] = blob.w[threadIdx.x];
+        const char *here = reinterpret_cast<const char *>(&blob);
+        plan.chunks = reinterpret_cast<const kvp_chunk *>(here + (reinterpret_cast<const char *>(plan.chunks) - reinterpret_cast<const char *>(blob_dev)));
+        plan.delta = reinterpret_cast<const int32_t *>(here + (reinterpret_cast<const char *>(plan.delta) - reinterpret_cast<const char *>(blob_dev)));
+    }
     if ((int)blockIdx.x < n_table) {
         const int e = blockIdx.x * 256 + threadIdx.x;
         if (e < n_rope * half_dim) table[e] = offset_cos_sin(plan.delta[e / half_dim], half_turns[e % half_dim]);
@@ -967,8 +974,9 @@ cudaError_t kvp_launch_upload(const void *host, void *dst, uint64_t bytes, volat
 
 cudaError_t kvp_launch_gather(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t n_chunks, int32_t n_rope,
                               const double *half_turns, const char *pool_k, const char *pool_v, char *ws_k, char *ws_v,
-                              cudaStream_t st)
+                              const void *blob, uint32_t blob_bytes, char *blob_dev, cudaStream_t st)
 {
+    static_assert(KVP_INLINE_SMALL <= 256 * 16, "one word per thread of a block");
     const int vecs = sh.head_dim * sh.elem_bytes / 16, half = sh.head_dim / 2;
     const int planes = sh.n_layers * sh.n_kv_heads;
     const int n_table = (n_rope * half + 255) / 256;
@@ -981,11 +989,14 @@ cudaError_t kvp_launch_gather(const kvp_shape &sh, const kvp_plan_dev &plan, int
     groups = groups > most ? most : groups;
     const int grid = n_table + n_chunks * groups;
     float2 *table = const_cast<float2 *>(plan.rope);
+    auto go = [&](auto *kernel, const auto &b) {
+        return launch_pdl(kernel, grid, 256, 0, st, plan, b, (int)((blob_bytes + 15) / 16), (uint4 *)blob_dev, n_table, n_rope, groups,
+                          half_turns, table, pool_k, pool_v, ws_k, ws_v, sh.pool_rows, sh.ws_rows, vecs, half, sh.pairing);
+    };
+    const auto *small = reinterpret_cast<const kvp_blob<KVP_INLINE_SMALL> *>(blob);
     if (sh.dtype == KVP_DTYPE_BF16)
-        return launch_pdl(gather_kernel<__nv_bfloat16>, grid, 256, 0, st, plan, n_table, n_rope, groups, half_turns, table, pool_k,
-                          pool_v, ws_k, ws_v, sh.pool_rows, sh.ws_rows, vecs, half, sh.pairing);
-    return launch_pdl(gather_kernel<float>, grid, 256, 0, st, plan, n_table, n_rope, groups, half_turns, table, pool_k, pool_v, ws_k,
-                      ws_v, sh.pool_rows, sh.ws_rows, vecs, half, sh.pairing);
+        return blob ? go(gather_kernel<__nv_bfloat16, KVP_INLINE_SMALL>, *small) : go(gather_kernel<__nv_bfloat16, 0>, kvp_blob<0>());
+    return blob ? go(gather_kernel<float, KVP_INLINE_SMALL>, *small) : go(gather_kernel<float, 0>, kvp_blob<0>());
 }
 
 cudaError_t kvp_launch_append(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t batch, int32_t q_len,
