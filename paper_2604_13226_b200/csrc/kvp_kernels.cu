@@ -220,7 +220,9 @@ __device__ __forceinline__ float2 offset_cos_sin(int32_t offset, double half_tur
 // angles of its chunk's offset itself, so it waits for no table block.  V is a byte copy, K is a byte copy when the
 // offset is 0 and an fp32 rotation otherwise.  Bound by DRAM for a whole cache (materialised), by latency for adapter
 // rows; a thread has the loads of two (row, plane) pairs in flight.
-// With LB > 0 the plan comes along as a parameter: it is read from there, and block 0 stores it for everyone behind.
+// With LB > 0 the plan comes along as a parameter: it is read from there, and block 0 stores it for everyone behind.  Then
+// nothing that leads up to a block's first stores has to wait for the kernel in front: the angles and the rows of the pool
+// are there by the time it ends.
 template <typename T, int LB>
 __global__ void __launch_bounds__(256)
 gather_kernel(kvp_plan_dev plan, const __grid_constant__ kvp_blob<LB> blob, int blob_words, uint4 *blob_dev, int n_table, int n_rope, int groups, const double *__restrict__ half_turns,
@@ -229,17 +231,23 @@ gather_kernel(kvp_plan_dev plan, const __grid_constant__ kvp_blob<LB> blob, int 
               int half_dim, int pairing)
 {
     pdl_launch_dependents();
-    pdl_wait();
-    PDL_AFTER(pool_k); PDL_AFTER(pool_v); PDL_AFTER(plan.chunks); PDL_AFTER(plan.delta);
     if (LB > 0) {
-        if (blockIdx.x == 0 && (int)threadIdx.x < blob_words) blob_dev[threadIdx.x] = blob.w[threadIdx.x];
-        const char *here = reinterpret_cast<const char *>(&blob);
-        plan.chunks = reinterpret_cast<const kvp_chunk *>(here + (reinterpret_cast<const char *>(plan.chunks) - reinterpret_cast<const char *>(blob_dev)));
-        plan.delta = reinterpret_cast<const int32_t *>(here + (reinterpret_cast<const char *>(plan.delta) - reinterpret_cast<const char *>(blob_dev)));
+        const char *here = reinterpret_cast<const char *>(&blob), *there = reinterpret_cast<const char *>(blob_dev);
+        plan.chunks = reinterpret_cast<const kvp_chunk *>(here + (reinterpret_cast<const char *>(plan.chunks) - there));
+        plan.delta = reinterpret_cast<const int32_t *>(here + (reinterpret_cast<const char *>(plan.delta) - there));
+    } else {
+        pdl_wait();
+        PDL_AFTER(pool_k); PDL_AFTER(pool_v); PDL_AFTER(plan.chunks); PDL_AFTER(plan.delta);
     }
     if ((int)blockIdx.x < n_table) {
         const int e = blockIdx.x * 256 + threadIdx.x;
-        if (e < n_rope * half_dim) table[e] = offset_cos_sin(plan.delta[e / half_dim], half_turns[e % half_dim]);
+        const bool word = LB > 0 && blockIdx.x == 0 && (int)threadIdx.x < blob_words;
+        const uint4 mine = word ? blob.w[threadIdx.x] : uint4();
+        float2 angle = make_float2(0.f, 0.f);
+        if (e < n_rope * half_dim) angle = offset_cos_sin(plan.delta[e / half_dim], half_turns[e % half_dim]);
+        if (LB > 0) pdl_wait();
+        if (word) blob_dev[threadIdx.x] = mine;
+        if (e < n_rope * half_dim) table[e] = angle;
         return;
     }
     __shared__ float2 cs[64];
@@ -274,6 +282,7 @@ gather_kernel(kvp_plan_dev plan, const __grid_constant__ kvp_blob<LB> blob, int 
             va[u] = __ldg(sv);
             vb[u] = __ldg(sv + half_vecs);
         }
+        if (LB > 0 && w0 == (int)threadIdx.x) pdl_wait();
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             if (w0 + 256 * u >= n_items) break;
