@@ -496,14 +496,12 @@ __device__ __forceinline__ void append_rows(const Params &p, const Work &w, int 
 }
 
 // Start of a kernel whose work list comes along with the launch (a list in device memory costs a kernel of its own in front,
-// 4 us on the way to the first tile): the CTAs store it for the launches behind, before any of them is released.  Each takes
-// a few words, since lanes that read different words of a parameter are served one after the other.
+// 4 us on the way to the first tile): CTA 0 stores it for the launches behind, before any of them is released.
 template <int LB>
-__device__ __forceinline__ void store_list(const Params &p, const kvp_blob<LB> &list, uint32_t tid, uint32_t n_threads)
+__device__ __forceinline__ void store_list(const Params &p, const kvp_blob<LB> &list, int tid, int n_threads)
 {
-    const uint32_t words = p.list_bytes / 16, per = (words + gridDim.x - 1) / gridDim.x;
-    const uint32_t end = min(words, (blockIdx.x + 1) * per);
-    for (uint32_t i = blockIdx.x * per + tid; i < end; i += n_threads) p.list_dev[i] = list.w[i];
+    if (blockIdx.x != 0) return;
+    for (uint32_t i = tid; i < p.list_bytes / 16; i += n_threads) p.list_dev[i] = list.w[i];
     __threadfence();
 }
 

@@ -220,13 +220,13 @@ __device__ __forceinline__ float2 offset_cos_sin(int32_t offset, double half_tur
 // angles of its chunk's offset itself, so it waits for no table block.  V is a byte copy, K is a byte copy when the
 // offset is 0 and an fp32 rotation otherwise.  Bound by DRAM for a whole cache (materialised), by latency for adapter
 // rows; a thread has the loads of two (row, plane) pairs in flight.
-// With LB > 0 the plan comes along as a parameter: it is read from there, and the blocks store it for everyone behind.  Then
+// With LB > 0 the plan comes along as a parameter: it is read from there, and block 0 stores it for everyone behind.  Then
 // nothing that leads up to a block's first stores has to wait for the kernel in front: the angles and the rows of the pool
 // are there by the time it ends.
 template <typename T, int LB>
 __global__ void __launch_bounds__(256)
-gather_kernel(kvp_plan_dev plan, const __grid_constant__ kvp_blob<LB> blob, int blob_words, uint4 *blob_dev, int n_table,
-              int n_rope, int groups, const double *__restrict__ half_turns, float2 *__restrict__ table, const char *__restrict__ pool_k, const char *__restrict__ pool_v,
+gather_kernel(kvp_plan_dev plan, const __grid_constant__ kvp_blob<LB> blob, int blob_words, uint4 *blob_dev, int n_table, int n_rope, int groups, const double *__restrict__ half_turns,
+              float2 *__restrict__ table, const char *__restrict__ pool_k, const char *__restrict__ pool_v,
               char *__restrict__ ws_k, char *__restrict__ ws_v, int64_t pool_rows, int64_t ws_rows, int vecs_per_row,
               int half_dim, int pairing)
 {
@@ -239,15 +239,14 @@ gather_kernel(kvp_plan_dev plan, const __grid_constant__ kvp_blob<LB> blob, int 
         pdl_wait();
         PDL_AFTER(pool_k); PDL_AFTER(pool_v); PDL_AFTER(plan.chunks); PDL_AFTER(plan.delta);
     }
-    const int per_block = (blob_words + (int)gridDim.x - 1) / (int)gridDim.x, wi = blockIdx.x * per_block + threadIdx.x;
-    const bool word = LB > 0 && (int)threadIdx.x < per_block && wi < blob_words;
-    const uint4 mine = word ? blob.w[wi] : uint4();
     if ((int)blockIdx.x < n_table) {
         const int e = blockIdx.x * 256 + threadIdx.x;
+        const bool word = LB > 0 && blockIdx.x == 0 && (int)threadIdx.x < blob_words;
+        const uint4 mine = word ? blob.w[threadIdx.x] : uint4();
         float2 angle = make_float2(0.f, 0.f);
         if (e < n_rope * half_dim) angle = offset_cos_sin(plan.delta[e / half_dim], half_turns[e % half_dim]);
         if (LB > 0) pdl_wait();
-        if (word) blob_dev[wi] = mine;
+        if (word) blob_dev[threadIdx.x] = mine;
         if (e < n_rope * half_dim) table[e] = angle;
         return;
     }
@@ -294,10 +293,6 @@ gather_kernel(kvp_plan_dev plan, const __grid_constant__ kvp_blob<LB> blob, int 
             dv[0] = va[u];
             dv[half_vecs] = vb[u];
         }
-    }
-    if (word) {
-        pdl_wait();                              // (of a thread that had no row to move)
-        blob_dev[wi] = mine;
     }
 }
 
