@@ -544,7 +544,7 @@ int32_t build_schedule(kvp_ctx *ctx, kvp_assembly_host &as, int slot, int layer,
         memcpy(h + off_merges, sc.merges.data(), sizeof(kvp_merge_item) * sc.merges.size());
     };
     a.list_dev = ctx->slot_sched_dev[slot] + ctx->sched_bytes * li;
-    if (sc.n_ctas > 0 && used <= KVP_INLINE_LARGE) {               // comes along with the attention launch
+    if (sc.n_ctas > 0 && used <= (as.item_stride ? KVP_INLINE_LARGE : KVP_INLINE_SMALL)) {   // comes along with the attention launch
         pack(ctx->list_inline);
         a.list = ctx->list_inline;
         a.list_bytes = (uint32_t)round_up(used, 16);

@@ -225,8 +225,9 @@ __device__ __forceinline__ float2 offset_cos_sin(int32_t offset, double half_tur
 // are there by the time it ends.
 template <typename T, int LB>
 __global__ void __launch_bounds__(256)
-gather_kernel(kvp_plan_dev plan, const __grid_constant__ kvp_blob<LB> blob, int blob_words, uint4 *blob_dev, int n_table, int n_rope, int groups, const double *__restrict__ half_turns,
-              float2 *__restrict__ table, const char *__restrict__ pool_k, const char *__restrict__ pool_v,
+gather_kernel(kvp_plan_dev plan, const __grid_constant__ kvp_blob<LB> blob, int blob_words, uint4 *blob_dev, int n_table,
+              int n_rope, int groups, const double *__restrict__ half_turns, float2 *__restrict__ table,
+              const char *__restrict__ pool_k, const char *__restrict__ pool_v,
               char *__restrict__ ws_k, char *__restrict__ ws_v, int64_t pool_rows, int64_t ws_rows, int vecs_per_row,
               int half_dim, int pairing)
 {
