@@ -26,11 +26,14 @@ struct ws_layout {
 
 constexpr int kMaxCtas = 256;          // upper bound on persistent CTAs (one per SM)
 
-// Work list of the two-stream attention kernel: [cta_begin][works][merge items], packed.
+constexpr int kMaxJoint = 32;          // requests of a joint unit (a tile names them by a bit each)
+
+// Work list of the two-stream attention kernel: [cta_begin][works][merge items][tiles and offsets of joint units], packed.
 struct sched_layout {
     uint64_t total;
     int32_t max_works, max_merges;
 };
+kvp_plan_layout plan_layout(const kvp_config *c);
 
 sched_layout schedule_layout(const kvp_config *c)
 {
@@ -41,7 +44,10 @@ sched_layout schedule_layout(const kvp_config *c)
     s.max_works = (int32_t)std::min<int64_t>(units + kMaxCtas, 1 << 24);
     s.max_merges = 2 * kMaxCtas + 8 + (int32_t)std::min<int64_t>(units, KVP_MAX_SPLIT_UNITS);   // every unit has one with KVP_PARTIAL
     s.total = round_up(4 * (kMaxCtas + 1) + sizeof(kvp_work) * (uint64_t)s.max_works +
-                           sizeof(kvp_merge_item) * (uint64_t)s.max_merges + 2 * kPlanAlign, 256);
+                           sizeof(kvp_merge_item) * (uint64_t)s.max_merges + 4 * kPlanAlign, 256);
+    if (c->max_batch > 1 && c->head_dim == 128 && c->dtype == KVP_DTYPE_BF16 && c->max_compressed == 0)
+        s.total += round_up(sizeof(kvp_tile) * (uint64_t)plan_layout(c).max_tiles +
+                                4ull * c->max_slots * std::min<int32_t>(c->max_batch, kMaxJoint), 256);
     return s;
 }
 
@@ -272,15 +278,75 @@ bool use_pairs(const kvp_ctx *ctx, const kvp_assembly_host &as, int q_len, const
     return wide >= 6 * narrow;
 }
 
+// The tiles that the requests of an assembly hold between them (kvp_joint).  Returns whether walking them once saves a
+// fifth of the tiles.
+bool make_joint(kvp_assembly_host &as)
+{
+    struct use_t { int32_t row0, b, nth, rope, len; };
+    kvp_joint &jt = as.joint;
+    std::vector<use_t> uses;
+    jt.tiles.clear();
+    jt.ropes.clear();
+    for (int b = 0; b < as.batch; ++b) {
+        const kvp_item &it = as.items[b];
+        for (int i = it.tile_begin; i < it.tile_end; ++i) {       // adapter rows: this request's own
+            if (as.tiles[i].src == 0) continue;
+            jt.tiles.push_back(as.tiles[i]);
+            jt.tiles.back().rope = 0;
+            jt.tiles.back().pad = (int32_t)(1u << b);
+        }
+        for (int i = it.seg_begin; i < it.seg_end; ++i)
+            if (as.segs[i].pad[1] == 1) uses.push_back({as.segs[i].src_row0, b, 0, as.segs[i].rope, as.segs[i].len});
+    }
+    std::stable_sort(uses.begin(), uses.end(), [](const use_t &x, const use_t &y) { return x.row0 != y.row0 ? x.row0 < y.row0 : x.b < y.b; });
+    // a document that a request names twice is two runs
+    for (size_t i = 1; i < uses.size(); ++i)
+        if (uses[i].row0 == uses[i - 1].row0 && uses[i].b == uses[i - 1].b) uses[i].nth = uses[i - 1].nth + 1;
+    std::stable_sort(uses.begin(), uses.end(), [](const use_t &x, const use_t &y) { return x.row0 != y.row0 ? x.row0 < y.row0 : x.nth < y.nth; });
+    for (size_t i = 0; i < uses.size();) {
+        const size_t run0 = jt.ropes.size();
+        uint32_t who = 0;
+        size_t e = i;
+        jt.ropes.resize(run0 + as.batch, 0);
+        for (; e < uses.size() && uses[e].row0 == uses[i].row0 && uses[e].nth == uses[i].nth; ++e) {
+            who |= 1u << uses[e].b;
+            jt.ropes[run0 + uses[e].b] = uses[e].rope;
+        }
+        for (int32_t o = 0; o < uses[i].len; o += KVP_TILE_KEYS)
+            jt.tiles.push_back({uses[i].row0 + o, (int16_t)std::min<int32_t>(KVP_TILE_KEYS, uses[i].len - o), 0,
+                                (int32_t)(run0 / as.batch) + 1, (int32_t)who});
+        i = e;
+    }
+    return jt.tiles.size() * 5 <= as.tiles.size() * 4;
+}
+
+// Whether a call takes joint units: short queries of several requests, whose rows fit one query tile together, over
+// documents that requests share.  Such a call is bound by reading the cache, and the requests of a launch do not meet at
+// the same tiles by themselves (a decode step of 8 requests that draw 10 of 46 documents of 1024 tokens, 8 kv heads: 346 MB
+// read, 194 MB of them distinct).  The saving has to outweigh the merge of more and larger parts: two tiles per CTA.
+bool use_joint(const kvp_ctx *ctx, kvp_assembly_host &as, int q_len)
+{
+    const kvp_shape &sh = ctx->shape;
+    if (as.batch < 2 || as.batch > kMaxJoint || as.item_stride || (as.flags & KVP_MATERIALIZE) || sh.head_dim != 128 ||
+        (int64_t)as.batch * sh.group * q_len > KVP_TILE_ROWS || ctx->cfg.max_compressed > 0 || ctx->force_splits == 1)
+        return false;
+    if (as.joint.state < 0) as.joint.state = make_joint(as) ? 1 : 0;
+    return as.joint.state == 1 &&
+           (int64_t)(as.tiles.size() - as.joint.tiles.size()) * sh.n_kv_heads >= 2 * (int64_t)ctx->sm_count;
+}
+
+constexpr uint32_t kOptJoint = 1u << 31;       // in the options a work list was made with
+
 // q_lens: nullptr, or one query length per request (<= q_len, the stride of the padded tensors); a request's
 // work records and merge items then carry its own length.
 // opts: KVP_PARTIAL - every unit writes partial slots and gets merge items (even with one piece or none);
 // KVP_SKIP_QUERY_BLOCK - a unit's range starts behind the causal tiles of the query's own keys.
+// joint: one unit per kv head, of the rows of all requests (use_joint).
 int32_t plan_schedule(kvp_ctx *ctx, const kvp_assembly_host &as, int layer, int q_len, int q_pos0, const int32_t *q_lens,
-                      uint32_t opts, kvp_schedule &out)
+                      uint32_t opts, bool joint, kvp_schedule &out)
 {
     const kvp_shape &sh = ctx->shape;
-    out.pair = use_pairs(ctx, as, q_len, q_lens);
+    out.pair = !joint && use_pairs(ctx, as, q_len, q_lens);
     const int kPieceCost = out.pair ? kPieceCostPair : kPieceCostOne;
     const bool force_partial = (opts & KVP_PARTIAL) != 0, skip_tail = (opts & KVP_SKIP_QUERY_BLOCK) != 0;
     typedef kvp_schedule::unit unit_t;
@@ -292,7 +358,17 @@ int32_t plan_schedule(kvp_ctx *ctx, const kvp_assembly_host &as, int layer, int 
     // Row blocks outermost: the units of one (request, kv head) - which stream the same K/V - then lie a
     // whole number of CTA shares apart on the line (when their count divides the CTA count), so the CTAs
     // that hold them reach the same key tiles at the same time and all but the first find them in L2.
-    for (int row_base = 0; row_base < max_rows; row_base += 2 * KVP_TILE_ROWS)
+    for (int hk = 0; joint && hk < sh.n_kv_heads; ++hk) {
+        unit_t u = {};
+        u.hk = hk;
+        u.mode = 1;
+        u.n_tail = as.batch * ((q_pos0 + q_len - 1) / KVP_TILE_KEYS + 1);
+        u.n_all = u.n_tail + (int32_t)as.joint.tiles.size();
+        u.slot = -1;
+        units.push_back(u);
+        total += u.n_all + kPieceCost;
+    }
+    for (int row_base = 0; !joint && row_base < max_rows; row_base += 2 * KVP_TILE_ROWS)
         for (int b = 0; b < as.batch; ++b) {
             const int n_rows = sh.group * (q_lens ? q_lens[b] : q_len);
             if (row_base >= n_rows) continue;
@@ -501,7 +577,7 @@ int32_t plan_schedule(kvp_ctx *ctx, const kvp_assembly_host &as, int layer, int 
         if (u.n_pieces <= 1 && !force_partial) continue;
         max_pieces = std::max(max_pieces, u.n_pieces);
         u.slot = n_slots;
-        kvp_merge_item m = {u.b, u.hk, u.row_base, u.slot, u.n_pieces, {u.q_len, 0, 0}};
+        kvp_merge_item m = {u.b, u.hk, u.row_base, u.slot, u.n_pieces, {u.q_len, joint ? as.batch : 0, 0}};
         merges.push_back(m);
         n_slots += u.n_pieces;
         if (u.mode == 0) {
@@ -532,19 +608,26 @@ int32_t build_schedule(kvp_ctx *ctx, kvp_assembly_host &as, int slot, int layer,
                        uint32_t opts, kvp_attn2_args &a, cudaStream_t st)
 {
     kvp_schedule &sc = ctx->plan;
-    const int32_t rc = plan_schedule(ctx, as, layer, q_len, q_pos0, q_lens, opts, sc);
+    const int32_t rc = plan_schedule(ctx, as, layer, q_len, q_pos0, q_lens, opts & ~kOptJoint, (opts & kOptJoint) != 0, sc);
     if (rc != KVP_OK) return rc;
     const uint32_t off_works = (uint32_t)round_up(4 * sc.cta_begin.size(), kPlanAlign);
     const uint32_t off_merges = (uint32_t)round_up(off_works + sizeof(kvp_work) * sc.works.size(), kPlanAlign);
-    const size_t used = off_merges + sizeof(kvp_merge_item) * sc.merges.size();
+    const uint32_t off_joint = (uint32_t)round_up(off_merges + sizeof(kvp_merge_item) * sc.merges.size(), kPlanAlign);
+    const bool joint = (opts & kOptJoint) != 0;
+    const size_t tile_bytes = sizeof(kvp_tile) * as.joint.tiles.size(), rope_bytes = 4 * as.joint.ropes.size();
+    const size_t used = joint ? off_joint + tile_bytes + rope_bytes : off_merges + sizeof(kvp_merge_item) * sc.merges.size();
+    if (used > ctx->sched_bytes) return fail(ctx, KVP_ERR_CAPACITY, "query_prefill: work list overflow (%zu bytes)", used);
     const int li = as.item_stride ? layer : 0;                   // which of the assembly's work lists
     auto pack = [&](char *h) {
         memcpy(h, sc.cta_begin.data(), 4 * sc.cta_begin.size());
         memcpy(h + off_works, sc.works.data(), sizeof(kvp_work) * sc.works.size());
         memcpy(h + off_merges, sc.merges.data(), sizeof(kvp_merge_item) * sc.merges.size());
+        if (!joint) return;
+        memcpy(h + off_joint, as.joint.tiles.data(), tile_bytes);
+        memcpy(h + off_joint + tile_bytes, as.joint.ropes.data(), rope_bytes);
     };
     a.list_dev = ctx->slot_sched_dev[slot] + ctx->sched_bytes * li;
-    if (sc.n_ctas > 0 && used <= (as.item_stride ? KVP_INLINE_LARGE : KVP_INLINE_SMALL)) {   // comes along with the attention launch
+    if (!joint && sc.n_ctas > 0 && used <= (as.item_stride ? KVP_INLINE_LARGE : KVP_INLINE_SMALL)) {   // comes along with the attention launch
         pack(ctx->list_inline);
         a.list = ctx->list_inline;
         a.list_bytes = (uint32_t)round_up(used, 16);
@@ -569,6 +652,7 @@ int32_t build_schedule(kvp_ctx *ctx, kvp_assembly_host &as, int slot, int layer,
     ss.slots = sc.max_pieces;
     ss.off_works = off_works;
     ss.off_merges = off_merges;
+    ss.off_joint = off_joint;
     return KVP_OK;
 }
 
@@ -966,6 +1050,7 @@ static int32_t assemble_impl(kvp_ctx *ctx, int32_t batch, const int32_t *slot_of
     as.delta.assign(1, 0);
     as.appended.clear();
     as.sched.clear();
+    as.joint.state = -1;
     as.ragged = false;
     as.last_q_len = 0;
     as.flags = flags;
@@ -1335,18 +1420,23 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
         const bool same_lens = q_lens ? (as.sched[li].q_lens.size() == (size_t)as.batch &&
                                           std::equal(q_lens, q_lens + as.batch, as.sched[li].q_lens.begin()))
                                        : as.sched[li].q_lens.empty();
+        const bool joint = !pairs && !q_lens && !part_opts && !a.tail_direct && !a.precise && use_joint(ctx, as, q_len);
+        const uint32_t list_opts = part_opts | (joint ? kOptJoint : 0);
         a.fresh = 0;
         a.list = nullptr;
         a.list_bytes = a.list_works = 0;
         a.list_dev = nullptr;
         if (as.sched[li].q_len != q_len || as.sched[li].ctas == 0 || !same_lens ||
             (as.sched[li].q_pos0 != q_pos0 && (q_lens || !same_causal_tiles(sh, q_len, as.sched[li].q_pos0, q_pos0))) ||
-            as.sched[li].opts != part_opts) {
-            const int32_t rc = build_schedule(ctx, as, slot, layer, q_len, q_pos0, q_lens, part_opts, a, st);
+            as.sched[li].opts != list_opts) {
+            const int32_t rc = build_schedule(ctx, as, slot, layer, q_len, q_pos0, q_lens, list_opts, a, st);
             if (rc != KVP_OK) return rc;
         }
         const kvp_assembly_host::sched_state &ss = as.sched[li];
         const char *sd = ctx->slot_sched_dev[slot] + ctx->sched_bytes * li;
+        a.joint_batch = joint ? as.batch : 0;
+        a.joint_tiles = joint ? reinterpret_cast<const kvp_tile *>(sd + ss.off_joint) : nullptr;
+        a.joint_ropes = joint ? reinterpret_cast<const int32_t *>(a.joint_tiles + as.joint.tiles.size()) : nullptr;
         a.k_new = k_new;
         a.v_new = v_new;
         a.ws_k = ctx->slot_k[slot];
@@ -1495,7 +1585,7 @@ int32_t kvp_export_schedule(kvp_ctx *ctx, int32_t assembly_id, int32_t q_len, in
     if (slot < 0) return fail(ctx, KVP_ERR_NOT_FOUND, "export_schedule: unknown assembly %d", assembly_id);
     if (q_len <= 0 || q_len > ctx->cfg.max_query_tokens) return fail(ctx, KVP_ERR_INVALID, "export_schedule: bad q_len");
     kvp_schedule &sc = ctx->plan;
-    const int32_t rc = plan_schedule(ctx, ctx->slots[slot], 0, q_len, 0, nullptr, 0, sc);
+    const int32_t rc = plan_schedule(ctx, ctx->slots[slot], 0, q_len, 0, nullptr, 0, false, sc);
     if (rc != KVP_OK) return rc;
     counts[0] = sc.n_ctas;
     counts[1] = (int32_t)sc.works.size();

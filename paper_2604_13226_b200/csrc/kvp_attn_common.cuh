@@ -35,6 +35,9 @@ struct Params {
     int fresh;                 // the work list was uploaded by the kernel in front, or comes along with this launch
     uint32_t list_bytes, list_works;           // in the latter case: its size, where the pieces begin, and where it is stored for
     uint4 *list_dev;                           // the launches behind this one
+    int joint_batch;           // joint units (kvp_joint): their requests, tiles and offsets
+    const kvp_tile *joint_tiles;
+    const int32_t *joint_ropes;
     // l2_prefetch: the K/V tiles of a unit are read by at most two units of the launch, i.e. they come from DRAM
     // rather than from L2: the TMA warp then asks L2 for each tile a few loads before it fetches it
     int l2_prefetch;
@@ -242,8 +245,10 @@ struct Work {
     int n_tail, tile_begin, tail_row0, plane;
     int steps0, steps1;
     int q_len;                 // query tokens of this request (the call's q_len unless the work record carries its own)
+    int per;                   // joint units: causal tiles of each request
 };
 
+template <bool JOINT = false>
 __device__ __forceinline__ Work load_work(const Params &p, const kvp_work *works, int wi)
 {
     const int4 *w4 = reinterpret_cast<const int4 *>(works + wi);
@@ -254,9 +259,14 @@ __device__ __forceinline__ Work load_work(const Params &p, const kvp_work *works
     w.lo = c.x; w.n = c.y; w.slot0 = c.z; w.slot1 = c.w;
     w.tile_begin = e.x;                                       // the plan item's entries, carried in the work record
     w.tail_row0 = e.y;
-    const int n_rows = p.group * w.q_len;
-    const int last = min(n_rows - 1, w.row_base + (w.mode ? KVP_TILE_ROWS : 2 * KVP_TILE_ROWS) - 1);
-    w.n_tail = (p.q_pos0 + last / p.group) / KVP_TILE_KEYS + 1;
+    if (JOINT) {
+        w.per = (p.q_pos0 + p.q_len - 1) / KVP_TILE_KEYS + 1;
+        w.n_tail = p.joint_batch * w.per;
+    } else {
+        const int n_rows = p.group * w.q_len;
+        const int last = min(n_rows - 1, w.row_base + (w.mode ? KVP_TILE_ROWS : 2 * KVP_TILE_ROWS) - 1);
+        w.n_tail = (p.q_pos0 + last / p.group) / KVP_TILE_KEYS + 1;
+    }
     w.plane = p.layer * p.n_kv + w.hk;
     w.steps0 = w.mode ? (w.n + 1) >> 1 : w.n;
     w.steps1 = w.mode ? w.n >> 1 : w.n;
@@ -264,26 +274,32 @@ __device__ __forceinline__ Work load_work(const Params &p, const kvp_work *works
 }
 
 struct Tile {
-    int row0, n_keys, src, rope, qoff;
+    int row0, n_keys, src, rope;
 };
 
-// tile j of the unit's numbering
+// tile j of the unit's numbering.  Joint units: the causal tiles of request 0, 1, ..., then the joint prefix tiles, whose
+// `rope` is the number of a document run - what makes a new Q tile, as the offset does elsewhere.
+template <bool JOINT = false>
 __device__ __forceinline__ Tile get_tile(const Params &p, const Work &w, int j)
 {
     Tile t;
-    if (j < w.n_tail) {
+    if (JOINT && j < w.n_tail) {
+        const int b = j / w.per, at = (j - b * w.per) * KVP_TILE_KEYS;
+        t.row0 = p.plan.items[b].tail_row0 + at;
+        t.n_keys = min(KVP_TILE_KEYS, p.q_pos0 + p.q_len - at);
+        t.src = 1;
+        t.rope = 0;
+    } else if (j < w.n_tail) {
         t.row0 = p.tail_direct ? j * KVP_TILE_KEYS : w.tail_row0 + j * KVP_TILE_KEYS;
         t.n_keys = min(KVP_TILE_KEYS, p.q_pos0 + w.q_len - j * KVP_TILE_KEYS);
         t.src = p.tail_direct ? 2 : 1;               // 2: rows of the caller's k_new / v_new, by query token
         t.rope = 0;
-        t.qoff = j * KVP_TILE_KEYS;
     } else {
-        const int4 g = *reinterpret_cast<const int4 *>(p.plan.tiles + w.tile_begin + (j - w.n_tail));
+        const int4 g = *reinterpret_cast<const int4 *>((JOINT ? p.joint_tiles : p.plan.tiles + w.tile_begin) + (j - w.n_tail));
         t.row0 = g.x;
         t.n_keys = g.y & 0xFFFF;
         t.src = g.y >> 16;
         t.rope = g.z;
-        t.qoff = -1;
     }
     return t;
 }
@@ -318,6 +334,43 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
     uint64_t d;
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
+}
+
+__device__ __forceinline__ float bf16_lo(uint32_t u) { return __uint_as_float(u << 16); }
+__device__ __forceinline__ float bf16_hi(uint32_t u) { return __uint_as_float(u & 0xffff0000u); }
+
+// R(-Delta) on two partner chunks of a row (four words of bf16 pairs each); put(word, remainder word, x, y) takes the results.
+template <typename Put>
+__device__ __forceinline__ void rotate_chunks(int pairing, uint32_t *a, uint32_t *b, uint32_t *ar, uint32_t *br, const float4 *w4,
+                                              const Put &put)
+{
+                if (pairing == 0) {
+                    // pairs (i, i + D/2): word j of chunk c holds elements 8c+2j, 8c+2j+1; partners in chunk c + kCh
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float4 w = w4[j];                      // cos, sin of pair 8c+2j; cos, sin of pair 8c+2j+1
+                        const uint64_t va = pair(bf16_lo(a[j]), bf16_hi(a[j])), vb = pair(bf16_lo(b[j]), bf16_hi(b[j]));
+                        const uint64_t cc = pair(w.x, w.z), ss = pair(w.y, w.w), ns = pair(-w.y, -w.w);
+                        float x, y;
+                        unpair(fma2(vb, ss, mul2(va, cc)), x, y);    // R(-Delta): cos same, sin negated
+                        put(a[j], ar[j], x, y);
+                        unpair(fma2(va, ns, mul2(vb, cc)), x, y);
+                        put(b[j], br[j], x, y);
+                    }
+                } else {
+                    // pairs (2i, 2i+1): one word each; chunk c holds pairs 4c..4c+3 (w4[0], w4[1]), its partner w4[2], w4[3]
+#pragma unroll
+                    for (int j = 0; j < 4; j += 2) {
+                        float4 w = w4[j >> 1];
+                        float x0 = bf16_lo(a[j]), y0 = bf16_hi(a[j]), x1 = bf16_lo(a[j + 1]), y1 = bf16_hi(a[j + 1]);
+                        put(a[j], ar[j], x0 * w.x + y0 * w.y, y0 * w.x - x0 * w.y);
+                        put(a[j + 1], ar[j + 1], x1 * w.z + y1 * w.w, y1 * w.z - x1 * w.w);
+                        w = w4[2 + (j >> 1)];
+                        x0 = bf16_lo(b[j]); y0 = bf16_hi(b[j]); x1 = bf16_lo(b[j + 1]); y1 = bf16_hi(b[j + 1]);
+                        put(b[j], br[j], x0 * w.x + y0 * w.y, y0 * w.x - x0 * w.y);
+                        put(b[j + 1], br[j + 1], x1 * w.z + y1 * w.w, y1 * w.z - x1 * w.w);
+                    }
+                }
 }
 
 // The Q producer (128 threads) writes one 128-row query tile, counter-rotated by the offset of rope-table row
@@ -361,14 +414,12 @@ __device__ __forceinline__ void produce_q_tile(const Params &p, char *qbuf, char
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
     if (rope == 0) return;
-    auto lo_f = [](uint32_t u) { return __uint_as_float(u << 16); };
-    auto hi_f = [](uint32_t u) { return __uint_as_float(u & 0xffff0000u); };
     // word = bf16 pair of (x, y); rem = bf16 pair of what the rounding of the word dropped
     auto rotate = [&](auto rem_c) {
         constexpr bool kRem = decltype(rem_c)::value;
         auto put = [&](uint32_t &word, uint32_t &rem, float x, float y) {
             word = pack_bf16(x, y);
-            if (kRem) rem = pack_bf16(x - lo_f(word), y - hi_f(word));
+            if (kRem) rem = pack_bf16(x - bf16_lo(word), y - bf16_hi(word));
         };
 #pragma unroll 2
         for (int i = 0; i < kCh; ++i) {
@@ -380,33 +431,7 @@ __device__ __forceinline__ void produce_q_tile(const Params &p, char *qbuf, char
             uint4 ra, rb;                                        // remainders
             uint32_t *ar = reinterpret_cast<uint32_t *>(&ra);
             uint32_t *br = reinterpret_cast<uint32_t *>(&rb);
-            if (p.pairing == 0) {
-                // pairs (i, i + D/2): word j of chunk c holds elements 8c+2j, 8c+2j+1; partners in chunk c + kCh
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float4 w = w4[j];                      // cos, sin of pair 8c+2j; cos, sin of pair 8c+2j+1
-                    const uint64_t va = pair(lo_f(a[j]), hi_f(a[j])), vb = pair(lo_f(b[j]), hi_f(b[j]));
-                    const uint64_t cc = pair(w.x, w.z), ss = pair(w.y, w.w), ns = pair(-w.y, -w.w);
-                    float x, y;
-                    unpair(fma2(vb, ss, mul2(va, cc)), x, y);    // R(-Delta): cos same, sin negated
-                    put(a[j], ar[j], x, y);
-                    unpair(fma2(va, ns, mul2(vb, cc)), x, y);
-                    put(b[j], br[j], x, y);
-                }
-            } else {
-                // pairs (2i, 2i+1): one word each; chunk c holds pairs 4c..4c+3 (w4[0], w4[1]), its partner w4[2], w4[3]
-#pragma unroll
-                for (int j = 0; j < 4; j += 2) {
-                    float4 w = w4[j >> 1];
-                    float x0 = lo_f(a[j]), y0 = hi_f(a[j]), x1 = lo_f(a[j + 1]), y1 = hi_f(a[j + 1]);
-                    put(a[j], ar[j], x0 * w.x + y0 * w.y, y0 * w.x - x0 * w.y);
-                    put(a[j + 1], ar[j + 1], x1 * w.z + y1 * w.w, y1 * w.z - x1 * w.w);
-                    w = w4[2 + (j >> 1)];
-                    x0 = lo_f(b[j]); y0 = hi_f(b[j]); x1 = lo_f(b[j + 1]); y1 = hi_f(b[j + 1]);
-                    put(b[j], br[j], x0 * w.x + y0 * w.y, y0 * w.x - x0 * w.y);
-                    put(b[j + 1], br[j + 1], x1 * w.z + y1 * w.w, y1 * w.z - x1 * w.w);
-                }
-            }
+            rotate_chunks(p.pairing, a, b, ar, br, w4, put);
             *reinterpret_cast<uint4 *>(lo) = qa;
             *reinterpret_cast<uint4 *>(lo + hi_off) = qb;
             if (kRem) {
@@ -418,6 +443,43 @@ __device__ __forceinline__ void produce_q_tile(const Params &p, char *qbuf, char
     };
     if (qrem != nullptr) rotate(std::integral_constant<bool, true>{});
     else rotate(std::integral_constant<bool, false>{});
+}
+
+// The same for a joint unit: row r belongs to request r / (group * q_len) and takes that request's offset of document run
+// `run` (0, or a run that the request does not hold: as it is - such rows are masked).
+template <int D>
+__device__ __forceinline__ void produce_q_joint(const Params &p, char *qbuf, int t, int hk, int run)
+{
+    constexpr int kCh = D / 16, kRows = 128 / kCh;
+    const int c = t & (kCh - 1), r0 = t / kCh, per = p.group * p.q_len, n_rows = p.joint_batch * per;
+    const int at = r0 * 128 + ((c ^ (r0 & 7)) << 4);
+    const int hi_off = D == 128 ? kHalfBytes : (at ^ 64) - at;
+    auto put = [](uint32_t &word, uint32_t &, float x, float y) { word = pack_bf16(x, y); };
+#pragma unroll 2
+    for (int i = 0; i < kCh; ++i) {
+        const int r = r0 + kRows * i;
+        uint4 qa = make_uint4(0, 0, 0, 0), qb = qa;
+        if (r < n_rows) {
+            const int b = r / per, rr = r - b * per, tok = row_token(p, rr);
+            const int rope = run == 0 ? 0 : p.joint_ropes[(run - 1) * p.joint_batch + b];
+            const uint4 *src = reinterpret_cast<const uint4 *>(p.q) +
+                               (((long long)b * p.q_len + tok) * p.n_q + hk * p.group + rr - tok * p.group) * (D / 8);
+            qa = src[c];
+            qb = src[c + kCh];
+            if (rope > 0) {
+                const float4 *cs = reinterpret_cast<const float4 *>(p.plan.rope + (size_t)rope * (D / 2));
+                float4 w4[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    w4[j] = *(p.pairing == 0 ? cs + c * 4 + j : cs + (c + kCh * (j >> 1)) * 2 + (j & 1));
+                uint32_t *a = reinterpret_cast<uint32_t *>(&qa), *bb = reinterpret_cast<uint32_t *>(&qb);
+                rotate_chunks(p.pairing, a, bb, a, bb, w4, put);
+            }
+        }
+        char *lo = qbuf + at + i * (kRows * 128);
+        *reinterpret_cast<uint4 *>(lo) = qa;
+        *reinterpret_cast<uint4 *>(lo + hi_off) = qb;
+    }
 }
 
 // ---- softmax of a chunk: one thread per query row, 32 scores in registers ----------------------------------
@@ -533,6 +595,9 @@ inline Params make_params(const kvp_shape &sh, const kvp_attn2_args &a)
     p.list_bytes = a.list_bytes;
     p.list_works = a.list_works;
     p.list_dev = (uint4 *)a.list_dev;
+    p.joint_batch = a.joint_batch;
+    p.joint_tiles = a.joint_tiles;
+    p.joint_ropes = a.joint_ropes;
     p.l2_prefetch = a.l2_prefetch;
     p.k_new = (const uint4 *)a.k_new;
     p.v_new = (const uint4 *)a.v_new;

@@ -170,7 +170,7 @@ __device__ __forceinline__ void rescale_row(uint32_t s_addr, uint32_t o_addr, fl
     tc_wait_st();
 }
 
-template <int D>
+template <int D, bool JOINT>
 __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, const int S, const int t)
 {
     using C = Cfg<D>;
@@ -185,8 +185,9 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
         // what the loop needs of the piece; the rest is read again at its end (registers are short here)
         int steps, first, stride, n_tail, n_total, limit;
         const kvp_tile *tiles;
+        int row_b = 0, n_per = 1;                               // joint units: the row's request; causal tiles of each
         {
-            const Work w = load_work(p, c.works, wi);
+            const Work w = load_work<JOINT>(p, c.works, wi);
             steps = S == 0 ? w.steps0 : w.steps1;
             first = stream_tile(w, S, 0);
             stride = w.mode ? 2 : 1;
@@ -194,18 +195,32 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
             tiles = p.plan.tiles + w.tile_begin - n_tail;
             n_total = p.q_pos0 + w.q_len;
             const int r = w.row_base + (w.mode == 0 ? S * KVP_TILE_ROWS : 0) + t;
-            limit = p.q_pos0 + (r < p.group * w.q_len ? row_token(p, r) : w.q_len - 1) + 1;     // causal keys this row sees
+            if (JOINT) {
+                tiles = p.joint_tiles - n_tail;
+                n_per = w.per;
+                row_b = t / (p.group * p.q_len);
+                limit = p.q_pos0 + row_token(p, t - row_b * (p.group * p.q_len)) + 1;
+            } else {
+                limit = p.q_pos0 + (r < p.group * w.q_len ? row_token(p, r) : w.q_len - 1) + 1;     // causal keys this row sees
+            }
         }
         if (steps == 0) continue;
 
         float m_ref = -1e30f, l = 0.f;
-        auto keys_of = [&](int j) {                             // keys of tile j
+        // keys of tile j; joint units: with bit 8 set where the row's request holds the tile
+        auto keys_of = [&](int j) {
+            if (JOINT) {
+                if (j < n_tail) return min(KVP_TILE_KEYS, n_total - j % n_per * KVP_TILE_KEYS) | (j / n_per == row_b ? 256 : 0);
+                const int4 g = *reinterpret_cast<const int4 *>(tiles + j);
+                return (g.y & 0xffff) | (row_b < 32 && ((uint32_t)g.w >> row_b & 1u) ? 256 : 0);
+            }
             return j < n_tail ? min(KVP_TILE_KEYS, n_total - j * KVP_TILE_KEYS) : (int)tiles[j].n_keys;
         };
         int nk_next = keys_of(first);
 #pragma unroll 1
         for (int k = 0; k < steps; ++k) {
-            const int j = first + k * stride, n_keys = nk_next;
+            const int j = first + k * stride, n_keys = JOINT ? nk_next & 255 : nk_next;
+            const bool mine = !JOINT || (nk_next & 256) != 0;
             if (k + 1 < steps) nk_next = keys_of(j + stride);
             ok = mbar_wait(c.bar(C::kSFull + S), ph & 1, c.abort_flag(), p.status, 30 + S);
             ph ^= 1;
@@ -213,15 +228,16 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
             if (!ok) break;
             tc_fence_after();
 
-            const bool full = n_keys == KVP_TILE_KEYS && j >= n_tail;
-            const int lim = j >= n_tail ? n_keys : min(n_keys, limit - j * KVP_TILE_KEYS);       // visible keys: [0, lim)
+            const bool full = !JOINT && n_keys == KVP_TILE_KEYS && j >= n_tail;
+            int lim = j >= n_tail ? n_keys : min(n_keys, limit - (JOINT ? j % n_per : j) * KVP_TILE_KEYS);     // visible keys: [0, lim)
+            if (JOINT && !mine) lim = 0;
 
             // One pass over S, 32 columns at a time: the exponentials use the reference max carried over from earlier tiles;
             // a chunk's own max is reduced alongside and checked last, so that the two dependency chains overlap.  Only if it
             // exceeds the reference by more than 2^8 (first tile of a piece, or a rare jump) are l, O and the P chunks
             // already written rescaled.
             // a short tile (the end of a document, staged adapter rows) needs P only for the columns P V will read
-            const int n_ch = full ? 4 : max(1, (n_keys + 31) >> 5);
+            const int n_ch = full ? 4 : max(1, (n_keys + 31) >> 5);         // (a row that does not see the tile writes P = 0)
 #pragma unroll 1
             for (int ch = 0; ch < n_ch; ++ch) {
                 uint32_t v[32], pk[C::kSplit ? 32 : 16];
@@ -255,11 +271,11 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
         if (!ok) break;
 
         // ---- end of the piece: O of this stream is complete once its last P V has landed ----------
-        const Work w = load_work(p, c.works, wi);
-        const int n_rows = p.group * w.q_len;
-        const int r = w.row_base + (w.mode == 0 ? S * KVP_TILE_ROWS : 0) + t;
-        const bool valid = r < n_rows;
-        const int qi = valid ? row_token(p, r) : w.q_len - 1;
+        const Work w = load_work<JOINT>(p, c.works, wi);
+        const int n_rows = p.group * w.q_len, req = JOINT ? t / n_rows : 0;
+        const int r = JOINT ? t - req * n_rows : w.row_base + (w.mode == 0 ? S * KVP_TILE_ROWS : 0) + t;
+        const bool valid = JOINT ? req < p.joint_batch : r < n_rows;
+        const int qi = valid ? row_token(p, r) : w.q_len - 1, b = JOINT ? req : w.b;
         const int h = w.hk * p.group + (valid ? r - qi * p.group : 0);
         float2 *ml_smem = reinterpret_cast<float2 *>(c.smem() + C::kOffMl);
         ok = mbar_wait(c.bar(C::kOFull + S), (ph >> 1) & 1, c.abort_flag(), p.status, 32 + S);
@@ -296,7 +312,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
             w1 *= inv;
         }
         // un-normalised (partial slot) or normalised (output rows) O = w0 O_s (+ w1 O_1)
-        uint4 *orow_bf = (direct && valid) ? reinterpret_cast<uint4 *>(p.out + (((long long)w.b * p.q_len + qi) * p.n_q + h) * D) : nullptr;
+        uint4 *orow_bf = (direct && valid) ? reinterpret_cast<uint4 *>(p.out + (((long long)b * p.q_len + qi) * p.n_q + h) * D) : nullptr;
         // partial slot layout: [D / 4 float4 columns][128 rows], so that a warp's store covers 512 contiguous bytes
         uint4 *orow_f = direct || !valid ? nullptr : reinterpret_cast<uint4 *>(p.partial_o) + (long long)slot * (C::kCols4 * KVP_TILE_ROWS) + t;
 #pragma unroll 1
@@ -333,7 +349,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
         }
         if (direct) {
             if (valid && p.lse != nullptr)
-                p.lse[((long long)w.b * p.n_q + h) * p.q_len + qi] = m_ref * p.scale + logf(l);
+                p.lse[((long long)b * p.n_q + h) * p.q_len + qi] = m_ref * p.scale + logf(l);
         } else if (valid) {
             p.partial_ml[(long long)slot * KVP_TILE_ROWS + t] = make_float2(m_ref, l);
         }
@@ -344,7 +360,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
 }
 
 // ---- Q producer -----------------------------------------------------------------------------------------
-template <int D>
+template <int D, bool JOINT>
 __device__ __forceinline__ void producer_role(const Params &p, const Cta &c, const int t)
 {
     using C = Cfg<D>;
@@ -353,7 +369,7 @@ __device__ __forceinline__ void producer_role(const Params &p, const Cta &c, con
     bool ok = true;
     pdl_wait();
     for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
-        const Work w = load_work(p, c.works, wi);
+        const Work w = load_work<JOINT>(p, c.works, wi);
         const int n_rows = p.group * w.q_len;
         const int max_steps = max(w.steps0, w.steps1);
         int prev0 = 0, prev1 = 0;
@@ -370,7 +386,8 @@ __device__ __forceinline__ void producer_role(const Params &p, const Cta &c, con
             }
             char *qb = c.smem() + C::kOffQ + (2 * s + buf) * kQBufBytes;
             char *qrem = C::kSplit ? qb + kHalfBytes : one_buffer ? qb + kQBufBytes : nullptr;
-            produce_q_tile<D>(p, qb, qrem, t, p.q + (long long)w.b * p.q_len * p.n_q * D,
+            if (JOINT) produce_q_joint<D>(p, qb, t, w.hk, rope);
+            else produce_q_tile<D>(p, qb, qrem, t, p.q + (long long)w.b * p.q_len * p.n_q * D,
                            w.hk, w.row_base + (w.mode == 0 ? s * KVP_TILE_ROWS : 0), n_rows, rope);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             mbar_arrive(c.bar(C::kQFull + 2 * s + buf));
@@ -378,12 +395,12 @@ __device__ __forceinline__ void producer_role(const Params &p, const Cta &c, con
         };
         for (int k = 0; k < max_steps && ok; ++k) {
             if (k < w.steps0) {
-                const int rope = get_tile(p, w, stream_tile(w, 0, k)).rope;
+                const int rope = get_tile<JOINT>(p, w, stream_tile(w, 0, k)).rope;
                 if (k == 0 || rope != prev0) produce(0, rope, nEp0);
                 prev0 = rope;
             }
             if (ok && k < w.steps1) {
-                const int rope = get_tile(p, w, stream_tile(w, 1, k)).rope;
+                const int rope = get_tile<JOINT>(p, w, stream_tile(w, 1, k)).rope;
                 if (k == 0 || rope != prev1) produce(1, rope, nEp1);
                 prev1 = rope;
             }
@@ -408,7 +425,7 @@ __device__ __forceinline__ void append_role(const Params &p, const Cta &c, const
 }
 
 // ---- TMA producer (whole warp; lane 0 issues) ----------------------------------------------------------
-template <int D>
+template <int D, bool JOINT>
 __device__ __forceinline__ void tma_role(const Params &p, const Cta &c, const int lane, const CUtensorMap *tm_pool_k,
                                          const CUtensorMap *tm_pool_v, const CUtensorMap *tm_ws_k,
                                          const CUtensorMap *tm_ws_v, const CUtensorMap *tm_knew,
@@ -419,7 +436,7 @@ __device__ __forceinline__ void tma_role(const Params &p, const Cta &c, const in
     uint32_t ring_n = 0;                                   // loads issued before this piece
     bool ok = true;
     for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
-        const Work w = load_work(p, c.works, wi);
+        const Work w = load_work<JOINT>(p, c.works, wi);
         const int n_loads = 2 * w.n;
         for (int q0 = 0; q0 < n_loads && ok; q0 += 32) {
             // lane i looks up the tile of load q0 + i
@@ -432,7 +449,7 @@ __device__ __forceinline__ void tma_role(const Params &p, const Cta &c, const in
             else { r = (q - 2) >> 1; kv = 1; }
             int row0 = 0, src = 0;
             if (q < n_loads) {
-                const Tile tl = get_tile(p, w, w.lo + r);
+                const Tile tl = get_tile<JOINT>(p, w, w.lo + r);
                 row0 = tl.row0;
                 src = tl.src;
             }
@@ -479,7 +496,7 @@ struct MmaStream {
     Tile cur, nxt;
 };
 
-template <int D>
+template <int D, bool JOINT>
 __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
 {
     using C = Cfg<D>;
@@ -506,8 +523,8 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
         const bool shared_stage = (wq.mode == 0);                 // mode 0: both streams read the same K/V stage
         if (k == 0) {
             ms.prev_rope = 0;
-            ms.cur = get_tile(p, wq, stream_tile(wq, s, 0));
-            ms.nxt = n_steps > 1 ? get_tile(p, wq, stream_tile(wq, s, 1)) : ms.cur;
+            ms.cur = get_tile<JOINT>(p, wq, stream_tile(wq, s, 0));
+            ms.nxt = n_steps > 1 ? get_tile<JOINT>(p, wq, stream_tile(wq, s, 1)) : ms.cur;
         }
         const Tile tl = ms.cur;
         if (k == 0 || tl.rope != ms.prev_rope) {                  // first tile of a document: its own Q buffer
@@ -552,7 +569,7 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
         ms.prev_rope = tl.rope;
         ms.prev_keys = tl.n_keys;
         ms.cur = ms.nxt;
-        if (k + 2 < n_steps) ms.nxt = get_tile(p, wq, stream_tile(wq, s, k + 2));
+        if (k + 2 < n_steps) ms.nxt = get_tile<JOINT>(p, wq, stream_tile(wq, s, k + 2));
     };
 
     // ---- a piece in mode 0: both streams take every tile; loads arrive K(0) V(0) K(1) V(1) ... -----------------
@@ -573,7 +590,7 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
         auto refill = [&](int from) {
             b0 = from;
             if (from + lane < n) {
-                const Tile t = get_tile(p, w, w.lo + from + lane);
+                const Tile t = get_tile<JOINT>(p, w, w.lo + from + lane);
                 nk_l = t.n_keys;
                 rope_l = t.rope;
             }
@@ -675,8 +692,8 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
     };
 
     for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
-        const Work w = load_work(p, c.works, wi);
-        if (w.mode == 0) {
+        const Work w = load_work<JOINT>(p, c.works, wi);
+        if (!JOINT && w.mode == 0) {
             piece_mode0(w);
             ring_n += 2u * (uint32_t)w.n;
             continue;
@@ -741,7 +758,7 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
     }
 }
 
-template <int D, int LB>
+template <int D, int LB, bool JOINT>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_pool_k, const __grid_constant__ CUtensorMap tm_pool_v,
                   const __grid_constant__ CUtensorMap tm_ws_k, const __grid_constant__ CUtensorMap tm_ws_v,
@@ -805,14 +822,14 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_pool_k, const __grid_co
     c.tmem = ld_shared(c.tmem_slot());
 
     if (warp < 8) {
-        softmax_role<D>(p, c, warp >> 2, tid & 127);
+        softmax_role<D, JOINT>(p, c, warp >> 2, tid & 127);
     } else if (warp < 12) {
-        producer_role<D>(p, c, tid - 256);
+        producer_role<D, JOINT>(p, c, tid - 256);
     } else {
         if (warp == 12) {
-            mma_role<D>(p, c);
+            mma_role<D, JOINT>(p, c);
         } else if (warp == 13) {
-            tma_role<D>(p, c, lane, &tm_pool_k, &tm_pool_v, &tm_ws_k, &tm_ws_v, &tm_knew, &tm_vnew);
+            tma_role<D, JOINT>(p, c, lane, &tm_pool_k, &tm_pool_v, &tm_ws_k, &tm_ws_v, &tm_knew, &tm_vnew);
         } else {
             append_role<D>(p, c, tid - 448);
         }
@@ -851,7 +868,7 @@ struct MergeOut {
 // when a launch has few tiles (a short query over a long context: 8 tiles of 19 parts each took 22 us with 32 blocks that
 // walked the parts one by one, twice).
 template <int D, int CS>
-__device__ __forceinline__ void merge_tile(int b, int hk, int row_base, int item_q_len, const float4 *po, const float2 *pml,
+__device__ __forceinline__ void merge_tile(int b, int hk, int row_base, int item_q_len, int n_req, const float4 *po, const float2 *pml,
                                            int n, long long stride_o, long long stride_ml, int q_len, int n_q, int n_kv,
                                            int group, float scale, const MergeOut &mo)
 {
@@ -862,7 +879,8 @@ __device__ __forceinline__ void merge_tile(int b, int hk, int row_base, int item
     const int lane = threadIdx.x & 31, wv = threadIdx.x >> 5;
     const int row = blockIdx.y * 32 + lane;                     // row of the 128-row query tile
     const int col0 = CS > 1 ? blockIdx.z * (D / 4 / CS) : 0;    // first float4 column of this block
-    const int n_rows = group * (item_q_len ? item_q_len : q_len);       // q_len stays the stride of the padded tensors
+    // q_len stays the stride of the padded tensors; n_req > 1: the tile holds the rows of requests 0, 1, ... (kvp_joint)
+    const int per = group * (item_q_len ? item_q_len : q_len), n_rows = n_req > 1 ? per * n_req : per;
     const float c2 = scale * 1.4426950408889634f;
     // rows behind the request's last one exist in no partial (a decode step fills 4 of 128): nothing to read or write
     if (row_base + (int)blockIdx.y * 32 >= n_rows) return;
@@ -925,16 +943,19 @@ __device__ __forceinline__ void merge_tile(int b, int hk, int row_base, int item
         tile[lane][wv + 8 * j] = u;
     }
     const int r = row_base + row;
-    if (wv == 0 && col0 == 0 && r < n_rows && mo.lse != nullptr)
-        mo.lse[((long long)b * n_q + hk * group + r % group) * q_len + r / group] = M * scale + logf(L);
+    if (wv == 0 && col0 == 0 && r < n_rows && mo.lse != nullptr) {
+        const int rb = n_req > 1 ? r / per : b, rr = n_req > 1 ? r - rb * per : r;
+        mo.lse[((long long)rb * n_q + hk * group + rr % group) * q_len + rr / group] = M * scale + logf(L);
+    }
     __syncthreads();
     // 8 threads per output row (4 when the block's part of a row is 64 bytes)
     constexpr int kT = D / 8 / CS / kV;
     const int orow = threadIdx.x / kT, jt = threadIdx.x % kT;
     const int r2 = row_base + blockIdx.y * 32 + orow;
     if (orow < 32 && r2 < n_rows) {
-        const int i = r2 / group, h = hk * group + r2 % group;
-        uint4 *dst = reinterpret_cast<uint4 *>(mo.out + (((long long)b * q_len + i) * n_q + h) * D) + col0 / 2 + kV * jt;
+        const int rb = n_req > 1 ? r2 / per : b, rr = n_req > 1 ? r2 - rb * per : r2;
+        const int i = rr / group, h = hk * group + rr % group;
+        uint4 *dst = reinterpret_cast<uint4 *>(mo.out + (((long long)rb * q_len + i) * n_q + h) * D) + col0 / 2 + kV * jt;
 #pragma unroll
         for (int v = 0; v < kV; ++v) {
             const uint2 a0 = tile[orow][2 * (kV * jt + v)], a1 = tile[orow][2 * (kV * jt + v) + 1];
@@ -953,7 +974,7 @@ merge_list_kernel(const kvp_merge_item *__restrict__ merges, int q_len, int n_q,
     pdl_wait();
     PDL_AFTER(part_o); PDL_AFTER(part_ml); PDL_AFTER(merges);
     const kvp_merge_item mi = merges[blockIdx.x];
-    merge_tile<D, CS>(mi.b, mi.hk, mi.row_base, mi.pad[0], reinterpret_cast<const float4 *>(part_o) + (long long)mi.slot0 * (D / 4 * KVP_TILE_ROWS),
+    merge_tile<D, CS>(mi.b, mi.hk, mi.row_base, mi.pad[0], mi.pad[1], reinterpret_cast<const float4 *>(part_o) + (long long)mi.slot0 * (D / 4 * KVP_TILE_ROWS),
                part_ml + (long long)mi.slot0 * KVP_TILE_ROWS, mi.n_slots, D / 4 * KVP_TILE_ROWS, KVP_TILE_ROWS, q_len, n_q, n_kv,
                group, scale, mo);
 }
@@ -966,7 +987,7 @@ merge_ranks_kernel(const char *__restrict__ parts, int n_parts, long long part_b
 {
     const int c = blockIdx.x;
     const int rt = c % n_rt, hk = (c / n_rt) % n_kv, b = c / (n_rt * n_kv);
-    merge_tile<128, 1>(b, hk, rt * KVP_TILE_ROWS, 0, reinterpret_cast<const float4 *>(parts) + (long long)c * (32 * KVP_TILE_ROWS),
+    merge_tile<128, 1>(b, hk, rt * KVP_TILE_ROWS, 0, 1, reinterpret_cast<const float4 *>(parts) + (long long)c * (32 * KVP_TILE_ROWS),
                reinterpret_cast<const float2 *>(parts + ml_offset) + (long long)c * KVP_TILE_ROWS, n_parts, part_bytes / 16,
                part_bytes / 8, q_len, n_q, n_kv, group, scale, mo);
 }
@@ -977,9 +998,10 @@ template <int D>
 static cudaError_t prepare()
 {
     const cudaFuncAttribute what = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    cudaError_t rc = cudaFuncSetAttribute(attn_sm100_kernel<D, 0>, what, Cfg<D>::kSmemBytes);
-    if (rc == cudaSuccess) rc = cudaFuncSetAttribute(attn_sm100_kernel<D, KVP_INLINE_SMALL>, what, Cfg<D>::kSmemBytes);
-    if (rc == cudaSuccess) rc = cudaFuncSetAttribute(attn_sm100_kernel<D, KVP_INLINE_LARGE>, what, Cfg<D>::kSmemBytes);
+    cudaError_t rc = cudaFuncSetAttribute(attn_sm100_kernel<D, 0, false>, what, Cfg<D>::kSmemBytes);
+    if (rc == cudaSuccess) rc = cudaFuncSetAttribute(attn_sm100_kernel<D, KVP_INLINE_SMALL, false>, what, Cfg<D>::kSmemBytes);
+    if (rc == cudaSuccess) rc = cudaFuncSetAttribute(attn_sm100_kernel<D, KVP_INLINE_LARGE, false>, what, Cfg<D>::kSmemBytes);
+    if (rc == cudaSuccess && D == 128) rc = cudaFuncSetAttribute(attn_sm100_kernel<128, 0, true>, what, Cfg<128>::kSmemBytes);
     return rc;
 }
 cudaError_t kvp_attn_sm100_prepare(int32_t head_dim) { return head_dim == 64 ? prepare<64>() : prepare<128>(); }
@@ -996,14 +1018,15 @@ cudaError_t kvp_launch_attn_sm100(const kvp_shape &sh, const kvp_attn2_args &a, 
     };
     const auto *small = reinterpret_cast<const kvp_blob<KVP_INLINE_SMALL> *>(a.list);
     const auto *large = reinterpret_cast<const kvp_blob<KVP_INLINE_LARGE> *>(a.list);
+    if (a.joint_batch > 0) return go(attn_sm100_kernel<128, 0, true>, Cfg<128>::kSmemBytes, kvp_blob<0>());
     const int size = !a.list ? 0 : a.list_bytes <= KVP_INLINE_SMALL ? 1 : 2;
     if (sh.head_dim == 64)
-        return size == 0   ? go(attn_sm100_kernel<64, 0>, Cfg<64>::kSmemBytes, kvp_blob<0>())
-               : size == 1 ? go(attn_sm100_kernel<64, KVP_INLINE_SMALL>, Cfg<64>::kSmemBytes, *small)
-                           : go(attn_sm100_kernel<64, KVP_INLINE_LARGE>, Cfg<64>::kSmemBytes, *large);
-    return size == 0   ? go(attn_sm100_kernel<128, 0>, Cfg<128>::kSmemBytes, kvp_blob<0>())
-           : size == 1 ? go(attn_sm100_kernel<128, KVP_INLINE_SMALL>, Cfg<128>::kSmemBytes, *small)
-                       : go(attn_sm100_kernel<128, KVP_INLINE_LARGE>, Cfg<128>::kSmemBytes, *large);
+        return size == 0   ? go(attn_sm100_kernel<64, 0, false>, Cfg<64>::kSmemBytes, kvp_blob<0>())
+               : size == 1 ? go(attn_sm100_kernel<64, KVP_INLINE_SMALL, false>, Cfg<64>::kSmemBytes, *small)
+                           : go(attn_sm100_kernel<64, KVP_INLINE_LARGE, false>, Cfg<64>::kSmemBytes, *large);
+    return size == 0   ? go(attn_sm100_kernel<128, 0, false>, Cfg<128>::kSmemBytes, kvp_blob<0>())
+           : size == 1 ? go(attn_sm100_kernel<128, KVP_INLINE_SMALL, false>, Cfg<128>::kSmemBytes, *small)
+                       : go(attn_sm100_kernel<128, KVP_INLINE_LARGE, false>, Cfg<128>::kSmemBytes, *large);
 }
 
 cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_merges, const kvp_merge_item *merges,

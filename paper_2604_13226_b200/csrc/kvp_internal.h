@@ -86,7 +86,7 @@ struct kvp_merge_item {        // 128 packed rows whose result is spread over n_
     int32_t b, hk;
     int32_t row_base;
     int32_t slot0, n_slots;
-    int32_t pad[3];            // pad[0]: the request's own query length (0: the call's q_len)
+    int32_t pad[3];            // pad[0]: the request's own query length (0: the call's q_len); pad[1]: requests in the tile (0: one)
 };
 
 // Capacity of one plan blob (entries per array, bytes in all).
@@ -139,6 +139,16 @@ struct kvp_segment_host {
     std::vector<int32_t> kept;         // compressed packets: rows kept per plane (layer, kv head); else empty
 };
 
+// Short calls over documents that several requests share (decode steps, mostly): the rows of all requests lie in one query
+// tile and every document is walked once.  Prefix tiles of all requests together, staged adapter rows first, documents by
+// pool row; `rope` of a tile is the number of its document run (0: none), `pad` the requests that hold it, a bit each.
+// ropes[(run - 1) * batch + b]: rope-table index of run `run` in request b (where it holds it).
+struct kvp_joint {
+    int32_t state = -1;                    // -1: not looked at; 0: not worth it; 1: made
+    std::vector<kvp_tile> tiles;
+    std::vector<int32_t> ropes;
+};
+
 struct kvp_assembly_host {
     int32_t id = -1;
     uint32_t flags = 0;
@@ -157,8 +167,9 @@ struct kvp_assembly_host {
     bool waits_loads = false;              // uses packets that came from host memory: wait for the layer's load event
     // work lists of the two-stream kernel (one, or one per layer when the tile lists differ per layer), each
     // built for q_len query tokens at offset q_pos0 (q_len 0 = none yet)
-    struct sched_state { int32_t q_len = 0, q_pos0 = 0, ctas = 0, works = 0, merges = 0, slots = 0; uint32_t opts = 0, off_works = 0, off_merges = 0; std::vector<int32_t> q_lens; };
+    struct sched_state { int32_t q_len = 0, q_pos0 = 0, ctas = 0, works = 0, merges = 0, slots = 0; uint32_t opts = 0, off_works = 0, off_merges = 0, off_joint = 0; std::vector<int32_t> q_lens; };
     std::vector<sched_state> sched;
+    kvp_joint joint;
 };
 
 // Work list of the two-stream kernel for one assembly and query length, with the scratch it is built in.
@@ -359,6 +370,10 @@ struct kvp_attn2_args {
     // not null: the work list (list_bytes, padded to 16) comes along, works at list_works; the launch stores it at list_dev
     const void *list;
     uint32_t list_bytes, list_works;
+    // joint_batch > 0: a unit is one kv head, its rows are those of all requests (kvp_joint), its prefix tiles these
+    int32_t joint_batch;
+    const kvp_tile *joint_tiles;
+    const int32_t *joint_ropes;
     char *list_dev;
     int32_t l2_prefetch;           // the launch has at most two 256-row units per (request, kv head)
     const void *k_new, *v_new;
