@@ -627,7 +627,8 @@ int32_t build_schedule(kvp_ctx *ctx, kvp_assembly_host &as, int slot, int layer,
         memcpy(h + off_joint + tile_bytes, as.joint.ropes.data(), rope_bytes);
     };
     a.list_dev = ctx->slot_sched_dev[slot] + ctx->sched_bytes * li;
-    if (!joint && sc.n_ctas > 0 && used <= (as.item_stride ? KVP_INLINE_LARGE : KVP_INLINE_SMALL)) {   // comes along with the attention launch
+    if (!joint && sc.n_ctas > 0 && used <= (as.item_stride || ctx->cfg.n_layers == 1 ? KVP_INLINE_LARGE : KVP_INLINE_SMALL)) {
+        // comes along with the attention launch
         pack(ctx->list_inline);
         a.list = ctx->list_inline;
         a.list_bytes = (uint32_t)round_up(used, 16);

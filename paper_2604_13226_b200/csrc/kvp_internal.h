@@ -19,9 +19,9 @@
 // Plans and work lists up to the first size travel as parameters of the kernel that needs them first: an upload kernel in
 // front costs 4 us on the way to the first tile, 4 KB of parameters next to nothing (one request of 5 documents x 512 tokens,
 // one layer: 24.4 -> 18.8 us; 2 x 8 documents in fp32: 41 -> 37.5).  A launch with 12 KB costs the GPU as much as the upload
-// does and saves host time only, so work lists up to the second size travel along where every layer has one of its own
-// (compressed packets, 4 layers: 244 -> 238 us), not where one list serves many launches (a 5 x 10 documents decode
-// was 0.8 % slower with it).
+// does and saves host time only, so work lists up to the second size travel along where a list serves one launch (compressed
+// packets, 4 layers: 244 -> 238 us; one layer, one call: 26.6 -> 24.8), not where it serves the launches of all layers (a
+// 5 x 10 documents decode was 0.8 % slower with it).
 #define KVP_INLINE_SMALL 4096
 #define KVP_INLINE_LARGE 16384
 #define KVP_UPLOAD_BLOCKS 16   // blocks of an upload, each with a completion flag of its own

@@ -43,7 +43,7 @@ def test_joint_only_where_it_saves():
     shape = gen.ModelShape(1, 32, 8, 128, "bf16", 500000.0, 0)
     for items, want in (([[(p, 0) for p in (0, 1, 2)], [(p, 0) for p in (3, 4, 5)]], False),
                         ([[(p, 0) for p in (0, 1, 2)], [(p, 0) for p in (2, 1, 0)]], True)):
-        wl = gen.make_workload(shape, [1024] * 6, items, q_len=5, seed=3)
+        wl = gen.make_workload(shape, [2048] * 6, items, q_len=5, seed=3)
         sess = Session(wl)
         sess.assemble()
         out, lse = run_chunks(wl, sess, [(0, 4), (4, 5)])
