@@ -323,7 +323,7 @@ bool make_joint(kvp_assembly_host &as)
 // Whether a call takes joint units: short queries of several requests, whose rows fit one query tile together, over
 // documents that requests share.  Such a call is bound by reading the cache, and the requests of a launch do not meet at
 // the same tiles by themselves (a decode step of 8 requests that draw 10 of 46 documents of 1024 tokens, 8 kv heads: 346 MB
-// read, 194 MB of them distinct).  The saving has to outweigh the merge of more and larger parts: two tiles per CTA.
+// read, 194 MB of them distinct; 4 layers, a prefill and 16 steps: 4520 -> 3558 us).  The saving has to outweigh the merge of more and larger parts: two tiles per CTA.
 bool use_joint(const kvp_ctx *ctx, kvp_assembly_host &as, int q_len)
 {
     const kvp_shape &sh = ctx->shape;
@@ -1052,6 +1052,7 @@ static int32_t assemble_impl(kvp_ctx *ctx, int32_t batch, const int32_t *slot_of
     as.appended.clear();
     as.sched.clear();
     as.joint.state = -1;
+    as.settled = false;
     as.ragged = false;
     as.last_q_len = 0;
     as.flags = flags;
@@ -1392,7 +1393,7 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
     // the CUDA-core kernel does the same when nothing has to be rotated and no row was appended before
     const bool core_append = !fast && ctx->fused_append && !rope_query && q_pos0 == 0 && (((uintptr_t)k_new | (uintptr_t)v_new) & 15) == 0;
     if (!a.tail_direct && !skip_block && !core_append) {
-        KVP_CUDA(ctx, kvp_launch_append(sh, plan, as.batch, q_len, q_pos0, q, k_new, v_new, ctx->slot_k[slot], ctx->slot_v[slot],
+        KVP_CUDA(ctx, kvp_launch_append(sh, plan, as.settled, as.batch, q_len, q_pos0, q, k_new, v_new, ctx->slot_k[slot], ctx->slot_v[slot],
                                         layer, rope_query, ctx->half_turns, ctx->q_scratch, st));
         ++launches;
     }
@@ -1463,6 +1464,7 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
                       : kvp_launch_attn_sm100(sh, a, ctx->tm_pool_k, ctx->tm_pool_v, ctx->tm_ws_k[slot], ctx->tm_ws_v[slot], st);
             if (launched != cudaSuccess) as.sched[li].q_len = 0;   // its work list never reached the device
             KVP_CUDA(ctx, launched);
+            as.settled = true;                                     // its first launch waits before it releases anyone
             KVP_CUDA(ctx, time_edge(ctx, 0, 1, st));
             ++launches;
         }
@@ -1470,7 +1472,7 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
             const bool partial = (flags & KVP_PARTIAL) != 0;
             const int64_t n_rt = ((int64_t)sh.group * q_len + KVP_TILE_ROWS - 1) / KVP_TILE_ROWS;
             KVP_CUDA(ctx, kvp_launch_merge_list(sh, q_len, ss.merges,
-                                                reinterpret_cast<const kvp_merge_item *>(sd + ss.off_merges),
+                                                reinterpret_cast<const kvp_merge_item *>(sd + ss.off_merges), ss.ctas > 0,
                                                 ctx->partial_o, ctx->partial_ml, out, lse, partial ? out : nullptr,
                                                 (int64_t)as.batch * sh.n_kv_heads * n_rt, st));
             ++launches;

@@ -873,7 +873,7 @@ __device__ __forceinline__ void merge_tile(int b, int hk, int row_base, int item
                                            int group, float scale, const MergeOut &mo)
 {
     constexpr int kC = D / 32 / CS;                             // float4 columns per warp
-    constexpr int U = kC == 1 ? 8 : 4;
+    constexpr int U = kC == 1 ? 20 : 4;
     constexpr int kV = D / 64 / CS > 0 ? D / 64 / CS : 1;       // 16-byte words of a row this block writes per thread
     __shared__ uint2 tile[32][D / 4 / CS + 1];
     const int lane = threadIdx.x & 31, wv = threadIdx.x >> 5;
@@ -967,13 +967,18 @@ __device__ __forceinline__ void merge_tile(int b, int hk, int row_base, int item
 // The partial slots of the units of one launch.  Grid (merge item, 4, CS).
 template <int D, int CS>
 __global__ void __launch_bounds__(256)
-merge_list_kernel(const kvp_merge_item *__restrict__ merges, int q_len, int n_q, int n_kv, int group, float scale,
+merge_list_kernel(const kvp_merge_item *__restrict__ merges, int list_there, int q_len, int n_q, int n_kv, int group, float scale,
                   const float *__restrict__ part_o, const float2 *__restrict__ part_ml, MergeOut mo)
 {
     pdl_launch_dependents();
-    pdl_wait();
-    PDL_AFTER(part_o); PDL_AFTER(part_ml); PDL_AFTER(merges);
-    const kvp_merge_item mi = merges[blockIdx.x];
+    if (!list_there) pdl_wait();                                // (no attention launch lies between the list's upload and this)
+    PDL_AFTER(merges);
+    kvp_merge_item mi;
+    int4 *m4 = reinterpret_cast<int4 *>(&mi);                   // (from L2: stored while this launch was being set up)
+    m4[0] = __ldcg(reinterpret_cast<const int4 *>(merges + blockIdx.x));
+    m4[1] = __ldcg(reinterpret_cast<const int4 *>(merges + blockIdx.x) + 1);
+    if (list_there) pdl_wait();
+    PDL_AFTER(part_o); PDL_AFTER(part_ml);
     merge_tile<D, CS>(mi.b, mi.hk, mi.row_base, mi.pad[0], mi.pad[1], reinterpret_cast<const float4 *>(part_o) + (long long)mi.slot0 * (D / 4 * KVP_TILE_ROWS),
                part_ml + (long long)mi.slot0 * KVP_TILE_ROWS, mi.n_slots, D / 4 * KVP_TILE_ROWS, KVP_TILE_ROWS, q_len, n_q, n_kv,
                group, scale, mo);
@@ -1029,7 +1034,7 @@ cudaError_t kvp_launch_attn_sm100(const kvp_shape &sh, const kvp_attn2_args &a, 
                        : go(attn_sm100_kernel<128, KVP_INLINE_LARGE, false>, Cfg<128>::kSmemBytes, *large);
 }
 
-cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_merges, const kvp_merge_item *merges,
+cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_merges, const kvp_merge_item *merges, bool list_there,
                                   const float *partial_o, const float2 *partial_ml, void *out, float *lse,
                                   void *part_out, int64_t part_tiles, cudaStream_t st)
 {
@@ -1046,7 +1051,7 @@ cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_
     // whole rows per block when that gives two blocks per SM, else quarter rows (halves with head dimension 64)
     const bool few = n_merges * (KVP_TILE_ROWS / 32) < 2 * 148;
     auto go = [&](auto *kernel, int cs) {
-        return launch_pdl(kernel, dim3(n_merges, KVP_TILE_ROWS / 32, cs), 256, 0, st, merges, q_len, sh.n_q_heads, sh.n_kv_heads,
+        return launch_pdl(kernel, dim3(n_merges, KVP_TILE_ROWS / 32, cs), 256, 0, st, merges, (int)list_there, q_len, sh.n_q_heads, sh.n_kv_heads,
                           sh.group, sh.scale, partial_o, partial_ml, mo);
     };
     if (sh.head_dim == 64) return few ? go(merge_list_kernel<64, 2>, 2) : go(merge_list_kernel<64, 1>, 1);

@@ -170,6 +170,7 @@ struct kvp_assembly_host {
     struct sched_state { int32_t q_len = 0, q_pos0 = 0, ctas = 0, works = 0, merges = 0, slots = 0; uint32_t opts = 0, off_works = 0, off_merges = 0, off_joint = 0; std::vector<int32_t> q_lens; };
     std::vector<sched_state> sched;
     kvp_joint joint;
+    bool settled = false;                  // an attention launch has waited for the plan
 };
 
 // Work list of the two-stream kernel for one assembly and query length, with the scratch it is built in.
@@ -321,7 +322,8 @@ cudaError_t kvp_launch_upload(const void *host, void *dst, uint64_t bytes, volat
 cudaError_t kvp_launch_gather(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t n_chunks, int32_t n_rope,
                               const double *half_turns, const char *pool_k, const char *pool_v, char *ws_k, char *ws_v,
                               const void *blob, uint32_t blob_bytes, char *blob_dev, cudaStream_t st);
-cudaError_t kvp_launch_append(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t batch, int32_t q_len,
+// plan_there: the plan was complete before the launch in front of this one was released
+cudaError_t kvp_launch_append(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t plan_there, int32_t batch, int32_t q_len,
                               int32_t q_pos0, const void *q, const void *k_new, const void *v_new, char *ws_k, char *ws_v,
                               int32_t layer, int32_t rope_query, const double *half_turns, void *q_rot,
                               cudaStream_t st);
@@ -389,7 +391,8 @@ cudaError_t kvp_launch_attn_sm100(const kvp_shape &sh, const kvp_attn2_args &a, 
                                   const CUtensorMap &tm_pool_v, const CUtensorMap &tm_ws_k,
                                   const CUtensorMap &tm_ws_v, cudaStream_t st);
 // part_out != nullptr: the merged tiles stay partials and go to a rank buffer of part_tiles query tiles
-cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_merges, const kvp_merge_item *merges,
+// list_there: the launch in front waited for the merge list before it released this one
+cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_merges, const kvp_merge_item *merges, bool list_there,
                                   const float *partial_o, const float2 *partial_ml, void *out, float *lse,
                                   void *part_out, int64_t part_tiles, cudaStream_t st);
 // n_parts rank buffers back to back -> final output rows

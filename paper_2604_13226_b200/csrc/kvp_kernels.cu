@@ -301,8 +301,9 @@ gather_kernel(kvp_plan_dev plan, const __grid_constant__ kvp_blob<LB> blob, int 
 // grid (batch*q_len); the rows go behind the q_pos0 rows appended earlier; with rope_query the raw
 // k_new and q are first rotated to positions prefix_len + q_pos0 + i, angles formed in double precision.
 // Latency is all there is (a decode step moves a few KB): a thread takes a pair of 16-byte words - the rotation partners -
-// of K and V or of Q, and every load is issued before the angles are formed.  One element at a time with the angles first
-// it took 9.4 us of a 75 us decode layer.
+// of K and V or of Q, the block is as wide as the token has pairs, and the angles are formed before the wait for the kernel
+// in front (plan_there: the plan is complete by then - not so right behind the gather that stores it).  One element at a
+// time with the angles first it took 9.4 us of a 75 us decode layer.
 template <typename T>
 __device__ __forceinline__ Vec16<T> load_vec(const T *p, bool aligned)
 {
@@ -317,8 +318,8 @@ __device__ __forceinline__ Vec16<T> load_vec(const T *p, bool aligned)
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256)
-append_kernel(kvp_plan_dev plan, int q_len, int q_pos0, const T *__restrict__ q, const T *__restrict__ k_new,
+__global__ void __launch_bounds__(512)
+append_kernel(kvp_plan_dev plan, int plan_there, int q_len, int q_pos0, const T *__restrict__ q, const T *__restrict__ k_new,
               const T *__restrict__ v_new, char *__restrict__ ws_k, char *__restrict__ ws_v,
               int64_t ws_rows, int layer, int n_q, int n_kv, int d, int pairing, int rope_query,
               const double *__restrict__ half_turns, T *__restrict__ q_rot)
@@ -326,36 +327,31 @@ append_kernel(kvp_plan_dev plan, int q_len, int q_pos0, const T *__restrict__ q,
     constexpr int EV = Elem<T>::kPerVec;
     __shared__ float2 cs[64];
     pdl_launch_dependents();
-    pdl_wait();
-    PDL_AFTER(q); PDL_AFTER(k_new); PDL_AFTER(v_new);
+    if (!plan_there) pdl_wait();
+    PDL_AFTER(plan.items);
     const int b = blockIdx.x / q_len, i = blockIdx.x % q_len;
     const kvp_item it = plan.items[b];
     const int half = d / 2, half_vecs = half / EV, vecs = 2 * half_vecs;
+    if (rope_query && (int)threadIdx.x < half) cs[threadIdx.x] = offset_cos_sin(it.prefix_len + q_pos0 + i, half_turns[threadIdx.x]);
+    __syncthreads();
+    if (plan_there) pdl_wait();
+    PDL_AFTER(q); PDL_AFTER(k_new); PDL_AFTER(v_new);
     const int64_t tok = (int64_t)b * q_len + i;
     const bool al_q = ((uintptr_t)q & 15) == 0, al_k = ((uintptr_t)k_new & 15) == 0, al_v = ((uintptr_t)v_new & 15) == 0;
     // keys and values: items [0, n_kv half_vecs); with rope_query the query rows behind them
     const int n_items = (n_kv + (rope_query ? n_q : 0)) * half_vecs;
-    bool first = rope_query != 0;
-    for (int w = threadIdx.x; w < n_items || first; w += 256) {
+    for (int w = threadIdx.x; w < n_items; w += blockDim.x) {
         Vec16<T> lo, hi, va, vb;
         const bool kv = w < n_kv * half_vecs;
         const int head = kv ? w / half_vecs : w / half_vecs - n_kv, c = w % half_vecs;
-        if (w < n_items) {
-            const T *src = (kv ? k_new + (tok * n_kv + head) * d : q + (tok * n_q + head) * d) + c * EV;
-            lo = load_vec<T>(src, kv ? al_k : al_q);
-            hi = load_vec<T>(src + half, kv ? al_k : al_q);
-            if (kv) {
-                const T *vs = v_new + (tok * n_kv + head) * d + c * EV;
-                va = load_vec<T>(vs, al_v);
-                vb = load_vec<T>(vs + half, al_v);
-            }
+        const T *src = (kv ? k_new + (tok * n_kv + head) * d : q + (tok * n_q + head) * d) + c * EV;
+        lo = load_vec<T>(src, kv ? al_k : al_q);
+        hi = load_vec<T>(src + half, kv ? al_k : al_q);
+        if (kv) {
+            const T *vs = v_new + (tok * n_kv + head) * d + c * EV;
+            va = load_vec<T>(vs, al_v);
+            vb = load_vec<T>(vs + half, al_v);
         }
-        if (first) {
-            if ((int)threadIdx.x < half) cs[threadIdx.x] = offset_cos_sin(it.prefix_len + q_pos0 + i, half_turns[threadIdx.x]);
-            __syncthreads();
-            first = false;
-        }
-        if (w >= n_items) break;
         if (rope_query) rotate_vec_pair<T>(lo, hi, cs, c, half_vecs, pairing);
         if (kv) {
             const int64_t drow = ((int64_t)(layer * n_kv + head)) * ws_rows + it.tail_row0 + q_pos0 + i;
@@ -1009,17 +1005,19 @@ cudaError_t kvp_launch_gather(const kvp_shape &sh, const kvp_plan_dev &plan, int
     return blob ? go(gather_kernel<float, KVP_INLINE_SMALL>, *small) : go(gather_kernel<float, 0>, kvp_blob<0>());
 }
 
-cudaError_t kvp_launch_append(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t batch, int32_t q_len,
+cudaError_t kvp_launch_append(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t plan_there, int32_t batch, int32_t q_len,
                               int32_t q_pos0, const void *q, const void *k_new, const void *v_new, char *ws_k, char *ws_v,
                               int32_t layer, int32_t rope_query, const double *half_turns, void *q_rot,
                               cudaStream_t st)
 {
     const int grid = batch * q_len;
+    const int pairs = (sh.n_kv_heads + (rope_query ? sh.n_q_heads : 0)) * (sh.head_dim * sh.elem_bytes / 32);
+    const int threads = pairs <= 64 ? 64 : pairs >= 512 ? 512 : (pairs + 31) / 32 * 32;     // (64: an angle each)
     if (sh.dtype == KVP_DTYPE_BF16)
-        return launch_pdl(append_kernel<__nv_bfloat16>, grid, 256, 0, st, plan, q_len, q_pos0, (const __nv_bfloat16 *)q,
+        return launch_pdl(append_kernel<__nv_bfloat16>, grid, threads, 0, st, plan, plan_there, q_len, q_pos0, (const __nv_bfloat16 *)q,
                           (const __nv_bfloat16 *)k_new, (const __nv_bfloat16 *)v_new, ws_k, ws_v, sh.ws_rows, layer, sh.n_q_heads,
                           sh.n_kv_heads, sh.head_dim, sh.pairing, rope_query, half_turns, (__nv_bfloat16 *)q_rot);
-    return launch_pdl(append_kernel<float>, grid, 256, 0, st, plan, q_len, q_pos0, (const float *)q, (const float *)k_new,
+    return launch_pdl(append_kernel<float>, grid, threads, 0, st, plan, plan_there, q_len, q_pos0, (const float *)q, (const float *)k_new,
                       (const float *)v_new, ws_k, ws_v, sh.ws_rows, layer, sh.n_q_heads, sh.n_kv_heads, sh.head_dim, sh.pairing,
                       rope_query, half_turns, (float *)q_rot);
 }
