@@ -1471,7 +1471,7 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
         if (ss.merges > 0) {
             const bool partial = (flags & KVP_PARTIAL) != 0;
             const int64_t n_rt = ((int64_t)sh.group * q_len + KVP_TILE_ROWS - 1) / KVP_TILE_ROWS;
-            KVP_CUDA(ctx, kvp_launch_merge_list(sh, q_len, ss.merges,
+            KVP_CUDA(ctx, kvp_launch_merge_list(sh, q_len, ss.merges, ss.slots,
                                                 reinterpret_cast<const kvp_merge_item *>(sd + ss.off_merges), ss.ctas > 0,
                                                 ctx->partial_o, ctx->partial_ml, out, lse, partial ? out : nullptr,
                                                 (int64_t)as.batch * sh.n_kv_heads * n_rt, st));

@@ -867,13 +867,12 @@ struct MergeOut {
 // (m, l) together, and folded in by the online rule, so that a tile of up to U parts costs one memory round trip.  CS > 1
 // when a launch has few tiles (a short query over a long context: 8 tiles of 19 parts each took 22 us with 32 blocks that
 // walked the parts one by one, twice).
-template <int D, int CS>
+template <int D, int CS, int U>
 __device__ __forceinline__ void merge_tile(int b, int hk, int row_base, int item_q_len, int n_req, const float4 *po, const float2 *pml,
                                            int n, long long stride_o, long long stride_ml, int q_len, int n_q, int n_kv,
                                            int group, float scale, const MergeOut &mo)
 {
     constexpr int kC = D / 32 / CS;                             // float4 columns per warp
-    constexpr int U = kC == 1 ? 20 : 4;
     constexpr int kV = D / 64 / CS > 0 ? D / 64 / CS : 1;       // 16-byte words of a row this block writes per thread
     __shared__ uint2 tile[32][D / 4 / CS + 1];
     const int lane = threadIdx.x & 31, wv = threadIdx.x >> 5;
@@ -965,7 +964,7 @@ __device__ __forceinline__ void merge_tile(int b, int hk, int row_base, int item
 }
 
 // The partial slots of the units of one launch.  Grid (merge item, 4, CS).
-template <int D, int CS>
+template <int D, int CS, int U>
 __global__ void __launch_bounds__(256)
 merge_list_kernel(const kvp_merge_item *__restrict__ merges, int list_there, int q_len, int n_q, int n_kv, int group, float scale,
                   const float *__restrict__ part_o, const float2 *__restrict__ part_ml, MergeOut mo)
@@ -979,7 +978,7 @@ merge_list_kernel(const kvp_merge_item *__restrict__ merges, int list_there, int
     m4[1] = __ldcg(reinterpret_cast<const int4 *>(merges + blockIdx.x) + 1);
     if (list_there) pdl_wait();
     PDL_AFTER(part_o); PDL_AFTER(part_ml);
-    merge_tile<D, CS>(mi.b, mi.hk, mi.row_base, mi.pad[0], mi.pad[1], reinterpret_cast<const float4 *>(part_o) + (long long)mi.slot0 * (D / 4 * KVP_TILE_ROWS),
+    merge_tile<D, CS, U>(mi.b, mi.hk, mi.row_base, mi.pad[0], mi.pad[1], reinterpret_cast<const float4 *>(part_o) + (long long)mi.slot0 * (D / 4 * KVP_TILE_ROWS),
                part_ml + (long long)mi.slot0 * KVP_TILE_ROWS, mi.n_slots, D / 4 * KVP_TILE_ROWS, KVP_TILE_ROWS, q_len, n_q, n_kv,
                group, scale, mo);
 }
@@ -992,7 +991,7 @@ merge_ranks_kernel(const char *__restrict__ parts, int n_parts, long long part_b
 {
     const int c = blockIdx.x;
     const int rt = c % n_rt, hk = (c / n_rt) % n_kv, b = c / (n_rt * n_kv);
-    merge_tile<128, 1>(b, hk, rt * KVP_TILE_ROWS, 0, 1, reinterpret_cast<const float4 *>(parts) + (long long)c * (32 * KVP_TILE_ROWS),
+    merge_tile<128, 1, 4>(b, hk, rt * KVP_TILE_ROWS, 0, 1, reinterpret_cast<const float4 *>(parts) + (long long)c * (32 * KVP_TILE_ROWS),
                reinterpret_cast<const float2 *>(parts + ml_offset) + (long long)c * KVP_TILE_ROWS, n_parts, part_bytes / 16,
                part_bytes / 8, q_len, n_q, n_kv, group, scale, mo);
 }
@@ -1034,7 +1033,7 @@ cudaError_t kvp_launch_attn_sm100(const kvp_shape &sh, const kvp_attn2_args &a, 
                        : go(attn_sm100_kernel<128, KVP_INLINE_LARGE, false>, Cfg<128>::kSmemBytes, *large);
 }
 
-cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_merges, const kvp_merge_item *merges, bool list_there,
+cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_merges, int32_t max_parts, const kvp_merge_item *merges, bool list_there,
                                   const float *partial_o, const float2 *partial_ml, void *out, float *lse,
                                   void *part_out, int64_t part_tiles, cudaStream_t st)
 {
@@ -1054,8 +1053,12 @@ cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_
         return launch_pdl(kernel, dim3(n_merges, KVP_TILE_ROWS / 32, cs), 256, 0, st, merges, (int)list_there, q_len, sh.n_q_heads, sh.n_kv_heads,
                           sh.group, sh.scale, partial_o, partial_ml, mo);
     };
-    if (sh.head_dim == 64) return few ? go(merge_list_kernel<64, 2>, 2) : go(merge_list_kernel<64, 1>, 1);
-    return few ? go(merge_list_kernel<128, 4>, 4) : go(merge_list_kernel<128, 1>, 1);
+    // 20 parts per round trip where a tile has more than 8 (a unit per kv head: 148 CTAs / 8; a decode layer 52 -> 50 us), 8
+    // elsewhere: the longer code cost launches of a few parts 2-5 us.
+    const bool many = max_parts > 8;
+    if (sh.head_dim == 64)
+        return !few ? go(merge_list_kernel<64, 1, 4>, 1) : many ? go(merge_list_kernel<64, 2, 20>, 2) : go(merge_list_kernel<64, 2, 8>, 2);
+    return !few ? go(merge_list_kernel<128, 1, 4>, 1) : many ? go(merge_list_kernel<128, 4, 20>, 4) : go(merge_list_kernel<128, 4, 8>, 4);
 }
 
 cudaError_t kvp_launch_merge_ranks(const kvp_shape &sh, int32_t batch, int32_t q_len, const void *parts, int32_t n_parts,

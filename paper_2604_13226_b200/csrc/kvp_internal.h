@@ -392,7 +392,7 @@ cudaError_t kvp_launch_attn_sm100(const kvp_shape &sh, const kvp_attn2_args &a, 
                                   const CUtensorMap &tm_ws_v, cudaStream_t st);
 // part_out != nullptr: the merged tiles stay partials and go to a rank buffer of part_tiles query tiles
 // list_there: the launch in front waited for the merge list before it released this one
-cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_merges, const kvp_merge_item *merges, bool list_there,
+cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_merges, int32_t max_parts, const kvp_merge_item *merges, bool list_there,
                                   const float *partial_o, const float2 *partial_ml, void *out, float *lse,
                                   void *part_out, int64_t part_tiles, cudaStream_t st);
 // n_parts rank buffers back to back -> final output rows
