@@ -399,6 +399,7 @@ __device__ __forceinline__ void produce_q_tile(const Params &p, char *qbuf, char
         for (int j = 0; j < 4; ++j)
             w4[j] = *(p.pairing == 0 ? cs + c * 4 + j : cs + (c + kCh * (j >> 1)) * 2 + (j & 1));
     }
+    pdl_wait();                                              // (plan and work list are there before; the query rows may not be)
 #pragma unroll 1
     for (int i = 0; i < kCh; ++i) {
         const int r = row_base + r0 + kRows * i;
@@ -455,23 +456,26 @@ __device__ __forceinline__ void produce_q_joint(const Params &p, char *qbuf, int
     const int at = r0 * 128 + ((c ^ (r0 & 7)) << 4);
     const int hi_off = D == 128 ? kHalfBytes : (at ^ 64) - at;
     auto put = [](uint32_t &word, uint32_t &, float x, float y) { word = pack_bf16(x, y); };
-#pragma unroll 2
+#pragma unroll 1
     for (int i = 0; i < kCh; ++i) {
         const int r = r0 + kRows * i;
         uint4 qa = make_uint4(0, 0, 0, 0), qb = qa;
         if (r < n_rows) {
             const int b = r / per, rr = r - b * per, tok = row_token(p, rr);
             const int rope = run == 0 ? 0 : p.joint_ropes[(run - 1) * p.joint_batch + b];
+            float4 w4[4];
+            if (rope > 0) {
+                const float4 *cs = reinterpret_cast<const float4 *>(p.plan.rope + (size_t)rope * (D / 2));
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    w4[j] = *(p.pairing == 0 ? cs + c * 4 + j : cs + (c + kCh * (j >> 1)) * 2 + (j & 1));
+            }
+            pdl_wait();
             const uint4 *src = reinterpret_cast<const uint4 *>(p.q) +
                                (((long long)b * p.q_len + tok) * p.n_q + hk * p.group + rr - tok * p.group) * (D / 8);
             qa = src[c];
             qb = src[c + kCh];
             if (rope > 0) {
-                const float4 *cs = reinterpret_cast<const float4 *>(p.plan.rope + (size_t)rope * (D / 2));
-                float4 w4[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    w4[j] = *(p.pairing == 0 ? cs + c * 4 + j : cs + (c + kCh * (j >> 1)) * 2 + (j & 1));
                 uint32_t *a = reinterpret_cast<uint32_t *>(&qa), *bb = reinterpret_cast<uint32_t *>(&qb);
                 rotate_chunks(p.pairing, a, bb, a, bb, w4, put);
             }

@@ -352,7 +352,6 @@ __device__ __forceinline__ void producer_role(const Params &p, const Cta &c, con
     const uint32_t stride = p.precise ? 2 * kQBufBytes : kQBufBytes;
     uint32_t ep = 0;
     bool ok = true;
-    pdl_wait();
     for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
         const Work w = load_work(p, c.works, wi);
         const int n_rows = p.group * w.q_len;
@@ -379,6 +378,7 @@ __device__ __forceinline__ void producer_role(const Params &p, const Cta &c, con
             if (k == 0 && w.lo == 0 && p.tail_direct) append_rows<16, 128>(p, w, w.row_base + c.rank * KVP_TILE_ROWS, KVP_TILE_ROWS, t);
         }
     }
+    pdl_wait();                                               // (a role that gave up early)
 }
 
 // Loads of a piece with n tiles in the order the MMA warp takes them: Q K^T runs three tiles ahead of P V, so

@@ -367,7 +367,6 @@ __device__ __forceinline__ void producer_role(const Params &p, const Cta &c, con
     const bool one_buffer = !C::kSplit && p.precise;
     uint32_t nEp0 = 0, nEp1 = 0;
     bool ok = true;
-    pdl_wait();
     for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
         const Work w = load_work<JOINT>(p, c.works, wi);
         const int n_rows = p.group * w.q_len;
@@ -406,6 +405,7 @@ __device__ __forceinline__ void producer_role(const Params &p, const Cta &c, con
             }
         }
     }
+    pdl_wait();                                               // (a role that gave up early)
 }
 
 // ---- append (the two spare warps) -------------------------------------------------------------------------------
