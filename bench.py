@@ -857,7 +857,7 @@ def main():
                 roof = {"bound": "hbm", "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                         "frac": ach / peaks["hbm_gbs"], "frac_nominal": ach / NOMINAL_GBS, "peak_nominal": NOMINAL_GBS,
                         "traffic": traffic, "peak_source": peaks["source"]}
-            roof.update({"kernel": "attn_sm100_kernel", "launches_timed": len(attn_ms), "avg_launch_ms": a_ms,
+            roof.update({"kernel": "attn_pair_kernel, or attn_sm100_kernel where units do not fill 256 rows", "launches_timed": len(attn_ms), "avg_launch_ms": a_ms,
                          "algorithmic_flops_per_launch": flops, "algorithmic_bytes_per_launch": bytes_,
                          "attn_share_of_step": a_ms * L * args.steps / ms_total,     # every launch counted at the sampled mean
                          "gather_avg_ms": statistics.mean(gather_ms) if gather_ms else None})

@@ -124,7 +124,8 @@ KVP_API int32_t kvp_register_packet(kvp_ctx *ctx, const void *k, const void *v, 
 /*
  * Register one packet whose K/V stay in host memory until a request uses it (the CPU-to-GPU cache transfer
  * that the paper counts inside time-to-first-token, Section 4.3).  Pool rows are reserved now; nothing is copied.
- * The first kvp_assemble that names the packet enqueues the copy on a stream the context owns, layer by layer,
+ * The first kvp_assemble that names the packet enqueues the copy on a stream the context owns, layer by layer (one
+ * kernel per layer reads the packets over the host link; unpinned buffers are copied by the driver instead),
  * and kvp_query_prefill(layer) makes its stream wait for that layer only: the transfer of layer l+1 runs while
  * layer l is attended to.  After that the packet is resident like any other, until kvp_evict_packet.
  *   k_host, v_host   host, layout [n_layers][n_kv_heads][n_tokens][head_dim] (the pool's own plane order, so a
@@ -183,8 +184,9 @@ KVP_API int32_t kvp_register_adapter(kvp_ctx *ctx, const void *hk, const void *h
  * Positions are dense from 0; a segment cached at p0 and placed at slot offset t gets Delta = t - p0
  * (0 for every segment when KVP_REBASE is not set).  All three index arrays are host arrays.
  *
- * Host work: validation, segment table, tile list, cos/sin of Delta*theta_i in double precision.
- * Device work on `stream`: one plan upload and one gather kernel that copies + re-bases either the
+ * Host work: validation, segment table, tile list.  Device work on `stream`: one gather kernel (a plan of more than
+ * 4 KB travels by an upload kernel in front of it) that forms cos/sin of Delta*theta_i in double precision and
+ * copies + re-bases either the
  * adapter tokens only (default: documents are read in place by kvp_query_prefill) or, with
  * KVP_MATERIALIZE, the whole prefix into the workspace cache.
  * prefix_len (host, [batch]) is written before return.  Errors: INVALID, NOT_FOUND, CAPACITY, CUDA.
@@ -301,7 +303,9 @@ KVP_API int32_t kvp_export_cache(kvp_ctx *ctx, int32_t assembly_id, int32_t laye
  * a unit is <= 256 packed rows (query token, head-in-group) of one request and kv head, its key tiles
  * numbered with the causal tiles of the query's own keys first and the request's prefix tiles after
  * them; mode 0 = two 128-row query tiles over every key tile, mode 1 = one query tile whose key tiles
- * alternate between the CTA's two streams; slot -1 = the piece covers the unit's whole key range and
+ * alternate between the CTA's two streams; a call whose units mostly fill 256 rows runs on CTA pairs (head_dim 128):
+ * an entry of cta_begin is then a pair and every piece has mode 0.  The list is that of a plain prefill; a short
+ * continued call over documents that requests share is planned otherwise.  Slot -1 = the piece covers the unit's whole key range and
  * writes the output directly.  A merge item is 8 ints {request, kv head, first packed row, first
  * partial slot, number of slots, 0, 0, 0}.  counts (4 ints): CTAs, pieces, merge items, partial slots.
  * Errors: NOT_FOUND, INVALID, CAPACITY (an output array is too small; counts is still written).
