@@ -490,7 +490,8 @@ int32_t plan_schedule(kvp_ctx *ctx, const kvp_assembly_host &as, int layer, int 
     // out and its cuts, counted from the first prefix tile of a unit, are used for all of them.  The CTAs that
     // hold the same (request, kv head) then stay on the same K/V tiles for the whole launch instead of drifting
     // apart by the tail tiles they have more or less (drift beyond what L2 holds per CTA turns re-reads into DRAM
-    // reads: 4 requests of 16 documents of 2048 tokens, 256 query tokens, read 1.37x their K/V).  Equal shares may leave a ninth of the CTAs idle: such
+    // reads: 4 requests of 16 documents of 2048 tokens, 256 query tokens, read 1.37x their K/V).  Equal shares may leave a
+    // ninth of the CTAs idle: such
     // launches are limited by power, and CTAs that do not run cost less than K/V read twice (74 pairs, 4 row blocks, 72
     // pairs used: 572 -> 548 us; 7 row blocks, 70 used: 1153 -> 1139; 11, 66 used: 784 -> 771).
     bool aligned = per_block && !q_lens && G / n_rb >= 1 && (G - n_rb * (G / n_rb)) * 9 <= G;
