@@ -404,7 +404,12 @@ int32_t plan_schedule(kvp_ctx *ctx, const kvp_assembly_host &as, int layer, int 
     // that holds its larger part.  The last CTA of the run takes all that is left, so g CTAs always suffice.
     std::vector<cut_t> &cuts = out.cuts;
     cuts.clear();
-    const int64_t min_budget = 8 + kPieceCost;
+    // Smallest share of a CTA: a sixth of the largest unit, between 3 and 8 single-stream tiles.  Short units gain by being
+    // cut finely (decode of 3 requests with 13 tiles each: 8 tiles a CTA 876 us, 4 719, 3 671; one layer, 2 x 16 tiles: 118,
+    // 91, 93); units of 20 tiles and more, cut into a dozen parts, pay for it in the merge (46 tiles: 18.4 us, 20.5).
+    int64_t largest = 0;
+    for (const unit_t &u : units) largest = std::max<int64_t>(largest, (int64_t)(u.n_all - u.t_first) * (u.mode ? 1 : 2));
+    const int64_t min_budget = std::min<int64_t>(8, std::max<int64_t>(3, (largest + 5) / 6)) + kPieceCost;
     auto fill = [&](size_t u_begin, size_t u_end, int g, std::vector<cut_t> *rec) -> int {
         std::vector<int64_t> &after = out.after;                      // weight of the units behind unit u
         after.resize(u_end - u_begin + 1);

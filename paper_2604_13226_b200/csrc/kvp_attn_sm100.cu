@@ -1053,9 +1053,9 @@ cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_
         return launch_pdl(kernel, dim3(n_merges, KVP_TILE_ROWS / 32, cs), 256, 0, st, merges, (int)list_there, q_len, sh.n_q_heads, sh.n_kv_heads,
                           sh.group, sh.scale, partial_o, partial_ml, mo);
     };
-    // 20 parts per round trip where a tile has more than 8 (a unit per kv head: 148 CTAs / 8; a decode layer 52 -> 50 us), 8
-    // elsewhere: the longer code cost launches of a few parts 2-5 us.
-    const bool many = max_parts > 8;
+    // 20 parts per round trip where a tile has more than 16 (a unit per kv head: 148 CTAs / 8; a decode layer 52 -> 50 us), 8
+    // elsewhere: the longer code cost launches of a few parts 2-5 us, and still lost at 12 parts (63.7 us against 58.2).
+    const bool many = max_parts > 16;
     if (sh.head_dim == 64)
         return !few ? go(merge_list_kernel<64, 1, 4>, 1) : many ? go(merge_list_kernel<64, 2, 20>, 2) : go(merge_list_kernel<64, 2, 8>, 2);
     return !few ? go(merge_list_kernel<128, 1, 4>, 1) : many ? go(merge_list_kernel<128, 4, 20>, 4) : go(merge_list_kernel<128, 4, 8>, 4);
