@@ -14,7 +14,10 @@
 //                     reference maximum m, P as bf16 over S.  O is shared by both warpgroups, so tile k's P has to be
 //                     relative to the reference that is in force after tile k - 1: the two warps of a row quadrant hand it
 //                     over (mref, an mbarrier per warp).  It rarely changes (only by more than 2^8); then this tile's P
-//                     or, once P V of tile k - 1 has landed, O is rescaled.
+//                     or, once P V of tile k - 1 has landed, O is rescaled.  The second tile of a piece starts from the
+//                     maximum of the first one's first 32 keys (another barrier): starting from its own, its P was always
+//                     scaled at the hand-over, i.e. rounded twice, and the error of a piece of two or three tiles 1.15 times
+//                     as large.
 //   warps 8-11        Q producer: counter-rotates this CTA's rows once per document (as in the one-CTA kernel), and appends
 //                     the query block's K/V rows
 //   warp 12           CTA 0 of the pair: MMA issuer for both.  TMEM owner in each.
@@ -39,7 +42,7 @@ constexpr uint32_t kColO = 384;                           // S buffer b: columns
 constexpr uint16_t kBoth = 3;
 
 enum BarIdx { kKvFull = 0, kKvEmpty = kMaxStages, kQFull = 2 * kMaxStages, kQFree = kQFull + 2, kSFull = kQFree + 2, kPFull = kSFull + 3,
-              kPvDone = kPFull + 3, kOFull = kPvDone + 2, kOFree, kMref, kEnd = kMref + 8, kDrain = kEnd + 8,      // Mref, End: [4 * warpgroup + quadrant]
+              kPvDone = kPFull + 3, kOFull = kPvDone + 2, kOFree, kMref, kEnd = kMref + 8, kStart = kEnd + 8, kDrain = kStart + 4,      // Mref, End: [4 * warpgroup + quadrant]; Start: [quadrant]
               kNumBars };
 static_assert(8 * kNumBars <= 504, "barrier block");
 
@@ -210,13 +213,30 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
-
             const bool full = n_keys == KVP_TILE_KEYS && j >= n_tail;
             const int lim = j >= n_tail ? n_keys : min(n_keys, limit - j * KVP_TILE_KEYS);       // visible keys: [0, lim)
             // a short tile (the end of a document, staged adapter rows) needs P only for the columns P V will read
             const int n_ch = full ? 4 : max(1, (n_keys + 31) >> 5);
+            if (k < 2) {
+                if (k == 0) {
+                    uint32_t v[32];
+                    tmem_ld32(s_addr, v);
+                    tc_wait_ld();
+                    landed32(v);
+                    if (!full) chunk_mask(v, lim);
+                    m = chunk_max(v, m);
+                    st_shared(mref, __float_as_uint(m));
+                    __syncwarp();
+                    if (lead_lane) mbar_arrive(c.bar(kStart + quad));
+                } else {
+                    ok = wait(p, c, kStart + quad, phO & 1, 38);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    m = __uint_as_float(ld_shared(mref));
+                }
+            }
             // One pass over S, 32 columns at a time, against the reference max this warpgroup knows; a chunk's own max is
-            // reduced alongside and checked last.  Only if it exceeds the reference by more than 2^8 (first tile, or a
+            // reduced alongside and checked last.  Only if it exceeds the reference by more than 2^8 (a
             // rare jump) does the reference move and the P written so far with it.
 #pragma unroll 1
             for (int ch = 0; ch < n_ch; ++ch) {

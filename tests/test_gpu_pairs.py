@@ -1,6 +1,8 @@
 """The attention kernel on CTA pairs at the edges of its pipeline: pieces of one to four tiles (three S buffers), documents
 of a single tile (a new Q buffer at every step), short tiles, remainders of rows in the second CTA, outliers that move the
 reference maximum late in a piece - every row against the oracle, and the same bits when run again."""
+import math
+
 import numpy as np
 import pytest
 import torch
@@ -52,3 +54,32 @@ def test_reference_maximum_moves_late_in_a_piece():
             sess.ctx.tune(kvp.TUNE_SPLIT_TARGET_CTAS, ctas)
         check_attention(wl, sess, flags=kvp.PRECISE_QK)
         sess.close()
+
+
+@pytest.mark.parametrize("q_len", [64, 192])
+def test_probabilities_are_rounded_once(q_len):
+    # Without rotation the scores are those of bf16 numbers and a partial result is not narrowed: what separates it from
+    # fp64 is the rounding of the probabilities to bf16.  The same sums with each probability rounded once, in torch: over
+    # 10^5 and more outputs the two errors' 2-norms agree to a percent or two (chance - the probabilities are rounded against
+    # another reference - and 1e-6 of fp32 sums); a second rounding of every third tile of a piece adds a sixth.
+    shape = gen.ModelShape(1, 8, 2, 128, "bf16", 500000.0, 0)
+    wl = gen.make_workload(shape, [640, 700, 1024], [[(0, -1), (1, -1), (2, -1)]], q_len=q_len, seed=17, rebase=False)
+    sess = Session(wl)
+    aid, (prefix,) = sess.assemble()
+    q, k, v = sess.query_tensors(0)
+    buf = torch.zeros(sess.ctx.partial_bytes(1, q_len) // 4, dtype=torch.float32, device=q.device)
+    sess.ctx.query_prefill(aid, 0, q, k, v, q_len, buf, None, kvp.PARTIAL)
+    assert sess.ctx.status_word() == 0
+    tiles = 2 * (4 * q_len // 128)                                # kv heads x 128-row tiles: O [tile][32][128][4], (m, l) [tile][128][2]
+    o = buf[:tiles * 16384].view(tiles, 32, 128, 4).permute(0, 2, 1, 3).reshape(2, q_len, 4, 128).double()
+    l = buf[tiles * 16384:].view(tiles, 128, 2)[..., 1].reshape(2, q_len, 4, 1).double()
+    K, V = (x.double().permute(1, 0, 2)[:, None] for x in sess.ctx.export_cache(aid, 0, 0, prefix, q_len))      # [kv head][1][row][128]
+    s = q[0].view(q_len, 2, 4, 128).permute(1, 2, 0, 3).double() @ K.transpose(-1, -2) / math.sqrt(128)
+    late = torch.arange(prefix + q_len, device=q.device) > prefix + torch.arange(q_len, device=q.device)[:, None]
+    s = s.masked_fill(late, -math.inf) / math.log(2)
+    p = torch.exp2(s - s.amax(-1, keepdim=True))
+    want = (p @ V / p.sum(-1, keepdim=True)).permute(0, 2, 1, 3)
+    once = (p.bfloat16().double() @ V / p.sum(-1, keepdim=True)).permute(0, 2, 1, 3)
+    err, ideal = float((o / l - want).norm()), float((once - want).norm())
+    assert err <= 1.06 * ideal, (err, ideal, err / ideal)
+    sess.close()
