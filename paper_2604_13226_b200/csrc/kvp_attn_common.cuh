@@ -275,6 +275,7 @@ __device__ __forceinline__ Work load_work(const Params &p, const kvp_work *works
 
 struct Tile {
     int row0, n_keys, src, rope;
+    uint32_t who;              // joint units: the requests that hold the tile, a bit each
 };
 
 // tile j of the unit's numbering.  Joint units: the causal tiles of request 0, 1, ..., then the joint prefix tiles, whose
@@ -289,6 +290,7 @@ __device__ __forceinline__ Tile get_tile(const Params &p, const Work &w, int j)
         t.n_keys = min(KVP_TILE_KEYS, p.q_pos0 + p.q_len - at);
         t.src = 1;
         t.rope = 0;
+        t.who = 1u << b;
     } else if (j < w.n_tail) {
         t.row0 = p.tail_direct ? j * KVP_TILE_KEYS : w.tail_row0 + j * KVP_TILE_KEYS;
         t.n_keys = min(KVP_TILE_KEYS, p.q_pos0 + w.q_len - j * KVP_TILE_KEYS);
@@ -300,6 +302,7 @@ __device__ __forceinline__ Tile get_tile(const Params &p, const Work &w, int j)
         t.n_keys = g.y & 0xFFFF;
         t.src = g.y >> 16;
         t.rope = g.z;
+        t.who = (uint32_t)g.w;
     }
     return t;
 }

@@ -81,6 +81,15 @@ __device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a, uint64_t b, uint3
         ::"r"(d), "r"(a), "l"(b), "r"(idesc), "r"(acc)
         : "memory");
 }
+// the same without the rows whose bit is set in (x, y, z, w), rows 0-31, 32-63, ...: they keep what they have
+__device__ __forceinline__ void mma_ts_rows(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t acc, const uint4 &off)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, {%5, %6, %7, %8}, p;\n\t}"
+        ::"r"(d), "r"(a), "l"(b), "r"(idesc), "r"(acc), "r"(off.x), "r"(off.y), "r"(off.z), "r"(off.w)
+        : "memory");
+}
 template <int ACC>
 __device__ __forceinline__ void mma_ts_c(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc)
 {
@@ -179,6 +188,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
     const uint32_t o_addr = c.tmem + lane_base + kColO + S * 128;
     const float c2 = p.scale_log2;
     uint32_t ph = 0;                                            // parities: bit 0 S full, bit 1 O full, bit 2 (m, l) full
+    uint32_t used = 0;                                          // joint units: pieces in which this stream had tiles
     bool ok = true;
 
     for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
@@ -231,6 +241,19 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
             const bool full = !JOINT && n_keys == KVP_TILE_KEYS && j >= n_tail;
             int lim = j >= n_tail ? n_keys : min(n_keys, limit - (JOINT ? j % n_per : j) * KVP_TILE_KEYS);     // visible keys: [0, lim)
             if (JOINT && !mine) lim = 0;
+            if (JOINT && k == 0) {
+                // P V leaves out the rows that do not hold a tile, so its first product does not set their O
+                if (__any_sync(0xffffffffu, !mine && row_b < p.joint_batch)) {
+                    if (used > 0) ok = mbar_wait(c.bar(C::kOFree + S), (used - 1) & 1, c.abort_flag(), p.status, 28 + S);   // the piece before has been read
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    tc_fence_after();
+                    uint32_t zero[32] = {};
+#pragma unroll 1
+                    for (int ch = 0; ch < D / 32; ++ch) tmem_st32(o_addr + ch * 32, zero);
+                }
+                ++used;
+            }
 
             // One pass over S, 32 columns at a time: the exponentials use the reference max carried over from earlier tiles;
             // a chunk's own max is reduced alongside and checked last, so that the two dependency chains overlap.  Only if it
@@ -493,6 +516,7 @@ __device__ __forceinline__ void tma_role(const Params &p, const Cta &c, const in
 struct MmaStream {
     uint32_t nP, nEpoch, nItems, qbuf;
     int prev_rope, prev_keys;
+    uint32_t prev_who;
     Tile cur, nxt;
 };
 
@@ -568,6 +592,7 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
         __syncwarp();
         ms.prev_rope = tl.rope;
         ms.prev_keys = tl.n_keys;
+        if (JOINT) ms.prev_who = tl.who;
         ms.cur = ms.nxt;
         if (k + 2 < n_steps) ms.nxt = get_tile<JOINT>(p, wq, stream_tile(wq, s, k + 2));
     };
@@ -698,6 +723,17 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
             ring_n += 2u * (uint32_t)w.n;
             continue;
         }
+        // Joint units: a row takes part in P V only where its request holds the tile.  P = 0 is not enough: one infinity or
+        // NaN among another request's values would make it NaN.
+        int req[4] = {};                                          // requests of the tile's rows lane, 32 + lane, ...
+        if (JOINT)
+            for (int i = 0; i < 4; ++i) req[i] = (32 * i + lane) / (p.group * p.q_len);
+        auto not_held = [&](uint32_t who) {
+            uint32_t m[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) m[i] = __ballot_sync(0xffffffffu, req[i] >= 32 || !(who >> (req[i] & 31) & 1u));
+            return make_uint4(m[0], m[1], m[2], m[3]);
+        };
         const int steps[2] = {w.steps0, w.steps1};
         const int max_steps = max(w.steps0, w.steps1);
         auto block = [&](auto s_c, int k) {
@@ -717,11 +753,16 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) return;
                 tc_fence_after();
+                const uint4 off = JOINT ? not_held(ms.prev_who) : uint4();
                 if (lead) {
                     const uint32_t v_lo = desc_lo(c.smem_base + C::kOffRing + stage * kTileBytes, kHalfBytes);
                     const uint32_t pa = c.tmem + kColS + s * 128;
                     const uint32_t oa = c.tmem + kColO + s * 128;
-                    if (ms.prev_keys == KVP_TILE_KEYS && k > 1) {
+                    if (JOINT) {
+                        const int ksteps = (ms.prev_keys + 15) >> 4;
+                        for (int kk = 0; kk < ksteps; ++kk)
+                            mma_ts_rows(oa, pa + p_col(kk), desc64(v_lo + kk * 128, kDescHi), idesc_pv, (k > 1 || kk > 0), off);
+                    } else if (ms.prev_keys == KVP_TILE_KEYS && k > 1) {
 #pragma unroll
                         for (int kk = 0; kk < 8; ++kk) {             // 16 keys per step: V advances 2048 bytes
                             mma_ts_c<1>(oa, pa + p_col(kk), desc64(v_lo + kk * 128, kDescHi), idesc_pv);

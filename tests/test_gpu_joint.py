@@ -1,7 +1,9 @@
 """Joint units: short calls of several requests over shared documents, whose rows share one query tile.  Steps against the
 oracle: batches of 2 to 32, groups of 1, 4 and 7, one and several tokens a step, a document that a request names twice,
 documents of a single key and of ragged lengths, causal tiles that a step enters, offsets of either sign and none."""
+import numpy as np
 import pytest
+import torch
 
 from paper_2604_13226_b200 import binding as kvp
 from paper_2604_13226_b200 import inputs as gen
@@ -50,3 +52,35 @@ def test_joint_only_where_it_saves():
         assert joint_used(sess, 8) == want
         check(wl, out, lse)
         sess.close()
+
+
+@pytest.mark.parametrize("group,steps", [(4, 3), (1, 2), (7, 4)])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_one_requests_values_stay_with_it(group, steps, bad):
+    # NaN or infinity among the values that only request 0 sees - a document of its own, rows it appends, a document it
+    # shares with request 2 - leaves every other request's bits alone.  (Not in the first 15 rows of a document: the last
+    # product over the document in front of it in the pool reaches that far, with weights of 0.)
+    shape = gen.ModelShape(1, 2 * group, 2, 128, "bf16", 500000.0, 0)
+    lens = [4096, 3000, 700, 130, 2048]
+    items = [[(0, 0), (2, 0), (4, -1)], [(0, 0), (1, 0)], [(1, -1), (0, 0), (4, 0)], [(0, -1), (1, 0), (3, 0)], [(1, 0), (0, 0)]]
+    outs = []
+    for poison in (None, "document", "appended", "shared"):
+        wl = gen.make_workload(shape, lens * 2, [it + [(p + 5, a) for p, a in it] for it in items], q_len=10 + steps, seed=9)
+        word = gen.to_stored(np.array([bad], dtype=np.float32), "bf16")[0]
+        if poison == "document":
+            wl.packets[2].v[0, [20, 131, 699], :, :] = word
+        elif poison == "shared":
+            wl.packets[9].v[0, 1027, :, 17] = word
+        elif poison == "appended":
+            wl.v_new[0][0, [3, 11], :, 40:] = word
+        sess = Session(wl)
+        sess.assemble()
+        outs.append(run_chunks(wl, sess, [(0, 10), (10, 10 + steps - 1), (10 + steps - 1, 10 + steps)])[0])
+        assert joint_used(sess, 2)
+        sess.close()
+    clean, rest = outs[0][:, 10:], [o[:, 10:] for o in outs[1:]]
+    assert torch.isfinite(clean).all()
+    for o, hit in zip(rest, ([0], [0], [0, 2])):
+        for b in range(5):
+            assert torch.equal(o[b], clean[b]) == (b not in hit), b
+            assert bool(torch.isfinite(o[b]).all()) == (b not in hit)
