@@ -414,6 +414,11 @@ __device__ __forceinline__ void produce_q_tile(const Params &p, char *qbuf, char
         } else {
             *reinterpret_cast<uint4 *>(lo) = make_uint4(0, 0, 0, 0);
             *reinterpret_cast<uint4 *>(lo + hi_off) = make_uint4(0, 0, 0, 0);
+            if (qrem != nullptr) {                           // (scores of what lay there before would move the warp's references)
+                char *rl = qrem + (lo - qbuf);
+                *reinterpret_cast<uint4 *>(rl) = make_uint4(0, 0, 0, 0);
+                *reinterpret_cast<uint4 *>(rl + hi_off) = make_uint4(0, 0, 0, 0);
+            }
         }
     }
     asm volatile("cp.async.wait_all;" ::: "memory");

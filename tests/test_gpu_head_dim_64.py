@@ -71,3 +71,22 @@ def test_continuation_and_raw_query_on_the_tensor_kernel():
     assert bool(((got - ref).abs() <= 2.0 ** -8 * ref.abs() + 1.6e-3).all())          # as above
     assert np.isfinite(lse.cpu().numpy()).all()
     sess.close()
+
+
+@pytest.mark.parametrize("q_len,batch", [(31, 8), (27, 8), (95, 4)])        # 124, 108 and 124 rows in a unit's last tile
+def test_the_same_bits_whatever_ran_before(q_len, batch):
+    # the rows that a query tile has beyond the request's share warps with the request's last ones: their scores must not
+    # depend on what shared memory held, or the probabilities next to them are taken apart into their two numbers again
+    shape = gen.ModelShape(1, 32, 8, 64, "bf16", 10000.0, 0)
+    lens = [2048, 1500, 900, 700]
+    wl = gen.make_workload(shape, lens, [[(p, 0) for p in range(4)]] * batch, q_len=q_len, seed=q_len)
+    sess = Session(wl)
+    sess.assemble()
+    q, k, v = sess.query_tensors(0)
+    want, want_lse = sess.prefill(0, qkv=(q, k, v))
+    for i in range(40):
+        sess.prefill(0, qkv=(q * 2.0 ** (i % 12), k, v))
+        out, lse = sess.prefill(0, qkv=(q, k, v))
+        assert sess.ctx.last_launch()["kind"] == 1
+        assert torch.equal(out, want) and torch.equal(lse, want_lse), i
+    sess.close()
