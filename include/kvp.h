@@ -14,6 +14,12 @@
  *   - "device" pointers are CUDA device addresses on the context's GPU, "host" pointers are ordinary
  *     host addresses; the library never allocates device memory: the caller lends it a pool and a
  *     workspace at kvp_create and keeps them alive until kvp_destroy;
+ *   - a context is used by one host thread at a time.  Its calls may go to several streams; the caller orders calls that
+ *     use one another's results (an assembly's prefills behind its assemble) and an assemble that takes the place of an
+ *     older assembly (max_assemblies) behind the work on that one.  fp32 calls, and bf16 calls with head_dim 64, need no
+ *     order beyond that; calls on one assembly run fastest on one stream (those on another one do without the space
+ *     for split key ranges).  bf16 calls with head_dim 128, and calls with KVP_ROPE_QUERY, share space of the context: they
+ *     have to be ordered among each other;
  *   - ids are dense int32 counted from 0 in registration order;
  *   - element type is the context's dtype (float32 or bfloat16) for every K/V/Q/out buffer.
  */

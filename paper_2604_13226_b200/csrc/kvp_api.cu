@@ -20,7 +20,7 @@ constexpr uint64_t kPlanAlign = 64;    // arrays of a plan blob
 inline uint64_t round_up(uint64_t x, uint64_t a) { return (x + a - 1) / a * a; }
 
 struct ws_layout {
-    uint64_t status, half_turns, slots, slot_stride, slot_plan, slot_sched, slot_k, slot_v, partial_o, partial_ml, arrived, q_scratch, total;
+    uint64_t status, half_turns, slots, slot_stride, slot_plan, slot_sched, slot_k, slot_v, own_o, own_ml, own_arrived, partial_o, partial_ml, q_scratch, total;
     uint64_t rows_bytes;
 };
 
@@ -101,6 +101,8 @@ kvp_plan_offsets plan_offsets(const kvp_assembly_host &as, size_t n_kept, int pl
     return p;
 }
 
+int own_slots(const kvp_config *c) { return c->dtype == KVP_DTYPE_BF16 && c->head_dim == 64 ? KVP_OWN_SLOTS_64 : KVP_OWN_SLOTS; }
+
 ws_layout workspace_layout(const kvp_config *c)
 {
     ws_layout w;
@@ -114,11 +116,14 @@ ws_layout workspace_layout(const kvp_config *c)
     w.slot_sched = round_up(p.total, kAlign);
     w.slot_k = round_up(w.slot_sched + schedule_layout(c).total * (c->max_compressed > 0 ? c->n_layers : 1), kAlign);
     w.slot_v = w.slot_k + w.rows_bytes;
-    w.slot_stride = w.slot_v + w.rows_bytes;
+    w.own_o = w.slot_v + w.rows_bytes;
+    w.own_ml = round_up(w.own_o + (uint64_t)own_slots(c) * KVP_TILE_ROWS * c->head_dim * 4, kAlign);
+    w.own_arrived = round_up(w.own_ml + (uint64_t)own_slots(c) * KVP_TILE_ROWS * 8, kAlign);
+    w.slot_stride = round_up(w.own_arrived + 4ull * KVP_CORE_UNITS, kAlign);
     w.slots = o;    o += w.slot_stride * c->max_assemblies;
-    w.partial_o = o;  o = round_up(o + (uint64_t)KVP_MAX_SPLIT_UNITS * KVP_TILE_ROWS * c->head_dim * 4, kAlign);
-    w.partial_ml = o; o = round_up(o + (uint64_t)KVP_MAX_SPLIT_UNITS * KVP_TILE_ROWS * 8, kAlign);
-    w.arrived = o;    o = round_up(o + 4ull * KVP_CORE_UNITS, kAlign);
+    const uint64_t shared = c->dtype == KVP_DTYPE_BF16 && c->head_dim == 128 ? KVP_MAX_SPLIT_UNITS : 0;
+    w.partial_o = o;  o = round_up(o + shared * KVP_TILE_ROWS * c->head_dim * 4, kAlign);
+    w.partial_ml = o; o = round_up(o + shared * KVP_TILE_ROWS * 8, kAlign);
     w.q_scratch = o;  o = round_up(o + (uint64_t)c->max_batch * c->max_query_tokens * c->n_q_heads * c->head_dim * e, kAlign);
     w.total = o;
     return w;
@@ -395,6 +400,7 @@ int32_t plan_schedule(kvp_ctx *ctx, const kvp_assembly_host &as, int layer, int 
     int G = std::min(ctx->sm_count, kMaxCtas);
     if (ctx->split_target_ctas > 0) G = std::min(ctx->split_target_ctas, kMaxCtas);
     if (out.pair) G /= 2;                                         // entries of cta_begin are pairs
+    if (sh.head_dim == 64) G = std::min(G, KVP_OWN_SLOTS_64 / 4); // a cut between two CTAs splits one unit, into at most four slots more
     const bool no_split = ctx->force_splits == 1;               // cuts only between units
 
     // Cut positions (unit, tile), non-decreasing.  A run of units is dealt out to g CTAs one after the other, each
@@ -602,7 +608,7 @@ int32_t plan_schedule(kvp_ctx *ctx, const kvp_assembly_host &as, int layer, int 
         if (u.mode == 0) works[i].slot1 = works[i].slot0 + u.n_pieces;
     }
     if (n_ctas > kMaxCtas || (int)works.size() > ctx->sched_max_works || (int)merges.size() > ctx->sched_max_merges ||
-        n_slots > KVP_MAX_SPLIT_UNITS)
+        n_slots > (sh.head_dim == 64 ? KVP_OWN_SLOTS_64 : KVP_MAX_SPLIT_UNITS))
         return fail(ctx, KVP_ERR_CAPACITY, "query_prefill: work list overflow (%d ctas, %zu pieces, %zu merges, %d slots)",
                     n_ctas, works.size(), merges.size(), n_slots);
 
@@ -676,6 +682,20 @@ bool same_causal_tiles(const kvp_shape &sh, int q_len, int from, int to)
         if ((from + last) / KVP_TILE_KEYS != (to + last) / KVP_TILE_KEYS) return false;
     }
     return true;
+}
+
+// Whether the assembly's scratch is this call's to use: that of the first stream that did.  Calls of one assembly on several
+// streams, which nothing orders, work without it: the CUDA-core kernel with whole key ranges.  (The scratch of one context
+// would not do for two assemblies on two streams: with counters that both add to, a block takes another's rows for its own.)
+bool owns_scratch(kvp_assembly_host &as, cudaStream_t st)
+{
+    unsigned long long id = 0;
+    if (st == cudaStreamPerThread || cudaStreamGetId(st, &id) != cudaSuccess) return false;
+    if (!as.owned) {
+        as.owned = true;
+        as.owner = id;
+    }
+    return as.owner == id;
 }
 
 thread_local std::string g_create_error;
@@ -767,10 +787,10 @@ int32_t kvp_create(const kvp_config *cfg, kvp_ctx **out)
         ctx->slot_sched_dev.push_back(s + w.slot_sched);
         ctx->slot_k.push_back(s + w.slot_k);
         ctx->slot_v.push_back(s + w.slot_v);
+        ctx->slot_own.push_back({(float *)(s + w.own_o), (float2 *)(s + w.own_ml), (int32_t *)(s + w.own_arrived)});
     }
     ctx->partial_o = (float *)(ws + w.partial_o);
     ctx->partial_ml = (float2 *)(ws + w.partial_ml);
-    ctx->arrived = (int32_t *)(ws + w.arrived);
     ctx->q_scratch = ws + w.q_scratch;
 
     // angles are formed on the device as (position offset) x (theta_i / pi), in half turns: sincospi reduces exactly
@@ -1061,6 +1081,7 @@ static int32_t assemble_impl(kvp_ctx *ctx, int32_t batch, const int32_t *slot_of
     as.sched.clear();
     as.joint.state = -1;
     as.settled = false;
+    as.owned = false;
     as.ragged = false;
     as.last_q_len = 0;
     as.flags = flags;
@@ -1372,6 +1393,15 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
         return fail(ctx, KVP_ERR_UNSUPPORTED, "query_prefill: KVP_ROPE_QUERY on an assembly made by kvp_assemble_at (the query's position is not prefix_len)");
     const bool skip_block = (flags & KVP_SKIP_QUERY_BLOCK) != 0;
 
+    // whether the work list made last also serves this call
+    const auto list_serves = [&](uint32_t list_opts) {
+        if (as.sched.empty()) return false;
+        const kvp_assembly_host::sched_state &ss = as.sched[as.item_stride ? layer : 0];
+        const bool same_lens = q_lens ? (ss.q_lens.size() == (size_t)as.batch && std::equal(q_lens, q_lens + as.batch, ss.q_lens.begin()))
+                                      : ss.q_lens.empty();
+        return ss.q_len == q_len && ss.ctas != 0 && same_lens && ss.opts == list_opts &&
+               (ss.q_pos0 == q_pos0 || (!q_lens && same_causal_tiles(sh, q_len, ss.q_pos0, q_pos0)));
+    };
     int launches = 0;
     bool fast = ctx->have_tma && !(flags & KVP_FORCE_SIMPLE);
     if (fast && sh.head_dim == 64) {
@@ -1381,8 +1411,14 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
         double keys = 0.0;
         for (int b = 0; b < as.batch; ++b) keys += as.items[b].prefix_len + q_pos0 + q_len;
         const double rows = (double)(((int64_t)sh.group * q_len + 15) / 16 * 16);
-        fast = 4.0 * sh.head_dim * sh.n_kv_heads * rows * keys >= kTcMinFlops64 && (((uintptr_t)q | (uintptr_t)out) & 15) == 0;
+        fast = 4.0 * sh.head_dim * sh.n_kv_heads * rows * keys >= kTcMinFlops64 && (((uintptr_t)q | (uintptr_t)out) & 15) == 0 &&
+               owns_scratch(as, st);
+        if (fast && !list_serves(0)) {                             // a list that is recorded would be read again at every replay
+            cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+            fast = cudaStreamIsCapturing(st, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone;
+        }
     }
+    const kvp_scratch &own = ctx->slot_own[slot];
     if (q_lens && !(tc128 && fast)) return fail(ctx, KVP_ERR_UNSUPPORTED, "query_prefill_ragged: needs the tcgen05 kernel (bf16, head_dim 128, sm_100)");
     // plain prefill on the two-stream kernel: it reads the query block's K/V from k_new / v_new and appends them itself
     kvp_attn2_args a;
@@ -1416,8 +1452,8 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
         int32_t n_tiles = 0;
         for (const kvp_item &it : as.items) n_tiles = std::max(n_tiles, it.tile_end - it.tile_begin);
         n_tiles += (q_pos0 + q_len - 1) / KVP_TILE_KEYS + 1;
-        const kvp_core_ws cw = {ctx->partial_o, ctx->partial_ml, ctx->arrived, (int64_t)KVP_MAX_SPLIT_UNITS * KVP_TILE_ROWS,
-                                KVP_CORE_UNITS, ctx->sm_count, core_append ? k_new : nullptr, core_append ? v_new : nullptr,
+        const kvp_core_ws cw = {own.partial_o, own.partial_ml, own.arrived,
+                                owns_scratch(as, st) ? (int64_t)own_slots(&ctx->cfg) * KVP_TILE_ROWS : 0, KVP_CORE_UNITS, ctx->sm_count, core_append ? k_new : nullptr, core_append ? v_new : nullptr,
                                 ctx->slot_k[slot], ctx->slot_v[slot]};
         KVP_CUDA(ctx, kvp_launch_attn_core(sh, plan, as.batch, q_len, q_pos0, layer, q_used, ctx->pool_k, ctx->pool_v,
                                            ctx->slot_k[slot], ctx->slot_v[slot], n_tiles, cw, out, lse, &ctas, st));
@@ -1427,18 +1463,15 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
     } else {
         const int li = as.item_stride ? layer : 0;
         if (as.sched.empty()) as.sched.resize(as.item_stride ? ctx->cfg.n_layers : 1);
-        const bool same_lens = q_lens ? (as.sched[li].q_lens.size() == (size_t)as.batch &&
-                                          std::equal(q_lens, q_lens + as.batch, as.sched[li].q_lens.begin()))
-                                       : as.sched[li].q_lens.empty();
         const bool joint = !pairs && !q_lens && !part_opts && !a.tail_direct && !a.precise && use_joint(ctx, as, q_len);
         const uint32_t list_opts = part_opts | (joint ? kOptJoint : 0);
         a.fresh = 0;
         a.list = nullptr;
         a.list_bytes = a.list_works = 0;
         a.list_dev = nullptr;
-        if (as.sched[li].q_len != q_len || as.sched[li].ctas == 0 || !same_lens ||
-            (as.sched[li].q_pos0 != q_pos0 && (q_lens || !same_causal_tiles(sh, q_len, as.sched[li].q_pos0, q_pos0))) ||
-            as.sched[li].opts != list_opts) {
+        float *const part_o = sh.head_dim == 64 ? own.partial_o : ctx->partial_o;
+        float2 *const part_ml = sh.head_dim == 64 ? own.partial_ml : ctx->partial_ml;
+        if (!list_serves(list_opts)) {
             const int32_t rc = build_schedule(ctx, as, slot, layer, q_len, q_pos0, q_lens, list_opts, a, st);
             if (rc != KVP_OK) return rc;
         }
@@ -1462,8 +1495,8 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
         a.q = q_used;
         a.out = out;
         a.lse = lse;
-        a.partial_o = ctx->partial_o;
-        a.partial_ml = ctx->partial_ml;
+        a.partial_o = part_o;
+        a.partial_ml = part_ml;
         a.status = ctx->status_dev;
         if (ss.ctas > 0) {                                         // (a rank may hold no key of any request)
             KVP_CUDA(ctx, time_edge(ctx, 0, 0, st));
@@ -1481,7 +1514,7 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
             const int64_t n_rt = ((int64_t)sh.group * q_len + KVP_TILE_ROWS - 1) / KVP_TILE_ROWS;
             KVP_CUDA(ctx, kvp_launch_merge_list(sh, q_len, ss.merges, ss.slots,
                                                 reinterpret_cast<const kvp_merge_item *>(sd + ss.off_merges), ss.ctas > 0,
-                                                ctx->partial_o, ctx->partial_ml, out, lse, partial ? out : nullptr,
+                                                part_o, part_ml, out, lse, partial ? out : nullptr,
                                                 (int64_t)as.batch * sh.n_kv_heads * n_rt, st));
             ++launches;
         }

@@ -15,6 +15,10 @@
 #define KVP_CHUNK_ROWS 32      // rows per gather work item
 #define KVP_MAX_SPLIT_UNITS 2048   // partial slots (128 query rows each) in the workspace
 #define KVP_CORE_UNITS 2048        // row tiles the CUDA-core kernel may split
+// Partial slots that every assembly has to itself: 320 hold what the CUDA-core kernel splits (148 x 2 CTAs of 64 rows, or 4
+// of 16, and as many row tiles again), 640 also the four per CTA of the tensor kernel with head dimension 64.
+#define KVP_OWN_SLOTS 320
+#define KVP_OWN_SLOTS_64 640
 #define KVP_SCHED_RING 8       // pinned staging buffers for work lists
 // Plans and work lists up to the first size travel as parameters of the kernel that needs them first: an upload kernel in
 // front costs 4 us on the way to the first tile, 4 KB of parameters next to nothing (one request of 5 documents x 512 tokens,
@@ -171,6 +175,10 @@ struct kvp_assembly_host {
     std::vector<sched_state> sched;
     kvp_joint joint;
     bool settled = false;                  // an attention launch has waited for the plan
+    // the stream (by its id, no handle is kept) whose calls use the assembly's scratch: its partial slots and counters and,
+    // with head dimension 64, its work list
+    bool owned = false;
+    unsigned long long owner = 0;
 };
 
 // Work list of the two-stream kernel for one assembly and query length, with the scratch it is built in.
@@ -187,6 +195,13 @@ struct kvp_schedule {
     std::vector<int64_t> after;
     std::vector<int32_t> order;            // emission order of the CTAs (indices into cuts)
     std::vector<int32_t> work_unit;        // unit of every piece
+};
+
+// Partial results of split key ranges, and the counters of the CUDA-core kernel's split row tiles.
+struct kvp_scratch {
+    float *partial_o;
+    float2 *partial_ml;
+    int32_t *arrived;
 };
 
 struct kvp_ctx {
@@ -212,6 +227,7 @@ struct kvp_ctx {
     kvp_plan_layout pl;
     std::vector<char *> slot_plan_dev;     // per assembly slot
     std::vector<char *> slot_k, slot_v;    // per assembly slot: workspace rows
+    std::vector<kvp_scratch> slot_own;     // per assembly slot
     std::vector<char *> slot_sched_dev;    // per assembly slot: cta ranges, work list, merge list
     // pinned staging of the same: a ring, so that the layers of an assembly with a list each, or the steps of a
     // decode, do not wait for one another's upload (which lies behind the attention kernels enqueued before it)
@@ -227,9 +243,9 @@ struct kvp_ctx {
     kvp_schedule plan;
     int32_t fused_append = 1;              // plain prefill: the attention kernel reads k_new / v_new itself and appends them
     void *encode_tiled = nullptr;          // cuTensorMapEncodeTiled
-    float *partial_o = nullptr;            // [units][128][head_dim]
-    float2 *partial_ml = nullptr;          // [units][128] (running max, running sum)
-    int32_t *arrived = nullptr;            // counters of the CUDA-core kernel's split row tiles
+    // bf16 with head dimension 128, all assemblies together: [units][128][head_dim]; [units][128] (running max, running sum)
+    float *partial_o = nullptr;
+    float2 *partial_ml = nullptr;
     char *q_scratch = nullptr;
     float2 *q_rope = nullptr;              // [max_batch*max_query][head_dim/2] for KVP_ROPE_QUERY
 
