@@ -871,10 +871,28 @@ int32_t kvp_destroy(kvp_ctx *ctx)
     return KVP_OK;
 }
 
+// A registration on `st` writes the pool.
+static void note_registration(kvp_ctx *ctx, cudaStream_t st)
+{
+    std::vector<cudaStream_t> &on = ctx->registered_on;
+    if (std::find(on.begin(), on.end(), st) != on.end()) return;
+    if (on.size() < 32) on.push_back(st); else ctx->registered_anywhere = true;
+}
+// Whether `st` has a registration on it that no assemble has come behind yet.
+static bool take_registration(kvp_ctx *ctx, cudaStream_t st)
+{
+    std::vector<cudaStream_t> &on = ctx->registered_on;
+    const auto it = std::find(on.begin(), on.end(), st);
+    if (it == on.end()) return ctx->registered_anywhere;
+    on.erase(it);
+    return true;
+}
+
 static int32_t store_segment(kvp_ctx *ctx, const void *k, const void *v, int32_t n, cudaStream_t st)
 {
     if (n == 0 || ctx->host_only) return KVP_OK;
     const kvp_shape &sh = ctx->shape;
+    note_registration(ctx, st);
     KVP_CUDA(ctx, kvp_launch_store_rows(sh, k, ctx->pool_k, sh.pool_rows, ctx->pool_rows_used, n, st));
     KVP_CUDA(ctx, kvp_launch_store_rows(sh, v, ctx->pool_v, sh.pool_rows, ctx->pool_rows_used, n, st));
     return KVP_OK;
@@ -1007,6 +1025,7 @@ int32_t kvp_register_packet_compressed(kvp_ctx *ctx, const void *k, const void *
     if (!ctx->host_only) {
         // plane (l, h) receives its run of kept rows; the runs lie back to back in the caller's buffers
         cudaStream_t st = (cudaStream_t)stream;
+        note_registration(ctx, st);
         KVP_CUDA(ctx, cudaSetDevice(ctx->cfg.device));
         const size_t row_bytes = (size_t)sh.head_dim * sh.elem_bytes;
         size_t src_off = 0;
@@ -1282,7 +1301,7 @@ static int32_t assemble_impl(kvp_ctx *ctx, int32_t batch, const int32_t *slot_of
         KVP_CUDA(ctx, time_edge(ctx, 1, 0, st));
         KVP_CUDA(ctx, kvp_launch_gather(ctx->shape, plan_dev(ctx, slot), n_chunks, n_rope, ctx->half_turns, ctx->pool_k,
                                         ctx->pool_v, ctx->slot_k[slot], ctx->slot_v[slot], blob, blob_bytes,
-                                        ctx->slot_plan_dev[slot], st));
+                                        ctx->slot_plan_dev[slot], !take_registration(ctx, st), st));
         ctx->slots[slot].id = id;                                 // from here on the device has the plan
         KVP_CUDA(ctx, time_edge(ctx, 1, 1, st));
     }

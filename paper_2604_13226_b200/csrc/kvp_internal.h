@@ -220,6 +220,9 @@ struct kvp_ctx {
     bool loads_recorded = false;
     std::vector<kvp_segment_host> adapter_h, adapter_t;
     int64_t pool_rows_used = 0;
+    // streams (compared, never used) that a registration was enqueued on and no assemble since
+    std::vector<cudaStream_t> registered_on;
+    bool registered_anywhere = false;               // more of them than are kept count of
 
     // device memory carved out of the caller's buffers
     char *pool_k = nullptr, *pool_v = nullptr;
@@ -277,8 +280,9 @@ struct kvp_ctx {
 // a kernel may have written just before or writes anything, so that launch latency and set-up - barriers, TMEM, filling
 // the grid - lie under the predecessor's tail.  Some thread of every block waits before the block can end, so a grid that
 // has ended implies that its predecessors have: later work in the stream needs no more than that.
-// Readable without waiting: the pool - its writers (registration, host copies) never release a successor early, so
-// whatever starts after them finds it complete - and tables that a kernel further in front has waited for before it
+// Readable without waiting: the pool - its writers (registration, host copies) never release a successor early, and between
+// them and whatever reads their rows lies a launch that waits for them: the gather (right behind a registration on its
+// stream it is launched in plain stream order; its successors start after it has) or a stream wait - and tables that a kernel further in front has waited for before it
 // released anyone: the attention kernel behind a fresh work list waits first and releases then, so that the launches
 // behind it find that list and the plan complete.
 #ifdef __CUDACC__
@@ -290,7 +294,7 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 
 template <typename T> struct as_given { typedef T type; };
 template <typename... P>
-cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, const typename as_given<P>::type &...args)
+cudaError_t launch_when(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, const typename as_given<P>::type &...args)
 {
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -301,9 +305,14 @@ cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = early ? 1 : 0;
     void *ptrs[] = {(void *)&args...};
     return cudaLaunchKernelExC(&cfg, (const void *)kernel, ptrs);
+}
+template <typename... P>
+cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, const typename as_given<P>::type &...args)
+{
+    return launch_when(true, kernel, grid, block, smem, st, args...);
 }
 
 // Tables that travel as a kernel's own parameters.  N = 0: none.
@@ -334,10 +343,10 @@ cudaError_t kvp_launch_load(const kvp_shape &sh, kvp_load_list &list, int32_t la
 cudaError_t kvp_launch_upload(const void *host, void *dst, uint64_t bytes, volatile uint32_t *flags, uint32_t seq,
                               int32_t *blocks, cudaStream_t st);
 // the rope table of an assembly and the gather of its chunks, one launch; blob not null: the plan (blob_bytes) comes along and
-// the launch stores it at blob_dev, where `plan` points
+// the launch stores it at blob_dev, where `plan` points.  early: it may begin before the kernel in front has ended
 cudaError_t kvp_launch_gather(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t n_chunks, int32_t n_rope,
                               const double *half_turns, const char *pool_k, const char *pool_v, char *ws_k, char *ws_v,
-                              const void *blob, uint32_t blob_bytes, char *blob_dev, cudaStream_t st);
+                              const void *blob, uint32_t blob_bytes, char *blob_dev, bool early, cudaStream_t st);
 // plan_there: the plan was complete before the launch in front of this one was released
 cudaError_t kvp_launch_append(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t plan_there, int32_t batch, int32_t q_len,
                               int32_t q_pos0, const void *q, const void *k_new, const void *v_new, char *ws_k, char *ws_v,

@@ -222,7 +222,7 @@ __device__ __forceinline__ float2 offset_cos_sin(int32_t offset, double half_tur
 // rows; a thread has the loads of two (row, plane) pairs in flight.
 // With LB > 0 the plan comes along as a parameter: it is read from there, and block 0 stores it for everyone behind.  Then
 // nothing that leads up to a block's first stores has to wait for the kernel in front: the angles and the rows of the pool
-// are there by the time it ends.
+// are there by the time it ends (behind a registration, which writes them, the launch waits as a whole).
 template <typename T, int LB>
 __global__ void __launch_bounds__(256)
 gather_kernel(kvp_plan_dev plan, const __grid_constant__ kvp_blob<LB> blob, int blob_words, uint4 *blob_dev, int n_table,
@@ -980,7 +980,7 @@ cudaError_t kvp_launch_upload(const void *host, void *dst, uint64_t bytes, volat
 
 cudaError_t kvp_launch_gather(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t n_chunks, int32_t n_rope,
                               const double *half_turns, const char *pool_k, const char *pool_v, char *ws_k, char *ws_v,
-                              const void *blob, uint32_t blob_bytes, char *blob_dev, cudaStream_t st)
+                              const void *blob, uint32_t blob_bytes, char *blob_dev, bool early, cudaStream_t st)
 {
     static_assert(KVP_INLINE_SMALL <= 256 * 16, "one word per thread of a block");
     const int vecs = sh.head_dim * sh.elem_bytes / 16, half = sh.head_dim / 2;
@@ -996,7 +996,7 @@ cudaError_t kvp_launch_gather(const kvp_shape &sh, const kvp_plan_dev &plan, int
     const int grid = n_table + n_chunks * groups;
     float2 *table = const_cast<float2 *>(plan.rope);
     auto go = [&](auto *kernel, const auto &b) {
-        return launch_pdl(kernel, grid, 256, 0, st, plan, b, (int)((blob_bytes + 15) / 16), (uint4 *)blob_dev, n_table, n_rope, groups,
+        return launch_when(early, kernel, grid, 256, 0, st, plan, b, (int)((blob_bytes + 15) / 16), (uint4 *)blob_dev, n_table, n_rope, groups,
                           half_turns, table, pool_k, pool_v, ws_k, ws_v, sh.pool_rows, sh.ws_rows, vecs, half, sh.pairing);
     };
     const auto *small = reinterpret_cast<const kvp_blob<KVP_INLINE_SMALL> *>(blob);
