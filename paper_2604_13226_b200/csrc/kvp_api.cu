@@ -225,17 +225,17 @@ int find_slot(kvp_ctx *ctx, int32_t assembly_id)
 }
 
 // Waits until the last upload from a staging buffer has read it.  That is nearly always so already; otherwise the flags
-// are polled, and after a while the stream is asked as well, so that an upload that never ran (an error on the device, a
-// stream that is being captured) ends the wait with an error.
+// are polled, and after a while the context's own stream is asked as well, so that an error on the device ends the wait.
+// (The caller's stream may be gone by then: destroying it does not take back what was enqueued.)
 int32_t stage_wait(kvp_ctx *ctx, kvp_stage &sg)
 {
+    if (sg.recorded) return fail(ctx, KVP_ERR_CUDA, "staging buffer in use: an upload from it was recorded into a graph");
     for (int b = 0; b < sg.blocks; ++b)
         for (uint32_t polls = 1; sg.flags[b] != sg.seq; ++polls) {
             if (polls % 4096) continue;
-            const cudaError_t rc = cudaStreamQuery(sg.stream);
-            if (rc == cudaErrorNotReady) continue;
-            if (rc != cudaSuccess) return fail(ctx, KVP_ERR_CUDA, "waiting for an upload: %s", cudaGetErrorString(rc));
-            if (sg.flags[b] != sg.seq) return fail(ctx, KVP_ERR_CUDA, "waiting for an upload: it was never run");
+            const cudaError_t rc = cudaStreamQuery(ctx->load_stream);
+            if (rc != cudaSuccess && rc != cudaErrorNotReady)
+                return fail(ctx, KVP_ERR_CUDA, "waiting for an upload: %s", cudaGetErrorString(rc));
         }
     return KVP_OK;
 }
@@ -244,11 +244,14 @@ cudaError_t stage_upload(kvp_stage &sg, char *dst, uint64_t bytes, cudaStream_t 
 {
     sg.blocks = 0;
     int32_t blocks = 0;
-    const cudaError_t rc = kvp_launch_upload(sg.host, dst, bytes, sg.flags, sg.seq + 1, &blocks, st);
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    cudaError_t rc = cudaStreamIsCapturing(st, &capture);
+    if (rc != cudaSuccess) return rc;
+    rc = kvp_launch_upload(sg.host, dst, bytes, sg.flags, sg.seq + 1, &blocks, st);
     if (rc != cudaSuccess) return rc;
     ++sg.seq;
     sg.blocks = blocks;
-    sg.stream = st;
+    sg.recorded = capture != cudaStreamCaptureStatusNone;
     return cudaSuccess;
 }
 

@@ -133,7 +133,7 @@ struct kvp_stage {
     volatile uint32_t *flags = nullptr;    // [KVP_UPLOAD_BLOCKS]
     uint32_t seq = 0;                      // number of the last upload from here
     int32_t blocks = 0;                    // and its blocks
-    cudaStream_t stream = nullptr;         // and its stream
+    bool recorded = false;                 // it was recorded into a graph, which reads the buffer whenever it is launched
 };
 
 // ---- host-side context -----------------------------------------------------------------------
