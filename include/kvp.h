@@ -131,13 +131,15 @@ KVP_API int32_t kvp_register_packet(kvp_ctx *ctx, const void *k, const void *v, 
  * Register one packet whose K/V stay in host memory until a request uses it (the CPU-to-GPU cache transfer
  * that the paper counts inside time-to-first-token, Section 4.3).  Pool rows are reserved now; nothing is copied.
  * The first kvp_assemble that names the packet enqueues the copy on a stream the context owns, layer by layer (one
- * kernel per layer reads the packets over the host link; unpinned buffers are copied by the driver instead),
+ * kernel per layer reads the packets over the host link; buffers that are not in one pinned range, or not 16-byte
+ * aligned, are copied by the driver instead),
  * and kvp_query_prefill(layer) makes its stream wait for that layer only: the transfer of layer l+1 runs while
  * layer l is attended to.  After that the packet is resident like any other, until kvp_evict_packet.
- *   k_host, v_host   host, layout [n_layers][n_kv_heads][n_tokens][head_dim] (the pool's own plane order, so a
- *                    layer of a packet is one strided copy); k post-RoPE for positions cache_pos0 + t.  The
- *                    buffers stay with the caller and must remain valid while the packet is registered; pinned
- *                    memory is needed for the copies to overlap anything.
+ *   k_host, v_host   host, layout [n_layers][n_kv_heads][n_tokens][head_dim] (the pool's own plane order); k
+ *                    post-RoPE for positions cache_pos0 + t.  The buffers stay with the caller and must remain
+ *                    valid while the packet is registered, and as they are - pinned or not - while a copy is under
+ *                    way; pinned memory is needed for the copies to overlap anything.  Whether they are pinned is
+ *                    looked at by every assemble that copies them.
  * In a host-only context the pointers may be NULL.  Not available for compressed packets.
  * Errors: INVALID, CAPACITY (max_packets or pool full).
  */

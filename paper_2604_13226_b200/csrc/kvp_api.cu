@@ -144,7 +144,10 @@ int32_t fail(kvp_ctx *ctx, int32_t code, const char *fmt, ...)
 #define KVP_CUDA(ctx, call)                                                                              \
     do {                                                                                                 \
         cudaError_t e_ = (call);                                                                         \
-        if (e_ != cudaSuccess) return fail(ctx, KVP_ERR_CUDA, "%s: %s", #call, cudaGetErrorString(e_));  \
+        if (e_ != cudaSuccess) {                                                                         \
+            (void)cudaGetLastError();      /* reported here, not to whoever asks next */                 \
+            return fail(ctx, KVP_ERR_CUDA, "%s: %s", #call, cudaGetErrorString(e_));                     \
+        }                                                                                                \
     } while (0)
 
 typedef CUresult (*encode_tiled_fn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -829,6 +832,12 @@ int32_t kvp_create(const kvp_config *cfg, kvp_ctx **out)
         if (cudaEventCreateWithFlags(&ctx->load_done[l], cudaEventDisableTiming) != cudaSuccess)
             return bail(KVP_ERR_CUDA, "load event creation failed");
 
+    {
+        void *fn = nullptr;                    // (without it host packets are copied by the driver)
+        cudaDriverEntryPointQueryResult qres;
+        if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &fn, cudaEnableDefault, &qres) == cudaSuccess && qres == cudaDriverEntryPointSuccess)
+            ctx->pointer_attributes = fn;
+    }
     if (kvp_attn_core_prepare(sh) != cudaSuccess) return bail(KVP_ERR_CUDA, "CUDA-core kernel attribute setup failed");
     if (sh.dtype == KVP_DTYPE_BF16 && cc_major == 10) {
         void *fn = nullptr;
@@ -918,17 +927,23 @@ int32_t kvp_register_packet(kvp_ctx *ctx, const void *k, const void *v, int32_t 
     return KVP_OK;
 }
 
-// The device address of a host buffer that is pinned from its first to its last byte and 16-byte aligned; else nullptr.
-static const char *pinned_address(const void *host, size_t bytes)
+// The device address of a host buffer that lies in one pinned range, now, and is 16-byte aligned; else nullptr.  Asked at
+// every load (0.3 us): a buffer may have been pinned or unpinned since it was registered.
+static const char *pinned_address(const kvp_ctx *ctx, const void *host, size_t bytes)
 {
-    cudaPointerAttributes first, last;
-    if (((uintptr_t)host & 15) == 0 && cudaPointerGetAttributes(&first, host) == cudaSuccess && first.type == cudaMemoryTypeHost &&
-        first.devicePointer && cudaPointerGetAttributes(&last, (const char *)host + bytes - 1) == cudaSuccess &&
-        last.type == cudaMemoryTypeHost && (char *)last.devicePointer == (char *)first.devicePointer + bytes - 1 &&
-        ((uintptr_t)first.devicePointer & 15) == 0)
-        return (const char *)first.devicePointer;
-    (void)cudaGetLastError();
-    return nullptr;
+    typedef CUresult (*attributes_fn)(unsigned int, CUpointer_attribute *, void **, CUdeviceptr);
+    CUpointer_attribute what[4] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                   CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    unsigned int type = 0;
+    CUdeviceptr device = 0, start = 0;
+    size_t size = 0;
+    void *to[4] = {&type, &device, &start, &size};
+    if (((uintptr_t)host & 15) || !ctx->pointer_attributes ||
+        ((attributes_fn)ctx->pointer_attributes)(4, what, to, (CUdeviceptr)(uintptr_t)host) != CUDA_SUCCESS)
+        return nullptr;
+    const uintptr_t at = (uintptr_t)host - (uintptr_t)start;     // (memory that is not pinned has type 0)
+    return type == CU_MEMORYTYPE_HOST && device && (device & 15) == 0 && start <= (CUdeviceptr)(uintptr_t)host && at + bytes <= size
+               ? (const char *)(uintptr_t)device : nullptr;
 }
 
 int32_t kvp_register_packet_host(kvp_ctx *ctx, const void *k_host, const void *v_host, int32_t n_tokens,
@@ -947,12 +962,6 @@ int32_t kvp_register_packet_host(kvp_ctx *ctx, const void *k_host, const void *v
     src.v = (const char *)v_host;
     src.from_host = true;
     src.resident = false;
-    if (!ctx->host_only) {
-        // what kernels may read themselves: pinned buffers, aligned for bulk copies
-        const size_t bytes = (size_t)ctx->shape.n_layers * ctx->shape.n_kv_heads * n_tokens * ctx->shape.head_dim * ctx->shape.elem_bytes;
-        src.dev_k = pinned_address(k_host, bytes);
-        src.dev_v = pinned_address(v_host, bytes);
-    }
     *packet_id = (int32_t)ctx->packets.size() - 1;
     return KVP_OK;
 }
@@ -979,14 +988,22 @@ static int32_t load_host_packets(kvp_ctx *ctx, const std::vector<int32_t> &ids, 
     // the rows may still be read by work the caller enqueued before (a packet that was evicted)
     KVP_CUDA(ctx, cudaEventRecord(ctx->load_fence, st));
     KVP_CUDA(ctx, cudaStreamWaitEvent(ctx->load_stream, ctx->load_fence, 0));
+    // what kernels may read themselves: pinned buffers, aligned for bulk copies
+    std::vector<std::pair<const char *, const char *>> dev;
+    for (int32_t id : ids) {
+        const kvp_ctx::host_src &src = ctx->packet_src[id];
+        const size_t bytes = (size_t)sh.n_layers * sh.n_kv_heads * ctx->packets[id].n * row_bytes;
+        dev.emplace_back(pinned_address(ctx, src.k, bytes), pinned_address(ctx, src.v, bytes));
+    }
     for (int l = 0; l < sh.n_layers; ++l) {
         kvp_load_list list;
         list.n_items = 0;
-        for (int32_t id : ids) {
+        for (size_t i = 0; i < ids.size(); ++i) {
+            const int32_t id = ids[i];
             const kvp_segment_host &pk = ctx->packets[id];
             const kvp_ctx::host_src &src = ctx->packet_src[id];
-            if (src.dev_k && src.dev_v) {
-                list.item[list.n_items++] = {src.dev_k, src.dev_v, pk.n, pk.row0, 0, 0};
+            if (dev[i].first && dev[i].second) {
+                list.item[list.n_items++] = {dev[i].first, dev[i].second, pk.n, pk.row0, 0, 0};
                 if (list.n_items == KVP_LOAD_ITEMS) {
                     KVP_CUDA(ctx, kvp_launch_load(sh, list, l, ctx->pool_k, ctx->pool_v, ctx->status_dev, ctx->load_stream));
                     list.n_items = 0;

@@ -211,8 +211,7 @@ struct kvp_ctx {
     std::vector<double> inv_freq;
     std::vector<kvp_segment_host> packets;
     // packets whose K/V wait in host memory until a request uses them (parallel to `packets`, grown on demand)
-    // (dev_k, dev_v: the same buffers as kernels see them, if they are pinned)
-    struct host_src { const char *k = nullptr, *v = nullptr, *dev_k = nullptr, *dev_v = nullptr; bool from_host = false, resident = true; };
+    struct host_src { const char *k = nullptr, *v = nullptr; bool from_host = false, resident = true; };
     std::vector<host_src> packet_src;
     cudaStream_t load_stream = nullptr;             // host -> pool copies, layer by layer
     cudaEvent_t load_fence = nullptr;               // the caller's stream at the assemble that starts a load
@@ -246,6 +245,7 @@ struct kvp_ctx {
     kvp_schedule plan;
     int32_t fused_append = 1;              // plain prefill: the attention kernel reads k_new / v_new itself and appends them
     void *encode_tiled = nullptr;          // cuTensorMapEncodeTiled
+    void *pointer_attributes = nullptr;    // cuPointerGetAttributes
     // bf16 with head dimension 128, all assemblies together: [units][128][head_dim]; [units][128] (running max, running sum)
     float *partial_o = nullptr;
     float2 *partial_ml = nullptr;

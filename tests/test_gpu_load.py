@@ -38,3 +38,61 @@ def test_host_packets_arrive_whole(dtype, d, n_kv, lens, pinned):
         ctx.close()
     for a, b in zip(*caches):
         assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+
+
+@pytest.mark.parametrize("pinned", ["whole", "unpinned later", "ends only", "pinned later"])
+def test_buffers_pinned_in_part_or_for_a_time(pinned):
+    # what is pinned when a packet is copied in decides who copies it, whatever it was at registration; a buffer that is
+    # pinned in part is no kernel's to read, and the driver refuses its copy with an error code
+    import mmap
+    L, hkv, d, n, page = 2, 2, 128, 3000, mmap.PAGESIZE
+    rt = torch.cuda.cudart()
+    ctx = kvp.Context(L, 4, hkv, d, "bf16", pool_tokens=n, max_packets=1, max_slots=1, max_prefix_tokens=n, max_query_tokens=1,
+                      max_ws_rows=n + 8)
+    maps = [mmap.mmap(-1, (L * hkv * n * d * 2 + page - 1) // page * page) for _ in range(2)]
+    buf = [torch.frombuffer(m, dtype=torch.bfloat16)[:L * hkv * n * d].view(L, hkv, n, d) for m in maps]
+    g = torch.Generator()
+    g.manual_seed(5)
+    ranges = []
+    for b, m in zip(buf, maps):
+        b.copy_(torch.randn(b.shape, generator=g))
+        at = b.data_ptr()
+        ranges += [(at, page), (at + len(m) - page, page)] if pinned == "ends only" else [(at, len(m))]
+
+    def pin():
+        for at, size in ranges:
+            assert int(rt.cudaHostRegister(at, size, 0)) == 0
+
+    def unpin():
+        for at, _ in ranges:
+            assert int(rt.cudaHostUnregister(at)) == 0
+
+    def check():
+        aid, _ = ctx.assemble([[(0, -1)]], 0)
+        for l in range(L):
+            k, v = ctx.export_cache(aid, l, 0, n, 0)
+            torch.cuda.synchronize()
+            assert torch.equal(k.cpu(), buf[0][l].transpose(0, 1)) and torch.equal(v.cpu(), buf[1][l].transpose(0, 1))
+        assert ctx.status_word() == 0
+
+    if pinned != "pinned later":
+        pin()
+    ctx.register_packet_host(buf[0], buf[1], n, 0)
+    if pinned == "unpinned later":
+        unpin()
+    if pinned == "ends only":
+        with pytest.raises(kvp.KvpError) as e:
+            ctx.assemble([[(0, -1)]], 0)
+        assert e.value.code == 6
+        unpin()
+        ctx.evict_packet(0)
+    check()
+    for b in buf:
+        b.mul_(2)
+    if pinned == "pinned later":
+        pin()
+    ctx.evict_packet(0)
+    check()
+    if pinned in ("whole", "pinned later"):
+        unpin()
+    ctx.close()
