@@ -252,7 +252,12 @@ template <bool JOINT = false>
 __device__ __forceinline__ Work load_work(const Params &p, const kvp_work *works, int wi)
 {
     const int4 *w4 = reinterpret_cast<const int4 *>(works + wi);
-    const int4 a = w4[0], c = w4[1], e = w4[2];
+    int4 a, c, e;
+    if (p.list_bytes != 0) {                                  // this launch's own parameters
+        a = w4[0]; c = w4[1]; e = w4[2];
+    } else {                                                  // from L2: the launch in front may have stored the list
+        a = __ldcg(w4); c = __ldcg(w4 + 1); e = __ldcg(w4 + 2);
+    }
     Work w;
     w.b = a.x; w.hk = a.y; w.row_base = a.z; w.mode = a.w & 0xff;
     w.q_len = (a.w >> 8) ? (a.w >> 8) : p.q_len;

@@ -645,8 +645,10 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap k_pool, const __grid_consta
     }
     // from here on: the Q producer, the append and the TMA warp (for anything but pool tiles) wait for the kernel in front;
     // everything else follows from what they deliver
-    c.item_begin = cta_begin[blockIdx.x >> 1];   // (the work list gives every pair at least one piece)
-    c.item_end = cta_begin[(blockIdx.x >> 1) + 1];
+    // (the work list gives every pair at least one piece)
+    const int32_t *range = cta_begin + (blockIdx.x >> 1);
+    c.item_begin = LB > 0 ? range[0] : __ldcg(range);
+    c.item_end = LB > 0 ? range[1] : __ldcg(range + 1);
     __syncwarp();
     tc_fence_before();
     cluster_sync();                                           // both CTAs' barriers and TMEM are there

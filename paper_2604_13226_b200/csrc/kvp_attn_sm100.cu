@@ -854,8 +854,10 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_pool_k, const __grid_co
     }
     // from here on: the Q producer, the append and the TMA warp (for anything but pool tiles) wait for the kernel in front;
     // everything else follows from what they deliver
-    c.item_begin = cta_begin[blockIdx.x];   // (the work list gives every CTA at least one piece)
-    c.item_end = cta_begin[(blockIdx.x) + 1];
+    // (the work list gives every CTA at least one piece)
+    const int32_t *range = cta_begin + (blockIdx.x);
+    c.item_begin = LB > 0 ? range[0] : __ldcg(range);
+    c.item_end = LB > 0 ? range[1] : __ldcg(range + 1);
     tc_fence_before();
     __syncthreads();
     if (LB > 0) pdl_launch_dependents();

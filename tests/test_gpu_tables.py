@@ -3,6 +3,7 @@ layer): attention of both layers (the second reads the stored list) and the expo
 against the oracle."""
 import numpy as np
 import pytest
+import torch
 
 from oracle import reference as orc
 from paper_2604_13226_b200 import binding as kvp
@@ -55,4 +56,31 @@ def test_list_per_layer(ctas):
         out, lse = sess.prefill(layer)
         assert sess.ctx.status_word() == 0
         check(wl, out, lse, layer)
+    sess.close()
+
+
+@pytest.mark.parametrize("batch,start", [(1, 126), (3, 126), (6, 124)])
+def test_lists_change_while_layers_follow_one_another(batch, start):
+    # a decode over four layers, each step layer after layer: the list changes when the appended rows enter another 128-key
+    # tile, in the place of the one before; the layers behind the first read it as that one's launch has stored it
+    L, n = 4, 5
+    shape = gen.ModelShape(L, 16, 2, 128, "bf16", 500000.0, 0)
+    lens = [900, 300, 1500]
+    wl = gen.make_workload(shape, lens, [[((b + i) % 3, 0) for i in range(1 + b % 3)] for b in range(batch)], q_len=start + n,
+                           seed=batch)
+    sess = Session(wl)
+    for _ in range(2):                                        # the second time over the first one's lists
+        sess.assemble()
+        outs, lses = [[] for _ in range(L)], [[] for _ in range(L)]
+        qkv = [sess.query_tensors(l) for l in range(L)]
+        cuts = [(0, start)] + [(start + i, start + i + 1) for i in range(n)]
+        parts = [[tuple(t[:, a:b].contiguous() for t in qkv[l]) for l in range(L)] for a, b in cuts]
+        for i, layers in enumerate(parts):
+            for l, x in enumerate(layers):
+                o, z = sess.prefill(l, kvp.CONTINUE if i else 0, qkv=x)
+                outs[l].append(o)
+                lses[l].append(z)
+        assert sess.ctx.status_word() == 0
+        for l in range(L):
+            check(wl, torch.cat(outs[l], dim=1), torch.cat(lses[l], dim=2), l)
     sess.close()
