@@ -21,7 +21,7 @@ STATUS_NAMES = {0: "KVP_OK", 1: "KVP_ERR_INVALID", 2: "KVP_ERR_CAPACITY", 3: "KV
 DTYPE_F32, DTYPE_BF16 = 0, 1
 REBASE, MATERIALIZE = 1, 2
 ROPE_QUERY, FORCE_SIMPLE, CONTINUE, PRECISE_QK, PARTIAL, SKIP_QUERY_BLOCK = 1, 2, 4, 8, 16, 32
-TUNE_SPLIT_TARGET_CTAS, TUNE_FORCE_SPLITS, TUNE_TIME_KERNELS, TUNE_FUSED_APPEND = 1, 2, 3, 5
+TUNE_SPLIT_TARGET_CTAS, TUNE_FORCE_SPLITS, TUNE_TIME_KERNELS, TUNE_FUSED_APPEND, TUNE_CTA_PAIRS = 1, 2, 3, 5, 6
 
 
 class KvpError(RuntimeError):

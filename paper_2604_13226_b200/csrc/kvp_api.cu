@@ -278,7 +278,8 @@ constexpr double kTcMinFlops64 = 1.5e8;
 bool use_pairs(const kvp_ctx *ctx, const kvp_assembly_host &as, int q_len, const int32_t *q_lens)
 {
     const kvp_shape &sh = ctx->shape;
-    if (!ctx->have_tma || sh.head_dim != 128 || ctx->split_target_ctas == 1) return false;
+    if (!ctx->pairs || !(ctx->have_tma || ctx->host_only) || sh.dtype != KVP_DTYPE_BF16 || sh.head_dim != 128 || ctx->split_target_ctas == 1)
+        return false;
     int64_t wide = 0, narrow = 0;                                 // units, weighted by their request's prefix
     for (int b = 0; b < as.batch; ++b) {
         const int64_t rows = (int64_t)sh.group * (q_lens ? q_lens[b] : q_len), rest = rows % (2 * KVP_TILE_ROWS);
@@ -486,10 +487,11 @@ int32_t plan_schedule(kvp_ctx *ctx, const kvp_assembly_host &as, int layer, int 
         rb_weight.back() += (int64_t)(units[u].n_all - units[u].t_first) * (units[u].mode ? 1 : 2) + kPieceCost;
     }
     rb_begin.push_back(units.size());
-    const int n_rb = (int)rb_weight.size();
-    std::vector<int> rb_ctas(n_rb, 0);
-    bool per_block = n_rb >= 2 && 2 * n_rb <= G && !no_split;
-    if (per_block) {
+    int n_rb = (int)rb_weight.size();
+    std::vector<int> rb_ctas;
+    // deals the CTAs out to the n_rb runs; how much more than its even share the worst served one has to do, at least one CTA each
+    auto deal = [&]() -> double {
+        rb_ctas.assign(n_rb, 0);
         int given = 0;
         std::vector<std::pair<int64_t, int>> rem;
         for (int r = 0; r < n_rb; ++r) {
@@ -500,8 +502,46 @@ int32_t plan_schedule(kvp_ctx *ctx, const kvp_assembly_host &as, int layer, int 
         }
         std::sort(rem.begin(), rem.end());
         for (int i = 0; given < G; ++i, ++given) ++rb_ctas[rem[i % n_rb].second];
-        for (int r = 0; r < n_rb; ++r) per_block = per_block && rb_ctas[r] >= 1;
+        double worst = 0.0;
+        for (int r = 0; r < n_rb; ++r)
+            worst = rb_ctas[r] ? std::max(worst, (double)rb_weight[r] * G / ((double)total * rb_ctas[r])) : 1e9;
+        return worst;
+    };
+    bool per_block = n_rb >= 2 && 2 * n_rb <= G && !no_split;
+    // Whole CTAs per row block round badly when there are only a few for each (16 row blocks on 74 pairs: 4 or 5, so the
+    // launch lasts as long as a quarter of a row block, 1.16 times the even share; 28: 2 or 3, 1.32).  Above an eighth,
+    // several row blocks following one another share a run, as few as bring it to a sixteenth, or else the number that
+    // rounds best; K/V are then read once per row block of a run, which calls with so many row blocks hide behind their
+    // arithmetic.  4 x 16 documents of 2048 tokens: 16 row blocks 2036 -> 1911 us; 28 (28/4 heads) 2004 -> 1712; 25 1945 ->
+    // 1507.
+    if (per_block && deal() > 1.125) {
+        const std::vector<size_t> begin = rb_begin;
+        const std::vector<int64_t> weight = rb_weight;
+        const int n_all = n_rb;
+        auto group = [&](int m) {
+            n_rb = (n_all + m - 1) / m;
+            rb_begin.clear();
+            rb_weight.assign(n_rb, 0);
+            for (int r = 0; r < n_all; ++r) {
+                if (r % m == 0) rb_begin.push_back(begin[r]);
+                rb_weight[r / m] += weight[r];
+            }
+            rb_begin.push_back(begin[n_all]);
+        };
+        int best = n_all;
+        double least = 1e9;
+        for (int m = 2; m <= n_all && least > 1.0625; ++m) {
+            group(m);
+            const double loss = deal();
+            if (loss < least) {
+                least = loss;
+                best = m;
+            }
+        }
+        group(best);
+        per_block = n_rb >= 2;
     }
+    if (per_block) per_block = deal() < 1e9;
     std::vector<int> rb_used(n_rb, 0);
     // Row blocks that differ only in a few causal tiles are cut at the same PREFIX tiles: one row block is dealt
     // out and its cuts, counted from the first prefix tile of a unit, are used for all of them.  The CTAs that
@@ -761,6 +801,7 @@ int32_t kvp_create(const kvp_config *cfg, kvp_ctx **out)
     ctx->slots.resize(cfg->max_assemblies);
     *out = ctx;
     if (ctx->host_only) {
+        ctx->pairs = false;
         if (sh.pool_rows <= 0) sh.pool_rows = INT32_MAX;      // sizes only: no pool behind it
         return KVP_OK;
     }
@@ -1700,8 +1741,9 @@ int32_t kvp_kernel_times(kvp_ctx *ctx, int32_t which, float *ms, int32_t cap, in
 int32_t kvp_tune(kvp_ctx *ctx, int32_t key, int32_t value)
 {
     if (!ctx) return KVP_ERR_INVALID;
-    if (key == KVP_TUNE_SPLIT_TARGET_CTAS || key == KVP_TUNE_FORCE_SPLITS) {
-        (key == KVP_TUNE_SPLIT_TARGET_CTAS ? ctx->split_target_ctas : ctx->force_splits) = value;
+    if (key == KVP_TUNE_SPLIT_TARGET_CTAS || key == KVP_TUNE_FORCE_SPLITS || key == KVP_TUNE_CTA_PAIRS) {
+        if (key == KVP_TUNE_CTA_PAIRS) ctx->pairs = value != 0;
+        else (key == KVP_TUNE_SPLIT_TARGET_CTAS ? ctx->split_target_ctas : ctx->force_splits) = value;
         for (kvp_assembly_host &as : ctx->slots) as.sched.clear();       // work lists are rebuilt on next use
     }
     else if (key == KVP_TUNE_FUSED_APPEND) ctx->fused_append = value != 0;

@@ -265,6 +265,7 @@ struct kvp_ctx {
 
     int32_t sm_count = 148;
     int32_t split_target_ctas = 0, force_splits = 0;
+    bool pairs = true;                     // KVP_TUNE_CTA_PAIRS
     // optional CUDA-event timing of the attention (0) and gather (1) kernels, for roofline reports
     int32_t time_kernels = 0;             // 0: off; p >= 1: every p-th attention / gather kernel is bracketed by events
     int32_t tev_seen[2] = {0, 0};

@@ -234,6 +234,42 @@ def test_schedule_covers_every_tile_once(case):
     assert max(cost) <= sum(cost) / len(cost) + 16
 
 
+@pytest.mark.parametrize("n_q,n_kv,batch,docs,doc", [(32, 8, 4, 16, 2048), (28, 4, 4, 16, 2048), (32, 8, 1, 16, 2048),
+                                                     (32, 8, 2, 8, 2048), (32, 8, 8, 10, 1024), (8, 1, 3, 40, 1024)])
+def test_pairs_share_the_work_of_many_row_blocks(n_q, n_kv, batch, docs, doc):
+    # 1 to 37 row blocks of 256 rows on 74 CTA pairs: every key tile of every unit once, and the heaviest pair within an eighth
+    # of the even share over all pairs (the equal cuts that neighbouring row blocks get may leave a ninth of them idle) and a
+    # fortieth for causal tiles and the two-tile granularity of pieces
+    g = n_q // n_kv
+    most = 37 * 256 // g
+    ctx = kvp.Context(1, n_q, n_kv, 128, "bf16", max_packets=docs, max_batch=batch, max_slots=batch * docs, max_prefix_tokens=docs * doc,
+                      max_query_tokens=most, max_ws_rows=batch * most, device=-1)
+    for _ in range(docs):
+        ctx.register_packet(None, None, doc, 0)
+    ctx.tune(kvp.TUNE_CTA_PAIRS, 1)
+    aid, _ = ctx.assemble([[(p, -1) for p in range(docs)]] * batch, kvp.REBASE)
+    n_prefix = docs * (doc // 128)
+    for n_rb in range(1, 38):
+        q_len = n_rb * 256 // g
+        cb, works, _, _ = ctx.export_schedule(aid, q_len)
+        assert len(cb) - 1 <= 74 and np.all(works[:, 3] == 0)
+        covered = {}
+        for b, hk, rb, _, lo, n in works[:, :6].tolist():
+            covered.setdefault((b, hk, rb), []).append((lo, n))
+        assert len(covered) == batch * n_kv * -(-g * q_len // 256)
+        for (b, hk, rb), pieces in covered.items():
+            pos = 0
+            for lo, n in sorted(pieces):
+                assert lo == pos
+                pos += n
+            assert pos == n_prefix + (min(g * q_len, rb + 256) - 1) // g // 128 + 1
+        if works[:, 5].sum() < 74 * 100:                     # fewer than a hundred tiles per pair: start and merge decide
+            continue
+        cost = np.array([2 * works[cb[c]:cb[c + 1], 5].sum() + 8 * (cb[c + 1] - cb[c]) for c in range(len(cb) - 1)])
+        assert cost.max() <= 1.15 * cost.sum() / 74, (n_rb, cost.max() * 74 / cost.sum())
+    ctx.close()
+
+
 def test_compressed_registration_and_per_layer_lists_host_only():
     shape = gen.ModelShape(3, 8, 2, 128, "bf16", 500000.0)
     wl = gen.make_workload(shape, [300, 700], [[(0, 0), (1, 0)]], q_len=8, seed=2, keep_rate=[0.5, None])
