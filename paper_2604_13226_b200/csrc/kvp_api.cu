@@ -274,8 +274,9 @@ constexpr double kTcMinFlops64 = 1.5e8;
 // Whether a call runs on CTA pairs (kvp_attn_pair.cu), whose units are 256 rows: a unit that holds no more than 128 costs
 // a pair as much as a full one (2 x 1,600 cycles per key tile; the one-CTA kernel 3,900, and 1,950 for a narrow unit).
 // With three narrow units to two wide ones pairs were 4 % slower, with one to four 1 % (ragged batches), without any
-// 2-10 % faster.
-bool use_pairs(const kvp_ctx *ctx, const kvp_assembly_host &as, int q_len, const int32_t *q_lens)
+// 2-10 % faster.  With KVP_PARTIAL (`partial`) every unit takes two partial slots, a narrow one too: only as far as there are
+// slots enough for that and for the cuts.
+bool use_pairs(const kvp_ctx *ctx, const kvp_assembly_host &as, int q_len, const int32_t *q_lens, bool partial)
 {
     const kvp_shape &sh = ctx->shape;
     if (!ctx->pairs || !(ctx->have_tma || ctx->host_only) || sh.dtype != KVP_DTYPE_BF16 || sh.head_dim != 128 || ctx->split_target_ctas == 1)
@@ -287,6 +288,8 @@ bool use_pairs(const kvp_ctx *ctx, const kvp_assembly_host &as, int q_len, const
         wide += keys * (rows / (2 * KVP_TILE_ROWS) + (rest > KVP_TILE_ROWS ? 1 : 0));
         narrow += keys * (rest > 0 && rest <= KVP_TILE_ROWS ? 1 : 0);
     }
+    const int64_t blocks = ((int64_t)sh.group * q_len + 2 * KVP_TILE_ROWS - 1) / (2 * KVP_TILE_ROWS);
+    if (partial && 2 * (blocks * as.batch * sh.n_kv_heads + std::min(ctx->sm_count, kMaxCtas)) > KVP_MAX_SPLIT_UNITS) return false;
     return wide >= 6 * narrow;
 }
 
@@ -358,7 +361,7 @@ int32_t plan_schedule(kvp_ctx *ctx, const kvp_assembly_host &as, int layer, int 
                       uint32_t opts, bool joint, kvp_schedule &out)
 {
     const kvp_shape &sh = ctx->shape;
-    out.pair = !joint && use_pairs(ctx, as, q_len, q_lens);
+    out.pair = !joint && use_pairs(ctx, as, q_len, q_lens, (opts & KVP_PARTIAL) != 0);
     const int kPieceCost = out.pair ? kPieceCostPair : kPieceCostOne;
     const bool force_partial = (opts & KVP_PARTIAL) != 0, skip_tail = (opts & KVP_SKIP_QUERY_BLOCK) != 0;
     typedef kvp_schedule::unit unit_t;
@@ -1504,7 +1507,7 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
     kvp_attn2_args a;
     a.tail_direct = 0;
     a.precise = (flags & KVP_PRECISE_QK) ? 1 : 0;
-    const bool pairs = fast && use_pairs(ctx, as, q_len, q_lens);
+    const bool pairs = fast && use_pairs(ctx, as, q_len, q_lens, part_opts != 0);
     if (fast && ctx->fused_append && !rope_query && q_pos0 == 0 && !skip_block &&
         (((uintptr_t)k_new | (uintptr_t)v_new) & 15) == 0 &&
         make_query_tensor_map((encode_tiled_fn)ctx->encode_tiled, &a.tm_knew, k_new, sh.head_dim, sh.n_kv_heads, q_len, as.batch,

@@ -107,3 +107,16 @@ def test_partial_flag_misuse_is_refused():
         sess.ctx.assemble(sub.items, kvp.REBASE, pos_base=[-1] * sub.batch)
     assert e.value.code == 1
     sess.close()
+
+
+def test_partials_up_to_the_slots_there_are():
+    # 150 requests of 13 row tiles: 1950 of 2048 partial slots on single CTAs; a CTA pair takes two for the last, narrow unit of
+    # each as well, 2100 in all
+    shape = gen.ModelShape(1, 32, 1, 128, "bf16", 500000.0, 0)
+    wl = gen.make_workload(shape, [100, 60], [[(b % 2, -1)] for b in range(150)], q_len=52, seed=4)
+    out, lse = run_sharded(wl, 1)
+    sess = Session(wl)
+    sess.assemble()
+    ref, ref_lse = sess.prefill(0)
+    assert float((out.float() - ref.float()).abs().max()) <= 2.0 ** -7 and float((lse - ref_lse).abs().max()) <= 1e-4
+    sess.close()
