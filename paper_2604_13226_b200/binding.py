@@ -10,7 +10,6 @@ from __future__ import annotations
 import ctypes
 import os
 import struct
-from itertools import accumulate
 from typing import List, Optional, Sequence, Tuple
 
 from . import build as _build
@@ -106,6 +105,14 @@ EXPORTED = ["kvp_version", "kvp_token_bytes", "kvp_workspace_bytes", "kvp_create
 
 def _i32_array(xs: Sequence[int]):
     return (ctypes.c_int32 * max(1, len(xs)))(*[int(x) for x in xs])
+
+
+def _i32_packed(xs: List[int]):
+    # a ctypes array costs six times as much to fill; it takes what is not an int, or not one of 32 bits
+    try:
+        return struct.pack(f"{len(xs)}i", *xs)
+    except struct.error:
+        return _i32_array(xs)
 
 
 def _ptr(t) -> Optional[int]:
@@ -230,12 +237,13 @@ class Context:
         """items[b] = [(packet_id, adapter_id), ...].  Returns (assembly_id, prefix_len list).
         pos_base (one position per request) -> ``kvp_assemble_at``: this rank's part of a sharded request."""
         B = len(items)
-        pids = [p for it in items for p, _ in it]
-        aids = [a for it in items for _, a in it]
-        n = len(pids)
-        # packed ints: a ctypes array costs six times as much to fill
-        offs = struct.pack(f"{B + 1}i", 0, *accumulate(map(len, items)))
-        pids, aids = struct.pack(f"{n}i", *pids), struct.pack(f"{n}i", *aids)
+        offs, pids, aids = [0], [], []
+        for it in items:
+            for pid, aid in it:
+                pids.append(pid)
+                aids.append(aid)
+            offs.append(len(pids))
+        offs, pids, aids = _i32_packed(offs), _i32_packed(pids), _i32_packed(aids)
         plen = (ctypes.c_int32 * max(1, B))()
         aid = ctypes.c_int32(-1)
         if pos_base is not None:

@@ -369,3 +369,17 @@ def test_packets_registered_from_host_memory_plan_like_any_other():
     a.close()
     b.close()
 
+
+
+def test_assemble_takes_any_pairs_of_numbers():
+    # requests as iterators, ids that are not ints, and ids beyond 32 bits, which are unknown ids like any other
+    wl = ragged_workload()
+    ctx = host_ctx(wl.shape, wl)
+    want = ctx.assemble(wl.items)[1]
+    assert ctx.assemble([iter(it) for it in wl.items])[1] == want
+    assert ctx.assemble([[(float(p), np.int64(a)) for p, a in it] for it in wl.items])[1] == want
+    for bad in (2 ** 31, -2 ** 40 - 1):
+        with pytest.raises(kvp.KvpError) as e:
+            ctx.assemble([[(bad, -1)]])
+        assert e.value.code == 3
+    ctx.close()
