@@ -124,7 +124,7 @@ upload_kernel(const uint4 *__restrict__ host, uint4 *__restrict__ dst, int n_wor
 // take pieces in turn, one thread each, with bulk copies host -> shared memory -> pool in a ring of three.  Bound by the
 // host link: reads from the SMs reach 51.2 GB/s whatever the sizes, where a copy per packet, layer and K/V costs 4 us
 // beside its transfer (1 MB each: 45.7 GB/s, 256 KB: 28.8; one copy of 128 MB: 55.2).  A block is one warp with 12 KB, so
-// that the attention kernel on CTA pairs fits beside it.
+// that the attention kernel on CTA pairs fits beside it (the one-CTA kernel, with 226 KB, does not).
 constexpr int kLoadPiece = 4096, kLoadStages = 3;
 
 __device__ __forceinline__ uint32_t shared_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -964,8 +964,11 @@ cudaError_t kvp_launch_load(const kvp_shape &sh, kvp_load_list &list, int32_t la
         pieces += 2ll * sh.n_kv_heads * (((int64_t)list.item[i].n * row_bytes + kLoadPiece - 1) / kLoadPiece);
     }
     list.n_pieces = (int32_t)pieces;
-    // 64 blocks have 768 KB in flight, several times what the link's latency takes
-    load_kernel<<<(int)std::min<int64_t>(64, pieces), 32, 0, st>>>(list, layer, sh.n_kv_heads, row_bytes, sh.pool_rows, pool_k, pool_v, status);
+    // 20 blocks have 240 KB in flight, just what the link's latency takes, and as few SMs as that needs: the one-CTA attention
+    // kernel does not fit beside a block, and its CTAs there wait for the load to end.  Of 50.1 GB/s with 64 blocks: 12 blocks
+    // 47.0, 16 49.9, 20 and more 50.0; four short layers over 10 x 1024 tokens on another stream meanwhile (85 us alone):
+    // 64 blocks 495 us, 32 290, 20 200, 16 185.
+    load_kernel<<<(int)std::min<int64_t>(20, pieces), 32, 0, st>>>(list, layer, sh.n_kv_heads, row_bytes, sh.pool_rows, pool_k, pool_v, status);
     return cudaGetLastError();
 }
 
