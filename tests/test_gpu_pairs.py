@@ -15,13 +15,21 @@ from test_gpu_parity import check_attention
 pytestmark = pytest.mark.gpu
 
 
+def on_pairs(sess, q_len):
+    # an entry of a pair plan's list is two CTAs
+    cta_begin = sess.ctx.export_schedule(sess.assembly_id, q_len)[0]
+    launch = sess.ctx.last_launch()
+    return launch["kind"] == 1 and launch["ctas"] == 2 * (len(cta_begin) - 1)
+
+
 @pytest.mark.parametrize("lens,q_len,ctas,flags", [
     ([1], 64, 0, 0),                                   # two or three tiles in all
     ([128], 33, 2, 0),                                 # 132 rows: four in the second CTA; one pair walks everything
     ([100, 1, 128, 127, 31, 33, 64], 64, 0, 0),        # a document per tile
     ([100, 1, 128, 127, 31, 33, 64], 64, 4, kvp.PRECISE_QK),
-    ([129, 257, 385, 513], 70, 148, 0),                # many pieces of two tiles
-    ([640, 1024], 150, 6, kvp.PRECISE_QK),             # two causal tiles, several pieces per pair
+    ([129, 257, 385, 513], 64, 148, 0),                # many pieces of two tiles
+    ([640, 1024], 192, 6, kvp.PRECISE_QK),             # two causal tiles, several pieces per pair
+    ([300, 200], 409, 0, 0),                           # six units of 256 rows and one of 100 per kv head
 ])
 def test_pipeline_edges(lens, q_len, ctas, flags):
     shape = gen.ModelShape(1, 32, 8, 128, "bf16", 500000.0, 0)
@@ -31,7 +39,7 @@ def test_pipeline_edges(lens, q_len, ctas, flags):
     if ctas:
         sess.ctx.tune(kvp.TUNE_SPLIT_TARGET_CTAS, ctas)
     check_attention(wl, sess, flags=flags)
-    assert sess.ctx.last_launch()["kind"] == 1 and sess.ctx.last_launch()["ctas"] % 2 == 0
+    assert on_pairs(sess, q_len)
     qkv = sess.query_tensors(0)
     first, _ = sess.prefill(0, flags, qkv=qkv)
     for _ in range(20):
@@ -53,6 +61,7 @@ def test_reference_maximum_moves_late_in_a_piece():
         if ctas:
             sess.ctx.tune(kvp.TUNE_SPLIT_TARGET_CTAS, ctas)
         check_attention(wl, sess, flags=kvp.PRECISE_QK)
+        assert on_pairs(sess, 64)
         sess.close()
 
 
@@ -82,4 +91,18 @@ def test_probabilities_are_rounded_once(q_len):
     once = (p.bfloat16().double() @ V / p.sum(-1, keepdim=True)).permute(0, 2, 1, 3)
     err, ideal = float((o / l - want).norm()), float((once - want).norm())
     assert err <= 1.06 * ideal, (err, ideal, err / ideal)
+    sess.close()
+
+
+@pytest.mark.parametrize("q_len", [64, 96, 150, 409])
+def test_either_kernel_on_request(q_len):
+    # KVP_TUNE_CTA_PAIRS: off, on again; 96 and 150 tokens (384 and 600 rows) have a narrow unit to one or two wide ones
+    shape = gen.ModelShape(1, 32, 8, 128, "bf16", 500000.0, 0)
+    wl = gen.make_workload(shape, [300, 700], [[(0, 0), (1, 0)]], q_len=q_len, seed=q_len)
+    sess = Session(wl)
+    sess.assemble()
+    for pairs in (0, 1):
+        sess.ctx.tune(kvp.TUNE_CTA_PAIRS, pairs)
+        check_attention(wl, sess)
+        assert on_pairs(sess, q_len) == (pairs == 1 and q_len in (64, 409))
     sess.close()

@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 BF16_MAX_ABS, BF16_MEAN_ABS = 2e-2, 2e-3
 
 
-def run_ragged(wl, q_lens, layer=0, split_ctas=0):
+def run_ragged(wl, q_lens, layer=0, split_ctas=0, pairs=None):
     sess = Session(wl)
     sess.assemble()
     if split_ctas:
@@ -26,6 +26,8 @@ def run_ragged(wl, q_lens, layer=0, split_ctas=0):
     sess.ctx.query_prefill_ragged(sess.assembly_id, layer, q, kn, vn, wl.q_len, q_lens, out, lse)
     torch.cuda.synchronize()
     assert sess.ctx.status_word() == 0
+    if pairs is not None:                                        # of three CTAs to be used, two make a pair
+        assert split_ctas == 3 and sess.ctx.last_launch()["ctas"] == (2 if pairs else 3)
     s = wl.shape
     o = orc.widen(torch_to_np(out, s.dtype), s.dtype)           # [B][Lq][Hq][d]
     l = lse.cpu().numpy().astype(np.float64)                     # [B][Hq][Lq]
@@ -64,6 +66,13 @@ def test_ragged_query_lengths_against_the_oracle(q_lens):
 def test_ragged_query_lengths_with_split_units():
     run_ragged(ragged_wl(200), [150, 37, 1, 200], split_ctas=148)
     run_ragged(ragged_wl(200), [150, 37, 1, 200], split_ctas=3)
+
+
+# group 4: rows in blocks of 256 and a remainder above 128 (pairs), at most 128 to six full ones (pairs), more of those (not)
+@pytest.mark.parametrize("q_lens,pairs", [([64, 192, 256, 100], True), ([256, 64, 64, 128], True), ([33, 63, 97, 191], True),
+                                          ([256, 256, 25, 64], True), ([25, 256, 64, 33], False), ([150, 37, 1, 200], False)])
+def test_ragged_query_lengths_on_cta_pairs(q_lens, pairs):
+    run_ragged(ragged_wl(256), q_lens, split_ctas=3, pairs=pairs)
 
 
 def test_ragged_rejects_bad_lengths_and_other_paths():

@@ -270,6 +270,40 @@ def test_pairs_share_the_work_of_many_row_blocks(n_q, n_kv, batch, docs, doc):
     ctx.close()
 
 
+@pytest.mark.parametrize("n_q,n_kv,lens,items,q_len", [
+    (32, 8, [1024] * 10, [[(i, 0) for i in range(10)]] * 4, 128),         # two row blocks, split
+    (28, 4, [300, 1000, 257, 640], [[(0, 0), (1, 0)], [(2, 0), (3, 0), (0, -1)]], 146),      # g = 7: 1022 rows, ragged
+    (32, 8, [512] * 5, [[(i, 0) for i in range(5)]], 64),                 # little work
+    (4, 4, [200, 3000], [[(0, 0)], [(1, 0), (0, 0)]], 750),               # g = 1, a last block of 238 rows
+    (32, 8, [2048] * 4, [[(i, 0) for i in range(4)]], 409),               # a last block of 100 rows
+])
+def test_pair_plan_covers_every_tile_and_slot_once(n_q, n_kv, lens, items, q_len):
+    ctx, aid, plen, shape = _schedule_case(n_q, n_kv, lens, items, q_len)
+    ctx.tune(kvp.TUNE_CTA_PAIRS, 1)
+    cb, works, merges, n_slots = ctx.export_schedule(aid, q_len)
+    g, n_rows = n_q // n_kv, n_q // n_kv * q_len
+    assert cb[0] == 0 and cb[-1] == len(works) and np.all(np.diff(cb) > 0) and len(cb) - 1 <= 74 and np.all(works[:, 3] == 0)
+    units, slots = {}, []
+    for b, hk, rb, _, lo, n, s0, s1 in works.tolist():
+        units.setdefault((b, hk, rb), []).append((lo, n, s0, s1))
+    assert sorted(units) == [(b, hk, rb) for b in range(len(items)) for hk in range(n_kv) for rb in range(0, n_rows, 256)]
+    for (b, hk, rb), pieces in units.items():
+        docs = [n for n in (int(s[1]) for s in ctx.export_plan(aid, b)[2]) if n != 16]
+        n_ad = sum(1 for s in ctx.export_plan(aid, b)[2] if s[1] == 16)
+        pos = 0
+        for lo, n, s0, s1 in sorted(pieces):
+            assert lo == pos
+            pos += n
+            assert (s0 >= 0) == (s1 >= 0) == (len(pieces) > 1)
+            slots += [s0, s1] if s0 >= 0 else []
+        assert pos == -(-16 * n_ad // 128) + sum(-(-n // 128) for n in docs) + (min(n_rows, rb + 256) - 1) // g // 128 + 1
+    named = [s for m in merges.tolist() for s in range(m[3], m[3] + m[4])]
+    assert sorted(slots) == sorted(named) == list(range(n_slots))
+    cost = [sum(2 * int(works[i][5]) + 8 for i in range(cb[c], cb[c + 1])) for c in range(len(cb) - 1)]
+    assert max(cost) <= sum(cost) / len(cost) + 20            # a piece's start and write-out, and two tiles
+    ctx.close()
+
+
 def test_compressed_registration_and_per_layer_lists_host_only():
     shape = gen.ModelShape(3, 8, 2, 128, "bf16", 500000.0)
     wl = gen.make_workload(shape, [300, 700], [[(0, 0), (1, 0)]], q_len=8, seed=2, keep_rate=[0.5, None])
