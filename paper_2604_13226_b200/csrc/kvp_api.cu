@@ -426,7 +426,7 @@ int32_t plan_schedule(kvp_ctx *ctx, const kvp_assembly_host &as, int layer, int 
     int64_t largest = 0;
     for (const unit_t &u : units) largest = std::max<int64_t>(largest, (int64_t)(u.n_all - u.t_first) * (u.mode ? 1 : 2));
     const int64_t min_budget = std::min<int64_t>(8, std::max<int64_t>(3, (largest + 5) / 6)) + kPieceCost;
-    auto fill = [&](size_t u_begin, size_t u_end, int g, std::vector<cut_t> *rec) -> int {
+    auto fill = [&](size_t u_begin, size_t u_end, int g, std::vector<cut_t> *rec) {
         std::vector<int64_t> &after = out.after;                      // weight of the units behind unit u
         after.resize(u_end - u_begin + 1);
         after[u_end - u_begin] = 0;
@@ -446,7 +446,7 @@ int32_t plan_schedule(kvp_ctx *ctx, const kvp_assembly_host &as, int layer, int 
             const int64_t to_share = left_all + (int64_t)kPieceCost * (ctas_left - 1);
             const int64_t budget = ctas_left == 1 ? left_all : std::max(min_budget, (to_share + ctas_left - 1) / ctas_left);
             ++used;
-            if (rec) rec->push_back({(int32_t)u, t});
+            rec->push_back({(int32_t)u, t});
             int64_t cost = 0;
             while (u < u_end) {
                 const int w = units[u].mode ? 1 : 2;
@@ -471,11 +471,6 @@ int32_t plan_schedule(kvp_ctx *ctx, const kvp_assembly_host &as, int layer, int 
                 if (cost >= budget) break;
             }
         }
-        return used;
-    };
-    auto cut_range = [&](size_t u_begin, size_t u_end, int64_t weight, int g) {
-        (void)weight;
-        fill(u_begin, u_end, g, &cuts);
     };
     // Each row block gets its own run of CTAs, in proportion to its work, and is cut on its own: row blocks of
     // equal work then get the same cuts, so the CTAs of units that share K/V walk the same tiles in step.  With
@@ -589,11 +584,11 @@ int32_t plan_schedule(kvp_ctx *ctx, const kvp_assembly_host &as, int layer, int 
     } else if (per_block) {
         for (int r = 0; r < n_rb; ++r) {
             const size_t before = cuts.size();
-            cut_range(rb_begin[r], rb_begin[r + 1], rb_weight[r], rb_ctas[r]);
+            fill(rb_begin[r], rb_begin[r + 1], rb_ctas[r], &cuts);
             rb_used[r] = (int)(cuts.size() - before);
         }
     } else {
-        cut_range(0, units.size(), total, G);
+        fill(0, units.size(), G, &cuts);
     }
     cuts.push_back({(int32_t)units.size(), 0});
 
@@ -1595,7 +1590,7 @@ static int32_t query_prefill_impl(kvp_ctx *ctx, int32_t assembly_id, int32_t lay
         if (ss.merges > 0) {
             const bool partial = (flags & KVP_PARTIAL) != 0;
             const int64_t n_rt = ((int64_t)sh.group * q_len + KVP_TILE_ROWS - 1) / KVP_TILE_ROWS;
-            KVP_CUDA(ctx, kvp_launch_merge_list(sh, q_len, ss.merges, ss.slots,
+            KVP_CUDA(ctx, kvp_launch_merge_list(sh, q_len, ss.merges, ss.slots, ctx->sm_count,
                                                 reinterpret_cast<const kvp_merge_item *>(sd + ss.off_merges), ss.ctas > 0,
                                                 part_o, part_ml, out, lse, partial ? out : nullptr,
                                                 (int64_t)as.batch * sh.n_kv_heads * n_rt, st));

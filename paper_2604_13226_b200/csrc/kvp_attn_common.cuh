@@ -352,33 +352,33 @@ template <typename Put>
 __device__ __forceinline__ void rotate_chunks(int pairing, uint32_t *a, uint32_t *b, uint32_t *ar, uint32_t *br, const float4 *w4,
                                               const Put &put)
 {
-                if (pairing == 0) {
-                    // pairs (i, i + D/2): word j of chunk c holds elements 8c+2j, 8c+2j+1; partners in chunk c + kCh
+    if (pairing == 0) {
+        // pairs (i, i + D/2): word j of chunk c holds elements 8c+2j, 8c+2j+1; partners in chunk c + kCh
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const float4 w = w4[j];                      // cos, sin of pair 8c+2j; cos, sin of pair 8c+2j+1
-                        const uint64_t va = pair(bf16_lo(a[j]), bf16_hi(a[j])), vb = pair(bf16_lo(b[j]), bf16_hi(b[j]));
-                        const uint64_t cc = pair(w.x, w.z), ss = pair(w.y, w.w), ns = pair(-w.y, -w.w);
-                        float x, y;
-                        unpair(fma2(vb, ss, mul2(va, cc)), x, y);    // R(-Delta): cos same, sin negated
-                        put(a[j], ar[j], x, y);
-                        unpair(fma2(va, ns, mul2(vb, cc)), x, y);
-                        put(b[j], br[j], x, y);
-                    }
-                } else {
-                    // pairs (2i, 2i+1): one word each; chunk c holds pairs 4c..4c+3 (w4[0], w4[1]), its partner w4[2], w4[3]
+        for (int j = 0; j < 4; ++j) {
+            const float4 w = w4[j];                      // cos, sin of pair 8c+2j; cos, sin of pair 8c+2j+1
+            const uint64_t va = pair(bf16_lo(a[j]), bf16_hi(a[j])), vb = pair(bf16_lo(b[j]), bf16_hi(b[j]));
+            const uint64_t cc = pair(w.x, w.z), ss = pair(w.y, w.w), ns = pair(-w.y, -w.w);
+            float x, y;
+            unpair(fma2(vb, ss, mul2(va, cc)), x, y);    // R(-Delta): cos same, sin negated
+            put(a[j], ar[j], x, y);
+            unpair(fma2(va, ns, mul2(vb, cc)), x, y);
+            put(b[j], br[j], x, y);
+        }
+    } else {
+        // pairs (2i, 2i+1): one word each; chunk c holds pairs 4c..4c+3 (w4[0], w4[1]), its partner w4[2], w4[3]
 #pragma unroll
-                    for (int j = 0; j < 4; j += 2) {
-                        float4 w = w4[j >> 1];
-                        float x0 = bf16_lo(a[j]), y0 = bf16_hi(a[j]), x1 = bf16_lo(a[j + 1]), y1 = bf16_hi(a[j + 1]);
-                        put(a[j], ar[j], x0 * w.x + y0 * w.y, y0 * w.x - x0 * w.y);
-                        put(a[j + 1], ar[j + 1], x1 * w.z + y1 * w.w, y1 * w.z - x1 * w.w);
-                        w = w4[2 + (j >> 1)];
-                        x0 = bf16_lo(b[j]); y0 = bf16_hi(b[j]); x1 = bf16_lo(b[j + 1]); y1 = bf16_hi(b[j + 1]);
-                        put(b[j], br[j], x0 * w.x + y0 * w.y, y0 * w.x - x0 * w.y);
-                        put(b[j + 1], br[j + 1], x1 * w.z + y1 * w.w, y1 * w.z - x1 * w.w);
-                    }
-                }
+        for (int j = 0; j < 4; j += 2) {
+            float4 w = w4[j >> 1];
+            float x0 = bf16_lo(a[j]), y0 = bf16_hi(a[j]), x1 = bf16_lo(a[j + 1]), y1 = bf16_hi(a[j + 1]);
+            put(a[j], ar[j], x0 * w.x + y0 * w.y, y0 * w.x - x0 * w.y);
+            put(a[j + 1], ar[j + 1], x1 * w.z + y1 * w.w, y1 * w.z - x1 * w.w);
+            w = w4[2 + (j >> 1)];
+            x0 = bf16_lo(b[j]); y0 = bf16_hi(b[j]); x1 = bf16_lo(b[j + 1]); y1 = bf16_hi(b[j + 1]);
+            put(b[j], br[j], x0 * w.x + y0 * w.y, y0 * w.x - x0 * w.y);
+            put(b[j + 1], br[j + 1], x1 * w.z + y1 * w.w, y1 * w.z - x1 * w.w);
+        }
+    }
 }
 
 // The Q producer (128 threads) writes one 128-row query tile, counter-rotated by the offset of rope-table row

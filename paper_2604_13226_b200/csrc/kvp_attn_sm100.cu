@@ -539,12 +539,11 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
     uint32_t ring_n = 0;
     bool ok = true;
 
-    // ---- S_s = Q_s K^T of step k of piece wq (whose loads start at ring position `base`) ----------------
+    // ---- mode 1: S_s = Q_s K^T of step k of piece wq (whose loads start at ring position `base`) ---------
     auto issue_qk = [&](auto s_c, const Work &wq, uint32_t base, int k) {
         constexpr int s = decltype(s_c)::value;
         MmaStream &ms = st[s];
         const int n_steps = s == 0 ? wq.steps0 : wq.steps1;
-        const bool shared_stage = (wq.mode == 0);                 // mode 0: both streams read the same K/V stage
         if (k == 0) {
             ms.prev_rope = 0;
             ms.cur = get_tile<JOINT>(p, wq, stream_tile(wq, s, 0));
@@ -559,7 +558,7 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
         const int r = wq.mode ? 2 * k + s : k;
         const uint32_t g = base + (uint32_t)load_seq(wq.mode, wq.n, r, 0);
         const uint32_t stage = g % kStages, par = (g / kStages) & 1;
-        if (ok && !(shared_stage && s == 1)) ok = mbar_wait(c.bar(C::kKvFull + stage), par, c.abort_flag(), p.status, 22);
+        if (ok) ok = mbar_wait(c.bar(C::kKvFull + stage), par, c.abort_flag(), p.status, 22);
         ok = __all_sync(0xffffffffu, ok);                         // the lanes stay together
         if (!ok) return;
         tc_fence_after();
@@ -586,7 +585,7 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
                 }
             }
             tc_commit(c.bar(C::kSFull + s));
-            if (!shared_stage || s == 1) tc_commit(c.bar(C::kKvEmpty + stage));
+            tc_commit(c.bar(C::kKvEmpty + stage));
             if (last) tc_commit(c.bar(C::kQFree + 2 * s + ms.qbuf));
         }
         __syncwarp();
@@ -739,13 +738,12 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
         auto block = [&](auto s_c, int k) {
             constexpr int s = decltype(s_c)::value;
             MmaStream &ms = st[s];
-            const bool shared_stage = (w.mode == 0);
             if (k >= 1 && k <= steps[s]) {
                 // ---- O_s += P_s V of step k-1 -------------------------------------------------------
                 const int r = w.mode ? 2 * (k - 1) + s : k - 1;
                 const uint32_t g = ring_n + (uint32_t)load_seq(w.mode, w.n, r, 1);
                 const uint32_t stage = g % kStages, par = (g / kStages) & 1;
-                if (!(shared_stage && s == 1)) ok = mbar_wait(c.bar(C::kKvFull + stage), par, c.abort_flag(), p.status, 23);
+                ok = mbar_wait(c.bar(C::kKvFull + stage), par, c.abort_flag(), p.status, 23);
                 if (ok) ok = mbar_wait(c.bar(C::kPFull + s), ms.nP & 1, c.abort_flag(), p.status, 24 + s);
                 ++ms.nP;
                 if (ok && k == 1 && ms.nItems > 0)
@@ -775,7 +773,7 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
                             if (C::kSplit) mma_ts_c<1>(oa, pa + p_col(kk) + 16, desc64(v_lo + kk * 128, kDescHi), idesc_pv);
                         }
                     }
-                    if (!shared_stage || s == 1) tc_commit(c.bar(C::kKvEmpty + stage));
+                    tc_commit(c.bar(C::kKvEmpty + stage));
                     if (k == steps[s]) {
                         tc_commit(c.bar(C::kOFull + s));
                     }
@@ -1076,7 +1074,7 @@ cudaError_t kvp_launch_attn_sm100(const kvp_shape &sh, const kvp_attn2_args &a, 
                        : go(attn_sm100_kernel<128, KVP_INLINE_LARGE, false>, Cfg<128>::kSmemBytes, *large);
 }
 
-cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_merges, int32_t max_parts, const kvp_merge_item *merges, bool list_there,
+cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_merges, int32_t max_parts, int32_t sm_count, const kvp_merge_item *merges, bool list_there,
                                   const float *partial_o, const float2 *partial_ml, void *out, float *lse,
                                   void *part_out, int64_t part_tiles, cudaStream_t st)
 {
@@ -1091,7 +1089,7 @@ cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_
         mo.part_ml = reinterpret_cast<float2 *>((char *)part_out + (uint64_t)part_tiles * (32ull * KVP_TILE_ROWS * 16));
     }
     // whole rows per block when that gives two blocks per SM, else quarter rows (halves with head dimension 64)
-    const bool few = n_merges * (KVP_TILE_ROWS / 32) < 2 * 148;
+    const bool few = n_merges * (KVP_TILE_ROWS / 32) < 2 * sm_count;
     auto go = [&](auto *kernel, int cs) {
         return launch_pdl(kernel, dim3(n_merges, KVP_TILE_ROWS / 32, cs), 256, 0, st, merges, (int)list_there, q_len, sh.n_q_heads, sh.n_kv_heads,
                           sh.group, sh.scale, partial_o, partial_ml, mo);

@@ -238,7 +238,7 @@ struct kvp_ctx {
     const double *half_turns = nullptr;    // device [head_dim/2]: theta_i / pi (angles in half turns per position)
     uint64_t sched_bytes = 0;
     int32_t sched_max_works = 0, sched_max_merges = 0;
-    // planning scratch, kept so that a call allocates nothing once the sizes have been seen
+    // planning scratch: the large arrays of a call are kept from one to the next
     kvp_assembly_host build;
     std::vector<int32_t> rope_hash, kept_row_of;
     alignas(16) char list_inline[KVP_INLINE_LARGE], plan_inline[KVP_INLINE_SMALL];
@@ -250,7 +250,6 @@ struct kvp_ctx {
     float *partial_o = nullptr;
     float2 *partial_ml = nullptr;
     char *q_scratch = nullptr;
-    float2 *q_rope = nullptr;              // [max_batch*max_query][head_dim/2] for KVP_ROPE_QUERY
 
     char *staging = nullptr;               // the pinned block that all staging buffers and their flags lie in
     std::vector<kvp_stage> plan_ring;      // staging of plans: one more than assemblies alive
@@ -418,7 +417,7 @@ cudaError_t kvp_launch_attn_sm100(const kvp_shape &sh, const kvp_attn2_args &a, 
                                   const CUtensorMap &tm_ws_v, cudaStream_t st);
 // part_out != nullptr: the merged tiles stay partials and go to a rank buffer of part_tiles query tiles
 // list_there: the launch in front waited for the merge list before it released this one
-cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_merges, int32_t max_parts, const kvp_merge_item *merges, bool list_there,
+cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_merges, int32_t max_parts, int32_t sm_count, const kvp_merge_item *merges, bool list_there,
                                   const float *partial_o, const float2 *partial_ml, void *out, float *lse,
                                   void *part_out, int64_t part_tiles, cudaStream_t st);
 // n_parts rank buffers back to back -> final output rows
