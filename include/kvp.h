@@ -227,7 +227,7 @@ KVP_API int32_t kvp_assemble_at(kvp_ctx *ctx, int32_t batch, const int32_t *slot
  *   out    device [batch][q_len][n_q_heads][head_dim]
  *   lse    device float [batch][n_q_heads][q_len] or NULL: natural-log sum of exp(scaled scores)
  * bf16 with head_dim 64: large calls run on the tensor cores, with the rotated query and the probabilities in two bf16
- * numbers each (2^-17 relative).  lse is then off by 4.5e-7 (2-norm) and 1.7e-6 at most for keys and queries of unit
+ * numbers each (2^-17 relative).  lse is then off by 4.5e-7 (root mean square) and 1.7e-6 at most for keys and queries of unit
  * variance, where the CUDA cores, which small calls and KVP_FORCE_SIMPLE run on, give 3.7e-7 and 1.4e-6 (half a unit in
  * the last place of an lse of 8 is 4.8e-7); 2^-17 |q| |k| scale bounds it.
  * By default q and k_new are already rotated for positions prefix_len[b] + i; KVP_ROPE_QUERY makes
