@@ -1425,7 +1425,7 @@ int32_t kvp_export_cache(kvp_ctx *ctx, int32_t assembly_id, int32_t layer, int32
     if (as.waits_loads) KVP_CUDA(ctx, cudaStreamWaitEvent((cudaStream_t)stream, ctx->load_done[layer], 0));
     KVP_CUDA(ctx, kvp_launch_export(ctx->shape, plan_dev(ctx, slot), b, layer, as.items[b].prefix_len, n_query_rows,
                                     ctx->pool_k, ctx->pool_v, ctx->slot_k[slot], ctx->slot_v[slot], k_out, v_out,
-                                    k_as_f32, (cudaStream_t)stream));
+                                    k_as_f32, as.settled, (cudaStream_t)stream));
     return KVP_OK;
 }
 

@@ -288,8 +288,9 @@ struct kvp_ctx {
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// Loads the compiler may take for invariant (const __restrict__ parameters) could be moved in front of the wait; a pointer
-// that passes through here cannot be used before this point.
+// Loads the compiler may take for invariant (const __restrict__ parameters) could be moved in front of the wait, or made
+// non-coherent; a pointer that passes through here cannot be used before this point.  What a kernel in front may have
+// written is not read with __ldg either: that is for what nothing writes while the kernel is there, and it is there early.
 #define PDL_AFTER(p) asm volatile("" : "+l"(p)::"memory")
 
 template <typename T> struct as_given { typedef T type; };
@@ -352,9 +353,10 @@ cudaError_t kvp_launch_append(const kvp_shape &sh, const kvp_plan_dev &plan, int
                               int32_t q_pos0, const void *q, const void *k_new, const void *v_new, char *ws_k, char *ws_v,
                               int32_t layer, int32_t rope_query, const double *half_turns, void *q_rot,
                               cudaStream_t st);
+// early: it may begin before the kernel in front has ended; the prefix was complete before that one released anyone
 cudaError_t kvp_launch_export(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t b, int32_t layer,
                               int32_t prefix_len, int32_t n_query_rows, const char *pool_k, const char *pool_v,
-                              const char *ws_k, const char *ws_v, void *k_out, void *v_out, int32_t k_as_f32,
+                              const char *ws_k, const char *ws_v, void *k_out, void *v_out, int32_t k_as_f32, bool early,
                               cudaStream_t st);
 cudaError_t kvp_launch_segment_mass(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t batch, int32_t q_len,
                                     int32_t q_pos0, int32_t layer, const void *q, const float *lse, const char *pool_k,

@@ -309,7 +309,7 @@ __device__ __forceinline__ Vec16<T> load_vec(const T *p, bool aligned)
 {
     Vec16<T> v;
     if (aligned) {
-        v.u = __ldg(reinterpret_cast<const uint4 *>(p));
+        v.u = *reinterpret_cast<const uint4 *>(p);
     } else {
 #pragma unroll
         for (int e = 0; e < Elem<T>::kPerVec; ++e) v.e[e] = p[e];
@@ -371,7 +371,9 @@ append_kernel(kvp_plan_dev plan, int plan_there, int q_len, int q_pos0, const T 
 // ---- export of the logical composed cache of one (layer, request) ---------------------------------
 // A block takes kExportRows rows of all kv heads: where each row lies is looked up once (prefix rows come from where
 // attention reads them: the materialised cache or the staged adapter rows, already re-based, else the pool, rotated
-// here), then every thread moves pairs of 16-byte words, two in flight.  Bound by DRAM: one element per thread and one
+// here), then every thread moves pairs of 16-byte words, two in flight.  The prefix lies there since before the launch (the
+// caller sees to that with `early`); only blocks that reach the appended rows need loads that are coherent, which are slower
+// (all blocks with them: a handover pass 182 -> 189 us).  Bound by DRAM: one element per thread and one
 // row and head per block took 39 us for 9,000 rows of 8 heads of 128 (73 MB), 1.9 TB/s.
 constexpr int kExportRows = 16;
 
@@ -426,6 +428,7 @@ export_kernel(kvp_plan_dev plan, int b, int layer, int prefix_len, int n_rows, c
     __syncthreads();
     const int half = d / 2, half_vecs = half / EV, vecs = 2 * half_vecs;
     const int n_items = min(kExportRows, n_rows - t0) * n_kv * half_vecs;
+    const bool appended = t0 + kExportRows > prefix_len;     // rows that the launch in front may have written
     const bool al_k = ((uintptr_t)k_out & 15) == 0, al_v = ((uintptr_t)v_out & 15) == 0;
     for (int w0 = threadIdx.x; w0 < n_items; w0 += 512) {
         Vec16<T> lo[2], hi[2], va[2], vb[2];
@@ -437,10 +440,17 @@ export_kernel(kvp_plan_dev plan, int b, int layer, int prefix_len, int n_rows, c
             const int64_t src = ((int64_t)(layer * n_kv + hk) * (s_pool[r] ? pool_rows : ws_rows) + s_row[r]) * vecs + c;
             const uint4 *ks = reinterpret_cast<const uint4 *>(s_pool[r] ? pool_k : ws_k) + src;
             const uint4 *vs = reinterpret_cast<const uint4 *>(s_pool[r] ? pool_v : ws_v) + src;
-            lo[u].u = __ldg(ks);
-            hi[u].u = __ldg(ks + half_vecs);
-            va[u].u = __ldg(vs);
-            vb[u].u = __ldg(vs + half_vecs);
+            if (appended) {
+                lo[u].u = *ks;
+                hi[u].u = *(ks + half_vecs);
+                va[u].u = *vs;
+                vb[u].u = *(vs + half_vecs);
+            } else {
+                lo[u].u = __ldg(ks);
+                hi[u].u = __ldg(ks + half_vecs);
+                va[u].u = __ldg(vs);
+                vb[u].u = __ldg(vs + half_vecs);
+            }
         }
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
@@ -565,7 +575,7 @@ attn_core_kernel(kvp_plan_dev plan, int q_len, int q_pos0, int layer, const T *_
             Vec16<T> x;
             x.u = make_uint4(0, 0, 0, 0);
             if (rr < n_rows)
-                x.u = __ldg(reinterpret_cast<const uint4 *>(q + (((int64_t)b * q_len + rr / group) * n_q + hk * group + rr % group) * D + c));
+                x.u = *reinterpret_cast<const uint4 *>(q + (((int64_t)b * q_len + rr / group) * n_q + hk * group + rr % group) * D + c);
 #pragma unroll
             for (int e = 0; e < EV; e += 4)
                 *reinterpret_cast<float4 *>(Qs + (w / (D / EV)) * LD + c + e) =
@@ -644,10 +654,10 @@ attn_core_kernel(kvp_plan_dev plan, int q_len, int q_pos0, int layer, const T *_
                         kr = k_new + src;
                         vr = v_new + src;
                     }
-                    ka[u].u = __ldg(kr);
-                    kc[u].u = __ldg(kr + CP);
-                    va[u].u = __ldg(vr);
-                    vc[u].u = __ldg(vr + CP);
+                    ka[u].u = *kr;
+                    kc[u].u = *(kr + CP);
+                    va[u].u = *vr;
+                    vc[u].u = *(vr + CP);
                     if (fresh && rt == 0) {
                         uint4 *kw = reinterpret_cast<uint4 *>(ws_k_out) + (row + kk) * (2 * CP) + c;
                         uint4 *vw = reinterpret_cast<uint4 *>(ws_v_out) + (row + kk) * (2 * CP) + c;
@@ -671,13 +681,13 @@ attn_core_kernel(kvp_plan_dev plan, int q_len, int q_pos0, int layer, const T *_
                     if (pairing == 0) {
 #pragma unroll
                         for (int e = 0; e < EV; ++e) {
-                            const float2 r = __ldg(cs + c * EV + e);
+                            const float2 r = *(cs + c * EV + e);
                             rotate_pair(a[e], x[e], r.x, r.y);
                         }
                     } else {
 #pragma unroll
                         for (int e = 0; e < EV; e += 2) {
-                            const float2 r = __ldg(cs + (c * EV + e) / 2), r2 = __ldg(cs + (c * EV + HALF + e) / 2);
+                            const float2 r = *(cs + (c * EV + e) / 2), r2 = *(cs + (c * EV + HALF + e) / 2);
                             rotate_pair(a[e], a[e + 1], r.x, r.y);
                             rotate_pair(x[e], x[e + 1], r2.x, r2.y);
                         }
@@ -1027,17 +1037,17 @@ cudaError_t kvp_launch_append(const kvp_shape &sh, const kvp_plan_dev &plan, int
 
 cudaError_t kvp_launch_export(const kvp_shape &sh, const kvp_plan_dev &plan, int32_t b, int32_t layer,
                               int32_t prefix_len, int32_t n_query_rows, const char *pool_k, const char *pool_v,
-                              const char *ws_k, const char *ws_v, void *k_out, void *v_out, int32_t k_as_f32,
+                              const char *ws_k, const char *ws_v, void *k_out, void *v_out, int32_t k_as_f32, bool early,
                               cudaStream_t st)
 {
     const int n_rows = prefix_len + n_query_rows;
     if (n_rows <= 0) return cudaSuccess;
     const int grid = (n_rows + kExportRows - 1) / kExportRows;
     if (sh.dtype == KVP_DTYPE_BF16)
-        return launch_pdl(export_kernel<__nv_bfloat16>, grid, 256, 0, st, plan, b, layer, prefix_len, n_rows, pool_k, pool_v, ws_k,
+        return launch_when(early, export_kernel<__nv_bfloat16>, grid, 256, 0, st, plan, b, layer, prefix_len, n_rows, pool_k, pool_v, ws_k,
                           ws_v, sh.pool_rows, sh.ws_rows, sh.n_kv_heads, sh.head_dim, sh.pairing, k_out, (__nv_bfloat16 *)v_out,
                           k_as_f32);
-    return launch_pdl(export_kernel<float>, grid, 256, 0, st, plan, b, layer, prefix_len, n_rows, pool_k, pool_v, ws_k, ws_v,
+    return launch_when(early, export_kernel<float>, grid, 256, 0, st, plan, b, layer, prefix_len, n_rows, pool_k, pool_v, ws_k, ws_v,
                       sh.pool_rows, sh.ws_rows, sh.n_kv_heads, sh.head_dim, sh.pairing, k_out, (float *)v_out, k_as_f32);
 }
 
