@@ -196,6 +196,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
         int steps, first, stride, n_tail, n_total, limit;
         const kvp_tile *tiles;
         int row_b = 0, n_per = 1;                               // joint units: the row's request; causal tiles of each
+        bool idle;                                              // none of this warp's rows exists
         {
             const Work w = load_work<JOINT>(p, c.works, wi);
             steps = S == 0 ? w.steps0 : w.steps1;
@@ -205,6 +206,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
             tiles = p.plan.tiles + w.tile_begin - n_tail;
             n_total = p.q_pos0 + w.q_len;
             const int r = w.row_base + (w.mode == 0 ? S * KVP_TILE_ROWS : 0) + t;
+            idle = !JOINT && r - t + (t & ~31) >= p.group * w.q_len;
             if (JOINT) {
                 tiles = p.joint_tiles - n_tail;
                 n_per = w.per;
@@ -238,9 +240,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
             if (!ok) break;
             tc_fence_after();
 
-            const bool full = !JOINT && n_keys == KVP_TILE_KEYS && j >= n_tail;
-            int lim = j >= n_tail ? n_keys : min(n_keys, limit - (JOINT ? j % n_per : j) * KVP_TILE_KEYS);     // visible keys: [0, lim)
-            if (JOINT && !mine) lim = 0;
+            const int lim = j >= n_tail ? n_keys : min(n_keys, limit - (JOINT ? j % n_per : j) * KVP_TILE_KEYS);     // visible keys: [0, lim)
             if (JOINT && k == 0) {
                 // P V leaves out the rows that do not hold a tile, so its first product does not set their O
                 if (__any_sync(0xffffffffu, !mine && row_b < p.joint_batch)) {
@@ -259,8 +259,12 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
             // a chunk's own max is reduced alongside and checked last, so that the two dependency chains overlap.  Only if it
             // exceeds the reference by more than 2^8 (first tile of a piece, or a rare jump) are l, O and the P chunks
             // already written rescaled.
-            // a short tile (the end of a document, staged adapter rows) needs P only for the columns P V will read
-            const int n_ch = full ? 4 : max(1, (n_keys + 31) >> 5);         // (a row that does not see the tile writes P = 0)
+            // a short tile (the end of a document, staged adapter rows) needs P only for the columns P V will read (a row that
+            // does not see the tile writes P = 0).  Rows that do not exist have Q = 0, so S = 0, and that serves as P; what
+            // stands as P of rows that do not hold a joint tile, P V leaves out.  Launches of few rows are at the power limit
+            // like others: 16 tokens over 64 x 2048 (64 rows of 128) 115.9 -> 114.2 us, a decode layer (32 of 128) 48.8 -> 47.9.
+            const bool none = JOINT ? !__any_sync(0xffffffffu, mine) : idle;
+            const int n_ch = none ? 0 : max(1, (n_keys + 31) >> 5);
 #pragma unroll 1
             for (int ch = 0; ch < n_ch; ++ch) {
                 uint32_t v[32], pk[C::kSplit ? 32 : 16];
@@ -268,12 +272,12 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
                     tmem_ld32(s_addr + ch * 32, v);
                     tc_wait_ld();
                     landed32(v);
-                    if (!full) chunk_mask(v, lim - ch * 32);
+                    if (lim < ch * 32 + 32) chunk_mask(v, lim - ch * 32);
                 };
                 load();
                 const float cm = chunk_max(v, -INFINITY);
                 float ls = chunk_exp<C::kSplit>(v, c2, m_ref * c2, pk);
-                const bool need = (cm - m_ref) * c2 > 8.0f;
+                const bool need = mine && (cm - m_ref) * c2 > 8.0f;
                 if (__any_sync(0xffffffffu, need)) {
                     const float m_new = need ? cm : m_ref;
                     const float alpha = need ? ex2((m_ref - m_new) * c2) : 1.f;
@@ -285,7 +289,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
                 }
                 if (C::kSplit) tmem_st32(s_addr + ch * 32, pk);         // over this chunk's own scores
                 else tmem_st16(s_addr + ch * 16, pk);
-                l += ls;
+                if (mine) l += ls;
             }
             tc_wait_st();
             tc_fence_before();
