@@ -516,6 +516,11 @@ __device__ __forceinline__ void chunk_mask(uint32_t *v, int lim)
     for (int i = 0; i < 32; ++i)
         if (i >= lim) v[i] = 0xff800000u;                  // -inf
 }
+// A row's reference stays while the sum of a chunk's 32 exponentials is at most this; then it moves to the chunk's maximum,
+// which is at least 2^3 above it.  The sum is there anyway; taking the maximum of every chunk was 16 instructions per chunk
+// and 2 % of a tile's cycles.  (2^13: 3 % fewer cycles yet with outlier channels, but then fewer rows have their largest
+// probability exact, as that of the key the reference is.)
+constexpr float kJumpSum = 256.f;
 // p = exp2(s*c2 - mc) for 32 scores, packed as bf16 pairs into pk[0..15] (SPLIT: what that rounding dropped, as bf16
 // pairs, into pk[16..31]); returns their fp32 sum.
 // (Evaluating part of the exponentials by a polynomial on the FMA pipe was measured and lost: the

@@ -14,8 +14,8 @@
 //                     reference maximum m, P as bf16 over S.  O is shared by both warpgroups, so tile k's P has to be
 //                     relative to the reference that is in force after tile k - 1: the two warps of a row quadrant hand it
 //                     over (mref, an mbarrier per warp).  It rarely changes (only by more than 2^8); then this tile's P
-//                     or, once P V of tile k - 1 has landed, O is rescaled.  The second tile of a piece starts from the
-//                     maximum of the first one's first 32 keys (another barrier): starting from its own, its P was always
+//                     or, once P V of tile k - 1 has landed, O is rescaled.  The second tile of a piece starts from
+//                     where the first one does (another barrier): starting from its own maximum, its P was always
 //                     scaled at the hand-over, i.e. rounded twice, and the error of a piece of two or three tiles 1.15 times
 //                     as large.
 //   warps 8-11        Q producer: counter-rotates this CTA's rows once per document (as in the one-CTA kernel), and appends
@@ -187,6 +187,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
 
     for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
         int n, lo, n_tail, n_total, limit;
+        bool idle;                                        // none of this warp's rows exists
         const kvp_tile *tiles;
         {
             const Work w = load_work(p, c.works, wi);
@@ -196,6 +197,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
             tiles = p.plan.tiles + w.tile_begin - n_tail;
             n_total = p.q_pos0 + w.q_len;
             const int r = w.row_base + c.rank * KVP_TILE_ROWS + t;
+            idle = r - t + (t & ~31) >= p.group * w.q_len;
             limit = p.q_pos0 + (r < p.group * w.q_len ? row_token(p, r) : w.q_len - 1) + 1;     // causal keys this row sees
         }
         float m = -1e30f, l = 0.f;
@@ -213,18 +215,37 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
-            const bool full = n_keys == KVP_TILE_KEYS && j >= n_tail;
             const int lim = j >= n_tail ? n_keys : min(n_keys, limit - j * KVP_TILE_KEYS);       // visible keys: [0, lim)
-            // a short tile (the end of a document, staged adapter rows) needs P only for the columns P V will read
-            const int n_ch = full ? 4 : max(1, (n_keys + 31) >> 5);
+            // a short tile (the end of a document, staged adapter rows) needs P only for the columns P V will read; rows that
+            // do not exist have Q = 0, so S = 0, and that serves as P
+            const int n_ch = idle ? 0 : max(1, (n_keys + 31) >> 5);
             if (k < 2) {
                 if (k == 0) {
-                    uint32_t v[32];
-                    tmem_ld32(s_addr, v);
-                    tc_wait_ld();
-                    landed32(v);
-                    if (!full) chunk_mask(v, lim);
-                    m = chunk_max(v, m);
+                    // the reference a piece starts from: the maximum of its first tile, and of the second one too where the
+                    // first is the block of the query's own keys, of which its first rows see only a few.  (All eight warps
+                    // of a pair wait where one moves a reference: with the maximum of 32 keys, documents of outlier channels
+                    // 1177 -> 1135 us over two layers, the longest pair of one without them 102 -> 99.5 us.)
+                    auto max_of = [&](uint32_t addr, int seen_keys, int chunks) {
+#pragma unroll 1
+                        for (int ch = 0; ch < chunks; ++ch) {
+                            uint32_t v[32];
+                            tmem_ld32(addr + ch * 32, v);
+                            tc_wait_ld();
+                            landed32(v);
+                            if (seen_keys < ch * 32 + 32) chunk_mask(v, seen_keys - ch * 32);
+                            m = chunk_max(v, m);
+                        }
+                    };
+                    max_of(s_addr, lim, n_ch);
+                    if (lo == 0 && n_tail == 1 && n > 1) {
+                        const uint32_t use1 = (T + 1) / 3, buf1 = T + 1 - 3 * use1;
+                        ok = wait(p, c, kSFull + buf1, use1 & 1, 39);
+                        ok = __all_sync(0xffffffffu, ok);
+                        if (!ok) break;
+                        tc_fence_after();
+                        const int nk1 = keys_of(1);
+                        max_of(c.tmem + lane_base + buf1 * 128, nk1, idle ? 0 : (nk1 + 31) >> 5);
+                    }
                     st_shared(mref, __float_as_uint(m));
                     __syncwarp();
                     if (lead_lane) mbar_arrive(c.bar(kStart + quad));
@@ -235,9 +256,9 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
                     m = __uint_as_float(ld_shared(mref));
                 }
             }
-            // One pass over S, 32 columns at a time, against the reference max this warpgroup knows; a chunk's own max is
-            // reduced alongside and checked last.  Only if it exceeds the reference by more than 2^8 (a
-            // rare jump) does the reference move and the P written so far with it.
+            // One pass over S, 32 columns at a time, against the reference max this warpgroup knows.  Only if a chunk's sum
+            // shows that it exceeds the reference by far (kJumpSum) is its max formed, and the reference moves there and the
+            // P written so far with it.
 #pragma unroll 1
             for (int ch = 0; ch < n_ch; ++ch) {
                 uint32_t v[32], pk[16];
@@ -245,19 +266,18 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
                     tmem_ld32(s_addr + ch * 32, v);
                     tc_wait_ld();
                     landed32(v);
-                    if (!full) chunk_mask(v, lim - ch * 32);
+                    if (lim < ch * 32 + 32) chunk_mask(v, lim - ch * 32);
                 };
                 load();
-                const float cm = chunk_max(v, -INFINITY);
                 float ls = chunk_exp<false>(v, c2, m * c2, pk);
-                const bool need = (cm - m) * c2 > 8.0f;
+                const bool need = ls > kJumpSum;
                 if (__any_sync(0xffffffffu, need)) {
-                    const float m_new = need ? cm : m;
+                    load();                               // this chunk's scores again (P so far lies below them)
+                    const float m_new = need ? chunk_max(v, m) : m;
                     const float alpha = need ? ex2((m - m_new) * c2) : 1.f;
                     scale_p(s_addr, alpha, ch);
                     l *= alpha;
                     m = m_new;
-                    load();                               // this chunk's scores again (P so far lies below them)
                     ls = chunk_exp<false>(v, c2, m * c2, pk);
                 }
                 tmem_st16(s_addr + ch * 16, pk);
@@ -271,7 +291,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
                 if (!ok) break;
                 const float mp = __uint_as_float(ld_shared(mref));
                 if (__any_sync(0xffffffffu, mp != m)) {
-                    const bool raise = (m - mp) * c2 > 8.0f;              // O follows this tile; else this tile follows O
+                    const bool raise = m > mp;                            // O follows this tile; else this tile follows O
                     const float ap = raise ? 1.f : ex2((m - mp) * c2), ao = raise ? ex2((mp - m) * c2) : 1.f;
                     scale_p(s_addr, ap, n_ch);
                     l *= ap;

@@ -106,3 +106,21 @@ def test_either_kernel_on_request(q_len):
         check_attention(wl, sess)
         assert on_pairs(sess, q_len) == (pairs == 1 and q_len in (64, 409))
     sess.close()
+
+
+@pytest.mark.parametrize("lens,q_len,ctas", [([40], 33, 0), ([300, 500], 33, 2), ([300, 500], 64, 0), ([1500], 192, 4)])
+def test_first_rows_see_few_keys(lens, q_len, ctas):
+    # The first rows of the query block see one key, two, ... of it.  With those keys small and the documents' large, a
+    # chunk's exponentials sum to more than 2^8 against such a start (33 tokens: three of the second CTA's warps have no rows).
+    shape = gen.ModelShape(1, 32, 8, 128, "bf16", 500000.0, 0)
+    wl = gen.make_workload(shape, lens, [[(p, 0) for p in range(len(lens))]], q_len=q_len, seed=23 + q_len)
+    wl.k_new[0][:] = gen.to_stored(gen.bf16_bits_to_f32(wl.k_new[0]) * np.float32(0.05), "bf16")
+    for i, pk in enumerate(wl.packets):
+        pk.k[:] = gen.to_stored(gen.bf16_bits_to_f32(pk.k) * np.float32(1.5 + i), "bf16")
+    sess = Session(wl)
+    sess.assemble()
+    if ctas:
+        sess.ctx.tune(kvp.TUNE_SPLIT_TARGET_CTAS, ctas)
+    check_attention(wl, sess, flags=kvp.PRECISE_QK)
+    assert on_pairs(sess, q_len)
+    sess.close()
