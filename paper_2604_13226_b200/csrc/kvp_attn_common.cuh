@@ -33,6 +33,7 @@ struct Params {
     // epoch buffer instead of two) and Q K^T of a rotated tile takes both
     int precise;
     int fresh;                 // the work list was uploaded by the kernel in front, or comes along with this launch
+    int plan_there;            // the plan was complete before the launch in front of this one was released
     uint32_t list_bytes, list_works;           // in the latter case: its size, where the pieces begin, and where it is stored for
     uint4 *list_dev;                           // the launches behind this one
     int joint_batch;           // joint units (kvp_joint): their requests, tiles and offsets
@@ -579,14 +580,36 @@ __device__ __forceinline__ void append_rows(const Params &p, const Work &w, int 
     }
 }
 
-// Start of a kernel whose work list comes along with the launch (a list in device memory costs a kernel of its own in front,
-// 4 us on the way to the first tile): CTA 0 stores it for the launches behind, before any of them is released.
+// A work list that comes along with the launch (a list in device memory costs a kernel of its own in front, 4 us on the way
+// to the first tile) is stored for the launches behind by a warp of one CTA that has nothing to do yet.  That CTA releases
+// them behind its store, all others at once; a grid releases when its last CTA has.
 template <int LB>
-__device__ __forceinline__ void store_list(const Params &p, const kvp_blob<LB> &list, int tid, int n_threads)
+__device__ __forceinline__ void store_list(const Params &p, const kvp_blob<LB> &list, int lane)
 {
-    if (blockIdx.x != 0) return;
-    for (uint32_t i = tid; i < p.list_bytes / 16; i += n_threads) p.list_dev[i] = list.w[i];
+    pdl_wait();
+    for (uint32_t i = lane; i < p.list_bytes / 16; i += 32) p.list_dev[i] = list.w[i];
     __threadfence();
+    __syncwarp();
+    pdl_launch_dependents();
+}
+
+// First of all a launch releases the ones behind it, unless its list is new ...
+template <int LB>
+__device__ __forceinline__ void release_at_once(const Params &p)
+{
+    if (LB == 0 && !p.fresh) pdl_launch_dependents();
+}
+// ... and before it reads tables it waits for those that may not be there, and releases then.  `storing`: this CTA stores the list.
+template <int LB>
+__device__ __forceinline__ void wait_for_tables(const Params &p, bool storing)
+{
+    if (LB > 0) {
+        if (!p.plan_there) pdl_wait();
+        if (!storing) pdl_launch_dependents();
+    } else if (p.fresh) {
+        pdl_wait();
+        pdl_launch_dependents();
+    }
 }
 
 inline Params make_params(const kvp_shape &sh, const kvp_attn2_args &a)
@@ -614,6 +637,7 @@ inline Params make_params(const kvp_shape &sh, const kvp_attn2_args &a)
     p.tail_direct = a.tail_direct;
     p.precise = a.precise;
     p.fresh = a.fresh;
+    p.plan_there = a.plan_there;
     p.list_bytes = a.list_bytes;
     p.list_works = a.list_works;
     p.list_dev = (uint4 *)a.list_dev;

@@ -63,17 +63,23 @@ __device__ __forceinline__ uint32_t cluster_addr(uint32_t a, uint32_t rank)
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
     return r;
 }
-__device__ __forceinline__ void cluster_sync()
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// Every warp arrives at the cluster's barrier once its own part of the set-up is done (warp 0: barriers, warp 12: TMEM) and
+// waits there only when it has looked up its first piece and tile - the producers when they have formed the first Q tile.
+// First scores of a launch, 8.3 us after its entry with all of it in front of the look-ups: 7.0 (pruned documents: 7.9, 6.1;
+// the one-CTA kernel, where the look-ups lie behind one __syncthreads, lost 1 % with the same order).
+__device__ __forceinline__ void begin(Cta &c)
 {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    __syncwarp();
+    cluster_wait();
+    tc_fence_after();
+    c.tmem = ld_shared(c.tmem_slot());
 }
-// Shared memory written before it (the rotated Q) is released to the cluster.
-__device__ __forceinline__ void remote_arrive_release(uint32_t cluster_bar)
-{
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
-}
-// For what lies in TMEM, which tcgen05.fence::before_thread_sync orders: a release to the cluster waits for everything the
-// SM has in flight, 1,000 cycles and more per tile (it took half of the softmax warps' time).
+// What is handed over lies in TMEM, which tcgen05.fence::before_thread_sync orders, or in this CTA's own shared memory (the
+// rotated Q), written back to the tensor core's view by fence.proxy.async: a release to the cluster on top of that waits for
+// everything the SM has in flight, 1,000 cycles and more (per tile, it took half of the softmax warps' time; for Q, the
+// first scores of a launch came 1 us later).
 __device__ __forceinline__ void remote_arrive(uint32_t cluster_bar)
 {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
@@ -171,12 +177,12 @@ __device__ __forceinline__ void scale_o(uint32_t o_addr, float alpha)
     tc_wait_st();
 }
 
-__device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, const int G, const int t)
+__device__ __forceinline__ void softmax_role(const Params &p, Cta &c, const int G, const int t)
 {
     const int quad = t >> 5;
     const bool lead_lane = (t & 31) == 0;
     const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
-    const uint32_t o_addr = c.tmem + lane_base + kColO;
+    uint32_t o_addr = 0;
     const float c2 = p.scale_log2;
     const uint32_t mref = c.smem_base + kOffMref + 4 * t;
     const int own = 4 * G + quad, other = 4 * (G ^ 1) + quad;         // hand-over barriers of this row quadrant's two warps
@@ -205,6 +211,10 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
             return j < n_tail ? min(KVP_TILE_KEYS, n_total - j * KVP_TILE_KEYS) : (int)tiles[j].n_keys;
         };
         int nk_next = G < n ? keys_of(lo + G) : 0;
+        if (wi == c.item_begin) {
+            begin(c);
+            o_addr = c.tmem + lane_base + kColO;
+        }
 #pragma unroll 1
         for (int k = G; k < n; k += 2) {
             const int j = lo + k, n_keys = nk_next;
@@ -222,7 +232,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
             if (k < 2) {
                 if (k == 0) {
                     // the reference a piece starts from: the maximum of its first tile, and of the second one too where the
-                    // first is the block of the query's own keys, of which its first rows see only a few.  (All eight warps
+                    // first is the block of the query's own keys, of which its first rows see only a few (and more follow).  (All eight warps
                     // of a pair wait where one moves a reference: with the maximum of 32 keys, documents of outlier channels
                     // 1177 -> 1135 us over two layers, the longest pair of one without them 102 -> 99.5 us.)
                     auto max_of = [&](uint32_t addr, int seen_keys, int chunks) {
@@ -237,7 +247,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
                         }
                     };
                     max_of(s_addr, lim, n_ch);
-                    if (lo == 0 && n_tail == 1 && n > 1) {
+                    if (lo == 0 && n_tail == 1 && n > 2) {
                         const uint32_t use1 = (T + 1) / 3, buf1 = T + 1 - 3 * use1;
                         ok = wait(p, c, kSFull + buf1, use1 & 1, 39);
                         ok = __all_sync(0xffffffffu, ok);
@@ -320,6 +330,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
         if (!ok) break;
 
         // ---- end of the piece: O is complete once its last P V has landed ----------
+        const Work w = load_work(p, c.works, wi);
         ok = wait(p, c, kOFull, phO & 1, 32);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
@@ -337,7 +348,6 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
         const float M = ((n - 1) & 1) == G ? m : o.x;     // O is relative to the last tile's reference
         l = l * ex2((m - M) * c2) + o.y * ex2((o.x - M) * c2);
 
-        const Work w = load_work(p, c.works, wi);
         const int r = w.row_base + c.rank * KVP_TILE_ROWS + t;
         const bool valid = r < p.group * w.q_len;
         const int qi = valid ? row_token(p, r) : w.q_len - 1;
@@ -387,7 +397,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
 }
 
 // ---- Q producer: this CTA's 128 rows, once per document; append ------------------------------------------------
-__device__ __forceinline__ void producer_role(const Params &p, const Cta &c, const int t)
+__device__ __forceinline__ void producer_role(const Params &p, Cta &c, const int t)
 {
     const uint32_t stride = p.precise ? 2 * kQBufBytes : kQBufBytes;
     uint32_t ep = 0;
@@ -410,8 +420,9 @@ __device__ __forceinline__ void producer_role(const Params &p, const Cta &c, con
             produce_q_tile<128>(p, qb, p.precise ? qb + kQBufBytes : nullptr, t, p.q + (long long)w.b * p.q_len * p.n_q * 128, w.hk,
                                 w.row_base + c.rank * KVP_TILE_ROWS, n_rows, rope);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            if (ep == 0) begin(c);                            // (the first tile is formed while barriers and TMEM are set up)
             __syncwarp();
-            if ((t & 31) == 0) remote_arrive_release(c.lead(kQFull + buf));
+            if ((t & 31) == 0) remote_arrive(c.lead(kQFull + buf));
             ++ep;
             // the append (as in the one-CTA kernel): the tokens whose first packed row lies in this CTA's rows, behind the
             // piece's first Q tile
@@ -431,7 +442,7 @@ __device__ __forceinline__ void load_at(int n, int q, int &r, int &kv)
 }
 
 // ---- TMA producer (whole warp): this CTA's half of every tile ---------------------------------------------------
-__device__ __forceinline__ void tma_role(const Params &p, const Cta &c, const int lane, const CUtensorMap *k_pool,
+__device__ __forceinline__ void tma_role(const Params &p, Cta &c, const int lane, const CUtensorMap *k_pool,
                                          const CUtensorMap *v_pool, const CUtensorMap *k_ws, const CUtensorMap *v_ws,
                                          const CUtensorMap *k_new, const CUtensorMap *v_new)
 {
@@ -458,6 +469,7 @@ __device__ __forceinline__ void tma_role(const Params &p, const Cta &c, const in
             const int x = kv ? 64 * c.rank : 0, y = kv ? row0 : row0 + c.rank * (qk_n(n_keys) / 2);
             const int cnt = min(32, n_loads - q0);
             const bool ahead = p.l2_prefetch && lane < cnt && src != 2;
+            if (wi == c.item_begin && q0 == 0) begin(c);
 #pragma unroll 1
             for (int i = 0; i < cnt && ok; ++i) {
                 if (ahead && lane == i + 4) {             // tiles that come from DRAM: L2 is asked for the one four loads ahead
@@ -492,7 +504,7 @@ __device__ __forceinline__ void tma_role(const Params &p, const Cta &c, const in
 // wait in a queue that the sub-partition's special-function instructions go through too, so this warp's two softmax
 // neighbours are slower than the others (3,000 cycles per tile against 2,400); three issuing warps on three sub-partitions
 // in turn evened that out and did not help: the launch is then bound by power (1,000 W) or by the hand-over between them.
-__device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
+__device__ __forceinline__ void mma_role(const Params &p, Cta &c)
 {
     const uint32_t n_stages = p.precise ? 5 : 9;
     const uint32_t q_stride = p.precise ? 2 * kQBufBytes : kQBufBytes;
@@ -522,6 +534,7 @@ __device__ __forceinline__ void mma_role(const Params &p, const Cta &c)
             }
         };
         refill(0);
+        if (wi == c.item_begin) begin(c);
         int nk1 = 0, nk2 = 0, nk3 = 0;                    // key counts of the last three tiles
         int prev_rope = 0;
         uint32_t qbuf = 0;
@@ -634,54 +647,52 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap k_pool, const __grid_consta
     c.bar0 = c.smem_base + kOffBar;
     c.lead0 = cluster_addr(c.bar0, 0);
     c.rank = (int)(blockIdx.x & 1);
-    if (!p.fresh) pdl_launch_dependents();
+    release_at_once<LB>(p);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-    if (tid == 0) {
-        for (int i = 0; i < kNumBars; ++i) {
+    if (warp == 0) {
+        for (int i = lane; i < kNumBars; i += 32) {
             uint32_t count = 1;
             if (i >= kQFull && i < kQFree) count = 8;                   // four producer warps of both CTAs
             else if (i >= kPFull && i < kPvDone) count = 8;             // four softmax warps of both CTAs
             else if (i == kOFree) count = 16;                           // eight softmax warps of both CTAs
             mbar_init(c.bar(i), count);
         }
-        st_shared(c.abort_flag(), 0);
+        if (lane == 0) st_shared(c.abort_flag(), 0);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 12) {
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(c.tmem_slot()) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
-    const int32_t *cta_begin = p.cta_begin;
-    c.works = p.works;
-    if (LB > 0) {
-        pdl_wait();
-        store_list<LB>(p, list, tid, kThreads);
-        cta_begin = reinterpret_cast<const int32_t *>(&list);
-        c.works = reinterpret_cast<const kvp_work *>(reinterpret_cast<const char *>(&list) + p.list_works);
-    } else if (p.fresh) {
-        pdl_wait();
-        pdl_launch_dependents();
-    }
+    __syncwarp();
+    tc_fence_before();
+    cluster_arrive();
+    wait_for_tables<LB>(p, blockIdx.x == 1);
     // from here on: the Q producer, the append and the TMA warp (for anything but pool tiles) wait for the kernel in front;
     // everything else follows from what they deliver
     // (the work list gives every pair at least one piece)
+    const int32_t *cta_begin = p.cta_begin;
+    c.works = p.works;
+    if (LB > 0) {
+        cta_begin = reinterpret_cast<const int32_t *>(&list);
+        c.works = reinterpret_cast<const kvp_work *>(reinterpret_cast<const char *>(&list) + p.list_works);
+    }
     const int32_t *range = cta_begin + (blockIdx.x >> 1);
     c.item_begin = LB > 0 ? range[0] : __ldcg(range);
     c.item_end = LB > 0 ? range[1] : __ldcg(range + 1);
-    __syncwarp();
-    tc_fence_before();
-    cluster_sync();                                           // both CTAs' barriers and TMEM are there
-    if (LB > 0) pdl_launch_dependents();
-    tc_fence_after();
-    c.tmem = ld_shared(c.tmem_slot());
 
     if (warp < 8) {
         softmax_role(p, c, warp >> 2, tid & 127);
     } else if (warp < 12) {
         producer_role(p, c, tid - 256);
     } else if (warp == 12) {
-        if (c.rank == 0) mma_role(p, c);
+        if (c.rank == 0) {
+            mma_role(p, c);
+        } else {
+            if (LB > 0 && blockIdx.x == 1) store_list<LB>(p, list, lane);
+            begin(c);
+        }
     } else if (warp == 13) {
         tma_role(p, c, lane, &k_pool, &v_pool, &k_ws, &v_ws, &k_new, &v_new);
     }
@@ -693,7 +704,8 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap k_pool, const __grid_consta
     }
     __syncwarp();
     tc_fence_before();
-    cluster_sync();
+    cluster_arrive();
+    cluster_wait();
     if (warp == 12) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(c.tmem) : "memory");

@@ -206,7 +206,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
             tiles = p.plan.tiles + w.tile_begin - n_tail;
             n_total = p.q_pos0 + w.q_len;
             const int r = w.row_base + (w.mode == 0 ? S * KVP_TILE_ROWS : 0) + t;
-            idle = !JOINT && r - t + (t & ~31) >= p.group * w.q_len;
+            idle = D == 128 && !JOINT && p.group * w.q_len > 32 && r - t + (t & ~31) >= p.group * w.q_len;
             if (JOINT) {
                 tiles = p.joint_tiles - n_tail;
                 n_per = w.per;
@@ -240,6 +240,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
             if (!ok) break;
             tc_fence_after();
 
+            const bool full = n_keys == KVP_TILE_KEYS && j >= n_tail;
             const int lim = j >= n_tail ? n_keys : min(n_keys, limit - (JOINT ? j % n_per : j) * KVP_TILE_KEYS);     // visible keys: [0, lim)
             if (JOINT && k == 0) {
                 // P V leaves out the rows that do not hold a tile, so its first product does not set their O
@@ -262,9 +263,10 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
             // a short tile (the end of a document, staged adapter rows) needs P only for the columns P V will read (a row that
             // does not see the tile writes P = 0).  Rows that do not exist have Q = 0, so S = 0, and that serves as P; what
             // stands as P of rows that do not hold a joint tile, P V leaves out.  Launches of few rows are at the power limit
-            // like others: 16 tokens over 64 x 2048 (64 rows of 128) 115.9 -> 114.2 us, a decode layer (32 of 128) 48.8 -> 47.9.
+            // like others: 16 tokens over 64 x 2048 (64 rows of 128) 115.4 -> 112.5 us, a decode layer in joint units (32 of
+            // 128) 48.8 -> 47.9.  Not where one warp has all rows (a decode step's 7 rows per unit: 667 -> 672 us with it).
             const bool none = JOINT ? !__any_sync(0xffffffffu, mine) : idle;
-            const int n_ch = none ? 0 : max(1, (n_keys + 31) >> 5);
+            const int n_ch = none ? 0 : full ? 4 : max(1, (n_keys + 31) >> 5);
 #pragma unroll 1
             for (int ch = 0; ch < n_ch; ++ch) {
                 uint32_t v[32], pk[C::kSplit ? 32 : 16];
@@ -272,7 +274,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
                     tmem_ld32(s_addr + ch * 32, v);
                     tc_wait_ld();
                     landed32(v);
-                    if (lim < ch * 32 + 32) chunk_mask(v, lim - ch * 32);
+                    if (!full && lim < ch * 32 + 32) chunk_mask(v, lim - ch * 32);
                 };
                 load();
                 const float cm = chunk_max(v, -INFINITY);
@@ -813,8 +815,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_pool_k, const __grid_co
     Cta c;
     c.smem_base = (smem_u32(smem_raw) + 1023) & ~1023u;
     c.bar0 = c.smem_base + C::kOffBar;
-    if (!p.fresh) pdl_launch_dependents();
-
+    release_at_once<LB>(p);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     if (tid == 0) {
@@ -843,26 +844,21 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_pool_k, const __grid_co
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    const int32_t *cta_begin = p.cta_begin;
-    c.works = p.works;
-    if (LB > 0) {
-        pdl_wait();
-        store_list<LB>(p, list, tid, kThreads);
-        cta_begin = reinterpret_cast<const int32_t *>(&list);
-        c.works = reinterpret_cast<const kvp_work *>(reinterpret_cast<const char *>(&list) + p.list_works);
-    } else if (p.fresh) {
-        pdl_wait();
-        pdl_launch_dependents();
-    }
+    wait_for_tables<LB>(p, blockIdx.x == 0);
     // from here on: the Q producer, the append and the TMA warp (for anything but pool tiles) wait for the kernel in front;
     // everything else follows from what they deliver
     // (the work list gives every CTA at least one piece)
-    const int32_t *range = cta_begin + (blockIdx.x);
+    const int32_t *cta_begin = p.cta_begin;
+    c.works = p.works;
+    if (LB > 0) {
+        cta_begin = reinterpret_cast<const int32_t *>(&list);
+        c.works = reinterpret_cast<const kvp_work *>(reinterpret_cast<const char *>(&list) + p.list_works);
+    }
+    const int32_t *range = cta_begin + blockIdx.x;
     c.item_begin = LB > 0 ? range[0] : __ldcg(range);
     c.item_end = LB > 0 ? range[1] : __ldcg(range + 1);
     tc_fence_before();
     __syncthreads();
-    if (LB > 0) pdl_launch_dependents();
     tc_fence_after();
     c.tmem = ld_shared(c.tmem_slot());
 
@@ -876,6 +872,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_pool_k, const __grid_co
         } else if (warp == 13) {
             tma_role<D, JOINT>(p, c, lane, &tm_pool_k, &tm_pool_v, &tm_ws_k, &tm_ws_v, &tm_knew, &tm_vnew);
         } else {
+            if (LB > 0 && blockIdx.x == 0 && warp == 15) store_list<LB>(p, list, lane);
             append_role<D>(p, c, tid - 448);
         }
     }

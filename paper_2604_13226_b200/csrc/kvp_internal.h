@@ -396,6 +396,7 @@ struct kvp_attn2_args {
     int32_t tail_direct;
     int32_t precise;               // KVP_PRECISE_QK
     int32_t fresh;                 // the work list was uploaded just before, by a kernel this launch has to wait for
+    int32_t plan_there;            // the plan was complete before the launch in front of this one was released
     // not null: the work list (list_bytes, padded to 16) comes along, works at list_works; the launch stores it at list_dev
     const void *list;
     uint32_t list_bytes, list_works;
