@@ -1089,7 +1089,9 @@ cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_
         mo.part_o = reinterpret_cast<float4 *>(part_out);
         mo.part_ml = reinterpret_cast<float2 *>((char *)part_out + (uint64_t)part_tiles * (32ull * KVP_TILE_ROWS * 16));
     }
-    // whole rows per block when that gives two blocks per SM, else quarter rows (halves with head dimension 64)
+    // whole rows per block when that gives two blocks per SM, else quarter rows (halves with head dimension 64).  Whole rows
+    // take two parts per round trip: units are cut into two or three, and with four parts' registers two blocks fit an SM, so
+    // that 512 took two waves (pruned documents 220.6 -> 218.2 us, ragged batches 818 -> 807, 4 x 10 x 1024 869 -> 864)
     const bool few = n_merges * (KVP_TILE_ROWS / 32) < 2 * sm_count;
     auto go = [&](auto *kernel, int cs) {
         return launch_pdl(kernel, dim3(n_merges, KVP_TILE_ROWS / 32, cs), 256, 0, st, merges, (int)list_there, q_len, sh.n_q_heads, sh.n_kv_heads,
@@ -1100,7 +1102,7 @@ cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_
     const bool many = max_parts > 16;
     if (sh.head_dim == 64)
         return !few ? go(merge_list_kernel<64, 1, 4>, 1) : many ? go(merge_list_kernel<64, 2, 20>, 2) : go(merge_list_kernel<64, 2, 8>, 2);
-    return !few ? go(merge_list_kernel<128, 1, 4>, 1) : many ? go(merge_list_kernel<128, 4, 20>, 4) : go(merge_list_kernel<128, 4, 8>, 4);
+    return !few ? go(merge_list_kernel<128, 1, 2>, 1) : many ? go(merge_list_kernel<128, 4, 20>, 4) : go(merge_list_kernel<128, 4, 8>, 4);
 }
 
 cudaError_t kvp_launch_merge_ranks(const kvp_shape &sh, int32_t batch, int32_t q_len, const void *parts, int32_t n_parts,
