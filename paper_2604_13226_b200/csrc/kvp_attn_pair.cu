@@ -385,7 +385,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, Cta &c, const int 
         }
         tc_fence_before();
         __syncwarp();
-        if (lead_lane) remote_arrive(c.lead(kOFree));
+        if (lead_lane && wi + 1 < c.item_end) remote_arrive(c.lead(kOFree));     // (nobody waits for the last one)
         if (G == 0) {
             if (direct) {
                 if (valid && p.lse != nullptr) p.lse[((long long)w.b * p.n_q + h) * p.q_len + qi] = M * p.scale + logf(l);
@@ -704,7 +704,9 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap k_pool, const __grid_consta
     }
     __syncwarp();
     tc_fence_before();
-    cluster_arrive();
+    // (relaxed: a release waits for the stores of the partial results, 0.6 us, and nobody here reads them; every arrive at the
+    // other CTA has been waited for there, so none is under way.  Question of 5 x 512 tokens 22.4 -> 22.0 us.)
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     cluster_wait();
     if (warp == 12) {
         tc_fence_after();
