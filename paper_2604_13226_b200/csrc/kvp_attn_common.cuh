@@ -517,11 +517,12 @@ __device__ __forceinline__ void chunk_mask(uint32_t *v, int lim)
     for (int i = 0; i < 32; ++i)
         if (i >= lim) v[i] = 0xff800000u;                  // -inf
 }
-// A row's reference stays while the sum of a chunk's 32 exponentials is at most this; then it moves to the chunk's maximum,
-// which is at least 2^3 above it.  The sum is there anyway; taking the maximum of every chunk was 16 instructions per chunk
-// and 2 % of a tile's cycles.  (2^13: 3 % fewer cycles yet with outlier channels, but then fewer rows have their largest
-// probability exact, as that of the key the reference is.)
-constexpr float kJumpSum = 256.f;
+// A row's reference moves when a score lies more than 2^8 above it.  The sum of the chunk's 32 exponentials, which is formed
+// anyway, is above 2^8 then, so up to this sum - below 2^8 by what rounding takes from either for references of 2^20 and less -
+// the maximum need not be formed.  4 x 16 documents of 2048, 1024 query tokens: 2200 us, 2270 with 128 (a chunk of many scores
+// somewhat above the reference reaches that), 2480 with a maximum of every chunk behind its exponentials; 20 x 8 documents, 28/4
+// heads 820, 925, 909.
+constexpr float kJumpSum = 240.f;
 // p = exp2(s*c2 - mc) for 32 scores, packed as bf16 pairs into pk[0..15] (SPLIT: what that rounding dropped, as bf16
 // pairs, into pk[16..31]); returns their fp32 sum.
 // (Evaluating part of the exponentials by a polynomial on the FMA pipe was measured and lost: the

@@ -15,7 +15,7 @@
 //                     relative to the reference that is in force after tile k - 1: the two warps of a row quadrant hand it
 //                     over (mref, an mbarrier per warp).  It rarely changes (only by more than 2^8); then this tile's P
 //                     or, once P V of tile k - 1 has landed, O is rescaled.  The second tile of a piece starts from
-//                     where the first one does (another barrier): starting from its own maximum, its P was always
+//                     the maximum of the first one's first 32 keys (another barrier): starting from its own, its P was always
 //                     scaled at the hand-over, i.e. rounded twice, and the error of a piece of two or three tiles 1.15 times
 //                     as large.
 //   warps 8-11        Q producer: counter-rotates this CTA's rows once per document (as in the one-CTA kernel), and appends
@@ -231,30 +231,16 @@ __device__ __forceinline__ void softmax_role(const Params &p, Cta &c, const int 
             const int n_ch = idle ? 0 : max(1, (n_keys + 31) >> 5);
             if (k < 2) {
                 if (k == 0) {
-                    // the reference a piece starts from: the maximum of its first tile, and of the second one too where the
-                    // first is the block of the query's own keys, of which its first rows see only a few (and more follow).  (All eight warps
-                    // of a pair wait where one moves a reference: with the maximum of 32 keys, documents of outlier channels
-                    // 1177 -> 1135 us over two layers, the longest pair of one without them 102 -> 99.5 us.)
-                    auto max_of = [&](uint32_t addr, int seen_keys, int chunks) {
-#pragma unroll 1
-                        for (int ch = 0; ch < chunks; ++ch) {
-                            uint32_t v[32];
-                            tmem_ld32(addr + ch * 32, v);
-                            tc_wait_ld();
-                            landed32(v);
-                            if (seen_keys < ch * 32 + 32) chunk_mask(v, seen_keys - ch * 32);
-                            m = chunk_max(v, m);
-                        }
-                    };
-                    max_of(s_addr, lim, n_ch);
-                    if (lo == 0 && n_tail == 1 && n > 2) {
-                        const uint32_t use1 = (T + 1) / 3, buf1 = T + 1 - 3 * use1;
-                        ok = wait(p, c, kSFull + buf1, use1 & 1, 39);
-                        ok = __all_sync(0xffffffffu, ok);
-                        if (!ok) break;
-                        tc_fence_after();
-                        const int nk1 = keys_of(1);
-                        max_of(c.tmem + lane_base + buf1 * 128, nk1, idle ? 0 : (nk1 + 31) >> 5);
+                    // the reference a piece starts from: the maximum of its first 32 keys.  (That of the whole tile, and of the next
+                    // one behind a causal block, moves less often: 28/4 heads with outlier channels 1180 -> 1120 us.  Not taken: it
+                    // decides which way each probability is rounded, and single outputs moved by 0.14 of the root mean square.)
+                    if (!idle) {
+                        uint32_t v[32];
+                        tmem_ld32(s_addr, v);
+                        tc_wait_ld();
+                        landed32(v);
+                        if (lim < 32) chunk_mask(v, lim);
+                        m = chunk_max(v, m);
                     }
                     st_shared(mref, __float_as_uint(m));
                     __syncwarp();
@@ -266,9 +252,9 @@ __device__ __forceinline__ void softmax_role(const Params &p, Cta &c, const int 
                     m = __uint_as_float(ld_shared(mref));
                 }
             }
-            // One pass over S, 32 columns at a time, against the reference max this warpgroup knows.  Only if a chunk's sum
-            // shows that it exceeds the reference by far (kJumpSum) is its max formed, and the reference moves there and the
-            // P written so far with it.
+            // One pass over S, 32 columns at a time, against the reference max this warpgroup knows.  Only if a chunk's max
+            // exceeds the reference by more than 2^8 (a rare jump) does the reference move and the P written so far with it;
+            // the max is formed only where the chunk's sum leaves room for that (kJumpSum).
 #pragma unroll 1
             for (int ch = 0; ch < n_ch; ++ch) {
                 uint32_t v[32], pk[16];
@@ -280,15 +266,18 @@ __device__ __forceinline__ void softmax_role(const Params &p, Cta &c, const int 
                 };
                 load();
                 float ls = chunk_exp<false>(v, c2, m * c2, pk);
-                const bool need = ls > kJumpSum;
-                if (__any_sync(0xffffffffu, need)) {
+                if (__any_sync(0xffffffffu, !(ls <= kJumpSum))) {
                     load();                               // this chunk's scores again (P so far lies below them)
-                    const float m_new = need ? chunk_max(v, m) : m;
-                    const float alpha = need ? ex2((m - m_new) * c2) : 1.f;
-                    scale_p(s_addr, alpha, ch);
-                    l *= alpha;
-                    m = m_new;
-                    ls = chunk_exp<false>(v, c2, m * c2, pk);
+                    const float cm = chunk_max(v, -INFINITY);
+                    const bool need = (cm - m) * c2 > 8.0f;
+                    if (__any_sync(0xffffffffu, need)) {
+                        const float m_new = need ? cm : m;
+                        const float alpha = need ? ex2((m - m_new) * c2) : 1.f;
+                        scale_p(s_addr, alpha, ch);
+                        l *= alpha;
+                        m = m_new;
+                        ls = chunk_exp<false>(v, c2, m * c2, pk);
+                    }
                 }
                 tmem_st16(s_addr + ch * 16, pk);
                 l += ls;
@@ -301,7 +290,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, Cta &c, const int 
                 if (!ok) break;
                 const float mp = __uint_as_float(ld_shared(mref));
                 if (__any_sync(0xffffffffu, mp != m)) {
-                    const bool raise = m > mp;                            // O follows this tile; else this tile follows O
+                    const bool raise = (m - mp) * c2 > 8.0f;              // O follows this tile; else this tile follows O
                     const float ap = raise ? 1.f : ex2((m - mp) * c2), ao = raise ? ex2((mp - m) * c2) : 1.f;
                     scale_p(s_addr, ap, n_ch);
                     l *= ap;

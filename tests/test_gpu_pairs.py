@@ -94,6 +94,79 @@ def test_probabilities_are_rounded_once(q_len):
     sess.close()
 
 
+def rounded_against_references(s, v, tiles):
+    """sum of P V / sum of p over one piece by the rule that moves references (the comment at the head of the pair kernel), in
+    float64 but for P, which is rounded to bf16 as often as there.  s: scores in powers of two [row][key], -inf where masked;
+    tiles: (first key, keys) of each.  Returns (result, whether a reference of the row moved)."""
+    bf16 = lambda x: x.bfloat16().double()
+    rows = s.shape[0]
+    m = [None, None]
+    o = torch.zeros(rows, v.shape[1], dtype=torch.float64, device=s.device)
+    moved = torch.zeros(rows, dtype=torch.bool, device=s.device)
+    for k, (at, n) in enumerate(tiles):
+        g = k & 1
+        if k == 0:
+            m[0] = m[1] = s[:, at:at + min(32, n)].amax(1)                # where a piece starts from
+        p = torch.zeros(rows, 0, dtype=torch.float64, device=s.device)
+        for c in range(at, at + n, 32):
+            x = s[:, c:min(c + 32, at + n)]
+            need = x.amax(1) - m[g] > 8
+            new = torch.where(need, x.amax(1), m[g])
+            p = torch.cat([bf16(p * torch.exp2(m[g] - new)[:, None]), bf16(torch.exp2(x - new[:, None]))], 1)
+            m[g], moved = new, moved | need
+        if k > 0:                                                         # against the one in force after the tile before
+            raised = m[g] - in_force > 8
+            p = torch.where(raised[:, None], p, bf16(p * torch.exp2(m[g] - in_force)[:, None]))
+            o *= torch.where(raised, torch.exp2(in_force - m[g]), 1.0)[:, None]
+            m[g] = torch.where(raised, m[g], in_force)
+        in_force = m[g]
+        o += p @ v[at:at + n]
+    return o / torch.exp2(s - in_force[:, None]).sum(1, keepdim=True), moved
+
+
+@pytest.mark.parametrize("loud,own", [(8, 1), (1, 6)])
+def test_references_that_probabilities_are_rounded_against(loud, own):
+    # Probabilities are rounded to bf16 against a reference: another one rounds others up or down, by 2^-9 of a value that is
+    # many times the root mean square where a row attends to one key.  The reference is the maximum of a piece's first 32
+    # keys, of the causal block to begin with, until a score exceeds it by 2^8.  `loud`: two channels of the documents' keys;
+    # `own`: the query block's keys from the 40th on, so that references move in the first tile and the second one starts from
+    # where the first did.  fp32 scores and exponentials put a few probabilities in 2,000 on the other side of a tie (a
+    # twelfth of the rounding error of all); against another reference the results are 1.4 of it apart.
+    q_len, lens = 64, [640, 700, 1024]
+    shape = gen.ModelShape(1, 8, 2, 128, "bf16", 500000.0, 0)
+    wl = gen.make_workload(shape, lens, [[(i, -1) for i in range(3)]], q_len=q_len, seed=29, rebase=False)
+    for pk in wl.packets:
+        x = gen.bf16_bits_to_f32(pk.k)
+        x[..., [5, 77]] *= np.float32(loud)
+        pk.k[:] = gen.to_stored(x, "bf16")
+    x = gen.bf16_bits_to_f32(wl.k_new[0])
+    x[:, 40:] *= np.float32(own)
+    wl.k_new[0][:] = gen.to_stored(x, "bf16")
+    sess = Session(wl)
+    aid, (prefix,) = sess.assemble()
+    sess.ctx.tune(kvp.TUNE_SPLIT_TARGET_CTAS, 2)                          # one pair: units in one piece
+    q, k, v = sess.query_tensors(0)
+    buf = torch.zeros(sess.ctx.partial_bytes(1, q_len) // 4, dtype=torch.float32, device=q.device)
+    sess.ctx.query_prefill(aid, 0, q, k, v, q_len, buf, None, kvp.PARTIAL)
+    assert sess.ctx.status_word() == 0 and sess.ctx.last_launch()["ctas"] == 2
+    o = buf[:4 * 16384].view(2, 2, 32, 128, 4).permute(0, 1, 3, 2, 4).reshape(2, 4 * q_len, 128).double()
+    l = buf[4 * 16384:].view(2, 2, 128, 2)[..., 1].reshape(2, 4 * q_len, 1).double()
+    K, V = (x.double() for x in sess.ctx.export_cache(aid, 0, 0, prefix, q_len))                  # [row][kv head][128]
+    token = torch.arange(4 * q_len, device=q.device) // 4                                         # packed row: token, head in group
+    tiles = [(prefix, q_len)] + [(sum(lens[:i]) + t, min(128, n - t)) for i, n in enumerate(lens) for t in range(0, n, 128)]
+    apart = ideal = some = 0.0
+    for h in range(2):
+        s = q[0, :, 4 * h:4 * h + 4].reshape(-1, 128).double() @ K[:, h].T / math.sqrt(128) / math.log(2)
+        s = s.masked_fill(torch.arange(prefix + q_len, device=q.device) > prefix + token[:, None], -math.inf)
+        rounded, moved = rounded_against_references(s, V[:, h], tiles)
+        apart += float((o[h] / l[h] - rounded).square().sum())
+        ideal += float((rounded - torch.softmax(s * math.log(2), 1) @ V[:, h]).square().sum())
+        some += float(moved.double().mean()) / 2
+    assert (some > 0.2) == (own > 1), some
+    assert apart <= 0.2 ** 2 * ideal, (apart / ideal) ** 0.5
+    sess.close()
+
+
 @pytest.mark.parametrize("q_len", [64, 96, 150, 409])
 def test_either_kernel_on_request(q_len):
     # KVP_TUNE_CTA_PAIRS: off, on again; 96 and 150 tokens (384 and 600 rows) have a narrow unit to one or two wide ones
