@@ -20,7 +20,7 @@
 //                     as large.
 //   warps 8-11        Q producer: counter-rotates this CTA's rows once per document (as in the one-CTA kernel), and appends
 //                     the query block's K/V rows
-//   warp 12           CTA 0 of the pair: MMA issuer for both.  TMEM owner in each.
+//   warp 12           CTA 0 of the pair: MMA issuer for both.  CTA 1: tells it of the Q tiles formed there.  TMEM owner in each.
 //   warp 13           TMA producer of this CTA's halves; its bytes are counted on CTA 0's barriers
 //
 // Barriers that CTA 0's MMA warp waits for live in CTA 0 and are arrived at from both CTAs; those they signal
@@ -41,7 +41,7 @@ constexpr int kSmemBytes = kOffMl + 2048 + 1024;          // + alignment slack
 constexpr uint32_t kColO = 384;                           // S buffer b: columns [128 b, 128 b + 128)
 constexpr uint16_t kBoth = 3;
 
-enum BarIdx { kKvFull = 0, kKvEmpty = kMaxStages, kQFull = 2 * kMaxStages, kQFree = kQFull + 2, kSFull = kQFree + 2, kPFull = kSFull + 3,
+enum BarIdx { kKvFull = 0, kKvEmpty = kMaxStages, kQFull = 2 * kMaxStages, kQPeer = kQFull + 2, kQFree = kQPeer + 2, kSFull = kQFree + 2, kPFull = kSFull + 3,
               kPvDone = kPFull + 3, kOFull = kPvDone + 2, kOFree, kMref, kEnd = kMref + 8, kStart = kEnd + 8, kDrain = kStart + 4,      // Mref, End: [4 * warpgroup + quadrant]; Start: [quadrant]
               kNumBars };
 static_assert(8 * kNumBars <= 504, "barrier block");
@@ -67,8 +67,8 @@ __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 // Every warp arrives at the cluster's barrier once its own part of the set-up is done (warp 0: barriers, warp 12: TMEM) and
 // waits there only when it has looked up its first piece and tile - the producers when they have formed the first Q tile.
-// First scores of a launch, 8.3 us after its entry with all of it in front of the look-ups: 7.0 (pruned documents: 7.9, 6.1;
-// the one-CTA kernel, where the look-ups lie behind one __syncthreads, lost 1 % with the same order).
+// Pruned documents 240 us with all of it in front of the look-ups, so 230, both with Q released by its producers (the one-CTA
+// kernel, where the look-ups lie behind one __syncthreads, lost 1 % with the same order).
 __device__ __forceinline__ void begin(Cta &c)
 {
     __syncwarp();
@@ -76,13 +76,16 @@ __device__ __forceinline__ void begin(Cta &c)
     tc_fence_after();
     c.tmem = ld_shared(c.tmem_slot());
 }
-// What is handed over lies in TMEM, which tcgen05.fence::before_thread_sync orders, or in this CTA's own shared memory (the
-// rotated Q), written back to the tensor core's view by fence.proxy.async: a release to the cluster on top of that waits for
-// everything the SM has in flight, 1,000 cycles and more (per tile, it took half of the softmax warps' time; for Q, the
-// first scores of a launch came 1 us later).
+// For what lies in TMEM, which tcgen05.fence::before_thread_sync orders: a release to the cluster waits for everything the SM
+// has in flight, 1,000 cycles and more per tile (it took half of the softmax warps' time).
 __device__ __forceinline__ void remote_arrive(uint32_t cluster_bar)
 {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
+}
+// For shared memory that this CTA has written: wait_cluster acquires it.
+__device__ __forceinline__ void remote_arrive_release(uint32_t cluster_bar)
+{
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
 }
 
 // the waits of this kernel; one that runs out also raises the other CTA's abort flag
@@ -96,6 +99,20 @@ __device__ __forceinline__ bool wait(const Params &p, const Cta &c, int i, uint3
 {
     if (mbar_try_wait(c.bar(i), parity)) return true;
     return wait_slow(c.bar(i), parity, c.abort_flag(), c.rank, p.status, code);
+}
+// the same, and what the arrives released to the cluster is acquired (a complete phase stays so until this CTA goes on)
+__device__ __forceinline__ bool wait_cluster(const Params &p, const Cta &c, int i, uint32_t parity, int code)
+{
+    if (!wait(p, c, i, parity, code)) return false;
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(c.bar(i)), "r"(parity)
+        : "memory");
+    return ok != 0;
 }
 
 __device__ __forceinline__ void load_3d(uint32_t dst, const CUtensorMap *tm, int x, int y, int z, uint32_t cluster_bar)
@@ -411,7 +428,7 @@ __device__ __forceinline__ void producer_role(const Params &p, Cta &c, const int
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             if (ep == 0) begin(c);                            // (the first tile is formed while barriers and TMEM are set up)
             __syncwarp();
-            if ((t & 31) == 0) remote_arrive(c.lead(kQFull + buf));
+            if ((t & 31) == 0) mbar_arrive(c.bar(kQFull + buf));
             ++ep;
             // the append (as in the one-CTA kernel): the tokens whose first packed row lies in this CTA's rows, behind the
             // piece's first Q tile
@@ -419,6 +436,34 @@ __device__ __forceinline__ void producer_role(const Params &p, Cta &c, const int
         }
     }
     pdl_wait();                                               // (a role that gave up early)
+}
+
+// ---- Q tiles of CTA 1 (its warp 12) ------------------------------------------------------------------------------
+// Their MMAs are issued by a thread of CTA 0, so the tiles are released to the cluster, which takes 1,000 cycles and more: an
+// arrive alone orders this CTA's threads only.  From here 4 x 20 documents of 100-200 tokens take 148 us, pruned documents
+// 215; the producers themselves held up their next tile with it, 169 and 230.
+// `first`: what else this warp has to do, behind the first one.
+template <typename First>
+__device__ __forceinline__ void peer_role(const Params &p, Cta &c, const int lane, const First &first)
+{
+    uint32_t ep = 0;
+    bool ok = true;
+    for (int wi = c.item_begin; wi < c.item_end && ok; ++wi) {
+        const Work w = load_work(p, c.works, wi);
+        for (int k0 = 0; k0 < w.n && ok; k0 += 32) {
+            const int k = k0 + lane;
+            const bool newq = k < w.n && (k == 0 || get_tile(p, w, w.lo + k).rope != get_tile(p, w, w.lo + k - 1).rope);
+            int count = __popc(__ballot_sync(0xffffffffu, newq));
+            if (ep == 0) begin(c);
+            for (; count > 0 && ok; --count) {
+                ok = wait(p, c, kQFull + (ep & 1), (ep >> 1) & 1, 42);
+                ok = __all_sync(0xffffffffu, ok);
+                if (ok && lane == 0) remote_arrive_release(c.lead(kQPeer + (ep & 1)));
+                if (ep == 0) first();
+                ++ep;
+            }
+        }
+    }
 }
 
 // Loads of a piece with n tiles in the order the MMA warp takes them: Q K^T runs three tiles ahead of P V, so
@@ -549,6 +594,7 @@ __device__ __forceinline__ void mma_role(const Params &p, Cta &c)
                 if (newq) {
                     qbuf = ep & 1;
                     if (ok) ok = wait(p, c, kQFull + qbuf, (ep >> 1) & 1, 20);
+                    if (ok) ok = wait_cluster(p, c, kQPeer + qbuf, (ep >> 1) & 1, 21);
                     ++ep;
                 }
             }
@@ -642,7 +688,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap k_pool, const __grid_consta
     if (warp == 0) {
         for (int i = lane; i < kNumBars; i += 32) {
             uint32_t count = 1;
-            if (i >= kQFull && i < kQFree) count = 8;                   // four producer warps of both CTAs
+            if (i >= kQFull && i < kQPeer) count = 4;                   // four producer warps
             else if (i >= kPFull && i < kPvDone) count = 8;             // four softmax warps of both CTAs
             else if (i == kOFree) count = 16;                           // eight softmax warps of both CTAs
             mbar_init(c.bar(i), count);
@@ -679,8 +725,9 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap k_pool, const __grid_consta
         if (c.rank == 0) {
             mma_role(p, c);
         } else {
-            if (LB > 0 && blockIdx.x == 1) store_list<LB>(p, list, lane);
-            begin(c);
+            peer_role(p, c, lane, [&] {
+                if (LB > 0 && blockIdx.x == 1) store_list<LB>(p, list, lane);
+            });
         }
     } else if (warp == 13) {
         tma_role(p, c, lane, &k_pool, &v_pool, &k_ws, &v_ws, &k_new, &v_new);

@@ -417,3 +417,20 @@ def test_assemble_takes_any_pairs_of_numbers():
             ctx.assemble([[(bad, -1)]])
         assert e.value.code == 3
     ctx.close()
+
+
+def test_rotated_queries_are_released_to_the_cluster():
+    # What a thread wrote to its CTA's shared memory is there for a thread of the pair's other CTA only behind a release and
+    # an acquire of cluster scope; a plain arrive has the scope of the CTA.  It serves barriers that hand TMEM over, which
+    # tcgen05's own fences order.  No run can be relied on to show a missing one, so the source is read.
+    src = open(os.path.join(os.path.dirname(kvp.__file__), "csrc", "kvp_attn_pair.cu")).read()
+    body = {name: src[src.index("__forceinline__ %s(" % name):].split("\n}\n")[0] for name in ("void remote_arrive_release", "bool wait_cluster")}
+    assert "mbarrier.arrive.release.cluster.shared::cluster" in body["void remote_arrive_release"]
+    assert ".acquire.cluster." in body["bool wait_cluster"]
+    arrives = set(re.findall(r"(remote_arrive\w*)\(c\.lead\((k\w+)", src))
+    assert {b for f, b in arrives if f == "remote_arrive"} == {"kPFull", "kOFree"}
+    released = {b for f, b in arrives if f == "remote_arrive_release"}
+    waits = set(re.findall(r"(wait\w*)\(p, c, (k\w+)", src))
+    assert released and all({f for f, b in waits if b == r} == {"wait_cluster"} for r in released)
+    # and the producers' own barrier is arrived at and waited for within a CTA
+    assert "mbar_arrive(c.bar(kQFull" in src and ("wait", "kQFull") in waits
