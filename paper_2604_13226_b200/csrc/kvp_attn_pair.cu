@@ -42,7 +42,7 @@ constexpr uint32_t kColO = 384;                           // S buffer b: columns
 constexpr uint16_t kBoth = 3;
 
 enum BarIdx { kKvFull = 0, kKvEmpty = kMaxStages, kQFull = 2 * kMaxStages, kQPeer = kQFull + 2, kQFree = kQPeer + 2, kSFull = kQFree + 2, kPFull = kSFull + 3,
-              kPvDone = kPFull + 3, kOFull = kPvDone + 2, kOFree, kMref, kEnd = kMref + 8, kStart = kEnd + 8, kDrain = kStart + 4,      // Mref, End: [4 * warpgroup + quadrant]; Start: [quadrant]
+              kOFull = kPFull + 3, kOFree, kMref, kEnd = kMref + 8, kStart = kEnd + 8, kDrain = kStart + 4,      // Mref, End: [4 * warpgroup + quadrant]; Start: [quadrant]
               kNumBars };
 static_assert(8 * kNumBars <= 504, "barrier block");
 
@@ -160,6 +160,16 @@ __device__ __forceinline__ uint32_t instr_desc(uint32_t n, uint32_t b_mn_major)
 }
 // N of a tile's Q K^T: its keys rounded up to what M = 256 takes; CTA r holds keys [r N / 2, (r + 1) N / 2)
 __device__ __forceinline__ int qk_n(int n_keys) { return max(32, (n_keys + 31) & ~31); }
+
+// Loads of a piece with n tiles in the order the MMA warp takes them: Q K^T runs three tiles ahead of P V, so
+// K0 K1 K2 V0 K3 V1 K4 ... V(n-1).  Load q is tile r's K (kv = 0) or V (kv = 1).
+__device__ __forceinline__ void load_at(int n, int q, int &r, int &kv)
+{
+    if (q < min(n, 3)) { r = q; kv = 0; }
+    else if (q >= n + max(n - 3, 0)) { r = q - n; kv = 1; }
+    else { kv = (q - 3) & 1 ? 0 : 1; r = (q - 3) / 2 + (kv ? 0 : 3); }
+}
+__device__ __forceinline__ int v_load(int n, int r) { return r < n - 3 ? 3 + 2 * r : n + r; }                // which load is tile r's V
 
 // ---- softmax / epilogue of warpgroup G (tiles G, G + 2, ... of a piece) ------------------------------------
 // Scales P of a tile (n_chunks x 16 columns of packed pairs) by alpha.
@@ -313,9 +323,10 @@ __device__ __forceinline__ void softmax_role(const Params &p, Cta &c, const int 
                     l *= ap;
                     if (!raise) m = mp;
                     if (__any_sync(0xffffffffu, raise)) {
-                        // O is quiet then: P V of tile k waits for this warp (tiles take two barriers in turn: S of this
-                        // tile shows that P V of tile k - 3 is done, so the phase meant here is the next or the last one)
-                        ok = wait(p, c, kPvDone + ((T - 1) & 1), ((T - 1) >> 1) & 1, 37);
+                        // O is quiet once P V of tile k - 1 is done, as the stage of that V being free shows: P V of tile k
+                        // waits for this warp (so the stage, five or nine loads later in use again, is not free once more)
+                        const uint32_t n_stages = p.precise ? 5 : 9, load = 2 * T0 + v_load(n, k - 1);
+                        ok = wait(p, c, kKvEmpty + load % n_stages, (load / n_stages) & 1, 37);
                         ok = __all_sync(0xffffffffu, ok);
                         if (!ok) break;
                         tc_fence_after();
@@ -436,6 +447,9 @@ __device__ __forceinline__ void producer_role(const Params &p, Cta &c, const int
         }
     }
     pdl_wait();                                               // (a role that gave up early)
+    // the last arrive at each of this CTA's barriers, see the teardown (so far every one but the last has been waited for)
+    for (uint32_t buf = 0; buf < 2 && ok; ++buf)
+        if (ep > buf) ok = wait(p, c, kQFree + buf, ((ep - 1 - buf) >> 1) & 1, 41);
 }
 
 // ---- Q tiles of CTA 1 (its warp 12) ------------------------------------------------------------------------------
@@ -464,15 +478,6 @@ __device__ __forceinline__ void peer_role(const Params &p, Cta &c, const int lan
             }
         }
     }
-}
-
-// Loads of a piece with n tiles in the order the MMA warp takes them: Q K^T runs three tiles ahead of P V, so
-// K0 K1 K2 V0 K3 V1 K4 ... V(n-1).  Load q is tile r's K (kv = 0) or V (kv = 1).
-__device__ __forceinline__ void load_at(int n, int q, int &r, int &kv)
-{
-    if (q < min(n, 3)) { r = q; kv = 0; }
-    else if (q >= n + max(n - 3, 0)) { r = q - n; kv = 1; }
-    else { kv = (q - 3) & 1 ? 0 : 1; r = (q - 3) / 2 + (kv ? 0 : 3); }
 }
 
 // ---- TMA producer (whole warp): this CTA's half of every tile ---------------------------------------------------
@@ -531,6 +536,9 @@ __device__ __forceinline__ void tma_role(const Params &p, Cta &c, const int lane
             }
         }
     }
+    // the last arrive at each of this CTA's barriers, see the teardown
+    const uint32_t uses = use + ((uint32_t)lane < stage ? 1 : 0);
+    if (ok && (uint32_t)lane < n_stages && uses > 0) wait(p, c, kKvEmpty + lane, (uses - 1) & 1, 11);
 }
 
 // ---- MMA issuer (one warp of CTA 0, convergent; one elected lane issues) ----------------------------------------
@@ -549,7 +557,6 @@ __device__ __forceinline__ void mma_role(const Params &p, Cta &c)
     uint32_t stage = 0, par = 0;                          // ring position of the next load to be used
     uint32_t bufS = 0;                                    // S buffer of the next Q K^T
     uint32_t bufP = 0, parP = 0;                          // of the next P V
-    uint32_t T = 0;                                       // its running number
     uint32_t ep = 0, pieces = 0;
     bool ok = true;
     auto advance = [&] { if (++stage == n_stages) { stage = 0; par ^= 1; } };
@@ -620,12 +627,10 @@ __device__ __forceinline__ void mma_role(const Params &p, Cta &c)
                             mma_ts(oa, pa + kk * 8, desc64(v_lo + kk * 128, kDescHi), idesc_pv, (k > 3 || kk > 0));
                     }
                     commit_both(c.bar(kKvEmpty + stage));
-                    commit_both(c.bar(kPvDone + (T & 1)));
                     if (k == n + 2) commit_both(c.bar(kOFull));
                 }
                 __syncwarp();
                 advance();
-                ++T;
                 if (++bufP == 3) { bufP = 0; parP ^= 1; }
             }
             if (k < n) {
@@ -689,7 +694,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap k_pool, const __grid_consta
         for (int i = lane; i < kNumBars; i += 32) {
             uint32_t count = 1;
             if (i >= kQFull && i < kQPeer) count = 4;                   // four producer warps
-            else if (i >= kPFull && i < kPvDone) count = 8;             // four softmax warps of both CTAs
+            else if (i >= kPFull && i < kOFull) count = 8;             // four softmax warps of both CTAs
             else if (i == kOFree) count = 16;                           // eight softmax warps of both CTAs
             mbar_init(c.bar(i), count);
         }
@@ -740,8 +745,10 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap k_pool, const __grid_consta
     }
     __syncwarp();
     tc_fence_before();
-    // (relaxed: a release waits for the stores of the partial results, 0.6 us, and nobody here reads them; every arrive at the
-    // other CTA has been waited for there, so none is under way.  Question of 5 x 512 tokens 22.4 -> 22.0 us.)
+    // (Every arrive at this CTA's barriers has been waited for, those of the MMAs' completion (kSFull and kOFull by the softmax,
+    // kKvEmpty and kQFree to their last phase by the roles that use them) and, but for the last piece's kOFree, which is left
+    // out, those of threads of the other CTA: none is under way when this CTA says so.  Relaxed: a release waits for the stores
+    // of the partial results, 0.6 us, and nobody here reads them.  Question of 5 x 512 tokens 22.4 -> 22.0 us.)
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     cluster_wait();
     if (warp == 12) {

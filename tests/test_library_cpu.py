@@ -434,3 +434,14 @@ def test_rotated_queries_are_released_to_the_cluster():
     assert released and all({f for f, b in waits if b == r} == {"wait_cluster"} for r in released)
     # and the producers' own barrier is arrived at and waited for within a CTA
     assert "mbar_arrive(c.bar(kQFull" in src and ("wait", "kQFull") in waits
+
+
+def test_a_cta_of_a_pair_leaves_when_every_arrive_at_its_barriers_is_in():
+    # tcgen05.commit arrives at barriers of both CTAs, so each role that uses such a barrier waits for the last phase too,
+    # although nothing else follows it: an arrive at a CTA that is gone may land in another block's shared memory.
+    src = open(os.path.join(os.path.dirname(kvp.__file__), "csrc", "kvp_attn_pair.cu")).read()
+    role = {name: src[src.index("void %s_role(" % name):].split("\n}\n")[0] for name in ("softmax", "producer", "tma")}
+    behind = {name: role[name][role[name].rindex("\n    }\n"):] for name in ("producer", "tma")}      # what follows the loop over the pieces
+    assert set(re.findall(r"commit_both\(c\.bar\((k\w+)", src)) == {"kSFull", "kOFull", "kKvEmpty", "kQFree"}
+    assert "wait(p, c, kSFull" in role["softmax"] and "wait(p, c, kOFull" in role["softmax"]       # every tile's, every piece's
+    assert "wait(p, c, kQFree" in behind["producer"] and "wait(p, c, kKvEmpty" in behind["tma"]
