@@ -711,7 +711,6 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap k_pool, const __grid_consta
     wait_for_tables<LB>(p, blockIdx.x == 1);
     // from here on: the Q producer, the append and the TMA warp (for anything but pool tiles) wait for the kernel in front;
     // everything else follows from what they deliver
-    // (the work list gives every pair at least one piece)
     const int32_t *cta_begin = p.cta_begin;
     c.works = p.works;
     if (LB > 0) {
@@ -721,6 +720,8 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap k_pool, const __grid_consta
     const int32_t *range = cta_begin + (blockIdx.x >> 1);
     c.item_begin = LB > 0 ? range[0] : __ldcg(range);
     c.item_end = LB > 0 ? range[1] : __ldcg(range + 1);
+    // (the work list gives every pair a piece; without one the roles would not get to it, and warps arrive twice)
+    if (c.item_begin >= c.item_end) begin(c);
 
     if (warp < 8) {
         softmax_role(p, c, warp >> 2, tid & 127);

@@ -445,3 +445,20 @@ def test_a_cta_of_a_pair_leaves_when_every_arrive_at_its_barriers_is_in():
     assert set(re.findall(r"commit_both\(c\.bar\((k\w+)", src)) == {"kSFull", "kOFull", "kKvEmpty", "kQFree"}
     assert "wait(p, c, kSFull" in role["softmax"] and "wait(p, c, kOFull" in role["softmax"]       # every tile's, every piece's
     assert "wait(p, c, kQFree" in behind["producer"] and "wait(p, c, kKvEmpty" in behind["tma"]
+
+
+def test_every_entry_of_a_work_list_has_a_piece():
+    # a CTA (or pair) without one would find nothing to do, but also nothing of what the roles set up with their first piece
+    rng = np.random.default_rng(5)
+    for _ in range(60):
+        n_docs, batch, q_len = int(rng.integers(1, 6)), int(rng.integers(1, 5)), int(rng.integers(1, 700))
+        lens = [int(x) for x in rng.integers(1, 900, n_docs)]
+        ctx = kvp.Context(1, 32, 8, 128, "bf16", max_packets=n_docs, max_batch=batch, max_slots=batch * n_docs, max_prefix_tokens=sum(lens),
+                          max_query_tokens=q_len, max_ws_rows=batch * q_len, device=-1)
+        for n in lens:
+            ctx.register_packet(None, None, n, 0)
+        aid, _ = ctx.assemble([[(int(p), -1) for p in rng.permutation(n_docs)[: rng.integers(1, n_docs + 1)]] for _ in range(batch)], kvp.REBASE)
+        for ctas in (0, 2, 3, 40):
+            ctx.tune(kvp.TUNE_SPLIT_TARGET_CTAS, ctas)
+            cb, works, _, _ = ctx.export_schedule(aid, q_len)
+            assert cb[0] == 0 and cb[-1] == len(works) and np.all(np.diff(cb) > 0) and np.all(works[:, 5] > 0)
