@@ -36,7 +36,8 @@ constexpr int kStageBytes = 16384;                       // half a K or V tile
 constexpr int kMaxStages = 9;
 constexpr int kOffBar = 208 * 1024;
 constexpr int kOffMref = kOffBar + 512;                   // float[128]
-constexpr int kOffMl = kOffMref + 512;                    // float2[2][128]: (m, l) of both warpgroups at the end of a piece
+constexpr int kOffStart = kOffMref + 512;                 // float[128]: the reference a piece starts from
+constexpr int kOffMl = kOffStart + 512;                   // float2[2][128]: (m, l) of both warpgroups at the end of a piece
 constexpr int kSmemBytes = kOffMl + 2048 + 1024;          // + alignment slack
 constexpr uint32_t kColO = 384;                           // S buffer b: columns [128 b, 128 b + 128)
 constexpr uint16_t kBoth = 3;
@@ -269,14 +270,15 @@ __device__ __forceinline__ void softmax_role(const Params &p, Cta &c, const int 
                         if (lim < 32) chunk_mask(v, lim);
                         m = chunk_max(v, m);
                     }
-                    st_shared(mref, __float_as_uint(m));
+                    // (in a place of its own: the second tile may look when this one's reference has moved on)
+                    st_shared(mref + kOffStart - kOffMref, __float_as_uint(m));
                     __syncwarp();
                     if (lead_lane) mbar_arrive(c.bar(kStart + quad));
                 } else {
                     ok = wait(p, c, kStart + quad, phO & 1, 38);
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
-                    m = __uint_as_float(ld_shared(mref));
+                    m = __uint_as_float(ld_shared(mref + kOffStart - kOffMref));
                 }
             }
             // One pass over S, 32 columns at a time, against the reference max this warpgroup knows.  Only if a chunk's max

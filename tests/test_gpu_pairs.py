@@ -167,6 +167,29 @@ def test_references_that_probabilities_are_rounded_against(loud, own):
     sess.close()
 
 
+def test_same_bits_whenever_the_second_tile_arrives():
+    # References move in the first tile of a piece (the query's own keys, from the 40th on).  The second one starts from where
+    # the first did, also when its keys come from memory so late that the first is done by then: after a write of 256 MB,
+    # and with them in L2.
+    shape = gen.ModelShape(1, 32, 8, 128, "bf16", 500000.0, 0)
+    wl = gen.make_workload(shape, [100, 128, 60, 300], [[(p, -1) for p in range(4)]], q_len=64, seed=31)
+    x = gen.bf16_bits_to_f32(wl.k_new[0])
+    x[:, 40:] *= np.float32(6)
+    wl.k_new[0][:] = gen.to_stored(x, "bf16")
+    sess = Session(wl)
+    sess.assemble()
+    sess.ctx.tune(kvp.TUNE_SPLIT_TARGET_CTAS, 8)
+    qkv = sess.query_tensors(0)
+    first, _ = sess.prefill(0, qkv=qkv)
+    assert on_pairs(sess, 64)
+    far = torch.empty(1 << 28, dtype=torch.uint8, device=first.device)
+    for i in range(30):
+        if i % 3:
+            far.fill_(i)
+        assert torch.equal(first, sess.prefill(0, qkv=qkv)[0])
+    sess.close()
+
+
 @pytest.mark.parametrize("q_len", [64, 96, 150, 409])
 def test_either_kernel_on_request(q_len):
     # KVP_TUNE_CTA_PAIRS: off, on again; 96 and 150 tokens (384 and 600 rows) have a narrow unit to one or two wide ones
