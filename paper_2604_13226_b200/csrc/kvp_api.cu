@@ -272,11 +272,11 @@ constexpr int kPieceCostOne = 4, kPieceCostPair = 8;
 constexpr double kTcMinFlops64 = 1.5e8;
 
 // Whether a call runs on CTA pairs (kvp_attn_pair.cu), whose units are 256 rows: a unit that holds no more than 128 costs
-// a pair as much as a full one (2 x 1,600 cycles per key tile; the one-CTA kernel 3,900, and 1,950 for a narrow unit).
+// a pair as much as a full one (2 x 1,600 to 1,800 cycles per key tile; the one-CTA kernel 3,900, and 1,950 for a narrow unit).
 // Times of both over 8 documents of 400-1000 tokens (4 layers, four or eight requests): one wide unit to a narrow one 243 us on
 // single CTAs, 253 on pairs; two 359, 365 (the narrow one nearly full 374, 374); 2.4 517, 489; 2.6 555, 543; three 482, 475;
-// four 600, 582.  24 short ragged batches of 2.3 to 6: 0.79 to 1.08 times as long on pairs, 0.91 on average.  Up to six wide
-// units to a narrow one pairs also have to make up for the CTA that an odd number of them leaves over (three CTAs: two work).
+// four 600, 582.  24 short ragged batches of 2.3 to 6: 0.79 to 1.08 times as long on pairs, 0.91 on average.  That is with 148
+// CTAs; of an odd number pairs leave one over (three: two work), and there the line lies at six to one.
 // With KVP_PARTIAL (`partial`) every unit takes two partial slots, a narrow one too: only as far as there are
 // slots enough for that and for the cuts.
 bool use_pairs(const kvp_ctx *ctx, const kvp_assembly_host &as, int q_len, const int32_t *q_lens, bool partial)
@@ -293,9 +293,8 @@ bool use_pairs(const kvp_ctx *ctx, const kvp_assembly_host &as, int q_len, const
     }
     const int64_t blocks = ((int64_t)sh.group * q_len + 2 * KVP_TILE_ROWS - 1) / (2 * KVP_TILE_ROWS);
     if (partial && 2 * (blocks * as.batch * sh.n_kv_heads + std::min(ctx->sm_count, kMaxCtas)) > KVP_MAX_SPLIT_UNITS) return false;
-    if (wide >= 6 * narrow) return true;
-    const int64_t G = ctx->split_target_ctas > 0 ? std::min(ctx->split_target_ctas, kMaxCtas) : std::min(ctx->sm_count, kMaxCtas);
-    return 2 * wide >= 5 * narrow && (wide + narrow) * 3200 * G <= (wide * 3900 + narrow * 1950) * (G / 2 * 2);
+    const int ctas = std::min(ctx->split_target_ctas > 0 ? ctx->split_target_ctas : ctx->sm_count, kMaxCtas);
+    return ctas % 2 == 0 ? 2 * wide >= 5 * narrow : wide >= 6 * narrow;
 }
 
 // The tiles that the requests of an assembly hold between them (kvp_joint).  Returns whether walking them once saves a

@@ -15,9 +15,10 @@ pytestmark = pytest.mark.gpu
 BF16_MAX_ABS, BF16_MEAN_ABS = 2e-2, 2e-3
 
 
-def run_ragged(wl, q_lens, layer=0, split_ctas=0, pairs=None):
+def run_ragged(wl, q_lens, layer=0, split_ctas=0, pairs=None, allow_pairs=1):
     sess = Session(wl)
     sess.assemble()
+    sess.ctx.tune(kvp.TUNE_CTA_PAIRS, allow_pairs)
     if split_ctas:
         sess.ctx.tune(kvp.TUNE_SPLIT_TARGET_CTAS, split_ctas)
     q, kn, vn = sess.query_tensors(layer)
@@ -49,6 +50,7 @@ def run_ragged(wl, q_lens, layer=0, split_ctas=0, pairs=None):
         with pytest.raises(kvp.KvpError):
             sess.ctx.export_cache(sess.assembly_id, layer, b, sess.prefix_len[b], 1)
     sess.close()
+    return out
 
 
 def ragged_wl(q_len, seed=11, n_layers=1):
@@ -68,11 +70,21 @@ def test_ragged_query_lengths_with_split_units():
     run_ragged(ragged_wl(200), [150, 37, 1, 200], split_ctas=3)
 
 
-# group 4: rows in blocks of 256 and a remainder above 128 (pairs), at most 128 to six full ones (pairs), more of those (not)
+# group 4: rows in blocks of 256 and a remainder above 128 (pairs), at most 128 to six full ones (pairs), more of those (not, with
+# an odd number of CTAs)
 @pytest.mark.parametrize("q_lens,pairs", [([64, 192, 256, 100], True), ([256, 64, 64, 128], True), ([33, 63, 97, 191], True),
                                           ([256, 256, 25, 64], True), ([25, 256, 64, 33], False), ([150, 37, 1, 200], False)])
 def test_ragged_query_lengths_on_cta_pairs(q_lens, pairs):
     run_ragged(ragged_wl(256), q_lens, split_ctas=3, pairs=pairs)
+
+
+# an even number of CTAs: 2.2 wide units to a narrow one (weighted by their keys), 2.5, 3.5, 4.8
+@pytest.mark.parametrize("q_lens,pairs", [([256, 25, 96, 80], False), ([150, 70, 64, 64], True), ([64, 64, 64, 17], True), ([128, 64, 50, 20], True)])
+@pytest.mark.parametrize("ctas", [4, 0])                         # units in a few pieces; cut finely, narrow ones too
+def test_ragged_batches_between_the_kernels(q_lens, pairs, ctas):
+    # which kernel ran shows in the roundings: other bits than without pairs, or the same
+    either, single = (run_ragged(ragged_wl(256), q_lens, split_ctas=ctas, allow_pairs=allow) for allow in (1, 0))
+    assert torch.equal(either, single) == (not pairs)
 
 
 def test_ragged_rejects_bad_lengths_and_other_paths():

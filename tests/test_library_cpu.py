@@ -462,3 +462,20 @@ def test_every_entry_of_a_work_list_has_a_piece():
             ctx.tune(kvp.TUNE_SPLIT_TARGET_CTAS, ctas)
             cb, works, _, _ = ctx.export_schedule(aid, q_len)
             assert cb[0] == 0 and cb[-1] == len(works) and np.all(np.diff(cb) > 0) and np.all(works[:, 5] > 0)
+
+
+@pytest.mark.parametrize("ctas", [0, 148, 4, 147, 3])
+@pytest.mark.parametrize("rows,wide", [(1024, 99), (640, 2), (896, 3), (1408, 5), (1664, 6)])      # wide units to a narrow one
+def test_which_batches_run_on_cta_pairs(ctas, rows, wide):
+    # from five wide units to two narrow ones on, with an odd number of CTAs from six to one on; pairs know no narrow units
+    ctx = kvp.Context(1, 8, 2, 128, "bf16", max_packets=1, max_batch=2, max_slots=2, max_prefix_tokens=3000, max_query_tokens=rows // 4,
+                      max_ws_rows=2 * rows, device=-1)
+    ctx.register_packet(None, None, 3000, 0)
+    ctx.tune(kvp.TUNE_CTA_PAIRS, 1)
+    ctx.tune(kvp.TUNE_CTA_PAIRS, 1)
+    if ctas:
+        ctx.tune(kvp.TUNE_SPLIT_TARGET_CTAS, ctas)
+    aid, _ = ctx.assemble([[(0, -1)]] * 2, kvp.REBASE)
+    cb, works, _, _ = ctx.export_schedule(aid, rows // 4)
+    pairs = wide >= (6 if ctas % 2 else 2.5)
+    assert np.all(works[:, 3] == 0) == pairs and len(cb) - 1 <= (ctas or 148) // (2 if pairs else 1)
