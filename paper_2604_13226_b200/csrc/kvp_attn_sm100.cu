@@ -206,7 +206,7 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
             tiles = p.plan.tiles + w.tile_begin - n_tail;
             n_total = p.q_pos0 + w.q_len;
             const int r = w.row_base + (w.mode == 0 ? S * KVP_TILE_ROWS : 0) + t;
-            idle = D == 128 && !JOINT && p.group * w.q_len > 32 && r - t + (t & ~31) >= p.group * w.q_len;
+            idle = D == 128 && !JOINT && r - t + (t & ~31) >= p.group * w.q_len;
             if (JOINT) {
                 tiles = p.joint_tiles - n_tail;
                 n_per = w.per;
@@ -263,8 +263,8 @@ __device__ __forceinline__ void softmax_role(const Params &p, const Cta &c, cons
             // a short tile (the end of a document, staged adapter rows) needs P only for the columns P V will read (a row that
             // does not see the tile writes P = 0).  Rows that do not exist have Q = 0, so S = 0, and that serves as P; what
             // stands as P of rows that do not hold a joint tile, P V leaves out.  Launches of few rows are at the power limit
-            // like others: 16 tokens over 64 x 2048 (64 rows of 128) 115.4 -> 112.5 us, a decode layer in joint units (32 of
-            // 128) 48.8 -> 47.9.  Not where one warp has all rows (a decode step's 7 rows per unit: 667 -> 672 us with it).
+            // like others: 16 tokens over 64 x 2048 (64 rows of 128) 115.4 -> 112.5 us; 16 decode steps of 4 requests over
+            // documents of their own (4 rows of 128), 4 layers, 2755 -> 2690, of 8 4800 -> 4680 (7 rows of 28/4 heads 1782, 1788).
             const bool none = JOINT ? !__any_sync(0xffffffffu, mine) : idle;
             const int n_ch = none ? 0 : full ? 4 : max(1, (n_keys + 31) >> 5);
 #pragma unroll 1

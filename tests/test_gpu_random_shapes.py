@@ -130,3 +130,20 @@ def test_random_large_shapes_long_queries_pruned_packets_and_three_chunk_continu
         d = (torch.cat(outs, dim=1).float() - ref.float()).abs()
         assert float(d.max()) <= 3e-2 and float(d.mean()) <= 2e-3, (seed, cuts, float(d.max()), float(d.mean()))
     sess.close()
+
+
+@pytest.mark.parametrize("group,q_len", [(4, 1), (7, 1), (4, 8), (7, 5), (4, 24), (1, 97), (4, 33), (7, 23), (4, 63)])
+@pytest.mark.parametrize("flags", [0, kvp.PRECISE_QK])
+def test_warps_without_rows(group, q_len, flags):
+    # 4 to 252 rows per kv head: the last rows of a unit in each warp of a tile, those behind it empty, of either tile; whole
+    # units and pieces of them
+    shape = gen.ModelShape(1, 2 * group, 2, 128, "bf16", 500000.0, 0)
+    wl = gen.make_workload(shape, [300, 1, 700, 129], [[(0, 0), (1, 0), (2, -1)], [(3, 0), (2, 0)]], q_len=q_len, seed=q_len)
+    sess = Session(wl)
+    sess.ctx.tune(kvp.TUNE_CTA_PAIRS, 0)
+    for ctas in (3, 148):
+        sess.ctx.tune(kvp.TUNE_SPLIT_TARGET_CTAS, ctas)
+        sess.assemble()
+        check_attention(wl, sess, flags=flags)
+        assert sess.ctx.last_launch()["kind"] == 1
+    sess.close()
