@@ -1090,8 +1090,10 @@ cudaError_t kvp_launch_merge_list(const kvp_shape &sh, int32_t q_len, int32_t n_
         mo.part_ml = reinterpret_cast<float2 *>((char *)part_out + (uint64_t)part_tiles * (32ull * KVP_TILE_ROWS * 16));
     }
     // whole rows per block when that gives two blocks per SM, else quarter rows (halves with head dimension 64).  Whole rows
-    // take two parts per round trip: units are cut into two or three, and with four parts' registers two blocks fit an SM, so
-    // that 512 took two waves (pruned documents 220.6 -> 218.2 us, ragged batches 818 -> 807, 4 x 10 x 1024 869 -> 864)
+    // take two parts per round trip, which leaves room for three blocks per SM (70 registers), where four leave it for two
+    // (108): pruned documents 220.6 -> 218.2 us, ragged batches 818 -> 807, 4 x 10 x 1024 869 -> 864.  Units are cut into two or
+    // three; a long request among short ones into up to seven, which two serve no worse: 10000 + 5 x 1666 tokens over 8
+    // layers (five parts) 280.4 -> 279.4, 10000 + 6 x 1250 (six) 271.0 -> 267.9, 30000 + 4 x 5000 (seven) 589, 591.
     const bool few = n_merges * (KVP_TILE_ROWS / 32) < 2 * sm_count;
     auto go = [&](auto *kernel, int cs) {
         return launch_pdl(kernel, dim3(n_merges, KVP_TILE_ROWS / 32, cs), 256, 0, st, merges, (int)list_there, q_len, sh.n_q_heads, sh.n_kv_heads,

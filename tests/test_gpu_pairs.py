@@ -190,6 +190,18 @@ def test_same_bits_whenever_the_second_tile_arrives():
     sess.close()
 
 
+def test_a_long_request_among_short_ones():
+    # 90 query tiles to be merged, of which those of the short requests have two parts and those of the long one five
+    shape = gen.ModelShape(1, 32, 8, 128, "bf16", 500000.0, 0)
+    wl = gen.make_workload(shape, [10000] + [1666] * 5, [[(p, -1)] for p in range(6)], q_len=64, seed=41)
+    sess = Session(wl)
+    sess.assemble()
+    check_attention(wl, sess)
+    merges = sess.ctx.export_schedule(sess.assembly_id, 64)[2]
+    assert on_pairs(sess, 64) and len(merges) == 90 and merges[:, 4].min() == 2 and merges[:, 4].max() == 5
+    sess.close()
+
+
 @pytest.mark.parametrize("q_len", [64, 96, 150, 409])
 def test_either_kernel_on_request(q_len):
     # KVP_TUNE_CTA_PAIRS: off, on again; 96 and 150 tokens (384 and 600 rows) have a narrow unit to one or two wide ones
