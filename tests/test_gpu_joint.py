@@ -84,3 +84,30 @@ def test_one_requests_values_stay_with_it(group, steps, bad):
         for b in range(5):
             assert torch.equal(o[b], clean[b]) == (b not in hit), b
             assert bool(torch.isfinite(o[b]).all()) == (b not in hit)
+
+
+@pytest.mark.parametrize("group,batch,steps", [(4, 16, 2), (4, 8, 3), (7, 6, 3)])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), 3e38])
+def test_one_requests_keys_stay_with_it(group, batch, steps, bad):
+    # Scores of rows over documents that their request does not hold are not masked, and warps with no other rows leave them
+    # where P would stand: NaN and infinity among the keys of request 0's own document and of one that it shares with the last
+    # request, which lies in another warp, leave every other request's bits alone.
+    shape = gen.ModelShape(1, 2 * group, 2, 128, "bf16", 500000.0, 0)
+    lens = [4096, 2048, 300, 130]
+    items = [[(0, 0), (1, 0)] for _ in range(batch)]
+    items[0] = [(2, 0), (0, 0), (1, -1), (3, 0)]
+    items[-1] = [(0, -1), (3, 0), (1, 0)]
+    outs = []
+    for poison in (None, 2, 3):
+        wl = gen.make_workload(shape, lens, items, q_len=5 + steps, seed=19)
+        if poison is not None:
+            wl.packets[poison].k[0, 5::7, :, ::3] = gen.to_stored(np.array([bad], dtype=np.float32), "bf16")[0]
+        sess = Session(wl)
+        sess.assemble()
+        outs.append(run_chunks(wl, sess, [(0, 5), (5, 5 + steps - 1), (5 + steps - 1, 5 + steps)])[0][:, 5:])
+        assert joint_used(sess, 2)
+        sess.close()
+    assert torch.isfinite(outs[0]).all()
+    for o, hit in zip(outs[1:], ([0], [0, batch - 1])):
+        for b in range(batch):
+            assert torch.equal(o[b], outs[0][b]) == (b not in hit), b

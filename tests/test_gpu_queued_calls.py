@@ -47,3 +47,34 @@ def test_queued_calls(dtype, d, hq, hkv, q_len, kind):
         runs.append(got)
     assert all(torch.equal(a, b) for a, b in zip(*runs))
     sess.close()
+
+
+@pytest.mark.parametrize("layers,kept", [(1, None), (4, 0.5)])
+def test_queued_calls_with_lists_of_their_own(layers, kept):
+    # Every call has a new work list, in the place of the one before: it comes along with the launch, one warp stores it and the
+    # other CTAs release the merge and the next call before that; the same list again is read where it was stored.  Pairs (64
+    # tokens), single CTAs (20) and one of several row blocks (100), layer after layer; `kept`: a list per layer.
+    shape = gen.ModelShape(layers, 32, 8, 128, "bf16", 10000.0, 0)
+    wl = gen.make_workload(shape, [700, 1024, 300], [[(0, -1), (1, -1)], [(1, -1), (2, -1), (0, -1)]], q_len=100, seed=3)
+    if kept:
+        gen.draw_kept(wl.packets, [kept] * 3, 4, layers, 8)
+    sess = Session(wl)
+    calls = [(l, n, again) for n in (64, 20, 100, 20, 64) for l in range(layers) for again in (0, 1)]
+    qkv = [tuple(t[:, :n].contiguous() for t in sess.query_tensors(l)) for l, n, _ in calls]
+    runs = []
+    for queued in (False, True, True):
+        got = []
+        torch.cuda.synchronize()
+        if queued:
+            torch.cuda._sleep(40_000_000)
+        sess.assemble()
+        for (l, _, _), x in zip(calls, qkv):
+            got += sess.prefill(l, qkv=x)
+            if not queued:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        assert sess.ctx.status_word() == 0
+        runs.append(got)
+    for run in runs[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(runs[0], run))
+    sess.close()
