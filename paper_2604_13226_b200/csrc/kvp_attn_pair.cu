@@ -287,16 +287,12 @@ __device__ __forceinline__ void softmax_role(const Params &p, Cta &c, const int 
 #pragma unroll 1
             for (int ch = 0; ch < n_ch; ++ch) {
                 uint32_t v[32], pk[16];
-                auto load = [&] {
-                    tmem_ld32(s_addr + ch * 32, v);
-                    tc_wait_ld();
-                    landed32(v);
-                    if (lim < ch * 32 + 32) chunk_mask(v, lim - ch * 32);
-                };
-                load();
+                tmem_ld32(s_addr + ch * 32, v);
+                tc_wait_ld();
+                landed32(v);
+                if (lim < ch * 32 + 32) chunk_mask(v, lim - ch * 32);
                 float ls = chunk_exp<false>(v, c2, m * c2, pk);
                 if (__any_sync(0xffffffffu, !(ls <= kJumpSum))) {
-                    load();                               // this chunk's scores again (P so far lies below them)
                     const float cm = chunk_max(v, -INFINITY);
                     const bool need = (cm - m) * c2 > 8.0f;
                     if (__any_sync(0xffffffffu, need)) {
